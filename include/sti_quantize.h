@@ -49,7 +49,7 @@ size_t sti_quantize_workspace_bytes(uint32_t n_units, uint32_t n_weights);
 #define STI_QUANTIZE_SELECT 0
 #define STI_QUANTIZE_SORT 1
 
-/* Quantizes n_units units (one CTA per unit), asynchronously on `stream` (a cudaStream_t,
+/* Quantizes n_units units, asynchronously on `stream` (a cudaStream_t,
  * NULL = default stream) of `device`; the caller's current device is left as it was.  All pointers are
  * device pointers owned by the caller:
  *   w_dev            [n_units][n_weights] fp32, read only, 16-byte aligned

@@ -20,13 +20,23 @@
 //   6. the indexes are packed into the upload format: index i at stream bits [i k, i k + k), LSB first.
 // All decisions that yield integers (outlier test, sort order, cluster of a rank, nearest centroid) are taken
 // in fp64 / exact integer arithmetic.  Units are independent: the grid is the number of units.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stddef.h>
 #include <stdint.h>
 
+#include <mutex>
+#include <type_traits>
+
 #include "../../include/sti_quantize.h"
+#include "sti_device.cuh"
 
 namespace {
+
+namespace cg = cooperative_groups;
+using sti::pdl_launch_dependents;
+using sti::pdl_wait;
 
 constexpr int kQThreads = 1024;
 constexpr int kQWarps = kQThreads / 32;
@@ -128,7 +138,8 @@ quantize_units_kernel(const float* w_all, uint32_t n, int bits, uint32_t* codes_
   QuantShared& sm = *reinterpret_cast<QuantShared*>(q_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t unit = blockIdx.x;
-  if (only_marked != nullptr && only_marked[unit] == 0) return;      // the selection kernel has done this unit
+  pdl_wait();                                                         // for the selection kernel's marks
+  if (only_marked[unit] == 0) return;                                 // it has done this unit
   const uint32_t K = 1u << bits;
   const float* w = w_all + static_cast<size_t>(unit) * n;
   uint32_t* codes = codes_all + static_cast<size_t>(unit) * (static_cast<size_t>(n) * bits / 32);
@@ -384,87 +395,137 @@ quantize_units_kernel(const float* w_all, uint32_t n, int bits, uint32_t* codes_
 // ---------------------------------------------------------------------------------------------------------------
 // Selection kernel.  The stable sorted order of the inliers is the lexicographic order of (key, offset) pairs, and
 // cluster c starts at sorted rank floor(c n'/2^k).  So a weight's index is the number of boundary elements (the
-// elements at those ranks, c = 1 .. 2^k - 1) whose pair is not above its own - no sort needed once the boundary
-// elements are known.  They are found in two levels: a histogram of the inliers over kSelBins equal-width value
-// bins between the two outlier thresholds (the bin is a monotone function of the value, so bins partition the
-// sorted order), then, for the few bins that hold a boundary rank, their members are gathered and the member with
-// the wanted number of smaller pairs is picked by counting.  One CTA per unit; every warp owns one contiguous
-// 1/32 of the unit in all passes (a lane reads four consecutive weights at a time), so outlier lists come out in
-// ascending offsets from per-warp counts alone.  Cluster sums are plain fp64 additions in a fixed order (every cell
-// of a shared-memory table has one writing thread, the columns are then added in a fixed tree), so the output is
-// deterministic.
+// elements at those ranks, c = 1 .. 2^k - 1) whose pair is not above its own, and nothing has to be sorted but the
+// few weights that share a value bin with a boundary.  A cluster of C CTAs (C = 1 .. 16, chosen by the number of units
+// in the call) works on one unit:
+//   1. fp64 moments, one pass, about a provisional centre;
+//   2. a histogram of the inliers over equal-width value bins between the two outlier thresholds (the bin is a
+//      monotone function of the value, so bins partition the sorted order), one per CTA, added up through
+//      distributed shared memory; its prefix gives the bin and the in-bin rank of every boundary;
+//   3. ONE pass that gives every weight outside the boundary bins its index (bin -> number of boundaries in lower
+//      bins), adds the cluster sums, packs the stream and writes the outlier lists; the weights of boundary bins are
+//      set aside as pairs, their indexes left zero in the stream;
+//   4. a warp per boundary bin ranks its pairs by counting, ORs their indexes into the stream and adds their values to
+//      the sums in rank order; then the centroids and the outliers' indexes.
+// Every warp owns one contiguous run of the unit in all passes (a lane reads four consecutive weights at a time), so
+// outlier lists come out in ascending offsets from per-warp counts alone.  Cluster sums are plain fp64 additions in a
+// fixed order (every cell of a shared-memory table has one writing thread or threads that take turns, columns and
+// CTAs are added in a fixed tree), so the output is deterministic.
 //
-// The fp64 outlier test is taken only where it can matter: a weight whose bin is neither the first nor the last
-// lies at least half a bin (3e-5 of the threshold distance) inside the thresholds, far more than the rounding of
-// the bin's fp32 arithmetic (about 1e-6 bins while |mean| < 10 threshold distances; otherwise every weight is
-// tested), so it is an inlier.
+// The fp64 outlier test is monotone on either side of the mean, so it is taken once per unit, to find the smallest and
+// the largest fp32 value that pass it; a weight is then an inlier if it lies between these two.
+//
+// Two CTAs of 512 threads share an SM: while one waits at a cluster barrier or for memory the other has the pipes.
+//
+// Bound: with few units the chain of seven cluster barriers and the table passes between them (half of the 31 us that
+// 12 units of 196,608 weights take at 4 bits; one CTA of 1024 threads per unit and five passes took 126 us); with many
+// units shared memory - the histogram's atomics, about 5 cycles for a warp's 32 weights on an SM, and in the last pass
+// the table lookup and the fp64 read-modify-write of the sums, about 9 (384 units of 524,288 weights at 3 bits: 1055 ->
+// 625 us, 1.4 TB/s of the 6.5 a copy moves; 16 such units at 6 bits, where four lanes take turns at the sums, 435 -> 95).
 
-constexpr int kSelBins = 16384;
-constexpr int kSelMaxSeg = 1024;           // members of one boundary bin the counting selection accepts
+constexpr int kSelThreads = 512;
+constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kSelMaxCluster = 16;
+constexpr int kSelBins = 16384;            // most value bins; half of them for units of at most 2^18 weights
+constexpr int kSelMaxSeg = 1024;           // weights of one boundary bin that are ranked by counting
+constexpr int kSelSmemSeg = 256;           // ... in shared memory; more than that in the workspace
 constexpr int kSelGroups = 4;              // groups of 128 consecutive weights (four per lane) a warp classifies per step
 constexpr int kSelStep = kSelGroups * 128; // weights of one step of one warp
-constexpr int kAccCells = 16384;           // fp64 cells of the cluster-sum table: 2^k clusters x columns
+constexpr int kAccCells = 8192;            // fp64 cells of the cluster-sum table: 2^k clusters x columns
 
 struct SelShared {
-  double red[kQWarps];
-  unsigned long long bnd_pair[64];         // (key << 32 | offset) of the element at the boundary rank
-  uint32_t warp_out[kQWarps];              // outliers of each warp's part -> their exclusive prefix
-  uint32_t scan[kQWarps];
-  uint32_t n_out, fallback;
+  double red[2][kSelWarps];
+  double moments[2][kSelMaxCluster][2];    // of every CTA of the cluster: sum and sum of squares (the second set: the repeated pass)
+  double part[kSelMaxCluster][64];         // cluster sums of every CTA
+  double extra_lo[64], extra_hi[64];       // sums of cluster c's weights from the bin of its lower / only of its upper boundary
+  uint32_t warp_out[kSelWarps];            // outliers of each warp's run -> their exclusive prefix
+  uint32_t warp_in[kSelWarps];             // inliers in each warp's run of bins -> their exclusive prefix
+  uint32_t cta_out[kSelMaxCluster], range_in[kSelMaxCluster];   // of every CTA: outliers found, inliers in its range of bins
   uint32_t bounds[65];
-  uint32_t bnd_bin[64], bnd_rho[64], seg_start[64], seg_len[64], seg_fill[64];
+  uint32_t bnd_bin[64], bnd_rho[64], seg_len[64];   // of boundary c: its bin, its rank in the bin, the bin's population
+  uint32_t seg_start[64];                  // where the pairs of the bin that boundary c is the first of begin
+  uint32_t seg_fill[64];                   // next free place of this CTA in that list
+  uint32_t longest;
   float cents[64];
-  uint8_t binfo[kSelBins];                 // boundaries in lower bins (6 bits) | 0x80 when the bin holds a boundary rank
-  alignas(16) uint32_t stage[kQWarps][kSelStep / 4];   // a step's indexes of one warp, a byte each, in element order
-  union {
-    uint32_t hist[kSelBins];               // first the inlier histogram, in place its exclusive prefix
+  alignas(16) uint8_t binfo[kSelBins];     // boundaries in lower bins (6 bits) | 0x80: holds a boundary
+  alignas(16) uint32_t stage[kSelWarps][2 * 128 * 6 / 32];       // the packed indexes of two groups
+  union alignas(16) {
+    uint32_t hist[kSelBins];               // this CTA's inlier histogram; in its own range of bins the cluster's, then its prefix
     double acc[kAccCells];                 // later the cluster sums
+    unsigned long long pairs[kSelWarps][2][kSelSmemSeg];         // and last the boundary bins: as gathered, in order
   } u;
 };
-static_assert(offsetof(SelShared, stage) % 16 == 0 && offsetof(SelShared, u) % 8 == 0 && offsetof(SelShared, bnd_pair) % 8 == 0,
-              "vector and 64-bit accesses into the shared layout");
-static_assert(sizeof(SelShared) <= 227 * 1024, "shared memory of one CTA");
+static_assert(2 * (sizeof(SelShared) + 1024) <= 228 * 1024, "two CTAs on an SM");
 
-// Nearest integer of x inv_w + off, clamped to the bins: monotone in x, and no conversion instructions (a float in
-// [0, 2^23) plus 2^23 has its integer value in the low mantissa bits).  NaN goes to bin 0.
-__device__ __forceinline__ int value_bin(float x, float inv_w, float off) {
-  const float t = fminf(fmaxf(fmaf(x, inv_w, off), 0.f), static_cast<float>(kSelBins - 1));
-  return __float_as_int(t + 8388608.0f) - 0x4B000000;
-}
-__device__ __forceinline__ bool edge_bin(int b) { return static_cast<unsigned>(b - 1) >= static_cast<unsigned>(kSelBins - 2); }
+constexpr uint32_t kInfoBoundary = 0x80u;
 
-struct SelUnit {                           // what every pass needs to classify a weight
-  double mu, inv2var, c0;
-  float inv_w, off;
-  bool test_all;                           // the bins' arithmetic is too coarse to clear weights of inner bins
-  // bins of the lane's four weights; bit j of the result: weight j is an outlier
-  __device__ __forceinline__ uint32_t classify(const float4& x, int (&b)[4]) const {
-    b[0] = value_bin(x.x, inv_w, off); b[1] = value_bin(x.y, inv_w, off);
-    b[2] = value_bin(x.z, inv_w, off); b[3] = value_bin(x.w, inv_w, off);
-    uint32_t om = 0;
-    if (test_all || edge_bin(b[0]) || edge_bin(b[1]) || edge_bin(b[2]) || edge_bin(b[3])) {
-      const float v[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if ((test_all || edge_bin(b[j])) && is_outlier(v[j], mu, inv2var, c0)) om |= 1u << j;
-    }
-    return om;
-  }
+// What classifies a weight of a unit.
+struct SelUnit {
+  float least, most;                       // the inliers' range
+  float inv, off, last;                    // place of a value between the thresholds: 0 .. 1; the last bin's number
+  __device__ __forceinline__ bool inlier(float x) const { return x >= least && x <= most; }
+  // 2^23 + bin: the nearest integer of a clamped value in [0, last], monotone in x.  NaN goes to bin 0.
+  __device__ __forceinline__ float place(float x) const { return fmaf(__saturatef(fmaf(x, inv, off)), last, 8388608.0f); }
 };
+__device__ __forceinline__ uint32_t bin_of(float place) { return static_cast<uint32_t>(__float_as_int(place) - 0x4B000000); }
 
 __device__ __forceinline__ float4 load4(const float* w, uint32_t i, uint32_t n) {
   return i < n ? *reinterpret_cast<const float4*>(w + i) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
+// Sum and sum of squares of x - shift over the cluster, in fp64 and in a fixed order.
+__device__ __forceinline__ void cluster_moments(cg::cluster_group& cluster, SelShared& sm, int set, const float* w, uint32_t n,
+                                                uint32_t base, uint32_t part, double shift, int tid, double& sum, double& squares) {
+  const int lane = tid & 31, warp = tid >> 5;
+  double s[2] = {0.0, 0.0}, q[2] = {0.0, 0.0};
+  float4 next[kSelGroups];
+#pragma unroll
+  for (int u = 0; u < kSelGroups; ++u) next[u] = load4(w, base + u * 128u, n);
+  for (uint32_t e0 = 0; e0 < part; e0 += kSelStep) {
+    float4 x[kSelGroups];
+#pragma unroll
+    for (int u = 0; u < kSelGroups; ++u) {
+      x[u] = next[u];
+      if (e0 + kSelStep < part) next[u] = load4(w, base + e0 + kSelStep + u * 128u, n);
+    }
+#pragma unroll
+    for (int u = 0; u < kSelGroups; ++u) {
+      if (base + e0 + u * 128u >= n) continue;
+      const double d0 = static_cast<double>(x[u].x) - shift, d1 = static_cast<double>(x[u].y) - shift;
+      const double d2 = static_cast<double>(x[u].z) - shift, d3 = static_cast<double>(x[u].w) - shift;
+      s[0] += d0 + d1; s[1] += d2 + d3;
+      q[0] = fma(d0, d0, q[0]); q[1] = fma(d1, d1, q[1]);
+      q[0] = fma(d2, d2, q[0]); q[1] = fma(d3, d3, q[1]);
+    }
+  }
+  double a = s[0] + s[1], b = q[0] + q[1];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) { a += __shfl_xor_sync(0xffffffffu, a, o); b += __shfl_xor_sync(0xffffffffu, b, o); }
+  if (lane == 0) { sm.red[0][warp] = a; sm.red[1][warp] = b; }
+  __syncthreads();
+  if (set == 0) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");      // the cluster's CTAs have all started
+  const int n_ctas = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
+  if (tid < n_ctas) {                      // thread t hands this CTA's sums to CTA t
+    a = b = 0.0;
+    for (int v = 0; v < kSelWarps; ++v) { a += sm.red[0][v]; b += sm.red[1][v]; }
+    double* to = cluster.map_shared_rank(&sm.moments[set][rank][0], tid);
+    to[0] = a; to[1] = b;
+  }
+  cluster.sync();
+  sum = squares = 0.0;
+  for (int r = 0; r < n_ctas; ++r) { sum += sm.moments[set][r][0]; squares += sm.moments[set][r][1]; }
+}
+
 template <int BITS>      // the index width is a compile-time constant: the packing and the table addressing unroll to immediates
-__global__ void __launch_bounds__(kQThreads, 1)
-quantize_select_kernel(const float* w_all, uint32_t n, uint32_t* codes_all, float* cent_all, uint32_t* ooff_all,
+__global__ void __launch_bounds__(kSelThreads, 2)
+quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t* codes_all, float* cent_all, uint32_t* ooff_all,
                        float* oval_all, uint32_t max_out, uint32_t* n_out_all, uint8_t* ws_all, size_t ws_per_unit,
                        uint8_t* marks) {
   extern __shared__ __align__(16) uint8_t q_smem[];
   SelShared& sm = *reinterpret_cast<SelShared*>(q_smem);
+  cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const uint32_t unit = blockIdx.x;
+  const uint32_t n_ctas = cluster.num_blocks(), rank = cluster.block_rank(), unit = blockIdx.x / n_ctas;
   constexpr uint32_t bits = BITS, K = 1u << BITS;
   const float* w = w_all + static_cast<size_t>(unit) * n;
   uint32_t* codes = codes_all + static_cast<size_t>(unit) * (static_cast<size_t>(n) * bits / 32);
@@ -473,196 +534,269 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t* codes_all, floa
   float* oval = oval_all + static_cast<size_t>(unit) * max_out;
   unsigned long long* cand = reinterpret_cast<unsigned long long*>(ws_all + static_cast<size_t>(unit) * ws_per_unit);
   const uint32_t lt_mask = (1u << lane) - 1u;
+  pdl_launch_dependents();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");         // waited for before the first remote access
 
-  // ---- 1. Gaussian fit (shared with the sorting kernel, so both take the same outlier decisions)
-  double mu, var;
-  fit_gaussian(w, n, sm.red, tid, mu, var);
-  SelUnit un;
-  un.mu = mu;
-  un.c0 = -0.5 * log(2.0 * 3.14159265358979323846 * var);
-  un.inv2var = 1.0 / (2.0 * var);
+  // the warp's run: whole steps
+  const uint32_t steps = (n + kSelStep - 1u) / kSelStep, n_warps = n_ctas * kSelWarps;
+  const uint32_t part = ((steps + n_warps - 1u) / n_warps) * kSelStep;
+  const uint32_t base = (rank * kSelWarps + static_cast<uint32_t>(warp)) * part + 4u * lane;     // the lane's first weight
+
+  for (uint32_t i = tid; i < n_bins / 4; i += kSelThreads) reinterpret_cast<uint4*>(sm.u.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+
+  // ---- 1. Gaussian fit.  One pass about the mean of 32 weights; should that centre be far off, so that the squares
+  //         cancel, a second one about the mean found.
+  float centre = w[static_cast<size_t>(n / 32u) * lane] * 0.03125f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) centre += __shfl_xor_sync(0xffffffffu, centre, o);
+  const double count = static_cast<double>(n), shift = static_cast<double>(centre);
+  double sum, squares;
+  cluster_moments(cluster, sm, 0, w, n, base, part, shift, tid, sum, squares);
+  double mu = shift + sum / count;
+  double var = squares / count - (sum / count) * (sum / count);
+  if (!((sum / count) * (sum / count) <= 4.0 * var)) {                 // the same in every thread of the cluster
+    cluster_moments(cluster, sm, 1, w, n, base, part, mu, tid, sum, squares);
+    var = squares / count - (sum / count) * (sum / count);
+    mu += sum / count;
+  }
+  const double c0 = -0.5 * log(2.0 * 3.14159265358979323846 * var);
+  const double inv2var = 1.0 / (2.0 * var);
   // inliers satisfy (x - mu)^2 <= 2 var (c0 + 4): the bins span that interval, values outside are clamped
-  const double radius = sqrt(2.0 * var * (un.c0 + 4.0));
-  un.inv_w = static_cast<float>(static_cast<double>(kSelBins - 1) / (2.0 * radius));
-  un.off = -static_cast<float>(mu - radius) * un.inv_w;
-  un.test_all = !(fabs(mu) < 10.0 * radius);
-  if (!(var > 0.0) || !(radius > 0.0) || !(un.inv_w > 0.f) || !(un.inv_w < 3.0e38f) || !(fabsf(un.off) < 3.0e38f)) {
-    if (tid == 0) marks[unit] = 1;                                   // every thread sees the same values: all leave
+  const double radius = sqrt(2.0 * var * (c0 + 4.0));
+  SelUnit un;
+  un.inv = static_cast<float>(1.0 / (2.0 * radius));
+  un.off = -static_cast<float>(mu - radius) * un.inv;
+  un.last = static_cast<float>(n_bins - 1u);
+  if (!(var > 0.0) || !(radius > 0.0) || !(un.inv > 0.f) || !(un.inv < 1.0e34f) || !(fabsf(un.off) < 1.0e34f)) {
+    if (rank == 0 && tid == 0) marks[unit] = 1;                        // every thread of the cluster leaves
     return;
   }
-
-  // the warp's part: whole steps
-  const uint32_t part = (((n + kQWarps - 1u) / kQWarps + kSelStep - 1u) / kSelStep) * kSelStep;
-  const uint32_t base = static_cast<uint32_t>(warp) * part + 4u * lane;     // the lane's first weight
+  {
+    // odd lanes look for the largest inlier, even ones for the smallest: from the rounded threshold towards the mean
+    // while the test calls a value an outlier, then away from it while it does not
+    const float away = (lane & 1) != 0 ? INFINITY : -INFINITY;
+    float t = static_cast<float>((lane & 1) != 0 ? mu + radius : mu - radius);
+    while (is_outlier(t, mu, inv2var, c0)) t = nextafterf(t, -away);
+    for (float further = nextafterf(t, away); fabsf(further) < INFINITY && !is_outlier(further, mu, inv2var, c0); further = nextafterf(t, away)) t = further;
+    un.least = __shfl_sync(0xffffffffu, t, 0);
+    un.most = __shfl_sync(0xffffffffu, t, 1);
+  }
 
   // ---- 2. outliers counted per warp, inliers into the histogram
-  for (int i = tid; i < kSelBins; i += kQThreads) sm.u.hist[i] = 0u;
-  if (tid < 64) { sm.bnd_pair[tid] = ~0ull; sm.seg_fill[tid] = 0u; sm.seg_len[tid] = 0u; sm.seg_start[tid] = 0u; }
-  __syncthreads();
   uint32_t my_out = 0;
+  float4 next[kSelGroups];
+#pragma unroll
+  for (int u = 0; u < kSelGroups; ++u) next[u] = load4(w, base + u * 128u, n);
   for (uint32_t e0 = 0; e0 < part; e0 += kSelStep) {
     float4 x[kSelGroups];
 #pragma unroll
-    for (int u = 0; u < kSelGroups; ++u) x[u] = load4(w, base + e0 + u * 128u, n);
+    for (int u = 0; u < kSelGroups; ++u) {
+      x[u] = next[u];
+      if (e0 + kSelStep < part) next[u] = load4(w, base + e0 + kSelStep + u * 128u, n);
+    }
 #pragma unroll
     for (int u = 0; u < kSelGroups; ++u) {
-      const bool valid = base + e0 + u * 128u < n;
-      int b[4];
-      const uint32_t om = valid ? un.classify(x[u], b) : 0xfu;
-      if (__any_sync(0xffffffffu, valid && om != 0u)) my_out += __reduce_add_sync(0xffffffffu, valid ? __popc(om) : 0u);
-      if (valid) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (!((om >> j) & 1u)) atomicAdd(&sm.u.hist[b[j]], 1u);
-      }
-    }
-  }
-  if (lane == 0) sm.warp_out[warp] = my_out;
-  __syncthreads();
-  if (warp == 0) {
-    const uint32_t mine = sm.warp_out[lane];
-    uint32_t inc = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
-    sm.warp_out[lane] = inc - mine;
-    if (lane == 31) sm.n_out = inc;
-  }
-  // exclusive prefix of the histogram, in place: thread t owns bins 16 t .. 16 t + 15
-  {
-    uint32_t c[16], tot = 0;
-#pragma unroll
-    for (int e = 0; e < 16; ++e) { c[e] = sm.u.hist[16 * tid + e]; tot += c[e]; }
-    uint32_t inc = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
-    if (lane == 31) sm.scan[warp] = inc;
-    __syncthreads();
-    uint32_t before = inc - tot;
-    for (int ww = 0; ww < warp; ++ww) before += sm.scan[ww];
-#pragma unroll
-    for (int e = 0; e < 16; ++e) { sm.u.hist[16 * tid + e] = before; before += c[e]; }
-  }
-  __syncthreads();
-  const uint32_t n_out = sm.n_out, n_in = n - n_out;
-
-  // ---- 3. the boundary ranks: their bin, their rank inside it, the bin's population
-  if (tid <= static_cast<int>(K)) {
-    const uint32_t r = static_cast<uint32_t>(static_cast<uint64_t>(tid) * n_in / K);
-    sm.bounds[tid] = r;
-    if (tid >= 1 && tid < static_cast<int>(K)) {
-      int lo = 0, hi = kSelBins - 1;                                  // the last bin whose prefix is <= r holds rank r
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (sm.u.hist[mid] <= r) lo = mid; else hi = mid - 1;
-      }
-      sm.bnd_bin[tid] = static_cast<uint32_t>(lo);
-      sm.bnd_rho[tid] = r - sm.u.hist[lo];
-      sm.seg_len[tid] = (lo + 1 < kSelBins ? sm.u.hist[lo + 1] : n_in) - sm.u.hist[lo];
-    }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    uint32_t start = 0, longest = 0;
-    for (uint32_t c = 1; c < K; ++c) {
-      if (c == 1 || sm.bnd_bin[c] != sm.bnd_bin[c - 1]) {             // the first boundary of a bin owns its member list
-        sm.seg_start[c] = start;
-        start += sm.seg_len[c];
-        longest = longest > sm.seg_len[c] ? longest : sm.seg_len[c];
-      } else {
-        sm.seg_start[c] = sm.seg_start[c - 1];
-      }
-    }
-    sm.fallback = longest > static_cast<uint32_t>(kSelMaxSeg) ? 1u : 0u;
-  }
-  __syncthreads();
-  if (sm.fallback) {
-    if (tid == 0) marks[unit] = 1;
-    return;
-  }
-  for (int b = tid; b < kSelBins; b += kQThreads) {
-    uint32_t below = 0;                                              // boundaries 1 .. below sit in lower bins (their bins ascend)
-    for (uint32_t step = K >> 1; step > 0; step >>= 1)
-      if (below + step < K && sm.bnd_bin[below + step] < static_cast<uint32_t>(b)) below += step;
-    const uint32_t here = (below + 1 < K && sm.bnd_bin[below + 1] == static_cast<uint32_t>(b)) ? 0x80u : 0u;
-    sm.binfo[b] = static_cast<uint8_t>(below | here);
-  }
-  __syncthreads();
-
-  // ---- 4. the members of the boundary bins, as (key, offset) pairs, in any order
-  for (uint32_t e0 = 0; e0 < part; e0 += kSelStep) {
-    float4 x[kSelGroups];
-#pragma unroll
-    for (int u = 0; u < kSelGroups; ++u) x[u] = load4(w, base + e0 + u * 128u, n);
-#pragma unroll
-    for (int u = 0; u < kSelGroups; ++u) {
-      const uint32_t i0 = base + e0 + u * 128u;
-      if (i0 >= n) continue;
+      if (base + e0 + u * 128u >= n) continue;
       const float v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int b = value_bin(v[j], un.inv_w, un.off);
-        const uint32_t info = sm.binfo[b];
-        if (info & 0x80u) {
-          if ((un.test_all || edge_bin(b)) && is_outlier(v[j], un.mu, un.inv2var, un.c0)) continue;
-          const uint32_t owner = (info & 63u) + 1u;
-          const uint32_t pos = atomicAdd(&sm.seg_fill[owner], 1u);
-          cand[sm.seg_start[owner] + pos] = (static_cast<unsigned long long>(sort_key(v[j])) << 32) | (i0 + j);
-        }
+        if (un.inlier(v[j])) atomicAdd(&sm.u.hist[bin_of(un.place(v[j]))], 1u);
+        else ++my_out;
       }
     }
   }
+  my_out = __reduce_add_sync(0xffffffffu, my_out);
+  if (lane == 0) sm.warp_out[warp] = my_out;
   __syncthreads();
-  // the member with exactly rho smaller members is the boundary element (all pairs are distinct)
-  for (uint32_t c = 1 + warp; c < K; c += kQWarps) {
-    const uint32_t m = sm.seg_len[c], rho = sm.bnd_rho[c];
-    const unsigned long long* seg = cand + sm.seg_start[c];
-    for (uint32_t j = lane; j < m; j += 32) {
-      const unsigned long long pj = seg[j];
-      uint32_t smaller = 0;
-      for (uint32_t t = 0; t < m; ++t) smaller += seg[t] < pj ? 1u : 0u;
-      if (smaller == rho) sm.bnd_pair[c] = pj;
+  if (warp == 0) {
+    const uint32_t mine = lane < kSelWarps ? sm.warp_out[lane] : 0u;
+    uint32_t inc = mine;
+#pragma unroll
+    for (int o = 1; o < kSelWarps; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
+    if (lane < kSelWarps) sm.warp_out[lane] = inc - mine;
+    const uint32_t total = __shfl_sync(0xffffffffu, inc, kSelWarps - 1);
+    if (lane < static_cast<int>(n_ctas)) *cluster.map_shared_rank(&sm.cta_out[rank], lane) = total;
+  }
+  cluster.sync();
+
+  // the cluster's histogram: CTA r adds up range r of the bins, in its own copy, and forms the prefix inside each warp's
+  // run of it
+  const uint32_t range = n_bins / n_ctas, range0 = rank * range, run = range / kSelWarps;
+  {
+    uint32_t* mine = sm.u.hist + range0 + warp * run;
+    for (uint32_t i = 4 * lane; i < run; i += 128) {                   // 32 bins or more
+      uint4 t = *reinterpret_cast<const uint4*>(mine + i);
+      for (uint32_t q0 = 1; q0 < n_ctas; q0 += 7) {                    // seven CTAs' counts in flight together
+        uint4 r[7];
+#pragma unroll
+        for (uint32_t q = 0; q < 7; ++q)
+          r[q] = q0 + q < n_ctas ? *cluster.map_shared_rank(reinterpret_cast<const uint4*>(mine + i), (rank + q0 + q) & (n_ctas - 1u))
+                                 : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (uint32_t q = 0; q < 7; ++q) { t.x += r[q].x; t.y += r[q].y; t.z += r[q].z; t.w += r[q].w; }
+      }
+      *reinterpret_cast<uint4*>(mine + i) = t;
+    }
+    __syncwarp();
+    uint32_t before = 0;
+    for (uint32_t i = lane; i < run; i += 32) {
+      const uint32_t t = mine[i];
+      uint32_t inc = t;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const uint32_t s = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += s; }
+      mine[i] = before + inc - t;
+      before += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    if (lane == 0) sm.warp_in[warp] = before;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t mine = lane < kSelWarps ? sm.warp_in[lane] : 0u;
+    uint32_t inc = mine;
+#pragma unroll
+    for (int o = 1; o < kSelWarps; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
+    if (lane < kSelWarps) sm.warp_in[lane] = inc - mine;
+    const uint32_t total = __shfl_sync(0xffffffffu, inc, kSelWarps - 1);
+    if (lane < static_cast<int>(n_ctas)) *cluster.map_shared_rank(&sm.range_in[rank], lane) = total;
+  }
+  cluster.sync();
+
+  // ---- the boundary ranks: the CTA whose range holds one finds its bin and tells the others
+  uint32_t n_out = 0, out_before = 0, in_before = 0;
+  for (uint32_t r = 0; r < n_ctas; ++r) {
+    if (r < rank) { out_before += sm.cta_out[r]; in_before += sm.range_in[r]; }
+    n_out += sm.cta_out[r];
+  }
+  const uint32_t n_in = n - n_out;
+  if (tid <= static_cast<int>(K)) {
+    const uint32_t r = static_cast<uint32_t>(static_cast<uint64_t>(tid) * n_in / K);
+    sm.bounds[tid] = r;
+    if (tid >= 1 && tid < static_cast<int>(K) && r >= in_before && r - in_before < sm.range_in[rank]) {
+      const uint32_t at = r - in_before;
+      uint32_t v = 0;                                                  // the last run, then bin, whose prefix is <= the rank holds it
+      for (uint32_t step = kSelWarps / 2; step > 0; step >>= 1) if (sm.warp_in[v + step] <= at) v += step;
+      const uint32_t* bins = sm.u.hist + range0 + v * run;
+      const uint32_t in_run = at - sm.warp_in[v];
+      uint32_t b = 0;
+      for (uint32_t step = run / 2; step > 0; step >>= 1) if (bins[b + step] <= in_run) b += step;
+      const uint32_t run_end = (v + 1 < kSelWarps ? sm.warp_in[v + 1] : sm.range_in[rank]) - sm.warp_in[v];
+      const uint32_t len = (b + 1 < run ? bins[b + 1] : run_end) - bins[b];
+      for (uint32_t q = 0; q < n_ctas; ++q) {
+        *cluster.map_shared_rank(&sm.bnd_bin[tid], q) = range0 + v * run + b;
+        *cluster.map_shared_rank(&sm.bnd_rho[tid], q) = in_run - bins[b];
+        *cluster.map_shared_rank(&sm.seg_len[tid], q) = len;
+      }
     }
   }
-  for (int i = tid; i < kAccCells; i += kQThreads) sm.u.acc[i] = 0.0;
+  cluster.sync();
+
+  // lists of the boundary bins' pairs: the first boundary of a bin owns its list, in which the CTAs' pairs follow one another
+  auto owns = [&](uint32_t c) { return c == 1u || sm.bnd_bin[c] != sm.bnd_bin[c - 1]; };
+  if (warp == kSelWarps - 1) {
+    uint32_t start = 0, longest = 0;
+    for (uint32_t c0 = 0; c0 < K; c0 += 32) {
+      const uint32_t c = c0 + lane;
+      const uint32_t len = c >= 1u && c < K && owns(c) ? sm.seg_len[c] : 0u;
+      uint32_t inc = len;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
+      if (c < K) sm.seg_start[c] = start + inc - len;
+      start += __shfl_sync(0xffffffffu, inc, 31);
+      longest = max(longest, __reduce_max_sync(0xffffffffu, len));
+    }
+    if (lane == 0) sm.longest = longest;
+  }
+  uint32_t fill = 0;                                                   // what the CTAs before this one put into boundary tid's bin
+  if (tid >= 1 && tid < static_cast<int>(K) && owns(tid)) {
+    const uint32_t b = sm.bnd_bin[tid], holder = b / range;            // the holder's own count made way for the cluster's
+    uint32_t others = 0, t[kSelMaxCluster];
+#pragma unroll
+    for (uint32_t r = 0; r < kSelMaxCluster; ++r)                      // all in flight together
+      t[r] = r < n_ctas && r != holder ? *cluster.map_shared_rank(&sm.u.hist[b], r) : 0u;
+#pragma unroll
+    for (uint32_t r = 0; r < kSelMaxCluster; ++r) {
+      others += t[r];
+      if (r < rank) fill += t[r];
+    }
+    if (holder < rank) fill += sm.seg_len[tid] - others;
+  }
+  for (uint32_t i = tid; i < n_bins / 16; i += kSelThreads) {          // sixteen bins a thread
+    uint32_t below = 0, packed[4];                                     // boundaries 1 .. below sit in lower bins (their bins ascend)
+#pragma unroll
+    for (uint32_t step = K >> 1; step > 0; step >>= 1)
+      if (sm.bnd_bin[below + step] < 16u * i) below += step;
+    uint32_t next = below + 1 < K ? sm.bnd_bin[below + 1] : 0xffffffffu;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      packed[q] = 0;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const uint32_t b = 16u * i + 4 * q + e;
+        while (next < b) { ++below; next = below + 1 < K ? sm.bnd_bin[below + 1] : 0xffffffffu; }
+        packed[q] |= (below | (next == b ? kInfoBoundary : 0u)) << (8 * e);
+      }
+    }
+    reinterpret_cast<uint4*>(sm.binfo)[i] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+  }
+  cluster.sync();                                                      // nobody looks at another CTA's histogram any more
+  if (sm.longest > static_cast<uint32_t>(kSelMaxSeg)) {
+    if (rank == 0 && tid == 0) marks[unit] = 1;
+    return;
+  }
+  if (tid < static_cast<int>(K)) sm.seg_fill[tid] = sm.seg_start[tid] + fill;
+  for (int i = tid; i < kAccCells / 2; i += kSelThreads) reinterpret_cast<uint4*>(sm.u.acc)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid < 64) sm.extra_lo[tid] = sm.extra_hi[tid] = 0.0;
   __syncthreads();
 
-  // ---- 5. indexes, outlier lists, cluster sums, the packed stream
-  // The cluster-sum table has one column per `share` neighbouring lanes (1, 2 or 4: 2^k columns of 1024 cells do not
+  // ---- 3. indexes, outlier lists, cluster sums, the packed stream
+  // The cluster-sum table has one column per `share` neighbouring lanes (1, 2 or 4: 2^k columns of 512 cells do not
   // fit above 16 clusters); the lanes of such a group add one after the other, so every cell sees a fixed order of
-  // additions.
-  constexpr uint32_t acc_cols = (kAccCells >> BITS) < kQThreads ? (kAccCells >> BITS) : kQThreads;
-  constexpr uint32_t share = kQThreads / acc_cols;
-  const uint32_t col = static_cast<uint32_t>(tid) / share;
-  uint32_t run_out = sm.warp_out[warp];
-  for (uint32_t e0 = 0; e0 < part; e0 += kSelStep) {
-    float4 x[kSelGroups];
+  // additions.  A weight without an index yet adds a zero to cluster 0.
+  constexpr uint32_t acc_cols = (kAccCells >> BITS) < kSelThreads ? (kAccCells >> BITS) : kSelThreads;
+  constexpr uint32_t share = kSelThreads / acc_cols;
+  double* column = sm.u.acc + static_cast<uint32_t>(tid) / share;
+  uint32_t run_out = out_before + sm.warp_out[warp];
+  next[0] = load4(w, base, n);
+  next[1] = load4(w, base + 128u, n);
+  for (uint32_t e0 = 0; e0 < part; e0 += 256u) {
+    if (base - 4u * lane + e0 >= n) break;                             // the whole warp
+    const float4 x[2] = {next[0], next[1]};
+    uint32_t packed[2];
+    next[0] = load4(w, base + e0 + 256u, n);                           // at the end of the run: the next warp's first, unused
+    next[1] = load4(w, base + e0 + 384u, n);
 #pragma unroll
-    for (int u = 0; u < kSelGroups; ++u) x[u] = load4(w, base + e0 + u * 128u, n);
-#pragma unroll
-    for (int u = 0; u < kSelGroups; ++u) {
+    for (int u = 0; u < 2; ++u) {
       const uint32_t i0 = base + e0 + u * 128u;
-      const bool valid = i0 < n;
-      const float v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
-      int b[4];
-      const uint32_t om = valid ? un.classify(x[u], b) : 0u;
-      uint32_t cw = 0xffffffffu;                                     // the four indexes, a byte each; 255 = nothing to add
-      if (valid) {
-        cw = 0u;
+      float v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+      uint32_t code[4], om = 0, flags = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t code = 255u;
-          if (!((om >> j) & 1u)) {
-            const uint32_t info = sm.binfo[b[j]];
-            code = info & 63u;
-            if (info & 0x80u) {
-              const unsigned long long pair = (static_cast<unsigned long long>(sort_key(v[j])) << 32) | (i0 + j);
-              while (code + 1u < K && sm.bnd_pair[code + 1u] <= pair) ++code;
-            }
-          }
-          cw |= code << (8 * j);
-        }
+      for (int j = 0; j < 4; ++j) {
+        code[j] = sm.binfo[bin_of(un.place(v[j]))];
+        flags |= un.inlier(v[j]) ? code[j] : kInfoBoundary;
       }
-      if (__any_sync(0xffffffffu, om != 0u)) {                       // outliers in this group of 128: in ascending offsets
+      if ((flags & kInfoBoundary) != 0u || i0 >= n) {
+        uint32_t later = 0xfu;                                         // weights without an index yet
+        if (i0 < n) {
+          later = 0u;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (!un.inlier(v[j])) om |= 1u << j;
+            else if ((code[j] & kInfoBoundary) != 0u) later |= 1u << j;
+          }
+          for (uint32_t left = later; left != 0u; left &= left - 1u) { // one as a rule
+            const uint32_t j = static_cast<uint32_t>(__ffs(static_cast<int>(left))) - 1u;
+            const float vj = j == 0 ? v[0] : j == 1 ? v[1] : j == 2 ? v[2] : v[3];
+            const uint32_t cj = j == 0 ? code[0] : j == 1 ? code[1] : j == 2 ? code[2] : code[3];
+            const uint32_t pos = atomicAdd(&sm.seg_fill[(cj & 63u) + 1u], 1u);
+            cand[pos] = (static_cast<unsigned long long>(sort_key(vj)) << 32) | (i0 + j);
+          }
+          later |= om;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if ((later >> j) & 1u) { code[j] = 0u; v[j] = 0.f; }
+      }
+      if (__any_sync(0xffffffffu, om != 0u)) {                         // outliers in this group of 128: in ascending offsets
         uint32_t before = 0, total = 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -674,79 +808,154 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t* codes_all, floa
         for (int j = 0; j < 4; ++j) {
           if ((om >> j) & 1u) {
             const uint32_t dst = run_out + before + __popc(om & ((1u << j) - 1u));
-            if (dst < max_out) { ooff[dst] = i0 + j; oval[dst] = v[j]; }
+            if (dst < max_out) { ooff[dst] = i0 + j; oval[dst] = j == 0 ? x[u].x : j == 1 ? x[u].y : j == 2 ? x[u].z : x[u].w; }
           }
         }
         run_out += total;
       }
-      // cluster sums: the lanes that share a column add in turns
+      packed[u] = code[0] | (code[1] << bits) | (code[2] << (2 * bits)) | (code[3] << (3 * bits));
 #pragma unroll
       for (uint32_t q = 0; q < share; ++q) {
-        if ((lane & (share - 1u)) == q) {
+        if (share == 1u || (lane & (share - 1u)) == q) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t code = (cw >> (8 * j)) & 255u;
-            if (code != 255u) sm.u.acc[code * acc_cols + col] += static_cast<double>(v[j]);
-          }
+          for (int j = 0; j < 4; ++j) column[code[j] * acc_cols] += static_cast<double>(v[j]);
         }
         if (share > 1u) __syncwarp();
       }
-      // an outlier's index is set in step 6: its bits stay zero here
-      sm.stage[warp][u * 32 + lane] = cw & ~(((cw & 0x80808080u) >> 7) * 255u);
     }
-    __syncwarp();
-    // 32 consecutive indexes are exactly `bits` words: lane r packs the r-th 32 weights of the step
-    if (lane < kSelStep / 32 && static_cast<uint32_t>(warp) * part + e0 + lane * 32u < n) {
-      const uint4 a = *reinterpret_cast<const uint4*>(&sm.stage[warp][lane * 8]);
-      const uint4 c = *reinterpret_cast<const uint4*>(&sm.stage[warp][lane * 8 + 4]);
-      const uint32_t src[8] = {a.x, a.y, a.z, a.w, c.x, c.y, c.z, c.w};
-      unsigned long long window = 0;
-      uint32_t fill = 0, out_w = ((static_cast<uint32_t>(warp) * part + e0) / 32u + lane) * bits;
+    // The stream: the lanes of a pair exchange so that each has the indexes of eight consecutive weights of one group,
+    // `bits` whole bytes (even lanes of the first group, odd ones of the second); the bytes go through shared memory.
+    uint8_t* stage = reinterpret_cast<uint8_t*>(sm.stage[warp]);
+    {
+      const bool odd = (lane & 1) != 0;
+      const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? packed[0] : packed[1], 1);
+      const uint32_t first = odd ? got : packed[0], second = odd ? packed[1] : got;
+      const uint64_t eight = first | (static_cast<uint64_t>(second) << (4 * bits));
+      uint8_t* to = stage + (lane & 1) * 16u * bits + (static_cast<uint32_t>(lane) >> 1) * bits;
+      if constexpr (BITS == 4) {
+        *reinterpret_cast<uint32_t*>(to) = static_cast<uint32_t>(eight);
+      } else if constexpr (BITS % 2 == 0) {
 #pragma unroll
-      for (int e = 0; e < 32; ++e) {
-        const uint32_t code = (src[e >> 2] >> (8 * (e & 3))) & 255u;
-        window |= static_cast<unsigned long long>(code) << fill;
-        fill += bits;
-        if (fill >= 32u) {
-          codes[out_w++] = static_cast<uint32_t>(window);
-          window >>= 32;
-          fill -= 32u;
-        }
+        for (int h = 0; h < BITS / 2; ++h) reinterpret_cast<uint16_t*>(to)[h] = static_cast<uint16_t>(eight >> (16 * h));
+      } else {
+#pragma unroll
+        for (int h = 0; h < BITS; ++h) to[h] = static_cast<uint8_t>(eight >> (8 * h));
       }
     }
     __syncwarp();
+    const uint32_t word0 = (base - 4u * lane + e0) / 32u * bits, n_words = n / 32u * bits;
+#pragma unroll
+    for (uint32_t i = lane; i < 8u * bits; i += 32)
+      if (word0 + i < n_words) codes[word0 + i] = sm.stage[warp][i];
+    __syncwarp();
   }
   __syncthreads();
-  // centroids: the columns of a cluster added in a fixed order
-  for (uint32_t c = warp; c < K; c += kQWarps) {
+  for (uint32_t c = warp; c < K; c += kSelWarps) {                     // the columns of a cluster in a fixed order
     double acc = 0.0;
     for (uint32_t t = lane; t < acc_cols; t += 32) acc += sm.u.acc[c * acc_cols + t];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) {
-      const uint32_t members = sm.bounds[c + 1] - sm.bounds[c];
-      const float m = members > 0 ? static_cast<float>(acc / static_cast<double>(members)) : 0.f;
-      sm.cents[c] = m;
-      cent[c] = m;
-    }
+    if (lane < static_cast<int>(n_ctas)) *cluster.map_shared_rank(&sm.part[rank][c], lane) = acc;
   }
-  if (tid == 0) { n_out_all[unit] = n_out; marks[unit] = 0; }
+  cluster.sync();                                                      // pairs and streams are complete as well
+
+  // ---- 4. the boundary bins, a warp each: a pair's rank is the number of smaller pairs of its bin (all are distinct)
+  for (uint32_t c = 1u + warp * n_ctas + rank; c < K; c += n_warps) {       // neighbours on different SMs
+    if (!owns(c)) continue;
+    const uint32_t m = sm.seg_len[c], bin = sm.bnd_bin[c];
+    uint32_t last = c;                                                 // the bin's boundaries: c .. last
+    while (last + 1u < K && sm.bnd_bin[last + 1u] == bin) ++last;
+    const unsigned long long* from = cand + sm.seg_start[c];
+    // in order: the second half of the unit's workspace takes what shared memory cannot
+    unsigned long long* sorted = m <= static_cast<uint32_t>(kSelSmemSeg) ? sm.u.pairs[warp][1] : cand + n + sm.seg_start[c];
+    if (m <= static_cast<uint32_t>(kSelSmemSeg)) {
+      for (uint32_t j = lane; j < m; j += 32) sm.u.pairs[warp][0][j] = from[j];
+      if (lane == 0 && (m & 1u) != 0u) sm.u.pairs[warp][0][m] = ~0ull;
+      from = sm.u.pairs[warp][0];
+      __syncwarp();
+    }
+    for (uint32_t j0 = 0; j0 < m; j0 += 128) {
+      unsigned long long mine[4];
+      uint32_t smaller[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) mine[e] = j0 + 32 * e + lane < m ? from[j0 + 32 * e + lane] : 0ull;
+      if (m <= static_cast<uint32_t>(kSelSmemSeg)) {
+        const ulonglong2* two = reinterpret_cast<const ulonglong2*>(sm.u.pairs[warp][0]);
+        auto rank_by_counting = [&](auto lists) {
+#pragma unroll 4
+          for (uint32_t t = 0; t < (m + 1) / 2; ++t) {                 // the list is padded with a largest pair
+            const ulonglong2 other = two[t];
+#pragma unroll
+            for (int e = 0; e < decltype(lists)::value; ++e)
+              smaller[e] += (other.x < mine[e] ? 1u : 0u) + (other.y < mine[e] ? 1u : 0u);
+          }
+        };
+        const uint32_t left = m - j0;
+        if (left <= 32) rank_by_counting(std::integral_constant<int, 1>());
+        else if (left <= 64) rank_by_counting(std::integral_constant<int, 2>());
+        else if (left <= 96) rank_by_counting(std::integral_constant<int, 3>());
+        else rank_by_counting(std::integral_constant<int, 4>());
+      } else {
+        for (uint32_t t = 0; t < m; ++t) {
+          const unsigned long long other = from[t];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) smaller[e] += other < mine[e] ? 1u : 0u;
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (j0 + 32 * e + lane >= m) continue;
+        sorted[smaller[e]] = mine[e];
+        uint32_t code = c - 1u;
+        while (code + 1u <= last && sm.bnd_rho[code + 1u] <= smaller[e]) ++code;
+        const uint64_t bit = (mine[e] & 0xffffffffull) * bits;
+        const uint32_t sh = static_cast<uint32_t>(bit & 31u);
+        atomicOr(&codes[bit >> 5], code << sh);
+        if (sh + bits > 32u) atomicOr(&codes[(bit >> 5) + 1], code >> (32u - sh));
+      }
+    }
+    __syncwarp();
+    for (uint32_t k = c - 1u; k <= last; ++k) {                        // the bin's share of clusters c - 1 .. last
+      const uint32_t lo = k == c - 1u ? 0u : sm.bnd_rho[k], hi = k == last ? m : sm.bnd_rho[k + 1u];
+      double acc = 0.0;
+      for (uint32_t t = lo + lane; t < hi; t += 32) acc += static_cast<double>(key_value(static_cast<uint32_t>(sorted[t] >> 32)));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      double* to = k == c - 1u ? &sm.extra_hi[k] : &sm.extra_lo[k];
+      if (lane < static_cast<int>(n_ctas)) *cluster.map_shared_rank(to, lane) = acc;
+    }
+    __syncwarp();                                                      // the buffers are free for the warp's next bin
+  }
+  cluster.sync();                                                      // the last access to another CTA's shared memory
+  if (tid < static_cast<int>(K)) {
+    double acc = sm.extra_lo[tid] + sm.extra_hi[tid];
+    for (uint32_t r = 0; r < n_ctas; ++r) acc += sm.part[r][tid];
+    const uint32_t members = sm.bounds[tid + 1] - sm.bounds[tid];
+    const float m = members > 0 ? static_cast<float>(acc / static_cast<double>(members)) : 0.f;
+    sm.cents[tid] = m;
+    if (rank == 0) cent[tid] = m;
+  }
+  if (rank == 0 && tid == 0) { n_out_all[unit] = n_out; marks[unit] = 0; }
   __syncthreads();
 
-  // ---- 6. an outlier's slot gets the nearest centroid's index (its bits in the stream are still zero)
-  if (n_out > 0) {
-    const bool listed = n_out <= max_out;                             // else the lists were cut short: scan the unit again
-    const uint32_t count = listed ? n_out : n;
-    for (uint32_t j = tid; j < count; j += kQThreads) {
+  // an outlier's slot gets the nearest centroid's index (its bits in the stream are still zero)
+  const uint32_t my_outs = sm.cta_out[rank];
+  if (my_outs > 0) {
+    const bool listed = out_before + my_outs <= max_out;               // else the list was cut short: this CTA's part again
+    const uint32_t first = listed ? out_before : min(n, rank * kSelWarps * part);
+    const uint32_t end = listed ? out_before + my_outs : min(n, (rank + 1u) * kSelWarps * part);
+    for (uint32_t j = first + tid; j < end; j += kSelThreads) {
       uint32_t i = j;
       float x;
       if (listed) { i = ooff[j]; x = oval[j]; }
-      else { x = w[j]; if (!is_outlier(x, un.mu, un.inv2var, un.c0)) continue; }
+      else { x = w[j]; if (un.inlier(x)) continue; }
+      auto distance = [&](uint32_t c) { return fabs(static_cast<double>(x) - static_cast<double>(sm.cents[c])); };
       uint32_t best = 0;
-      double bd = fabs(static_cast<double>(x) - static_cast<double>(sm.cents[0]));
-      for (uint32_t c = 1; c < K; ++c) {
-        const double dd = fabs(static_cast<double>(x) - static_cast<double>(sm.cents[c]));
-        if (dd < bd) { bd = dd; best = c; }
+      if (n_in >= K) {          // no empty cluster: the centroids ascend between the outliers of either side
+        if (x > un.most) for (best = K - 1u; best > 0u && distance(best - 1u) == distance(K - 1u);) --best;
+      } else {
+        for (uint32_t c = 1; c < K; ++c)
+          if (distance(c) < distance(best)) best = c;
       }
       const uint64_t bit = static_cast<uint64_t>(i) * bits;
       const uint32_t sh = static_cast<uint32_t>(bit & 31u);
@@ -756,28 +965,95 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t* codes_all, floa
   }
 }
 
-template <int BITS>
-bool select_configure_one() {
-  return cudaFuncSetAttribute(quantize_select_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(sizeof(SelShared))) == cudaSuccess;
-}
-bool select_configure(int bits) {
-  switch (bits) {
-    case 2: return select_configure_one<2>();
-    case 3: return select_configure_one<3>();
-    case 4: return select_configure_one<4>();
-    case 5: return select_configure_one<5>();
-    default: return select_configure_one<6>();
+
+// How many CTAs share a unit.  What an SM spends on its CTAs, in thousands of cycles: on a pair of CTAs 0.75 per
+// thousand weights of each and 10 + 1.3 C per CTA for the table passes and barriers of a cluster of C (more CTAs, more
+// remote reads); on a CTA that has the SM to itself 0.84 per thousand weights and 36 + 0.5 C, with nothing to fill its
+// waits.  Summed over the waves of clusters the device holds at a time.  Fitted to calls of 1 to 384 units of 32,768 to
+// 524,288 weights, whose fastest C it picks or comes within 6 % of; e.g. 12 units of 196,608 weights at 4 bits take
+// 107 / 64 / 42 / 32 / 36 us with C = 1 / 2 / 4 / 8 / 16, 384 of 524,288 at 3 bits 627 / 627 / 625 / 786 / 1198.
+uint32_t pick_cluster(uint32_t n_units, uint32_t n, int sm_count, const int (&resident)[5]) {
+  const uint32_t steps = (n + kSelStep - 1u) / kSelStep;
+  uint32_t best = 1;
+  double best_cost = -1.0;
+  for (int e = 0; e < 5; ++e) {
+    const uint32_t c = 1u << e;
+    if (e > 0 && (resident[e] < 1 || steps < c * kSelWarps)) break;    // at least a step for every warp
+    const uint32_t held = resident[e] > 0 ? static_cast<uint32_t>(resident[e]) : 1u;
+    const uint32_t full = (n_units - 1u) / held, last = n_units - full * held;     // full waves, clusters of the last one
+    const double weights = n / 1000.0 / c, paired = 0.75 * weights + 10.0 + 1.3 * c, alone = 0.84 * weights + 36.0 + 0.5 * c;
+    const double cost = 2.0 * full * paired + (last * c <= static_cast<uint32_t>(sm_count) ? alone : 2.0 * paired);
+    if (best_cost < 0.0 || cost < best_cost) { best = c; best_cost = cost; }
   }
+  return best;
 }
+
+// What a device's launches need to know, looked up once per device: the kernels' attributes are set then, too.
+struct QuantDevice {
+  bool ready = false;
+  int sm_count = 0;
+  int resident[5] = {0, 0, 0, 0, 0};       // clusters of 1, 2, 4, 8, 16 selection CTAs the device holds at a time
+};
+constexpr int kQuantMaxDevices = 64;
+
+cudaLaunchConfig_t select_config(uint32_t n_units, uint32_t n_ctas, cudaStream_t cs, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_units * n_ctas);
+  cfg.blockDim = dim3(kSelThreads);
+  cfg.dynamicSmemBytes = sizeof(SelShared);
+  cfg.stream = cs;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = n_ctas; attr->val.clusterDim.y = 1; attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+template <int BITS>
+cudaError_t select_configure_one(QuantDevice* d) {
+  cudaError_t e = cudaFuncSetAttribute(quantize_select_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(sizeof(SelShared)));
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(quantize_select_kernel<BITS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  for (int k = 0; k < 5 && BITS == 2; ++k) {                           // the widths' kernels have the same footprint
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = select_config(1, 1u << k, nullptr, &attr);
+    if (cudaOccupancyMaxActiveClusters(&d->resident[k], quantize_select_kernel<BITS>, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      d->resident[k] = 0;
+    }
+  }
+  return cudaSuccess;
+}
+
+// nullptr: the device cannot run the kernels.  The caller has made `device` current.
+const QuantDevice* quant_device(int device) {
+  static QuantDevice devices[kQuantMaxDevices];
+  static std::mutex lock;
+  if (device >= kQuantMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> hold(lock);
+  QuantDevice& d = devices[device];
+  if (d.ready) return &d;
+  if (cudaDeviceGetAttribute(&d.sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || d.sm_count < 1 ||
+      cudaFuncSetAttribute(quantize_units_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(sizeof(QuantShared))) != cudaSuccess ||
+      select_configure_one<2>(&d) != cudaSuccess || select_configure_one<3>(&d) != cudaSuccess ||
+      select_configure_one<4>(&d) != cudaSuccess || select_configure_one<5>(&d) != cudaSuccess ||
+      select_configure_one<6>(&d) != cudaSuccess)
+    return nullptr;
+  d.ready = true;
+  return &d;
+}
+
 template <typename... Args>
-void launch_select(int bits, uint32_t n_units, cudaStream_t cs, Args... args) {
+cudaError_t launch_select(int bits, const cudaLaunchConfig_t& cfg, Args... args) {
   switch (bits) {
-    case 2: quantize_select_kernel<2><<<n_units, kQThreads, sizeof(SelShared), cs>>>(args...); break;
-    case 3: quantize_select_kernel<3><<<n_units, kQThreads, sizeof(SelShared), cs>>>(args...); break;
-    case 4: quantize_select_kernel<4><<<n_units, kQThreads, sizeof(SelShared), cs>>>(args...); break;
-    case 5: quantize_select_kernel<5><<<n_units, kQThreads, sizeof(SelShared), cs>>>(args...); break;
-    default: quantize_select_kernel<6><<<n_units, kQThreads, sizeof(SelShared), cs>>>(args...); break;
+    case 2: return cudaLaunchKernelEx(&cfg, quantize_select_kernel<2>, args...);
+    case 3: return cudaLaunchKernelEx(&cfg, quantize_select_kernel<3>, args...);
+    case 4: return cudaLaunchKernelEx(&cfg, quantize_select_kernel<4>, args...);
+    case 5: return cudaLaunchKernelEx(&cfg, quantize_select_kernel<5>, args...);
+    default: return cudaLaunchKernelEx(&cfg, quantize_select_kernel<6>, args...);
   }
 }
 
@@ -804,40 +1080,53 @@ sti_status sti_quantize_units_by(int device, void* stream, const float* w_dev, u
     return STI_ERR_SHAPE;
   if (workspace_bytes < sti_quantize_workspace_bytes(n_units, n_weights)) return STI_ERR_SIZE;
   if ((reinterpret_cast<uintptr_t>(workspace_dev) & 15) != 0 || (reinterpret_cast<uintptr_t>(w_dev) & 15) != 0) return STI_ERR_ARG;
-  int n_dev = 0;
-  if (cudaGetDeviceCount(&n_dev) != cudaSuccess || device < 0 || device >= n_dev) {
+  int prev = 0;
+  if (device < 0 || cudaGetDevice(&prev) != cudaSuccess || (prev != device && cudaSetDevice(device) != cudaSuccess)) {
     (void)cudaGetLastError();
     return STI_ERR_CUDA;
   }
-  int prev = 0;
-  if (cudaGetDevice(&prev) != cudaSuccess || cudaSetDevice(device) != cudaSuccess) return STI_ERR_CUDA;
   sti_status st = STI_OK;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   uint8_t* ws = static_cast<uint8_t*>(workspace_dev);
   const size_t per_unit = ws_per_unit_bytes(n_weights);
   uint8_t* marks = ws + static_cast<size_t>(n_units) * per_unit;
-  if (cudaFuncSetAttribute(quantize_units_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(sizeof(QuantShared))) != cudaSuccess ||
-      !select_configure(bits))
+  const QuantDevice* dev = quant_device(device);
+  if (dev == nullptr) {
+    (void)cudaGetLastError();
     st = STI_ERR_CUDA;
+  }
+  // the sorting kernel follows at once (it leaves the units the selection has done) and is launched while the selection
+  // still runs
+  cudaLaunchAttribute early;
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t sort_cfg = {};
+  sort_cfg.gridDim = dim3(n_units);
+  sort_cfg.blockDim = dim3(kQThreads);
+  sort_cfg.dynamicSmemBytes = sizeof(QuantShared);
+  sort_cfg.stream = cs;
   if (st == STI_OK) {
     if (method == STI_QUANTIZE_SELECT) {
-      launch_select(bits, n_units, cs, w_dev, n_weights, codes_dev, centroids_dev, outlier_off_dev, outlier_val_dev,
-                    max_outliers, n_outliers_dev, ws, per_unit, marks);
+      cudaLaunchAttribute attr;
+      const cudaLaunchConfig_t cfg = select_config(n_units, pick_cluster(n_units, n_weights, dev->sm_count, dev->resident), cs, &attr);
+      const uint32_t n_bins = n_weights > (1u << 18) ? kSelBins : kSelBins / 2;      // about a hundred weights in a bin
+      if (launch_select(bits, cfg, w_dev, n_weights, n_bins, codes_dev, centroids_dev, outlier_off_dev, outlier_val_dev,
+                        max_outliers, n_outliers_dev, ws, per_unit, marks) != cudaSuccess)
+        st = STI_ERR_CUDA;
+      sort_cfg.attrs = &early;
+      sort_cfg.numAttrs = 1;
     } else if (cudaMemsetAsync(marks, 1, n_units, cs) != cudaSuccess) {
       st = STI_ERR_CUDA;
     }
   }
-  if (st == STI_OK) {
-    quantize_units_kernel<<<n_units, kQThreads, sizeof(QuantShared), cs>>>(
-        w_dev, n_weights, bits, codes_dev, centroids_dev, outlier_off_dev, outlier_val_dev, max_outliers, n_outliers_dev,
-        ws, per_unit, marks);
-    if (cudaGetLastError() != cudaSuccess) st = STI_ERR_CUDA;
-  }
+  if (st == STI_OK &&
+      cudaLaunchKernelEx(&sort_cfg, quantize_units_kernel, w_dev, n_weights, bits, codes_dev, centroids_dev, outlier_off_dev,
+                         outlier_val_dev, max_outliers, n_outliers_dev, ws, per_unit, static_cast<const uint8_t*>(marks)) != cudaSuccess)
+    st = STI_ERR_CUDA;
   if (st == STI_OK && sorted_units_dev != nullptr &&
       cudaMemcpyAsync(sorted_units_dev, marks, n_units, cudaMemcpyDeviceToDevice, cs) != cudaSuccess)
     st = STI_ERR_CUDA;
-  (void)cudaSetDevice(prev);
+  if (prev != device) (void)cudaSetDevice(prev);
   return st;
 }
 

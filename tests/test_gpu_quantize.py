@@ -145,6 +145,30 @@ def test_selection_is_deterministic():
         assert np.array_equal(x.view(np.uint32) if x.dtype == np.float32 else x, y.view(np.uint32) if y.dtype == np.float32 else y)
 
 
+@pytest.mark.parametrize("n_units,n,bits", [
+    (1, 16384 + 32, 6),          # two CTAs share a unit (a step of 512 weights for each of their warps), ragged end
+    (1, 32768, 5), (1, 65536 + 480, 4), (1, 131072 + 1056, 3), (2, 131072 + 8192, 6),      # four, eight, sixteen
+    (1, (1 << 18), 2), (1, (1 << 18) + 128, 2),      # the line between 8,192 and 16,384 value bins
+    (40, 16384, 3), (80, 33 * 1024, 4)])             # clusters by the dozen
+def test_units_shared_by_a_cluster_of_ctas(n_units, n, bits):
+    rng = np.random.default_rng(n + bits)
+    units = (rng.standard_normal((n_units, n)) * 0.02).astype(np.float32)
+    units[rng.random((n_units, n)) < 0.002] *= 10
+    ref = [Q.quantize_unit(units[u], bits) for u in range(n_units)]
+    assert not _check_one(units, bits, 4096, ref, sti.STI_QUANTIZE_SELECT).any()
+
+
+def test_units_whose_mean_is_far_off():
+    """A mean of many deviations, and a unit whose evenly spaced weights - the fit's provisional centre - are outliers."""
+    rng = np.random.default_rng(8)
+    n = 65536
+    shifted = (rng.standard_normal(n) * 0.001 + 3.0).astype(np.float32)
+    misled = (rng.standard_normal(n) * 0.02).astype(np.float32)
+    misled[:: n // 32] = 25.0
+    for bits in (3, 6):
+        _check(np.stack([shifted, misled]), bits)
+
+
 def test_outlier_lists_shorter_than_the_outliers_found():
     shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=1024, n_ffn_slices=4)
     mats = make_unit_weights(shape, 13, 0, FFN, 1, outlier_stress=0.01)

@@ -53,9 +53,12 @@ struct Unit {
   bool uploaded = false;
   std::vector<uint8_t> codes;          // re-tiled (or raw fp32), until finalize moves it into an arena
   std::vector<float> table;
-  std::vector<uint32_t> out_off;
+  // outliers in the order of the decode tasks (4096 weights each) and inside a task by offset, so that a warp finds its
+  // own in one run: row << 16 | column of the matrix, value, and where each task's run starts
+  std::vector<uint32_t> out_rc;
   std::vector<float> out_val;
-  size_t off_codes = 0, off_table = 0, off_ooff = 0, off_oval = 0, bytes = 0;   // inside the layer part
+  std::vector<uint32_t> task_first;
+  size_t off_codes = 0, off_table = 0, off_orc = 0, off_oval = 0, bytes = 0;   // inside the layer part
   uint8_t* dev = nullptr;              // where the unit's region starts in device memory
   size_t codes_bytes = 0;              // size of the index stream (known even when the bytes are not on the host)
   // Back-to-back executions (Section 3.2): a unit another plan already holds in device memory is taken over with
@@ -68,10 +71,10 @@ struct Unit {
 
 struct GemmTable {
   Job* jobs = nullptr;
-  Seg* segs = nullptr;
+  DecodeTask* tasks = nullptr;
   int n_jobs = 0;
   size_t smem = 0;
-  uint32_t w_bytes = 0, n_stages = 0, bps = 1, k_max = 0, hdr_bytes = 0, seg_stride = 0;
+  uint32_t w_bytes = 0, n_stages = 0, bps = 1, k_max = 0, hdr_bytes = 0, task_stride = 0;
   bool pair_ok = false;                // consecutive jobs can share two-CTA MMAs (64-row tiles, same K range)
   int n_split = 0;
 };
@@ -83,7 +86,7 @@ struct Layer {
   uint8_t* res_dev = nullptr;          // in the preload buffer
   uint8_t* str_host = nullptr;         // in the pinned arena
   int slot = -1;                       // ring slot of the streamed part
-  size_t tables_off = 0, tables_bytes = 0;   // this layer's tile-job descriptors inside the plan's table buffer
+  size_t tables_off = 0, tables_bytes = 0;   // this layer's job and task descriptors inside the plan's table buffer
   GemmTable qkv, o, f1, f2;
   GemmTable f2k;                       // FFN2 again, cut for the K-accumulating kernel (plans made for many tokens only)
   cudaEvent_t ev_loaded = nullptr, ev_done = nullptr, ev_copy_start = nullptr, ev_comp_start = nullptr;
@@ -138,7 +141,7 @@ struct sti_plan {
   uint8_t* pinned = nullptr;   size_t pinned_bytes = 0;
   uint8_t* ring = nullptr;     size_t slot_bytes = 0;      // a slot = its data followed by kGuardBytes of guard pattern
   uint8_t* ring_alloc = nullptr; uint8_t* preload_alloc = nullptr;   // the allocations: a leading guard, then `ring` / `preload`
-  uint8_t* tables = nullptr;   size_t tables_bytes = 0;       // job/segment descriptors
+  uint8_t* tables = nullptr;   size_t tables_bytes = 0;       // job and task descriptors
   std::vector<cudaEvent_t> slot_free, g_slot_free;   // direct launches / graph capture
   cudaEvent_t ev_copy_tail = nullptr, ev_begin = nullptr, ev_end = nullptr, ev_fork = nullptr, g_ev_join = nullptr;
   struct CachedGraph { ForwardKey key; cudaGraphExec_t exec = nullptr; uint64_t launches = 0; uint64_t last_use = 0; };
@@ -155,7 +158,7 @@ struct sti_plan {
   int max_partial = 1;
   float* zero_bias = nullptr;          // all-zero bias vector of sti_gemm_probe (allocated by its first call)
   uint8_t* rate_tables = nullptr;      // every layer's FFN1 tile jobs in one table (sti_decode_rate_probe, built by its first call)
-  int rate_jobs = 0; uint32_t rate_seg_stride = 0; uint64_t rate_packed_bytes = 0;
+  int rate_jobs = 0; uint32_t rate_task_stride = 0; uint64_t rate_packed_bytes = 0;
   unsigned long long* stamps = nullptr;   // [layer][kStampKernels][kStampWords] device, profiling level 3
   bool stamping = false;               // the forward being enqueued writes stamps
   bool overlap = true;                 // false: load every streamed layer, then execute (Load&Exec)
@@ -262,49 +265,97 @@ Unit* find_unit(sti_plan* p, int layer, sti_kind kind, int index) {
   return &v[index];
 }
 
-// Segment for rows [row0, row0 + n_rows) of matrix `m` of `u`.
-Seg make_seg(const sti_ctx* c, const Unit& u, sti_kind kind, int m, uint32_t row0, uint32_t n_rows, uint32_t koff) {
-  int nm;
-  const MatrixInfo* mi = unit_matrices(c, kind, &nm);
-  const int bits = u.cfg.bits;
-  size_t mat_off = 0;
-  for (int i = 0; i < m; ++i) mat_off += matrix_code_bytes(mi[i], bits);
-  Seg s{};
-  s.codes = reinterpret_cast<const uint4*>(u.dev + u.off_codes + mat_off +
-                                           static_cast<size_t>(row0) * mi[m].kc * bits / 8);
-  s.table = reinterpret_cast<const float*>(u.dev + u.off_table);
-  s.flat_base = mi[m].flat_base + row0 * mi[m].kc;
-  const uint32_t flat_end = s.flat_base + n_rows * mi[m].kc;
-  const size_t lo = std::lower_bound(u.out_off.begin(), u.out_off.end(), s.flat_base) - u.out_off.begin();
-  const size_t hi = std::lower_bound(u.out_off.begin(), u.out_off.end(), flat_end) - u.out_off.begin();
-  s.out_off = reinterpret_cast<const uint32_t*>(u.dev + u.off_ooff) + lo;
-  s.out_val = reinterpret_cast<const float*>(u.dev + u.off_oval) + lo;
-  s.n_out = static_cast<uint32_t>(hi - lo);
-  s.bits = bits;
-  s.kc = mi[m].kc;
-  s.koff = koff;
-  return s;
+// Shape of a matrix in decode tasks: 32 rows x 128 columns, 64 x 64 when it has 64 in-features.
+struct TaskGrid {
+  uint32_t rows, cols, per_row;      // of a task; tasks side by side
+};
+TaskGrid task_grid(const MatrixInfo& m) { return m.kc >= 128 ? TaskGrid{32, 128, m.kc / 128} : TaskGrid{64, 64, 1}; }
+
+// Number of tasks in the unit's matrices before matrix `m`.
+uint32_t tasks_before(const MatrixInfo* mi, int m) {
+  uint32_t n = 0;
+  for (int i = 0; i < m; ++i) n += mi[i].rows * mi[i].kc / 4096;
+  return n;
+}
+
+// The unit's outliers (flat offsets, ascending) into task order.
+void order_outliers(const MatrixInfo* mi, int nm, const uint32_t* off, const float* val, size_t n, Unit* u) {
+  const uint32_t n_tasks = tasks_before(mi, nm);
+  std::vector<uint32_t> task_of(n), rc(n);
+  u->task_first.assign(n_tasks + 1, 0);
+  for (size_t i = 0; i < n; ++i) {
+    int m = 0;
+    while (m + 1 < nm && off[i] >= mi[m + 1].flat_base) ++m;
+    const TaskGrid g = task_grid(mi[m]);
+    const uint32_t local = off[i] - mi[m].flat_base, row = local / mi[m].kc, col = local % mi[m].kc;
+    task_of[i] = tasks_before(mi, m) + row / g.rows * g.per_row + col / g.cols;
+    rc[i] = row << 16 | col;
+    ++u->task_first[task_of[i] + 1];
+  }
+  for (uint32_t t = 0; t < n_tasks; ++t) u->task_first[t + 1] += u->task_first[t];
+  u->out_rc.resize(n);
+  u->out_val.resize(n);
+  std::vector<uint32_t> next(u->task_first.begin(), u->task_first.end() - 1);
+  for (size_t i = 0; i < n; ++i) {
+    const uint32_t at = next[task_of[i]]++;
+    u->out_rc[at] = rc[i];
+    u->out_val[at] = val[i];
+  }
 }
 
 struct TableBuilder {
   std::vector<Job> jobs;
-  std::vector<std::vector<Seg>> job_segs;
-  std::vector<Seg> segs;               // filled by finish(): job j's segments start at j * seg_stride
-  uint32_t w_bytes = 0, k_max = 0, seg_stride = 0;
-  void add(Job j, const std::vector<Seg>& ss) {
-    j.n_seg = static_cast<uint32_t>(ss.size());
+  std::vector<std::vector<DecodeTask>> job_tasks;
+  std::vector<DecodeTask> tasks;       // filled by finish(): job j's tasks start at j * task_stride
+  uint32_t w_bytes = 0, k_max = 0, task_stride = 0;
+  void add(Job j) {
     jobs.push_back(j);
-    job_segs.push_back(ss);
+    job_tasks.emplace_back();
     w_bytes = std::max(w_bytes, static_cast<uint32_t>(gemm_weight_bytes(j.n_rows, j.k_total)));
     k_max = std::max(k_max, j.k_total);
-    seg_stride = std::max(seg_stride, j.n_seg);
   }
-  // A fixed stride lets a CTA fetch its job and its segments in the same memory round trip.
+  // Rows [row0, row0 + n_rows) of matrix `m` of `u` go to columns koff .. of the last job's tile.
+  void add_rows(const sti_ctx* c, const Unit& u, sti_kind kind, int m, uint32_t row0, uint32_t n_rows, uint32_t koff) {
+    int nm;
+    const MatrixInfo* mi = unit_matrices(c, kind, &nm);
+    const int bits = u.cfg.bits;
+    size_t mat_off = u.off_codes;
+    for (int i = 0; i < m; ++i) mat_off += matrix_code_bytes(mi[i], bits);
+    const TaskGrid g = task_grid(mi[m]);
+    for (uint32_t r = row0; r < row0 + n_rows; r += g.rows) {
+      for (uint32_t j = 0; j < g.per_row; ++j) {
+        const uint32_t in_matrix = r / g.rows * g.per_row + j, index = tasks_before(mi, m) + in_matrix;
+        DecodeTask t{};
+        size_t at;
+        if (bits == 32) {
+          at = mat_off + (static_cast<size_t>(r) * mi[m].kc + j * g.cols) * 4;
+          t.out_val = mi[m].kc * 4;                         // from row to row
+        } else {
+          at = mat_off + static_cast<size_t>(in_matrix) * 512 * bits;
+          const uint32_t first = u.task_first[index];
+          t.n_out = static_cast<uint16_t>(u.task_first[index + 1] - first);
+          t.table = static_cast<uint32_t>(u.off_table - at);
+          t.out_rc = static_cast<uint32_t>(u.off_orc + 4 * static_cast<size_t>(first) - at);
+          t.out_val = static_cast<uint32_t>(u.off_oval + 4 * static_cast<size_t>(first) - at);
+        }
+        t.codes = u.dev + at;
+        t.bits = static_cast<uint8_t>(bits);
+        t.narrow = g.cols == 64;
+        t.row0 = static_cast<uint16_t>(r - row0);
+        t.kcore0 = static_cast<uint16_t>((koff + j * g.cols) / 8);
+        t.origin = r << 16 | j * g.cols;
+        job_tasks.back().push_back(t);
+      }
+    }
+    jobs.back().n_tasks = static_cast<uint32_t>(job_tasks.back().size());
+    task_stride = std::max(task_stride, jobs.back().n_tasks);
+  }
+  // A fixed stride lets a CTA fetch its job and its tasks in the same memory round trip.
   void finish() {
-    segs.assign(jobs.size() * seg_stride, Seg{});
+    tasks.assign(jobs.size() * task_stride, DecodeTask{});
     for (size_t j = 0; j < jobs.size(); ++j) {
-      jobs[j].seg_begin = static_cast<uint32_t>(j * seg_stride);
-      std::copy(job_segs[j].begin(), job_segs[j].end(), segs.begin() + j * seg_stride);
+      jobs[j].task_begin = static_cast<uint32_t>(j * task_stride);
+      std::copy(job_tasks[j].begin(), job_tasks[j].end(), tasks.begin() + j * task_stride);
     }
   }
 };
@@ -323,7 +374,8 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
         j.n_rows = t.qkv_n; j.k_total = d.hidden; j.x_koff = 0;
         j.out_mat = static_cast<uint32_t>(hi * 3 + which); j.out_col = r0;
         j.bias_off = which * d.n_heads * 64 + h * 64 + static_cast<int>(r0);
-        tb[0].add(j, {make_seg(c, L.attn[h], STI_ATTN, which, r0, t.qkv_n, 0)});
+        tb[0].add(j);
+        tb[0].add_rows(c, L.attn[h], STI_ATTN, which, r0, t.qkv_n, 0);
       }
   }
   // O projection: K is split over groups of kept heads, each group writes its own partial sum
@@ -335,10 +387,8 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
       Job j{};
       j.n_rows = t.o_n; j.k_total = cnt * 64; j.x_koff = first * 64;
       j.out_mat = sp; j.out_col = n0; j.bias_off = -1;
-      std::vector<Seg> ss;
-      for (int i = 0; i < cnt; ++i)
-        ss.push_back(make_seg(c, L.attn[L.kept_heads[first + i]], STI_ATTN, 3, n0, t.o_n, i * 64));
-      tb[1].add(j, ss);
+      tb[1].add(j);
+      for (int i = 0; i < cnt; ++i) tb[1].add_rows(c, L.attn[L.kept_heads[first + i]], STI_ATTN, 3, n0, t.o_n, i * 64);
     }
   }
   // FFN1: one job per (kept slice, row tile); full K
@@ -349,7 +399,8 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
       j.n_rows = t.f1_n; j.k_total = d.hidden; j.x_koff = 0;
       j.out_mat = 0; j.out_col = static_cast<uint32_t>(ji * f + r0);
       j.bias_off = s * static_cast<int>(f) + static_cast<int>(r0);
-      tb[2].add(j, {make_seg(c, L.ffn[s], STI_FFN, 0, r0, t.f1_n, 0)});
+      tb[2].add(j);
+      tb[2].add_rows(c, L.ffn[s], STI_FFN, 0, r0, t.f1_n, 0);
     }
   }
   // FFN2: K split over groups of kept slices
@@ -361,10 +412,8 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
       Job j{};
       j.n_rows = t.f2_n; j.k_total = cnt * f; j.x_koff = first * f;
       j.out_mat = sp; j.out_col = n0; j.bias_off = -1;
-      std::vector<Seg> ss;
-      for (int i = 0; i < cnt; ++i)
-        ss.push_back(make_seg(c, L.ffn[L.kept_slices[first + i]], STI_FFN, 1, n0, t.f2_n, i * f));
-      tb[3].add(j, ss);
+      tb[3].add(j);
+      for (int i = 0; i < cnt; ++i) tb[3].add_rows(c, L.ffn[L.kept_slices[first + i]], STI_FFN, 1, n0, t.f2_n, i * f);
     }
   }
   // FFN2 for the K-accumulating kernel: 64-row tiles, K groups of at most 512 columns, group-major order
@@ -379,10 +428,8 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
         Job j{};
         j.n_rows = 64; j.k_total = cnt * f; j.x_koff = first * f;
         j.out_mat = 0; j.out_col = n0; j.bias_off = -1;
-        std::vector<Seg> ss;
-        for (int i = 0; i < cnt; ++i)
-          ss.push_back(make_seg(c, L.ffn[L.kept_slices[first + i]], STI_FFN, 1, n0, 64, i * f));
-        tb[4].add(j, ss);
+        tb[4].add(j);
+        for (int i = 0; i < cnt; ++i) tb[4].add_rows(c, L.ffn[L.kept_slices[first + i]], STI_FFN, 1, n0, 64, i * f);
       }
     }
   }
@@ -456,7 +503,7 @@ sti_status run_gemm(sti_plan* p, GemmKind kind, const GemmTable& tab, const void
   if (tab.n_jobs == 0) return STI_OK;
   GemmLaunch g{};
   g.stamps = stamps;
-  g.jobs = tab.jobs; g.segs = tab.segs; g.n_jobs = tab.n_jobs; g.m_ctas = m_ctas_for(tab.n_jobs, T, p->tune.cta_budget);
+  g.jobs = tab.jobs; g.tasks = tab.tasks; g.n_jobs = tab.n_jobs; g.m_ctas = m_ctas_for(tab.n_jobs, T, p->tune.cta_budget);
   const int n_mtiles = (T + 127) / 128;
   g.pair = tab.pair_ok && p->tune.pair_min_tiles > 0 && n_mtiles >= p->tune.pair_min_tiles;
   if (force_pair == 0) g.pair = false;
@@ -471,7 +518,7 @@ sti_status run_gemm(sti_plan* p, GemmKind kind, const GemmTable& tab, const void
   if (!make_xmap(&g.xmap, x, ldx, T)) return STI_ERR_CUDA;
   layer_ranges(p, prefetch_layer, g.pf_ptr, g.pf_bytes);
   g.x = x; g.ldx = ldx; g.T = T; g.out = out; g.ldo = ldo; g.bias = bias; g.err = p->ctx->err_dev;
-  g.smem_bytes = tab.smem; g.n_stages = tab.n_stages; g.bps = tab.bps; g.w_bytes = tab.w_bytes; g.hdr_bytes = tab.hdr_bytes; g.seg_stride = tab.seg_stride; g.simt_debug = p->ctx->simt_debug; g.pdl = p->ctx->pdl;
+  g.smem_bytes = tab.smem; g.n_stages = tab.n_stages; g.bps = tab.bps; g.w_bytes = tab.w_bytes; g.hdr_bytes = tab.hdr_bytes; g.task_stride = tab.task_stride; g.simt_debug = p->ctx->simt_debug; g.pdl = p->ctx->pdl;
   CUDA_TRY(launch_gemm(kind, g, p->ctx->compute));
   p->ctx->launches++;
   return STI_OK;
@@ -482,7 +529,7 @@ sti_status run_gemm_kacc(sti_plan* p, const GemmTable& tab, const void* x, int l
                          unsigned long long* stamps) {
   if (tab.n_jobs == 0 || tab.n_split == 0) return STI_ERR_STATE;
   KaccLaunch g{};
-  g.jobs = tab.jobs; g.segs = tab.segs; g.n_groups = tab.n_split; g.n_cols64 = tab.n_jobs / tab.n_split;
+  g.jobs = tab.jobs; g.tasks = tab.tasks; g.n_groups = tab.n_split; g.n_cols64 = tab.n_jobs / tab.n_split;
   const int n_mpairs = ((T + 127) / 128 + 1) / 2;
   g.m_ctas = std::max(1, std::min(n_mpairs, p->tune.cta_budget / g.n_cols64));
   if (!make_xmap(&g.xmap, x, ldx, T)) return STI_ERR_CUDA;
@@ -490,7 +537,7 @@ sti_status run_gemm_kacc(sti_plan* p, const GemmTable& tab, const void* x, int l
   // measured: 32 x 512 tokens (134 MB) 159 -> 149 us per launch, 8,192 tokens (67 MB) 79 -> 81
   g.x = static_cast<size_t>(T) * ldx * 2 > (100u << 20) ? x : nullptr; g.ldx = ldx;
   g.T = T; g.out = out; g.ldo = ldo; g.err = p->ctx->err_dev;
-  g.n_stages = tab.n_stages; g.bps = tab.bps; g.hdr_bytes = tab.hdr_bytes; g.seg_stride = tab.seg_stride; g.k_group = tab.k_max;
+  g.n_stages = tab.n_stages; g.bps = tab.bps; g.hdr_bytes = tab.hdr_bytes; g.task_stride = tab.task_stride; g.k_group = tab.k_max;
   g.pdl = p->ctx->pdl; g.stamps = stamps;
   CUDA_TRY(launch_gemm_kacc(g, p->ctx->compute));
   p->ctx->launches++;
@@ -1042,8 +1089,7 @@ sti_status sti_shard_upload(sti_plan* p, int layer, sti_kind kind, int index, co
   }
   u->table.clear();
   if (bits != 32) u->table.assign(blob->centroids, blob->centroids + (1u << bits));
-  u->out_off.assign(blob->outlier_off, blob->outlier_off + blob->n_outliers);
-  u->out_val.assign(blob->outlier_val, blob->outlier_val + blob->n_outliers);
+  order_outliers(mi, nm, blob->outlier_off, blob->outlier_val, blob->n_outliers, u);
   u->uploaded = true;
   return STI_OK;
 }
@@ -1067,7 +1113,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
       const size_t start = cursor;
       u.off_codes = cursor; cursor += align16(u.codes_bytes);
       u.off_table = cursor; cursor += align16(u.table.size() * 4);
-      u.off_ooff = cursor; cursor += align16(u.out_off.size() * 4);
+      u.off_orc = cursor; cursor += align16(u.out_rc.size() * 4);
       u.off_oval = cursor; cursor += align16(u.out_val.size() * 4);
       u.bytes = cursor - start;
       return true;
@@ -1123,8 +1169,8 @@ sti_status sti_plan_finalize(sti_plan* p) {
       auto at = [&](size_t off) { return u.cfg.resident ? staging.data() + (off - u.off_codes) : L.str_host + off; };
       memcpy(at(u.off_codes), u.codes.data(), u.codes.size());
       if (!u.table.empty()) memcpy(at(u.off_table), u.table.data(), u.table.size() * 4);
-      if (!u.out_off.empty()) {
-        memcpy(at(u.off_ooff), u.out_off.data(), u.out_off.size() * 4);
+      if (!u.out_rc.empty()) {
+        memcpy(at(u.off_orc), u.out_rc.data(), u.out_rc.size() * 4);
         memcpy(at(u.off_oval), u.out_val.data(), u.out_val.size() * 4);
       }
       u.dev = u.cfg.resident ? L.res_dev : p->ring + static_cast<size_t>(L.slot) * p->slot_bytes;
@@ -1141,7 +1187,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
   CUDA_TRY(cudaStreamSynchronize(c->compute));   // adopted units are in place before their source plan may go away
   // 3. tile-job tables
   std::vector<uint8_t> host_tables;
-  struct Fix { GemmTable* t; size_t jobs_off, segs_off; };
+  struct Fix { GemmTable* t; size_t jobs_off, tasks_off; };
   std::vector<Fix> fixes;
   p->max_partial = 1;
   for (auto& L : p->layers) {
@@ -1151,7 +1197,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
     GemmTable* gt[5] = {&L.qkv, &L.o, &L.f1, &L.f2, &L.f2k};
     for (int i = 0; i < 5; ++i) {
       tb[i].finish();
-      gt[i]->seg_stride = tb[i].seg_stride;
+      gt[i]->task_stride = tb[i].task_stride;
       gt[i]->n_jobs = static_cast<int>(tb[i].jobs.size());
       gt[i]->w_bytes = tb[i].w_bytes;
       gt[i]->n_stages = 2; gt[i]->bps = 1;
@@ -1180,9 +1226,9 @@ sti_status sti_plan_finalize(sti_plan* p) {
       fx.jobs_off = align16(host_tables.size());
       host_tables.resize(fx.jobs_off + tb[i].jobs.size() * sizeof(Job));
       if (!tb[i].jobs.empty()) memcpy(host_tables.data() + fx.jobs_off, tb[i].jobs.data(), tb[i].jobs.size() * sizeof(Job));
-      fx.segs_off = align16(host_tables.size());
-      host_tables.resize(fx.segs_off + tb[i].segs.size() * sizeof(Seg));
-      if (!tb[i].segs.empty()) memcpy(host_tables.data() + fx.segs_off, tb[i].segs.data(), tb[i].segs.size() * sizeof(Seg));
+      fx.tasks_off = align16(host_tables.size());
+      host_tables.resize(fx.tasks_off + tb[i].tasks.size() * sizeof(DecodeTask));
+      if (!tb[i].tasks.empty()) memcpy(host_tables.data() + fx.tasks_off, tb[i].tasks.data(), tb[i].tasks.size() * sizeof(DecodeTask));
       fixes.push_back(fx);
     }
     L.tables_bytes = host_tables.size() - L.tables_off;
@@ -1194,7 +1240,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
     CUDA_TRY(cudaMemcpy(p->tables, host_tables.data(), host_tables.size(), cudaMemcpyHostToDevice));
   for (auto& fx : fixes) {
     fx.t->jobs = reinterpret_cast<Job*>(p->tables + fx.jobs_off);
-    fx.t->segs = reinterpret_cast<Seg*>(p->tables + fx.segs_off);
+    fx.t->tasks = reinterpret_cast<DecodeTask*>(p->tables + fx.tasks_off);
   }
   // 4. activation scratch for max_batch * max_seq tokens
   const size_t Tmax = static_cast<size_t>(d.max_batch) * d.max_seq;
@@ -1312,13 +1358,21 @@ sti_status sti_shard_decode(sti_plan* p, int layer, sti_kind kind, int index, in
     if (p->copy_tail_valid) CUDA_TRY(cudaStreamWaitEvent(c->compute, p->ev_copy_tail, 0));
     if ((st = enqueue_layer_copy(p, layer, c->compute)) != STI_OK) return st;
   }
-  const Seg s = make_seg(c, *u, kind, matrix, 0, mi[matrix].rows, 0);
+  size_t mat_off = u->off_codes;
+  for (int i = 0; i < matrix; ++i) mat_off += matrix_code_bytes(mi[i], u->cfg.bits);
   DecodeLaunch dl{};
-  dl.codes = s.codes; dl.table = s.table; dl.out_off = s.out_off; dl.out_val = s.out_val; dl.n_out = s.n_out;
-  dl.flat_base = s.flat_base; dl.bits = s.bits; dl.rows = mi[matrix].rows; dl.kc = mi[matrix].kc;
+  dl.codes = reinterpret_cast<const uint4*>(u->dev + mat_off);
+  dl.bits = u->cfg.bits; dl.rows = mi[matrix].rows; dl.kc = mi[matrix].kc;
+  if (dl.bits != 32) {
+    const uint32_t first = u->task_first[tasks_before(mi, matrix)];
+    dl.table = reinterpret_cast<const float*>(u->dev + u->off_table);
+    dl.out_rc = reinterpret_cast<const uint32_t*>(u->dev + u->off_orc) + first;
+    dl.out_val = reinterpret_cast<const float*>(u->dev + u->off_oval) + first;
+    dl.n_out = u->task_first[tasks_before(mi, matrix + 1)] - first;
+  }
   dl.w = w_dev; dl.codes_out = codes_dev; dl.wbf16 = wbf16_dev;
   CUDA_TRY(launch_decode(dl, c->compute));
-  c->launches += (s.bits == 32 || s.n_out == 0) ? 1 : 2;
+  c->launches += dl.n_out == 0 ? 1 : 2;
   if (!u->cfg.resident) CUDA_TRY(cudaEventRecord(p->slot_free[L.slot], c->compute));
   return STI_OK;
 }
@@ -1385,39 +1439,39 @@ sti_status sti_decode_rate_probe(sti_plan* p, const void* x_bf16_dev, int tokens
   if (!p->rate_tables) {
     // one table with the FFN1 tile jobs of all layers; layer l's tiles write output columns l * ffn + ...
     std::vector<Job> jobs;
-    std::vector<Seg> segs;
+    std::vector<DecodeTask> tasks;
     uint32_t stride = 0;
-    for (auto& L : p->layers) stride = std::max(stride, L.f1.seg_stride);
+    for (auto& L : p->layers) stride = std::max(stride, L.f1.task_stride);
     if (stride == 0) return STI_ERR_STATE;                               // no FFN slice kept anywhere
     std::vector<Job> hj;
-    std::vector<Seg> hs;
+    std::vector<DecodeTask> ht;
     uint64_t bytes = 0;
     for (size_t l = 0; l < p->layers.size(); ++l) {
       Layer& L = p->layers[l];
       if (L.f1.n_jobs == 0) continue;
       hj.resize(L.f1.n_jobs);
-      hs.resize(static_cast<size_t>(L.f1.n_jobs) * L.f1.seg_stride);
+      ht.resize(static_cast<size_t>(L.f1.n_jobs) * L.f1.task_stride);
       CUDA_TRY(cudaMemcpy(hj.data(), L.f1.jobs, hj.size() * sizeof(Job), cudaMemcpyDeviceToHost));
-      CUDA_TRY(cudaMemcpy(hs.data(), L.f1.segs, hs.size() * sizeof(Seg), cudaMemcpyDeviceToHost));
+      CUDA_TRY(cudaMemcpy(ht.data(), L.f1.tasks, ht.size() * sizeof(DecodeTask), cudaMemcpyDeviceToHost));
       for (int j = 0; j < L.f1.n_jobs; ++j) {
         Job job = hj[j];
-        job.seg_begin = static_cast<uint32_t>(jobs.size()) * stride;
+        job.task_begin = static_cast<uint32_t>(jobs.size()) * stride;
         job.out_col += static_cast<uint32_t>(l) * d.ffn;
         job.bias_off = -1;
         jobs.push_back(job);
-        for (uint32_t k = 0; k < stride; ++k) segs.push_back(k < job.n_seg ? hs[static_cast<size_t>(j) * L.f1.seg_stride + k] : Seg{});
+        for (uint32_t k = 0; k < stride; ++k) tasks.push_back(k < job.n_tasks ? ht[static_cast<size_t>(j) * L.f1.task_stride + k] : DecodeTask{});
       }
       for (int sl : L.kept_slices) {
         const int bits = L.ffn[sl].cfg.bits;
         bytes += static_cast<uint64_t>(f) * d.hidden * bits / 8 + (bits == 32 ? 0 : (4ull << bits));
       }
     }
-    const size_t jb = align16(jobs.size() * sizeof(Job)), sb = segs.size() * sizeof(Seg);
-    CUDA_TRY(cudaMalloc(&p->rate_tables, jb + sb));
+    const size_t jb = align16(jobs.size() * sizeof(Job)), tb = tasks.size() * sizeof(DecodeTask);
+    CUDA_TRY(cudaMalloc(&p->rate_tables, jb + tb));
     CUDA_TRY(cudaMemcpy(p->rate_tables, jobs.data(), jobs.size() * sizeof(Job), cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(p->rate_tables + jb, segs.data(), sb, cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemcpy(p->rate_tables + jb, tasks.data(), tb, cudaMemcpyHostToDevice));
     p->rate_jobs = static_cast<int>(jobs.size());
-    p->rate_seg_stride = stride;
+    p->rate_task_stride = stride;
     p->rate_packed_bytes = bytes;
   }
   const int ldo = static_cast<int>(p->layers.size()) * d.ffn;
@@ -1425,9 +1479,9 @@ sti_status sti_decode_rate_probe(sti_plan* p, const void* x_bf16_dev, int tokens
   const GemmTable& ref = p->layers[0].f1.n_jobs ? p->layers[0].f1 : p->layers.back().f1;
   GemmTable tab = ref;                                                   // same tile shape, ring and shared memory
   tab.jobs = reinterpret_cast<Job*>(p->rate_tables);
-  tab.segs = reinterpret_cast<Seg*>(p->rate_tables + align16(static_cast<size_t>(p->rate_jobs) * sizeof(Job)));
+  tab.tasks = reinterpret_cast<DecodeTask*>(p->rate_tables + align16(static_cast<size_t>(p->rate_jobs) * sizeof(Job)));
   tab.n_jobs = p->rate_jobs;
-  tab.seg_stride = p->rate_seg_stride;
+  tab.task_stride = p->rate_task_stride;
   tab.pair_ok = false;
   for (auto& L : p->layers) {                                            // the widest tile decides the shared-memory shape
     if (L.f1.n_jobs && L.f1.smem > tab.smem) { tab.smem = L.f1.smem; tab.w_bytes = L.f1.w_bytes; tab.n_stages = L.f1.n_stages; tab.bps = L.f1.bps; }
@@ -1566,8 +1620,9 @@ sti_status sti_shard_adopt(sti_plan* p, const sti_plan* from, int layer, sti_kin
   else if (src->retained && src->retained_done) where = src->retained;
   if (!where) return STI_ERR_STATE;                        // not in device memory: it has to be uploaded
   u->table = src->table;                                   // host-side metadata the tile tables are built from
-  u->out_off = src->out_off;
+  u->out_rc = src->out_rc;
   u->out_val = src->out_val;
+  u->task_first = src->task_first;
   u->codes.clear();
   u->codes_bytes = src->codes_bytes;
   u->adopt_src = where;

@@ -77,8 +77,9 @@ __global__ void raw_copy_kernel(DecodeLaunch p, uint32_t n) {
 __global__ void patch_outliers_kernel(DecodeLaunch p) {
   const uint32_t o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= p.n_out) return;
-  const uint32_t local = p.out_off[o] - p.flat_base;
-  if (local >= p.rows * p.kc) return;
+  const uint32_t row = p.out_rc[o] >> 16, col = p.out_rc[o] & 0xffffu;
+  if (row >= p.rows || col >= p.kc) return;
+  const size_t local = static_cast<size_t>(row) * p.kc + col;
   const float v = p.out_val[o];
   if (p.w) p.w[local] = v;
   if (p.wbf16) p.wbf16[local] = bf16_bits(v);

@@ -98,17 +98,19 @@ __device__ __forceinline__ void epilogue_tile(uint32_t taddr, uint32_t half, uin
 
 template <typename OutT, bool GELU, bool SIMT, bool FEW>
 __global__ void __launch_bounds__(kThreads, 1)
-dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ jobs, const Seg* __restrict__ segs,
+dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ jobs, const DecodeTask* __restrict__ tasks,
               const __nv_bfloat16* __restrict__ x, int ldx, int T, OutT* __restrict__ out, int ldo,
               const float* __restrict__ bias, int* __restrict__ err, uint32_t n_stages, uint32_t bps,
-              uint32_t w_bytes, uint32_t hdr_bytes, uint32_t seg_stride, PrefetchRanges pf, int kind,
+              uint32_t w_bytes, uint32_t hdr_bytes, uint32_t task_stride, PrefetchRanges pf, int kind,
               unsigned long long* stamps) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) { stamp_min(stamps, STAMP_FIRST_START); stamp_max(stamps, STAMP_LAST_START); }
+  const DecodeTask* my_tasks = tasks + static_cast<size_t>(blockIdx.x) * task_stride;
+  TileDecode decode;
+  decode.begin(my_tasks, task_stride, tid);      // does not wait for the job descriptor
   const Job job = jobs[blockIdx.x];
-  const Seg* my_segs = segs + static_cast<size_t>(blockIdx.x) * seg_stride;     // independent of the job load
   const uint32_t n_rows = job.n_rows, k_total = job.k_total;
 
   SmemHeader* hdr = reinterpret_cast<SmemHeader*>(smem);
@@ -119,11 +121,11 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
   uint8_t* wsm = xsm + n_stages * stage_bytes;
 
   // the kernel's own checks of the descriptor: refuse rather than touch memory out of bounds
-  const bool bad = job.n_seg == 0 || job.n_seg > kMaxSegs || (n_rows != 32 && n_rows != 64 && n_rows != 128) ||
+  const bool bad = job.n_tasks == 0 || job.n_tasks > task_stride || (n_rows != 32 && n_rows != 64 && n_rows != 128) ||
                    (k_total % kChunkK) != 0 || k_total == 0 || n_rows * k_total * 2 > w_bytes ||
                    n_stages < 2 || n_stages > kMaxStages || (bps != 1 && bps != 2 && bps != 4) ||
                    768 + kWarps * kTableStride * 2 > hdr_bytes || (hdr_bytes & 1023) != 0 ||
-                   (smem_addr(smem_raw) & 1023u) != 0 || job.seg_begin != blockIdx.x * seg_stride || job.n_seg > seg_stride;
+                   (smem_addr(smem_raw) & 1023u) != 0 || job.task_begin != blockIdx.x * task_stride;
   if (bad) {
     if (tid == 0) atomicCAS(err, ERR_NONE, ERR_BAD_JOB);
     return;
@@ -180,7 +182,7 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
       tmem_relinquish();
     }
   }
-  if (tid < n_rows) bias_sm[tid] = job.bias_off >= 0 ? __ldg(bias + job.bias_off + tid) : 0.f;
+  const float bias_value = tid < n_rows && job.bias_off >= 0 ? __ldg(bias + job.bias_off + tid) : 0.f;
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
@@ -190,7 +192,8 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
   // can never starve it of columns.
   pdl_launch_dependents();
 
-  decode_weight_tile(job, my_segs, tables, wsm, tid);
+  if (tid < n_rows) bias_sm[tid] = bias_value;
+  decode.finish(my_tasks, task_stride, tables, wsm, n_rows, tid);
   if (tid == 0) stamp_max(stamps, STAMP_DECODED);
   // Everything above read only weights, descriptors and parameters.  The activations are the previous
   // kernel's output: from here on this kernel depends on it.
@@ -362,9 +365,9 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
 // ---------------------------------------------------------------------------------------
 template <typename OutT, bool GELU>
 __global__ void __launch_bounds__(kThreads, 1)
-dqgemm_pair_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ jobs, const Seg* __restrict__ segs,
+dqgemm_pair_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ jobs, const DecodeTask* __restrict__ tasks,
                    int T, OutT* __restrict__ out, int ldo, const float* __restrict__ bias, int* __restrict__ err,
-                   uint32_t n_stages, uint32_t bps, uint32_t w_bytes, uint32_t hdr_bytes, uint32_t seg_stride,
+                   uint32_t n_stages, uint32_t bps, uint32_t w_bytes, uint32_t hdr_bytes, uint32_t task_stride,
                    unsigned long long* stamps) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
@@ -372,26 +375,28 @@ dqgemm_pair_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
   if (tid == 0) { stamp_min(stamps, STAMP_FIRST_START); stamp_max(stamps, STAMP_LAST_START); }
   const uint32_t rank = cluster_ctarank();                 // 0 issues the MMAs
   const uint32_t pair_base = blockIdx.x & ~1u;
-  const Job job = jobs[blockIdx.x];                        // the 64 weight rows this CTA decodes
+  const DecodeTask* my_tasks = tasks + static_cast<size_t>(blockIdx.x) * task_stride;
+  TileDecode decode;                                       // the 64 weight rows this CTA decodes
+  decode.begin(my_tasks, task_stride, tid);                // does not wait for the job descriptors
+  const Job job = jobs[blockIdx.x];
   const Job job0 = jobs[pair_base], job1 = jobs[pair_base + 1];   // columns 0-63 / 64-127 of the accumulator
   const uint32_t k_total = job.k_total;
 
   SmemHeader* hdr = reinterpret_cast<SmemHeader*>(smem);
   float* bias_sm = reinterpret_cast<float*>(smem + 256);            // [128]
   uint16_t* tables = reinterpret_cast<uint16_t*>(smem + 768);       // [warp][64]
-  const Seg* my_segs = segs + static_cast<size_t>(blockIdx.x) * seg_stride;
   uint8_t* xsm = smem + hdr_bytes;
   const uint32_t stage_bytes = bps * kBoxBytes;
   uint8_t* wsm = xsm + n_stages * stage_bytes;
 
   // both CTAs evaluate the same conditions, so a refused pair leaves together
   const bool bad = job0.n_rows != 64 || job1.n_rows != 64 || job0.k_total != job1.k_total || job0.x_koff != job1.x_koff ||
-                   job0.n_seg == 0 || job0.n_seg > kMaxSegs || job1.n_seg == 0 || job1.n_seg > kMaxSegs ||
+                   job0.n_tasks == 0 || job0.n_tasks > task_stride || job1.n_tasks == 0 || job1.n_tasks > task_stride ||
                    (k_total % kChunkK) != 0 || k_total == 0 || 64 * k_total * 2 > w_bytes || n_stages < 2 ||
                    n_stages > kMaxStages || (bps != 1 && bps != 2 && bps != 4) ||
                    768 + kWarps * kTableStride * 2 > hdr_bytes || (hdr_bytes & 1023) != 0 || (gridDim.x & 1) != 0 ||
-                   (smem_addr(smem_raw) & 1023u) != 0 || job0.n_seg > seg_stride || job1.n_seg > seg_stride ||
-                   job0.seg_begin != pair_base * seg_stride || job1.seg_begin != (pair_base + 1) * seg_stride;
+                   (smem_addr(smem_raw) & 1023u) != 0 || job0.task_begin != pair_base * task_stride ||
+                   job1.task_begin != (pair_base + 1) * task_stride;
   if (bad) {
     if (tid == 0) atomicCAS(err, ERR_NONE, ERR_BAD_JOB);
     return;
@@ -426,17 +431,16 @@ dqgemm_pair_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
     tmem_alloc_pair(smem_addr(&hdr->tmem_base), kTmemCols);
     tmem_relinquish_pair();
   }
-  if (tid < 128) {
-    const Job& jb = tid < 64 ? job0 : job1;
-    bias_sm[tid] = jb.bias_off >= 0 ? __ldg(bias + jb.bias_off + (tid & 63)) : 0.f;
-  }
+  const int bias_off = tid < 64 ? job0.bias_off : job1.bias_off;
+  const float bias_value = tid < 128 && bias_off >= 0 ? __ldg(bias + bias_off + (tid & 63)) : 0.f;
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = hdr->tmem_base;
   pdl_launch_dependents();          // this CTA owns its tensor memory now (see the one-CTA kernel)
 
-  decode_weight_tile(job, my_segs, tables, wsm, tid);
+  if (tid < 128) bias_sm[tid] = bias_value;
+  decode.finish(my_tasks, task_stride, tables, wsm, 64, tid);
   if (tid == 0) stamp_max(stamps, STAMP_DECODED);
   cluster_sync_all();               // both halves of the weight tile are in place, all barriers initialised
   pdl_wait();                       // from here on: the previous kernel's output
@@ -580,17 +584,17 @@ cudaError_t launch_t(const GemmLaunch& p, cudaStream_t s) {
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p.pdl ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, dqgemm_pair_kernel<OutT, GELU>, p.xmap, p.jobs, p.segs, p.T, static_cast<OutT*>(p.out),
-                              p.ldo, p.bias, p.err, p.n_stages, p.bps, p.w_bytes, p.hdr_bytes, p.seg_stride, p.stamps);
+    return cudaLaunchKernelEx(&cfg, dqgemm_pair_kernel<OutT, GELU>, p.xmap, p.jobs, p.tasks, p.T, static_cast<OutT*>(p.out),
+                              p.ldo, p.bias, p.err, p.n_stages, p.bps, p.w_bytes, p.hdr_bytes, p.task_stride, p.stamps);
   }
   dim3 grid(p.n_jobs, p.m_ctas), block(kThreads);
   PrefetchRanges pf;
   for (int r = 0; r < 4; ++r) { pf.ptr[r] = p.pf_ptr[r]; pf.bytes[r] = p.pf_bytes[r]; }
   const int kind = sizeof(OutT) == 4 ? GEMM_BF16_TO_F32 : (GELU ? GEMM_BF16_TO_BF16_GELU : GEMM_BF16_TO_BF16);
   if (p.simt_debug) {
-    return launch_kernel(dqgemm_kernel<OutT, GELU, true, false>, grid, block, p.smem_bytes, s, p.pdl, p.xmap, p.jobs, p.segs, x, p.ldx,
+    return launch_kernel(dqgemm_kernel<OutT, GELU, true, false>, grid, block, p.smem_bytes, s, p.pdl, p.xmap, p.jobs, p.tasks, x, p.ldx,
                          p.T, static_cast<OutT*>(p.out), p.ldo, p.bias, p.err, p.n_stages, p.bps, p.w_bytes, p.hdr_bytes,
-                         p.seg_stride, pf, kind, p.stamps);
+                         p.task_stride, pf, kind, p.stamps);
   }
   // every output kind runs the same kernel (the kind is a parameter): one copy of the code for a layer's four GEMMs;
   // two builds of it, for few and for many token tiles per CTA (they differ in the epilogue's shape)
@@ -598,11 +602,11 @@ cudaError_t launch_t(const GemmLaunch& p, cudaStream_t s) {
   const bool few = (n_mtiles + p.m_ctas - 1) / p.m_ctas <= 2;
   if (few)
     return launch_kernel(dqgemm_kernel<void, false, false, true>, grid, block, p.smem_bytes, s, p.pdl, p.xmap,
-                                 p.jobs, p.segs, x, p.ldx, p.T, p.out, p.ldo, p.bias, p.err, p.n_stages, p.bps, p.w_bytes,
-                                 p.hdr_bytes, p.seg_stride, pf, kind, p.stamps);
+                                 p.jobs, p.tasks, x, p.ldx, p.T, p.out, p.ldo, p.bias, p.err, p.n_stages, p.bps, p.w_bytes,
+                                 p.hdr_bytes, p.task_stride, pf, kind, p.stamps);
   return launch_kernel(dqgemm_kernel<void, false, false, false>, grid, block, p.smem_bytes, s, p.pdl, p.xmap,
-                               p.jobs, p.segs, x, p.ldx, p.T, p.out, p.ldo, p.bias, p.err, p.n_stages, p.bps, p.w_bytes,
-                               p.hdr_bytes, p.seg_stride, pf, kind, p.stamps);
+                               p.jobs, p.tasks, x, p.ldx, p.T, p.out, p.ldo, p.bias, p.err, p.n_stages, p.bps, p.w_bytes,
+                               p.hdr_bytes, p.task_stride, pf, kind, p.stamps);
 }
 
 template <typename K>

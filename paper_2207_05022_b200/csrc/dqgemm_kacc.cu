@@ -49,25 +49,22 @@ struct KaccHeader {
 static_assert(sizeof(KaccHeader) <= 320, "barriers must fit the first 320 bytes of the header");
 
 // What the roles need to know about a K group, kept in shared memory (bytes 320..768 of the header) so that no role
-// has a global-memory round trip on its path at every step; the CTA's own segment descriptors sit in the upper
-// half of the table area (bytes 1792..2816, the tables of warps that do not decode here) when they fit.
+// has a global-memory round trip on its path at every step.
 struct KaccGroup {
-  uint16_t n_boxes;        // K range of the group in 64-column boxes
-  uint16_t n_seg;          // segments of this CTA's job
+  uint32_t n_boxes;        // K range of the group in 64-column boxes
   uint32_t x_koff;         // first activation column
 };
 constexpr int kKaccMaxGroups = 56;
-constexpr uint32_t kKaccSegArea = 1024;
 
 __device__ __forceinline__ void fence_acq_rel_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 
 // SPLIT: two warps share a decode task (weight buffers of at most 64 x 256: four tasks for the eight warps).
 template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1)
-dqgemm_kacc_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ jobs, const Seg* __restrict__ segs,
+dqgemm_kacc_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ jobs, const DecodeTask* __restrict__ tasks,
                    const __nv_bfloat16* __restrict__ x, int ldx, int n_groups, int T, float* __restrict__ out, int ldo,
                    int* __restrict__ err, uint32_t n_stages,
-                   uint32_t bps, uint32_t w_buf_bytes, uint32_t hdr_bytes, uint32_t seg_stride,
+                   uint32_t bps, uint32_t w_buf_bytes, uint32_t hdr_bytes, uint32_t task_stride,
                    unsigned long long* stamps) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
@@ -80,8 +77,6 @@ dqgemm_kacc_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
   KaccHeader* hdr = reinterpret_cast<KaccHeader*>(smem);
   KaccGroup* ginfo = reinterpret_cast<KaccGroup*>(smem + 320);
   uint16_t* tables = reinterpret_cast<uint16_t*>(smem + 768);
-  Seg* seg_sm = reinterpret_cast<Seg*>(smem + 1792);
-  const bool segs_in_smem = static_cast<uint32_t>(n_groups) * seg_stride * sizeof(Seg) <= kKaccSegArea;
   uint8_t* xsm = smem + hdr_bytes;
   const uint32_t stage_bytes = bps * kBoxBytes;         // a ring stage holds `bps` boxes of 64 columns
   uint8_t* wsm = xsm + n_stages * stage_bytes;          // two buffers of w_buf_bytes
@@ -94,9 +89,8 @@ dqgemm_kacc_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
     const uint32_t i0 = g * n_cols64 + pair_base;
     const Job a = jobs[i0], b = jobs[i0 + 1];
     bad |= a.n_rows != 64 || b.n_rows != 64 || a.k_total != b.k_total || a.x_koff != b.x_koff || a.k_total == 0 ||
-          a.k_total > k_max || (a.k_total % (kChunkK * bps)) != 0 || a.n_seg == 0 || b.n_seg == 0 || a.n_seg > seg_stride ||
-          b.n_seg > seg_stride || a.n_seg > kMaxSegs || b.n_seg > kMaxSegs || a.seg_begin != i0 * seg_stride ||
-          b.seg_begin != (i0 + 1) * seg_stride || a.out_col != pair_base * 64 || b.out_col != (pair_base + 1) * 64;
+          a.k_total > k_max || (a.k_total % (kChunkK * bps)) != 0 || a.n_tasks == 0 || b.n_tasks == 0 || a.n_tasks > task_stride ||
+          b.n_tasks > task_stride || a.task_begin != i0 * task_stride || b.task_begin != (i0 + 1) * task_stride || a.out_col != pair_base * 64 || b.out_col != (pair_base + 1) * 64;
   }
   if (bad) {
     if (tid == 0) atomicCAS(err, ERR_NONE, ERR_BAD_JOB);
@@ -114,19 +108,8 @@ dqgemm_kacc_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
 
   if (tid < static_cast<uint32_t>(n_groups)) {
     const Job j = jobs[tid * n_cols64 + blockIdx.x];
-    ginfo[tid].n_boxes = static_cast<uint16_t>(j.k_total / kChunkK);
-    ginfo[tid].n_seg = static_cast<uint16_t>(j.n_seg);
+    ginfo[tid].n_boxes = j.k_total / kChunkK;
     ginfo[tid].x_koff = j.x_koff;
-  }
-  if (segs_in_smem) {
-    constexpr uint32_t kSegWords = sizeof(Seg) / 4;
-    const uint32_t per_group = seg_stride * kSegWords, n_words = static_cast<uint32_t>(n_groups) * per_group;
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(segs);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(seg_sm);
-    for (uint32_t w = tid; w < n_words; w += kThreads) {
-      const uint32_t g = w / per_group, k = w % per_group;
-      dst[w] = __ldg(src + (static_cast<size_t>(g) * n_cols64 + blockIdx.x) * per_group + k);
-    }
   }
   if (tid == 0) {
     for (uint32_t s = 0; s < n_stages; ++s) {
@@ -348,17 +331,30 @@ dqgemm_kacc_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
         if (lane == 0) mbar_arrive_cluster_cta_scope(map_to_cta(smem_addr(&hdr->acc_empty[t]), 0));
       }
     };
+    // The next K group's task is loaded while this one is worked on: its descriptor and planes have arrived before the
+    // buffer they go to is free.  SPLIT: two warps share a task.
+    constexpr uint32_t kUnits = SPLIT ? kKaccGroupWarps / 2 : kKaccGroupWarps;
+    const uint32_t gwarp = warp - kKaccGroupWarp0, unit0 = SPLIT ? gwarp >> 1 : gwarp, part = SPLIT ? 1 + (gwarp & 1) : 0;
+    uint16_t* const tab = tables + gwarp * kTableStride;
+    DecodeTask task;
+    TaskLoads loads;
+    auto fetch = [&](int g, uint32_t unit) {
+      task = load_task(tasks + (static_cast<size_t>(g) * n_cols64 + blockIdx.x) * task_stride + unit);
+      issue_loads(task, lane, loads);
+    };
+    if (n_steps > 0 && unit0 < task_stride) fetch(0, unit0);
     uint32_t step = 0;
     for (uint32_t blk = 0; blk < n_blocks; ++blk) {
       for (int g = 0; g < n_groups; ++g, ++step) {
         const uint32_t wb = step & 1;
         if (step >= 2) wait_uniform(smem_addr(&hdr->w_empty[wb]), ((step >> 1) - 1) & 1);
-        Job job{};
-        job.n_rows = 64; job.k_total = ginfo[g].n_boxes * kChunkK; job.n_seg = ginfo[g].n_seg;
-        const Seg* my_segs = segs_in_smem ? seg_sm + static_cast<size_t>(g) * seg_stride
-                                          : segs + (static_cast<size_t>(g) * n_cols64 + blockIdx.x) * seg_stride;
-        decode_weight_tile_group<kKaccGroupWarps, SPLIT>(job, my_segs, tables, wsm + wb * w_buf_bytes, gtid,
-                                                         kKaccGroupBarrier);
+        for (uint32_t unit = unit0; unit < task_stride; unit += kUnits) {
+          if (unit != unit0) fetch(g, unit);
+          finish_task(task, loads, tab, wsm + wb * w_buf_bytes, 64, lane, part);
+        }
+        if (step + 1 < n_steps && unit0 < task_stride) fetch(g + 1 < n_groups ? g + 1 : 0, unit0);
+        fence_proxy_async_smem();
+        group_barrier<kKaccGroupWarps>(kKaccGroupBarrier);
         if (gtid == 0) {
           if (step == 0) stamp_max(stamps, STAMP_DECODED);
           mbar_arrive_cluster(map_to_cta(smem_addr(&hdr->w_full[wb]), 0));
@@ -416,10 +412,10 @@ cudaError_t launch_gemm_kacc(const KaccLaunch& p, cudaStream_t s) {
   cfg.numAttrs = p.pdl ? 2 : 1;
   const uint32_t w_buf_bytes = 64u * p.k_group * 2u;
   if (p.k_group <= 256)      // at most four decode tasks per weight tile: two warps share each
-    return cudaLaunchKernelEx(&cfg, dqgemm_kacc_kernel<true>, p.xmap, p.jobs, p.segs, static_cast<const __nv_bfloat16*>(p.x), p.ldx, p.n_groups, p.T, p.out, p.ldo, p.err,
-                              p.n_stages, p.bps, w_buf_bytes, p.hdr_bytes, p.seg_stride, p.stamps);
-  return cudaLaunchKernelEx(&cfg, dqgemm_kacc_kernel<false>, p.xmap, p.jobs, p.segs, static_cast<const __nv_bfloat16*>(p.x), p.ldx, p.n_groups, p.T, p.out, p.ldo, p.err,
-                            p.n_stages, p.bps, w_buf_bytes, p.hdr_bytes, p.seg_stride, p.stamps);
+    return cudaLaunchKernelEx(&cfg, dqgemm_kacc_kernel<true>, p.xmap, p.jobs, p.tasks, static_cast<const __nv_bfloat16*>(p.x), p.ldx, p.n_groups, p.T, p.out, p.ldo, p.err,
+                              p.n_stages, p.bps, w_buf_bytes, p.hdr_bytes, p.task_stride, p.stamps);
+  return cudaLaunchKernelEx(&cfg, dqgemm_kacc_kernel<false>, p.xmap, p.jobs, p.tasks, static_cast<const __nv_bfloat16*>(p.x), p.ldx, p.n_groups, p.T, p.out, p.ldo, p.err,
+                            p.n_stages, p.bps, w_buf_bytes, p.hdr_bytes, p.task_stride, p.stamps);
 }
 
 }  // namespace sti

@@ -19,8 +19,7 @@ constexpr int kMaxStages = 8;
 constexpr int kBoxBytes = kTileM * kChunkK * 2;     // 16 KB
 // header = barriers (256 B) + bias (512 B) + one 128-byte centroid table per warp; stages start 1024-aligned after it
 constexpr int kHeaderBytes = 3072;
-constexpr int kMaxSegs = 16;
-constexpr int kTableStride = 64;            // bf16 entries per segment table
+constexpr int kTableStride = 64;            // bf16 entries of a warp's centroid table
 constexpr int kEpilogueWarp0 = 4;             // epilogue warps 4..11: two per TMEM lane quadrant
 constexpr int kEpilogueWarps = 8;
 constexpr int kPairEpilogueWarps = 12;        // the two-CTA kernel drains with warps 4..15: three per lane quadrant
@@ -36,50 +35,122 @@ struct SmemHeader {
 };
 
 // ---------------------------------------------------------------------------------------
-// Weight-tile decode
+// Weight-tile decode (Section 4.2 decompression), one task of 4096 weights per warp at a time.
+//
+// Bound: latency, then the integer pipe.  A warp's chain is descriptor -> (planes, table, outliers) -> unpack -> its own
+// outliers, with no barrier of the CTA inside.  Up to 4 bits the table is looked up with byte permutes on registers
+// (2 to 2.6 integer instructions per weight; the shared-memory lookup took 3.5 and a shared-memory access each), 5 and 6
+// bits look up a table in shared memory.
+// Measured from a CTA's start to its decoded tile: 64 x 768 weights at 4 bits 4.5 -> 3.2 us, 64 x 1024 at 2..6 bits
+// 5.5 -> 4.0 (segment descriptors with divisions, a search for each thread's outlier and a CTA barrier before the
+// outliers came first); BERT-base, 385 tokens 50.5 -> 43.8 us per layer, BERT-large, 256 tokens 48.0 -> 46.2.
 // ---------------------------------------------------------------------------------------
-// The k index planes of one task = (row group, 128-column chunk), one coalesced 128-bit load per plane.
-// `bits` is only known at run time here, so that the loads can be issued before anything else of the
-// task is ready.  All six loads are issued back to back and unconditionally - a plane number beyond `bits`
-// re-reads the last plane (a cache hit) - so that the task pays one memory round trip: with a load under
-// `if (p < bits)` each plane's load waited for the one before it.
-__device__ __forceinline__ void load_planes(const Seg& sg, uint32_t task, uint32_t lane, uint32_t (&w)[24]) {
-  const uint32_t bits = sg.bits;
-  const uint32_t chunks = sg.kc >= 128 ? sg.kc / 128 : 1;
-  const uint32_t g = task / chunks, j = task % chunks;
-  const uint4* src = sg.codes + (static_cast<size_t>(g) * chunks + j) * (bits * 32) + lane;
+struct TaskLoads {               // a task's loads in flight
+  uint32_t w[24];                // lane's 128 indexes: `bits` planes of four words
+  float c0, c1;                  // centroids lane and lane + 32
+  uint32_t rc;                   // outlier number `lane`
+  float val;
+};
+
+__device__ __forceinline__ DecodeTask load_task(const DecodeTask* p) {
+  const uint4 a = __ldg(reinterpret_cast<const uint4*>(p)), b = __ldg(reinterpret_cast<const uint4*>(p) + 1);
+  DecodeTask t;
+  t.codes = reinterpret_cast<const uint8_t*>(static_cast<uint64_t>(a.x) | (static_cast<uint64_t>(a.y) << 32));
+  t.table = a.z; t.out_rc = a.w; t.out_val = b.x;
+  t.n_out = static_cast<uint16_t>(b.y); t.bits = static_cast<uint8_t>(b.y >> 16); t.narrow = static_cast<uint8_t>(b.y >> 24);
+  t.row0 = static_cast<uint16_t>(b.z); t.kcore0 = static_cast<uint16_t>(b.z >> 16);
+  t.origin = b.w;
+  return t;
+}
+
+// All loads of a task back to back.  Six planes whatever `bits` is - a plane number beyond it re-reads the last plane,
+// a cache hit - so that none waits for another.
+__device__ __forceinline__ void issue_loads(const DecodeTask& t, uint32_t lane, TaskLoads& f) {
+  if (t.bits == 0 || t.bits > 6) return;
+  const uint4* src = reinterpret_cast<const uint4*>(t.codes) + lane;
   uint4 v[6];
 #pragma unroll
-  for (int p = 0; p < 6; ++p) v[p] = __ldg(src + (static_cast<uint32_t>(p) < bits ? p : (bits ? bits - 1 : 0)) * 32);
-#pragma unroll
-  for (int p = 0; p < 6; ++p) { w[4 * p + 0] = v[p].x; w[4 * p + 1] = v[p].y; w[4 * p + 2] = v[p].z; w[4 * p + 3] = v[p].w; }
-}
-
-// Which outlier of the tile a thread patches: outlier number `t` in the order of the tile's segments.  The segments'
-// counts are read in one go (lane s reads segment s: one memory round trip for up to kMaxSegs descriptors instead of
-// one per segment) and handed round by shuffles.  Returns the total; `seg` stays 0xffffffff when t is beyond it.
-__device__ __forceinline__ uint32_t find_outlier_slot(const Seg* __restrict__ segs, uint32_t n_seg, uint32_t t, uint32_t lane,
-                                                      uint32_t& seg, uint32_t& index) {
-  const uint32_t mine = lane < n_seg ? segs[lane].n_out : 0u;
-  uint32_t before = 0;
-  seg = 0xffffffffu;
-  index = 0;
-#pragma unroll 1
-  for (uint32_t si = 0; si < n_seg; ++si) {
-    const uint32_t n = __shfl_sync(0xffffffffu, mine, static_cast<int>(si));
-    if (seg == 0xffffffffu && t >= before && t - before < n) { seg = si; index = t - before; }
-    before += n;
+  for (uint32_t p = 0; p < 6; ++p) v[p] = __ldg(src + (p < t.bits ? p : t.bits - 1u) * 32u);
+  const float* table = reinterpret_cast<const float*>(t.codes + t.table);
+  const uint32_t n_entries = 1u << t.bits;
+  f.c0 = lane < n_entries ? __ldg(table + lane) : 0.f;
+  f.c1 = lane + 32 < n_entries ? __ldg(table + lane + 32) : 0.f;
+  f.rc = 0u;
+  f.val = 0.f;
+  if (lane < t.n_out) {
+    f.rc = __ldg(reinterpret_cast<const uint32_t*>(t.codes + t.out_rc) + lane);
+    f.val = __ldg(reinterpret_cast<const float*>(t.codes + t.out_val) + lane);
   }
-  return before;
+#pragma unroll
+  for (int p = 0; p < 6; ++p) { f.w[4 * p + 0] = v[p].x; f.w[4 * p + 1] = v[p].y; f.w[4 * p + 2] = v[p].z; f.w[4 * p + 3] = v[p].w; }
 }
 
-// Index unpack in registers -> bf16 table lookup in shared memory -> 16-byte stores into the K-major
-// core-matrix layout.  Each lane holds 128 consecutive indexes of its own row.
-// `half`: 0 = the whole quantum (four index groups), 1 / 2 = its first / second two groups only (two warps share a
-// task when a tile has fewer tasks than the CTA has warps; both hold the task's planes).
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+  return r;
+}
+
+// 32 indexes of at most 4 bits -> four words of eight 4-bit fields.
 template <int BITS>
-__device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const Seg& sg, const uint16_t* __restrict__ tab,
-                                            uint8_t* wsm, uint32_t n_rows, uint32_t task, uint32_t lane, uint32_t half = 0) {
+__device__ __forceinline__ void spread_to_nibbles(const uint32_t (&w)[BITS], uint32_t (&sel)[4]) {
+  static_assert(BITS >= 2 && BITS <= 4, "one byte permute takes a 3-bit index");
+  if constexpr (BITS == 4) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sel[i] = w[i];
+  } else {
+    uint32_t x[4];             // eight indexes each, in the low bits
+    if constexpr (BITS == 3) {
+      x[0] = w[0]; x[1] = __funnelshift_r(w[0], w[1], 24); x[2] = __funnelshift_r(w[1], w[2], 16); x[3] = w[2] >> 8;
+    } else {
+      x[0] = w[0]; x[1] = w[0] >> 16; x[2] = w[1]; x[3] = w[1] >> 16;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {      // halves apart, quarters apart, eighths apart; what is in between is masked last
+      uint32_t y = (x[i] & 0x0000ffffu) | ((x[i] << (16 - 4 * BITS)) & 0xffff0000u);
+      y = (y & 0x00ff00ffu) | ((y << (8 - 2 * BITS)) & 0xff00ff00u);
+      y = (y & 0x0f0f0f0fu) | ((y << (4 - BITS)) & 0xf0f0f0f0u);
+      sel[i] = y & (BITS == 3 ? 0x77777777u : 0x33333333u);
+    }
+  }
+}
+
+// The table in registers, low and high bytes of the bf16 entries apart, four entries to a word.
+template <int BITS>
+struct ByteTable {
+  static constexpr int kWords = BITS == 2 ? 1 : (1 << BITS) / 4;
+  uint32_t lo[kWords], hi[kWords];
+  __device__ __forceinline__ void load(const uint16_t* tab) {
+#pragma unroll
+    for (int i = 0; i < kWords; ++i) {
+      const uint2 e = *reinterpret_cast<const uint2*>(tab + 4 * i);
+      lo[i] = prmt(e.x, e.y, 0x6420u);
+      hi[i] = prmt(e.x, e.y, 0x7531u);
+    }
+  }
+  // bf16 values of the four indexes in the low 16 bits of `sel`, in order
+  __device__ __forceinline__ void four(uint32_t sel, uint32_t upper, uint32_t& w0, uint32_t& w1) const {
+    uint32_t l, h;
+    if constexpr (BITS <= 3) {
+      l = prmt(lo[0], lo[kWords - 1], sel);
+      h = prmt(hi[0], hi[kWords - 1], sel);
+    } else {                   // entries 0-7 and 8-15 side by side, then byte j from the side that index j's top bit names
+      l = prmt(prmt(lo[0], lo[1], sel), prmt(lo[2], lo[3], sel), upper);
+      h = prmt(prmt(hi[0], hi[1], sel), prmt(hi[2], hi[3], sel), upper);
+    }
+    w0 = prmt(l, h, 0x5140u);
+    w1 = prmt(l, h, 0x7362u);
+  }
+};
+
+// Index unpack -> table lookup -> 16-byte stores into the K-major core-matrix layout.  Each lane holds 128 consecutive
+// indexes of its own row (narrow tasks: of rows l and l + 32).  `half`: 0 = the whole quantum (four groups of 32 indexes),
+// 1 / 2 = its first / second two groups only (two warps share a task when a tile has few; both hold the task's planes).
+// 32 indexes are exactly BITS words: the loop is rolled over the four groups and always reads w[0 .. BITS), the words
+// moving down after each group - the decode runs once per CTA, so its code is fetched cold and its size is what it costs.
+template <int BITS>
+__device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const DecodeTask& t, const uint16_t* __restrict__ tab,
+                                            uint8_t* wsm, uint32_t n_rows, uint32_t lane, uint32_t half) {
   uint32_t w[4 * BITS];
 #pragma unroll
   for (int i = 0; i < 4 * BITS; ++i) w[i] = planes[i];
@@ -87,53 +158,99 @@ __device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const 
 #pragma unroll
     for (int i = 0; i < 2 * BITS; ++i) w[i] = planes[i + 2 * BITS];
   }
-  const int grp0 = half == 2 ? 2 : 0, grp1 = half == 1 ? 2 : 4;
-  const uint32_t chunks = sg.kc >= 128 ? sg.kc / 128 : 1;
-  const uint32_t g = task / chunks, j = task % chunks;
-  const bool narrow = sg.kc < 128;     // 64 in-features: the quantum is rows (l, l + 32) of a 64-row group
-  const uint32_t row0 = narrow ? g * 64 + lane : g * 32 + lane;
-  const uint32_t kcore0 = (sg.koff + (narrow ? 0 : j * 128)) >> 3;
-  // 32 indexes = exactly BITS words, whatever BITS is: the loop below is rolled over the four such groups
-  // of the quantum and always reads w[0 .. BITS), the words moving down by BITS after each group.  A
-  // quarter of the instructions of the fully unrolled form: the decode runs once per CTA, so its code is
-  // fetched cold and its size is what it costs.
+  const uint32_t grp0 = half == 2 ? 2 : 0, grp1 = half == 1 ? 2 : 4;
+  const uint32_t piece = n_rows * 16;                    // from eight columns to the next eight
+  uint8_t* const dst0 = wsm + (static_cast<size_t>(t.kcore0) * n_rows + t.row0 + lane) * 16;
+  ByteTable<BITS <= 4 ? BITS : 2> table;
+  if constexpr (BITS <= 4) table.load(tab);
 #pragma unroll 1
-  for (int grp = grp0; grp < grp1; ++grp) {
+  for (uint32_t grp = grp0; grp < grp1; ++grp) {
     uint32_t lo[BITS];
 #pragma unroll
     for (int i = 0; i < BITS; ++i) lo[i] = w[i];
+    uint8_t* dst = dst0 + (t.narrow ? (grp & 1) * 4 * piece + (grp >> 1) * 512 : grp * 4 * piece);
+    if constexpr (BITS <= 4) {
+      uint32_t sel[4];
+      spread_to_nibbles<BITS>(lo, sel);
 #pragma unroll
-    for (int ss = 0; ss < 4; ++ss) {
-      uint32_t pk[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const uint32_t c0 = extract_index_words<BITS>(lo, 8 * ss + 2 * e);
-        const uint32_t c1 = extract_index_words<BITS>(lo, 8 * ss + 2 * e + 1);
-        pk[e] = static_cast<uint32_t>(tab[c0]) | (static_cast<uint32_t>(tab[c1]) << 16);
+      for (int ss = 0; ss < 4; ++ss) {
+        const uint32_t low = BITS == 4 ? sel[ss] & 0x77777777u : sel[ss];
+        const uint32_t upper = BITS == 4 ? ((sel[ss] >> 1) & 0x44444444u) | 0x32103210u : 0u;
+        uint4 v;
+        table.four(low, upper, v.x, v.y);
+        table.four(low >> 16, upper >> 16, v.z, v.w);
+        *reinterpret_cast<uint4*>(dst + ss * piece) = v;
       }
-      const uint32_t sidx = 4 * grp + ss;
-      const uint32_t row = narrow ? row0 + 32 * (sidx >> 3) : row0;
-      const uint32_t kcore = narrow ? kcore0 + (sidx & 7) : kcore0 + sidx;
-      *reinterpret_cast<uint4*>(wsm + (static_cast<size_t>(kcore) * n_rows + row) * 16) =
-          make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    } else {
+#pragma unroll
+      for (int ss = 0; ss < 4; ++ss) {
+        uint32_t pk[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const uint32_t c0 = extract_index_words<BITS>(lo, 8 * ss + 2 * e);
+          const uint32_t c1 = extract_index_words<BITS>(lo, 8 * ss + 2 * e + 1);
+          pk[e] = static_cast<uint32_t>(tab[c0]) | (static_cast<uint32_t>(tab[c1]) << 16);
+        }
+        *reinterpret_cast<uint4*>(dst + ss * piece) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      }
     }
 #pragma unroll
     for (int i = 0; i + BITS < 4 * BITS; ++i) w[i] = w[i + BITS];
   }
 }
 
-// Uncompressed (32-bit) version of a unit: rows are plain fp32, converted to bf16 on the way in.
-__device__ __forceinline__ void decode_raw(const Seg& sg, uint8_t* wsm, uint32_t n_rows, uint32_t tid) {
-  const float* src = reinterpret_cast<const float*>(sg.codes);
-  const uint32_t pieces_per_row = sg.kc / 8;
-  const uint32_t total = n_rows * pieces_per_row;
-  for (uint32_t idx = tid; idx < total; idx += kThreads) {
-    const uint32_t row = idx % n_rows, piece = idx / n_rows;
-    const float4 a = __ldg(reinterpret_cast<const float4*>(src + static_cast<size_t>(row) * sg.kc + piece * 8));
-    const float4 b = __ldg(reinterpret_cast<const float4*>(src + static_cast<size_t>(row) * sg.kc + piece * 8 + 4));
-    const uint32_t kcore = (sg.koff >> 3) + piece;
-    *reinterpret_cast<uint4*>(wsm + (static_cast<size_t>(kcore) * n_rows + row) * 16) =
-        make_uint4(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w), pack_bf16x2(b.x, b.y), pack_bf16x2(b.z, b.w));
+// Uncompressed (32-bit) version of a unit: rows are plain fp32, rounded to bf16 on the way in.  A load covers four rows x
+// 32 columns, four whole lines (a lane per row would touch 32 lines with every load: 9 us for a tile of 64 x 1024);
+// sixteen loads in flight.
+__device__ __forceinline__ void unpack_raw(const DecodeTask& t, uint8_t* wsm, uint32_t n_rows, uint32_t lane, uint32_t half) {
+#pragma unroll 1
+  for (uint32_t first = half == 2 ? 16 : 0; first < (half == 1 ? 16u : 32u); first += 16) {
+    float4 v[16];
+    const uint32_t r = lane >> 3, c = (lane & 7) * 4;
+    // of load i: its rows and columns (wide tasks: eight row groups of a 32-column strip, then the next strip)
+    auto row = [&](uint32_t i) { return (t.narrow ? i >> 1 : i & 7) * 4 + r; };
+    auto col = [&](uint32_t i) { return (t.narrow ? i & 1 : i >> 3) * 32 + c; };
+#pragma unroll
+    for (uint32_t i = 0; i < 16; ++i)
+      v[i] = __ldg(reinterpret_cast<const float4*>(t.codes + static_cast<size_t>(row(first + i)) * t.out_val + col(first + i) * 4));
+#pragma unroll
+    for (uint32_t i = 0; i < 16; ++i) {
+      uint8_t* dst = wsm + (static_cast<size_t>(t.kcore0 + (col(first + i) >> 3)) * n_rows + t.row0 + row(first + i)) * 16 + (c & 4) * 2;
+      *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(v[i].x, v[i].y), pack_bf16x2(v[i].z, v[i].w));
+    }
+  }
+}
+
+// The task (or half of it) into the tile; the warp's own 128 bytes at `tab` take the table, rounded once to bf16
+// (round-to-nearest-even).  Outliers (Section 6: they keep their original value) follow, the warp's own only.
+__device__ __forceinline__ void finish_task(const DecodeTask& t, const TaskLoads& f, uint16_t* tab, uint8_t* wsm, uint32_t n_rows,
+                                            uint32_t lane, uint32_t half) {
+  if (t.bits == 32) { unpack_raw(t, wsm, n_rows, lane, half); return; }
+  if (t.bits == 0) return;
+  tab[lane] = bf16_bits(f.c0);
+  tab[lane + 32] = bf16_bits(f.c1);
+  __syncwarp();
+  switch (t.bits) {
+    case 2: unpack_task<2>(f.w, t, tab, wsm, n_rows, lane, half); break;
+    case 3: unpack_task<3>(f.w, t, tab, wsm, n_rows, lane, half); break;
+    case 4: unpack_task<4>(f.w, t, tab, wsm, n_rows, lane, half); break;
+    case 5: unpack_task<5>(f.w, t, tab, wsm, n_rows, lane, half); break;
+    case 6: unpack_task<6>(f.w, t, tab, wsm, n_rows, lane, half); break;
+    default: break;
+  }
+  __syncwarp();                        // the slots below are written; the table may be overwritten by the next task
+  uint32_t rc = f.rc;
+  float val = f.val;
+  for (uint32_t o = lane; o < t.n_out;) {
+    const uint32_t at = rc - t.origin, row = at >> 16, col = at & 0xffffu;
+    const bool second = t.narrow ? row >= 32 : col >= 64;
+    if (half == 0 || second == (half == 2))
+      reinterpret_cast<uint16_t*>(wsm)[(static_cast<size_t>(t.kcore0 + (col >> 3)) * n_rows + t.row0 + row) * 8 + (col & 7)] = bf16_bits(val);
+    o += 32;
+    if (o < t.n_out) {
+      rc = __ldg(reinterpret_cast<const uint32_t*>(t.codes + t.out_rc) + o);
+      val = __ldg(reinterpret_cast<const float*>(t.codes + t.out_val) + o);
+    }
   }
 }
 
@@ -266,85 +383,41 @@ __device__ __forceinline__ void prefetch_range_l2(const uint8_t* ptr, uint32_t b
 }
 
 // ---------------------------------------------------------------------------------------
-// Decode of one job's weight tile (shared by every GEMM kernel)
+// Decode of one job's weight tile by all warps of the CTA.  The first task's loads are issued by `begin`, as early as
+// the caller can; `finish` ends with the tile visible to the tensor core (proxy fence + CTA barrier).
 // ---------------------------------------------------------------------------------------
-// One outlier (Section 6: outliers keep their original value) into its slot of the decoded tile.
-__device__ __forceinline__ void patch_outlier(const Seg& sg, uint32_t off, float val, uint8_t* wsm, uint32_t n_rows,
-                                              uint32_t k_total) {
-  const uint32_t local = off - sg.flat_base;
-  const uint32_t row = local / sg.kc, kk = sg.koff + local % sg.kc;
-  if (row < n_rows && kk < k_total)
-    reinterpret_cast<uint16_t*>(wsm)[(static_cast<size_t>(kk >> 3) * n_rows + row) * 8 + (kk & 7)] = bf16_bits(val);
-}
-
-// Decodes the job's weight tile into `wsm` (all threads of the CTA; ends with the tile visible to the tensor
-// core: proxy fence + CTA barrier).  `segs` are the job's own segments.  The whole prologue is two memory
-// round trips: the segment descriptors, then - issued together - the index planes, the centroid table and
-// the outliers.  A warp keeps the table of the segment it works on (rounded once to bf16, round-to-nearest-
-// even) in its own 128 bytes of `warp_tables`, so no CTA-wide barrier sits between the loads and the unpack.
-__device__ __forceinline__ void decode_weight_tile(const Job& job, const Seg* __restrict__ segs, uint16_t* warp_tables,
-                                                   uint8_t* wsm, uint32_t tid) {
-  const uint32_t lane = tid & 31, warp = tid >> 5;
-  const uint32_t n_rows = job.n_rows, k_total = job.k_total;
-  const Seg& s0 = segs[0];
-  const uint32_t rows_per_group = s0.kc >= 128 ? 32 : 64;
-  const uint32_t chunks = s0.kc >= 128 ? s0.kc / 128 : 1;
-  const uint32_t tasks_per_seg = (n_rows / rows_per_group) * chunks;
-  const uint32_t n_tasks = tasks_per_seg * job.n_seg;
-  // outlier number `tid` of the tile (segments in order): fetched now, applied once the tile is written
-  uint32_t o_seg, o_idx, o_off = 0;
-  float o_val = 0.f;
-  const uint32_t n_out_total = find_outlier_slot(segs, job.n_seg, tid, lane, o_seg, o_idx);
-  if (o_seg != 0xffffffffu) {
-    o_off = __ldg(segs[o_seg].out_off + o_idx);
-    o_val = __ldg(segs[o_seg].out_val + o_idx);
-  }
-  uint16_t* tab = warp_tables + warp * kTableStride;
+struct TileDecode {
+  DecodeTask task;
+  TaskLoads loads;
+  uint32_t unit, half;
   // a tile with at most half as many tasks as the CTA has warps: two warps share a task (half the decode latency)
-  const bool split = 2 * n_tasks <= kWarps;
-  const uint32_t n_units = split ? 2 * n_tasks : n_tasks;
-  for (uint32_t u = warp; u < n_units; u += kWarps) {
-    const uint32_t t = split ? u >> 1 : u, half = split ? 1 + (u & 1) : 0;
-    const uint32_t si = t / tasks_per_seg, task = t % tasks_per_seg;
-    const Seg& sg = segs[si];
-    const uint32_t bits = sg.bits;
-    if (bits > 6) continue;            // raw fp32 segments are handled below
-    const uint32_t n_entries = 1u << bits;
-    const float c0 = lane < n_entries ? __ldg(sg.table + lane) : 0.f;
-    const float c1 = lane + 32 < n_entries ? __ldg(sg.table + lane + 32) : 0.f;
-    uint32_t planes[24];
-    load_planes(sg, task, lane, planes);
-    tab[lane] = bf16_bits(c0);
-    tab[lane + 32] = bf16_bits(c1);
-    __syncwarp();
-    switch (bits) {
-      case 2: unpack_task<2>(planes, sg, tab, wsm, n_rows, task, lane, half); break;
-      case 3: unpack_task<3>(planes, sg, tab, wsm, n_rows, task, lane, half); break;
-      case 4: unpack_task<4>(planes, sg, tab, wsm, n_rows, task, lane, half); break;
-      case 5: unpack_task<5>(planes, sg, tab, wsm, n_rows, task, lane, half); break;
-      case 6: unpack_task<6>(planes, sg, tab, wsm, n_rows, task, lane, half); break;
-      default: break;
-    }
-    __syncwarp();                      // the table is overwritten by the warp's next task
-  }
-  for (uint32_t si = 0; si < job.n_seg; ++si) {
-    const Seg& sg = segs[si];
-    if (sg.bits == 32) decode_raw(sg, wsm, n_rows, tid);
-  }
-  __syncthreads();
-  if (o_seg != 0xffffffffu) patch_outlier(segs[o_seg], o_off, o_val, wsm, n_rows, k_total);
-  if (n_out_total > kThreads) {        // more outliers than threads: the rest, one pass per 512
-    uint32_t base = 0;
-    for (uint32_t si = 0; si < job.n_seg; ++si) {
-      const Seg& sg = segs[si];
-      for (uint32_t o = tid; o < sg.n_out; o += kThreads)
-        if (base + o >= kThreads) patch_outlier(sg, __ldg(sg.out_off + o), __ldg(sg.out_val + o), wsm, n_rows, k_total);
-      base += sg.n_out;
+  static __device__ __forceinline__ bool split(uint32_t task_stride) { return 2 * task_stride <= kWarps; }
+  __device__ __forceinline__ void begin(const DecodeTask* tasks, uint32_t task_stride, uint32_t tid) {
+    const uint32_t lane = tid & 31, warp = tid >> 5;
+    unit = split(task_stride) ? warp >> 1 : warp;
+    half = split(task_stride) ? 1 + (warp & 1) : 0;
+    task.bits = 0;
+    if (unit < task_stride) {
+      task = load_task(tasks + unit);
+      issue_loads(task, lane, loads);
     }
   }
-  fence_proxy_async_smem();
-  __syncthreads();
-}
+  __device__ __forceinline__ void finish(const DecodeTask* tasks, uint32_t task_stride, uint16_t* warp_tables, uint8_t* wsm,
+                                         uint32_t n_rows, uint32_t tid) {
+    const uint32_t lane = tid & 31, warp = tid >> 5;
+    uint16_t* tab = warp_tables + warp * kTableStride;
+    while (unit < task_stride) {
+      finish_task(task, loads, tab, wsm, n_rows, lane, half);
+      unit += split(task_stride) ? kWarps / 2 : kWarps;
+      if (unit < task_stride) {
+        task = load_task(tasks + unit);
+        issue_loads(task, lane, loads);
+      }
+    }
+    fence_proxy_async_smem();
+    __syncthreads();
+  }
+};
 
 // ---------------------------------------------------------------------------------------
 // Two-CTA (cta_group::2) forms of the tensor-memory, TMA and MMA helpers
@@ -391,102 +464,9 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
 }
 
 
-// ---------------------------------------------------------------------------------------
-// The same decode run by a group of NWARPS warps of the CTA (the others do something else meanwhile):
-// `gtid` is the thread's index inside the group, `warp_tables` the group's first centroid table, `bar_id`
-// a named barrier reserved for the group.  Ends with the tile visible to the tensor core (proxy fence +
-// group barrier).  Every thread of the group must call it the same number of times.
-// ---------------------------------------------------------------------------------------
 template <int NWARPS>
 __device__ __forceinline__ void group_barrier(uint32_t bar_id) {
   asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(NWARPS * 32) : "memory");
-}
-
-// SPLIT: every task is shared by two warps (unit u = 2 * task + half), for tiles with fewer tasks than warps.
-template <int NWARPS, bool SPLIT = false>
-__device__ __forceinline__ void decode_weight_tile_group(const Job& job, const Seg* __restrict__ segs,
-                                                         uint16_t* warp_tables, uint8_t* wsm, uint32_t gtid,
-                                                         uint32_t bar_id) {
-  constexpr uint32_t kGroupThreads = NWARPS * 32;
-  const uint32_t lane = gtid & 31, warp = gtid >> 5;
-  const uint32_t n_rows = job.n_rows, k_total = job.k_total;
-  const Seg& s0 = segs[0];
-  const uint32_t rows_per_group = s0.kc >= 128 ? 32 : 64;
-  const uint32_t chunks = s0.kc >= 128 ? s0.kc / 128 : 1;
-  const uint32_t tasks_per_seg = (n_rows / rows_per_group) * chunks;
-  const uint32_t n_tasks = tasks_per_seg * job.n_seg;
-  uint32_t o_seg, o_idx, o_off = 0;
-  float o_val = 0.f;
-  const uint32_t n_out_total = find_outlier_slot(segs, job.n_seg, gtid, lane, o_seg, o_idx);
-  if (o_seg != 0xffffffffu) {
-    o_off = __ldg(segs[o_seg].out_off + o_idx);
-    o_val = __ldg(segs[o_seg].out_val + o_idx);
-  }
-  uint16_t* tab = warp_tables + warp * kTableStride;
-  for (uint32_t u = warp; u < (SPLIT ? 2 * n_tasks : n_tasks); u += NWARPS) {
-    const uint32_t t = SPLIT ? u >> 1 : u;
-    const uint32_t si = t / tasks_per_seg, task = t % tasks_per_seg;
-    const Seg& sg = segs[si];
-    const uint32_t bits = sg.bits;
-    if (bits > 6) continue;
-    const uint32_t n_entries = 1u << bits;
-    const float c0 = lane < n_entries ? __ldg(sg.table + lane) : 0.f;
-    const float c1 = lane + 32 < n_entries ? __ldg(sg.table + lane + 32) : 0.f;
-    uint32_t planes[24];
-    load_planes(sg, task, lane, planes);
-    tab[lane] = bf16_bits(c0);
-    tab[lane + 32] = bf16_bits(c1);
-    __syncwarp();
-    if (SPLIT) {
-      switch (bits) {
-        case 2: unpack_task<2>(planes, sg, tab, wsm, n_rows, task, lane, 1 + (u & 1)); break;
-        case 3: unpack_task<3>(planes, sg, tab, wsm, n_rows, task, lane, 1 + (u & 1)); break;
-        case 4: unpack_task<4>(planes, sg, tab, wsm, n_rows, task, lane, 1 + (u & 1)); break;
-        case 5: unpack_task<5>(planes, sg, tab, wsm, n_rows, task, lane, 1 + (u & 1)); break;
-        case 6: unpack_task<6>(planes, sg, tab, wsm, n_rows, task, lane, 1 + (u & 1)); break;
-        default: break;
-      }
-    } else {
-    switch (bits) {
-      case 2: unpack_task<2>(planes, sg, tab, wsm, n_rows, task, lane); break;
-      case 3: unpack_task<3>(planes, sg, tab, wsm, n_rows, task, lane); break;
-      case 4: unpack_task<4>(planes, sg, tab, wsm, n_rows, task, lane); break;
-      case 5: unpack_task<5>(planes, sg, tab, wsm, n_rows, task, lane); break;
-      case 6: unpack_task<6>(planes, sg, tab, wsm, n_rows, task, lane); break;
-      default: break;
-    }
-    }
-    __syncwarp();
-  }
-  for (uint32_t si = 0; si < job.n_seg; ++si) {
-    const Seg& sg = segs[si];
-    if (sg.bits == 32) {             // uncompressed version: fp32 rows, rounded to bf16 on the way in
-      const float* src = reinterpret_cast<const float*>(sg.codes);
-      const uint32_t pieces_per_row = sg.kc / 8;
-      const uint32_t total = n_rows * pieces_per_row;
-      for (uint32_t idx = gtid; idx < total; idx += kGroupThreads) {
-        const uint32_t row = idx % n_rows, piece = idx / n_rows;
-        const float4 a = __ldg(reinterpret_cast<const float4*>(src + static_cast<size_t>(row) * sg.kc + piece * 8));
-        const float4 b = __ldg(reinterpret_cast<const float4*>(src + static_cast<size_t>(row) * sg.kc + piece * 8 + 4));
-        const uint32_t kcore = (sg.koff >> 3) + piece;
-        *reinterpret_cast<uint4*>(wsm + (static_cast<size_t>(kcore) * n_rows + row) * 16) =
-            make_uint4(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w), pack_bf16x2(b.x, b.y), pack_bf16x2(b.z, b.w));
-      }
-    }
-  }
-  group_barrier<NWARPS>(bar_id);
-  if (o_seg != 0xffffffffu) patch_outlier(segs[o_seg], o_off, o_val, wsm, n_rows, k_total);
-  if (n_out_total > kGroupThreads) {
-    uint32_t base = 0;
-    for (uint32_t si = 0; si < job.n_seg; ++si) {
-      const Seg& sg = segs[si];
-      for (uint32_t o = gtid; o < sg.n_out; o += kGroupThreads)
-        if (base + o >= kGroupThreads) patch_outlier(sg, __ldg(sg.out_off + o), __ldg(sg.out_val + o), wsm, n_rows, k_total);
-      base += sg.n_out;
-    }
-  }
-  fence_proxy_async_smem();
-  group_barrier<NWARPS>(bar_id);
 }
 
 }  // namespace

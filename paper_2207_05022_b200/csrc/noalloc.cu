@@ -109,7 +109,10 @@ extern "C" sti_status sti_matrix_decode_noalloc(int device, void* stream, int bi
   for (int i = 0; i < 64; ++i) g_host_table[i] = i < (1 << bits) ? centroids[i] : 0.f;
   // the outlier lists go through library-owned pageable buffers too: the caller's arrays may be pinned, and a copy
   // out of pinned memory would still be reading them after this call has returned
-  for (size_t i = 0; i < n_outliers; ++i) { g_host_off[i] = outlier_off[i]; g_host_val[i] = outlier_val[i]; }
+  for (size_t i = 0; i < n_outliers; ++i) {
+    g_host_off[i] = outlier_off[i] / cols << 16 | outlier_off[i] % cols;        // rows and columns fit: n <= 2^20, cols >= 64, rows >= 32
+    g_host_val[i] = outlier_val[i];
+  }
   auto fail = [] { (void)cudaGetLastError(); return STI_ERR_CUDA; };      // leave no sticky error behind
   if (cudaMemcpyAsync(scratch + kOffCodes, g_host_stage, stream_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaMemcpyAsync(scratch + kOffTable, g_host_table, kTableBytes, cudaMemcpyHostToDevice, s) != cudaSuccess)
@@ -122,10 +125,9 @@ extern "C" sti_status sti_matrix_decode_noalloc(int device, void* stream, int bi
   sti::DecodeLaunch dl{};
   dl.codes = reinterpret_cast<const uint4*>(scratch + kOffCodes);
   dl.table = reinterpret_cast<const float*>(scratch + kOffTable);
-  dl.out_off = reinterpret_cast<const uint32_t*>(scratch + kOffOutOff);
+  dl.out_rc = reinterpret_cast<const uint32_t*>(scratch + kOffOutOff);
   dl.out_val = reinterpret_cast<const float*>(scratch + kOffOutVal);
   dl.n_out = static_cast<uint32_t>(n_outliers);
-  dl.flat_base = 0;
   dl.bits = static_cast<uint32_t>(bits);
   dl.rows = rows;
   dl.kc = cols;

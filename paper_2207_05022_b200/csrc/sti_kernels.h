@@ -7,28 +7,28 @@
 
 namespace sti {
 
-// One contiguous run of a unit matrix's rows feeding a weight tile.
-// Index streams are held re-tiled (see retile.h): for every group of 32 rows (64 when the
-// matrix has 64 in-features) and every 128-column chunk, the k 16-byte planes of the 32
-// per-lane quanta are stored plane-major, so that a warp reads each plane as one coalesced
-// 512-byte line and every lane ends up with 128 consecutive indexes of one row.
-struct Seg {
-  const uint4* codes;       // device; first plane of the tile's first row group (raw fp32 rows when bits == 32)
-  const float* table;       // device; 2^bits fp32 centroids (unused when bits == 32)
-  const uint32_t* out_off;  // device; outliers whose flat offset falls inside this tile
-  const float* out_val;
-  uint32_t n_out;
-  uint32_t flat_base;       // flat offset, within the unit, of the tile's first weight
-  uint32_t bits;            // 2..6 or 32
-  uint32_t kc;              // in-features (row length) of the source matrix
-  uint32_t koff;            // where this segment starts in the job's K range
-  uint32_t pad_;
+// What one warp decodes of a weight tile: 4096 weights, 32 rows x 128 columns of a unit's matrix (64 x 64 when the
+// matrix has 64 in-features).  Index streams are held re-tiled (see retile.h): the k 16-byte planes of the 32 lanes'
+// quanta are stored plane-major, so that a warp reads each plane as one coalesced 512-byte line and every lane ends up
+// with 128 consecutive indexes of one row.  Everything the warp needs to issue its loads stands in these 32 bytes: one
+// memory round trip for the descriptor, one for planes, table and outliers together.
+struct alignas(16) DecodeTask {
+  const uint8_t* codes;     // device; first plane (uncompressed units: the fp32 rows, `out_val` bytes apart)
+  uint32_t table;           // byte distances from `codes`: the unit's 2^bits fp32 centroids,
+  uint32_t out_rc;          //   the task's outliers as (row << 16 | column) of the matrix,
+  uint32_t out_val;         //   and their values
+  uint16_t n_out;
+  uint8_t bits;             // 2..6 or 32; 0 = no task
+  uint8_t narrow;           // 1: 64 rows x 64 columns
+  uint16_t row0, kcore0;    // place in the tile: first row, first group of eight columns
+  uint32_t origin;          // (row << 16 | column) of the task's first weight in the matrix
 };
+static_assert(sizeof(DecodeTask) == 32, "two 16-byte loads");
 
 // One weight-stationary tile: n_rows output features x k_total input features.
 struct Job {
-  uint32_t seg_begin, n_seg;
-  uint32_t n_rows;          // 32, 64 or 128 (multiple of 64 when segments have kc == 64)
+  uint32_t task_begin, n_tasks;
+  uint32_t n_rows;          // 32, 64 or 128 (multiple of 64 when the matrices have 64 in-features)
   uint32_t k_total;         // multiple of 64
   uint32_t x_koff;          // first column of the activation operand
   uint32_t out_mat;         // output element (t, c) goes to out[(out_mat*T + t)*ldo + out_col + c]
@@ -44,7 +44,7 @@ enum GemmKind : int {
 
 struct GemmLaunch {
   const Job* jobs;
-  const Seg* segs;
+  const DecodeTask* tasks;
   int n_jobs;
   int m_ctas;               // CTAs along the token dimension (each loops over its M tiles)
   CUtensorMap xmap;         // TMA descriptor of x: [T rows, ldx columns] bf16, box 64 x 128, 128-byte swizzle
@@ -60,7 +60,7 @@ struct GemmLaunch {
   uint32_t bps;             // 16 KB boxes (64 columns) per stage: 1, 2 or 4
   uint32_t w_bytes;         // shared memory reserved for the weight tile (largest job)
   uint32_t hdr_bytes;       // barriers + bias + per-warp centroid tables
-  uint32_t seg_stride;      // the segments of job j start at segs[j * seg_stride]
+  uint32_t task_stride;     // the tasks of job j start at tasks[j * task_stride], unused ones have bits == 0
   const uint8_t* pf_ptr[4]; // what the next layer reads first (packed shards, tile descriptors, dense parameters):
   uint32_t pf_bytes[4];     // pulled into L2 by this launch's idle warps
   bool simt_debug;          // compute the products on the plain ALUs instead of the tensor cores
@@ -78,10 +78,10 @@ cudaError_t launch_gemm(GemmKind kind, const GemmLaunch& p, cudaStream_t s);
 
 // K-accumulating two-CTA dequant-GEMM (fp32 output written once, all K groups summed in tensor memory).
 // jobs: n_groups x n_cols64 tile jobs of 64 rows and at most k_group columns, job (g, c) at index g * n_cols64 + c,
-// segments at the fixed stride; out: [T][ldo] fp32, tile c writes columns [64 c, 64 c + 64).
+// tasks at the fixed stride; out: [T][ldo] fp32, tile c writes columns [64 c, 64 c + 64).
 struct KaccLaunch {
   const Job* jobs;
-  const Seg* segs;
+  const DecodeTask* tasks;
   int n_groups, n_cols64, m_ctas;
   CUtensorMap xmap;         // x: [T rows, ldx columns] bf16, box 64 x 128, 128-byte swizzle
   const void* x;            // the same operand as a plain pointer: idle warps prefetch it into L2; null = no prefetch
@@ -90,7 +90,7 @@ struct KaccLaunch {
   float* out;
   int ldo;
   int* err;
-  uint32_t n_stages, bps, hdr_bytes, seg_stride;   // ring: n_stages stages of bps boxes (1 or 2; K groups are multiples of 64 * bps)
+  uint32_t n_stages, bps, hdr_bytes, task_stride;   // ring: n_stages stages of bps boxes (1 or 2; K groups are multiples of 64 * bps)
   uint32_t k_group;         // columns of the widest K group (a multiple of 64): the size of the two weight buffers
   bool pdl;
   unsigned long long* stamps;
@@ -140,10 +140,9 @@ cudaError_t launch_cast_bf16(const float* in, uint16_t* out, size_t n, cudaStrea
 struct DecodeLaunch {
   const uint4* codes;       // re-tiled stream of the matrix (raw fp32 when bits == 32)
   const float* table;
-  const uint32_t* out_off;  // the unit's outliers restricted to this matrix
+  const uint32_t* out_rc;   // the matrix's outliers: row << 16 | column
   const float* out_val;
   uint32_t n_out;
-  uint32_t flat_base;       // flat offset of the matrix inside the unit
   uint32_t bits, rows, kc;
   float* w;                 // optional outputs
   uint8_t* codes_out;

@@ -30,68 +30,34 @@ namespace {
 // The kernel
 // ---------------------------------------------------------------------------------------
 // One accumulator tile's columns [half * ncol, (half + 1) * ncol) of this warp's 32 token rows: TMEM -> bias / erf-GELU -> global.
-// FEW (at most two token tiles per CTA): eight columns per step in a rolled loop - the epilogue then runs once or twice
-// per CTA, its instructions are fetched cold, and the kernel's code size is what it costs.  Otherwise 32 columns per step,
-// unrolled (each thread writes 128 or 64 contiguous bytes of its row).
+// FEW (at most two token tiles per CTA): the loop over blocks of 16 columns stays rolled - the epilogue then runs once or
+// twice per CTA, its instructions are fetched cold, and the kernel's code size is what it costs.
+// `first`: the row group_row(t) of the output at the tile's first column; rows_left counted from it.
+template <typename OutT, bool GELU>
+__device__ __forceinline__ void epilogue_block(uint32_t taddr, uint32_t col, const float* bias_sm, OutT* first, int ldo, int rows_left,
+                                               uint32_t lane) {
+  uint32_t r[16];
+  tmem_ld_32x32b_x16(taddr + col, r);
+  tc_wait_ld();
+  float v[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const float a = __uint_as_float(r[i]) + bias_sm[col + i];
+    v[i] = GELU ? gelu_erf(a) : a;
+  }
+  store_block16<OutT>(v, first + col, ldo, rows_left, lane);
+}
 template <typename OutT, bool GELU, bool FEW>
-__device__ __forceinline__ void epilogue_tile(uint32_t taddr, uint32_t half, uint32_t ncol, const float* bias_sm, OutT* drow,
-                                              bool row_ok) {
+__device__ __forceinline__ void epilogue_tile(uint32_t taddr, uint32_t half, uint32_t ncol, const float* bias_sm, OutT* first, int ldo,
+                                              int rows_left, uint32_t lane) {
   if constexpr (FEW) {
 #pragma unroll 1
-    for (uint32_t col = half * ncol; col < (half + 1) * ncol; col += 8) {
-      uint32_t r[8];
-      tmem_ld_32x32b_x8(taddr + col, r);
-      tc_wait_ld();
-      float v[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float a = __uint_as_float(r[i]) + bias_sm[col + i];
-        v[i] = GELU ? gelu_erf(a) : a;
-      }
-      if constexpr (sizeof(OutT) == 2) {
-        const uint4 o = make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
-                                   pack_bf16x2(v[6], v[7]));
-        if (row_ok) *reinterpret_cast<uint4*>(drow + col) = o;
-      } else {
-        if (row_ok) {
-          reinterpret_cast<float4*>(drow + col)[0] = make_float4(v[0], v[1], v[2], v[3]);
-          reinterpret_cast<float4*>(drow + col)[1] = make_float4(v[4], v[5], v[6], v[7]);
-        }
-      }
-    }
+    for (uint32_t col = half * ncol; col < (half + 1) * ncol; col += 16)
+      epilogue_block<OutT, GELU>(taddr, col, bias_sm, first, ldo, rows_left, lane);
   } else {
-    for (uint32_t col = half * ncol; col < (half + 1) * ncol; col += 32) {
-      if (col + 32 > (half + 1) * ncol) {            // 16-column tail of 32-row tiles
-        uint32_t r[16];
-        tmem_ld_32x32b_x16(taddr + col, r);
-        tc_wait_ld();
-        if (row_ok) {
-          float v[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float a = __uint_as_float(r[i]) + bias_sm[col + i];
-            v[i] = GELU ? gelu_erf(a) : a;
-          }
-          store_row16<OutT>(drow + col, v);
-        }
-        break;
-      }
-      uint32_t r[32];
-      tmem_ld_32x32b_x32(taddr + col, r);
-      tc_wait_ld();
-      if (row_ok) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float v[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float a = __uint_as_float(r[h * 16 + i]) + bias_sm[col + h * 16 + i];
-            v[i] = GELU ? gelu_erf(a) : a;
-          }
-          store_row16<OutT>(drow + col + h * 16, v);
-        }
-      }
-    }
+#pragma unroll 2
+    for (uint32_t col = half * ncol; col < (half + 1) * ncol; col += 16)
+      epilogue_block<OutT, GELU>(taddr, col, bias_sm, first, ldo, rows_left, lane);
   }
 }
 
@@ -230,7 +196,7 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
               v[c] = GELU ? gelu_erf(a) : a;
             }
             OutT* dst = out + (static_cast<size_t>(job.out_mat) * T + t) * ldo + job.out_col + chalf * ncol + cb * 16;
-            store_row16<OutT>(dst, v);
+            for (int c = 0; c < 16; ++c) dst[c] = static_cast<OutT>(v[c]);
           }
         }
       }
@@ -322,19 +288,22 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
         if (!ok) { failed = true; break; }
         tc_fence_after_sync();
         const int t = static_cast<int>((blockIdx.y + ti * gridDim.y) * kTileM + q * 32 + lane);
-        const size_t row_off = (static_cast<size_t>(job.out_mat) * T + (t < T ? t : 0)) * ldo + job.out_col;
         const uint32_t taddr = tmem_base + ((q * 32) << 16) + buf * n_rows;
+        auto drain = [&](auto* to, auto gelu) {
+          using Out = std::remove_pointer_t<decltype(to)>;
+          const int row = group_row<Out>(t, lane);           // past the end for the last tile's padding: nothing is stored
+          epilogue_tile<Out, decltype(gelu)::value, FEW>(
+              taddr, half, ncol, bias_sm, to + (static_cast<size_t>(job.out_mat) * T + (row < T ? row : 0)) * ldo + job.out_col, ldo,
+              T - row, lane);
+        };
         if constexpr (std::is_void<OutT>::value) {
           // one kernel for every GEMM of a layer: the output kind is a launch parameter, the code stays in the
           // instruction caches from launch to launch
-          if (kind == GEMM_BF16_TO_F32)
-            epilogue_tile<float, false, FEW>(taddr, half, ncol, bias_sm, static_cast<float*>(out) + row_off, t < T);
-          else if (kind == GEMM_BF16_TO_BF16_GELU)
-            epilogue_tile<__nv_bfloat16, true, FEW>(taddr, half, ncol, bias_sm, static_cast<__nv_bfloat16*>(out) + row_off, t < T);
-          else
-            epilogue_tile<__nv_bfloat16, false, FEW>(taddr, half, ncol, bias_sm, static_cast<__nv_bfloat16*>(out) + row_off, t < T);
+          if (kind == GEMM_BF16_TO_F32) drain(static_cast<float*>(out), std::false_type());
+          else if (kind == GEMM_BF16_TO_BF16_GELU) drain(static_cast<__nv_bfloat16*>(out), std::true_type());
+          else drain(static_cast<__nv_bfloat16*>(out), std::false_type());
         } else {
-          epilogue_tile<OutT, GELU, FEW>(taddr, half, ncol, bias_sm, out + row_off, t < T);
+          drain(out, std::integral_constant<bool, GELU>());
         }
         tc_fence_before_sync();
         __syncwarp();
@@ -527,28 +496,27 @@ dqgemm_pair_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
       if (!ok) { failed = true; break; }
       tc_fence_after_sync();
       const int t = tile_row0(ti) + static_cast<int>(q * 32 + lane);
-      const size_t trow = static_cast<size_t>(t < T ? t : 0);
-      OutT* drow0 = out + (static_cast<size_t>(job0.out_mat) * T + trow) * ldo + job0.out_col;
-      OutT* drow1 = out + (static_cast<size_t>(job1.out_mat) * T + trow) * ldo + job1.out_col;
+      const int row = group_row<OutT>(t, lane);
+      const size_t trow = static_cast<size_t>(row < T ? row : 0);
+      OutT* first0 = out + (static_cast<size_t>(job0.out_mat) * T + trow) * ldo + job0.out_col;
+      OutT* first1 = out + (static_cast<size_t>(job1.out_mat) * T + trow) * ldo + job1.out_col;
       const uint32_t taddr = tmem_base + ((q * 32) << 16) + buf * kAccCols;
       uint32_t r[3][16];
 #pragma unroll
       for (uint32_t c = 0; c < 3; ++c)
         if (chunk0 + c < chunk1) tmem_ld_32x32b_x16(taddr + (chunk0 + c) * 16, r[c]);
       tc_wait_ld();
-      if (t < T) {
 #pragma unroll
-        for (uint32_t c = 0; c < 3; ++c) {
-          if (chunk0 + c < chunk1) {
-            const uint32_t col = (chunk0 + c) * 16;            // 0..127: the first 64 are job 0's features
-            float v[16];
+      for (uint32_t c = 0; c < 3; ++c) {
+        if (chunk0 + c < chunk1) {
+          const uint32_t col = (chunk0 + c) * 16;            // 0..127: the first 64 are job 0's features
+          float v[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float a = __uint_as_float(r[c][i]) + bias_sm[col + i];
-              v[i] = GELU ? gelu_erf(a) : a;
-            }
-            store_row16<OutT>((col < 64 ? drow0 : drow1) + (col & 63), v);
+          for (int i = 0; i < 16; ++i) {
+            const float a = __uint_as_float(r[c][i]) + bias_sm[col + i];
+            v[i] = GELU ? gelu_erf(a) : a;
           }
+          store_block16<OutT>(v, (col < 64 ? first0 : first1) + (col & 63), ldo, T - row, lane);
         }
       }
       tc_fence_before_sync();

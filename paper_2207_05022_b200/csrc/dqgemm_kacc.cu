@@ -309,22 +309,18 @@ dqgemm_kacc_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
         wait_uniform(smem_addr(&hdr->acc_full[t]), blk & 1);
         tc_fence_after_sync();
         const int row = tile_row0(blk * kKaccTiles + t) + static_cast<int>(q * 32 + lane);
-        float* drow = out + static_cast<size_t>(row < T ? row : 0) * ldo + pair_base * 64 + half * 64;
+        const int first_row = group_row<float>(row, lane);
+        float* first = out + static_cast<size_t>(first_row < T ? first_row : 0) * ldo + pair_base * 64 + half * 64;
         const uint32_t taddr = tmem_base + ((q * 32) << 16) + t * kKaccAccCols + half * 64;
-#pragma unroll
-        for (uint32_t col = 0; col < 64; col += 32) {
-          uint32_t r[32];
-          tmem_ld_32x32b_x32(taddr + col, r);
+#pragma unroll 1
+        for (uint32_t col = 0; col < 64; col += 16) {
+          uint32_t r[16];
+          tmem_ld_32x32b_x16(taddr + col, r);
           tc_wait_ld();
-          if (row < T) {
+          float v[16];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              float v[16];
-#pragma unroll
-              for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[h * 16 + i]);
-              store_row16<float>(drow + col + h * 16, v);
-            }
-          }
+          for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+          store_block16<float>(v, first + col, ldo, T - first_row, lane);
         }
         tc_fence_before_sync();
         __syncwarp();

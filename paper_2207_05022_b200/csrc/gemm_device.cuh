@@ -348,20 +348,45 @@ __device__ __forceinline__ float gelu_erf(float v) {
   return fmaf(fabsf(h), erf_abs, h);
 }
 
+// 16 output columns of the warp's 32 rows: every lane comes with its own row's values, and the lanes of a group of G (two
+// for bf16, four for fp32) exchange 16-byte pieces so that a store covers whole 32- or 64-byte runs of fewer rows.  A lane
+// per row touches 32 lines with every store, and the load/store unit takes a cycle for each: 4096 cycles for a 128 x 128
+// fp32 tile, as long as 64 of its MMAs take.
+// `first` = row (lane - lane % G) of the output at the block's first column; rows_left = how many rows from there exist.
 template <typename OutT>
-__device__ __forceinline__ void store_row16(OutT* dst, const float (&v)[16]) {
-  if constexpr (sizeof(OutT) == 2) {
-    uint32_t p[8];
+__device__ __forceinline__ void store_block16(const float (&v)[16], OutT* first, int ldo, int rows_left, uint32_t lane) {
+  constexpr uint32_t G = sizeof(OutT) == 2 ? 2 : 4;
+  uint4 c[G];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) p[i] = pack_bf16x2(v[2 * i], v[2 * i + 1]);
-    reinterpret_cast<uint4*>(dst)[0] = make_uint4(p[0], p[1], p[2], p[3]);
-    reinterpret_cast<uint4*>(dst)[1] = make_uint4(p[4], p[5], p[6], p[7]);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      reinterpret_cast<float4*>(dst)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+  for (uint32_t i = 0; i < G; ++i) {
+    if constexpr (sizeof(OutT) == 2)
+      c[i] = make_uint4(pack_bf16x2(v[8 * i], v[8 * i + 1]), pack_bf16x2(v[8 * i + 2], v[8 * i + 3]),
+                        pack_bf16x2(v[8 * i + 4], v[8 * i + 5]), pack_bf16x2(v[8 * i + 6], v[8 * i + 7]));
+    else
+      c[i] = make_uint4(__float_as_uint(v[4 * i]), __float_as_uint(v[4 * i + 1]), __float_as_uint(v[4 * i + 2]), __float_as_uint(v[4 * i + 3]));
   }
+#pragma unroll
+  for (uint32_t step = 1; step < G; step <<= 1) {      // piece i of lane j <-> piece j of lane i, a bit at a time
+    const bool up = (lane & step) != 0;
+#pragma unroll
+    for (uint32_t i = 0; i < G; ++i) {
+      if (i & step) continue;
+      uint4 &lo = c[i], &hi = c[i | step];
+      const uint4 give = up ? lo : hi;
+      uint4 got;
+      got.x = __shfl_xor_sync(0xffffffffu, give.x, step); got.y = __shfl_xor_sync(0xffffffffu, give.y, step);
+      got.z = __shfl_xor_sync(0xffffffffu, give.z, step); got.w = __shfl_xor_sync(0xffffffffu, give.w, step);
+      if (up) lo = got; else hi = got;
+    }
+  }
+  OutT* dst = first + (lane & (G - 1)) * (16 / sizeof(OutT));
+#pragma unroll
+  for (uint32_t i = 0; i < G; ++i)
+    if (static_cast<int>(i) < rows_left) *reinterpret_cast<uint4*>(dst + static_cast<size_t>(i) * ldo) = c[i];
 }
+// The first row of the lane's exchange group.
+template <typename OutT>
+__device__ __forceinline__ int group_row(int t, uint32_t lane) { return t - static_cast<int>(lane & (sizeof(OutT) == 2 ? 1u : 3u)); }
 
 struct PrefetchRanges {
   const uint8_t* ptr[4];

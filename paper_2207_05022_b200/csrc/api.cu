@@ -45,7 +45,6 @@ struct Tuning {
   int f2_kacc_k = 512;                 // columns per K group there
   int f2_kacc_bps = 2;                 // boxes of 64 columns per ring stage there (1 or 2)
   int attn_tc_min_items = 96;          // tensor-core attention from this many (sequence, kept head) pairs on, seq >= 256 (0 = never)
-  int ln1_ctas = -1, ln2_ctas = -1;    // LayerNorm CTA counts: -1 = chosen per launch (see ln_ctas_hint), 0 = one row per CTA
 };
 
 struct Unit {
@@ -230,8 +229,6 @@ void parse_tuning(Tuning* t, int tmax, const sti_model_desc& d, int sm_count) {
         else if (k == "f2_kacc_bps") t->f2_kacc_bps = v == 1 ? 1 : 2;
         else if (k == "attn_tc_min_items") t->attn_tc_min_items = std::max(0, v);
         else if (k == "cta_budget") t->cta_budget = std::max(1, v);
-        else if (k == "ln1_ctas") t->ln1_ctas = std::max(-1, v);
-        else if (k == "ln2_ctas") t->ln2_ctas = std::max(-1, v);
       }
       pos = end + 1;
     }
@@ -544,18 +541,6 @@ sti_status run_gemm_kacc(sti_plan* p, const GemmTable& tab, const void* x, int l
   return STI_OK;
 }
 
-// How many CTAs a LayerNorm launch should use, given the GEMM that follows it.  A GEMM CTA needs a whole SM and its
-// CTAs are launched while the LayerNorm runs (they decode their weights meanwhile) - on SMs that hold no LayerNorm
-// CTA.  With one row per CTA the LayerNorm of a few hundred tokens spreads over about 64 SMs; when the next GEMM
-// wants more than the SMs it leaves free (84 of a B200's 148), its last CTAs start late and their decode lands on the critical path.  Then the
-// rows are packed into fewer CTAs (measured: 54.6 -> 50.5 us per BERT-large layer at 256 tokens; at 512 tokens
-// packing loses 1-3 us, at BERT-base sizes it changes nothing).  Otherwise one row per CTA.
-int ln_ctas_hint(int tuned, int T, int next_gemm_ctas, int sm_count) {
-  if (tuned >= 0) return tuned;
-  if (T > 256 || next_gemm_ctas <= sm_count - 64) return 0;      // at 512 tokens the packed LayerNorm itself costs more than it frees
-  return std::max(32, sm_count - next_gemm_ctas);
-}
-
 // The seven kernels of one layer on the compute stream.
 // `x_ready_bf16`: the bf16 copy of x already sits in p->x_bf16 (written by the previous layer's LayerNorm);
 // `want_next_bf16`: this layer's last kernel also writes y as bf16 into p->x_bf16 for the next layer.
@@ -617,7 +602,6 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     // With bf16 activations every activation that crosses a kernel boundary is bf16 (the layer's input and output are):
     // the second LayerNorm then takes its residual from the bf16 copy the FFN reads, and no fp32 copy is written.
     ln.out_f32 = bf16_act ? nullptr : p->h1_f32; ln.out_bf16 = p->h1_bf16;
-    ln.ctas_hint = ln_ctas_hint(p->tune.ln1_ctas, T, ns > 0 ? L.f1.n_jobs * m_ctas_for(L.f1.n_jobs, T, p->tune.cta_budget) : 0, c->sm_count);
     ln.stamps = stamp(4);
     CUDA_TRY(launch_layernorm(ln, c->compute, c->pdl));
     c->launches++;
@@ -648,15 +632,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   l2.gamma = dense + c->off_ln2g; l2.beta = dense + c->off_ln2b; l2.eps = d.ln_eps; l2.T = T; l2.d = d.hidden;
   l2.out_f32 = bf16_act ? nullptr : static_cast<float*>(y);
   l2.out_bf16 = bf16_act ? static_cast<uint16_t*>(y) : (want_next_bf16 ? p->x_bf16 : nullptr);
-  {
-    int next_ctas = 0;
-    if (next_layer >= 0 && next_layer < static_cast<int>(p->layers.size())) {
-      const GemmTable& q = p->layers[next_layer].qkv;
-      next_ctas = q.n_jobs * m_ctas_for(q.n_jobs, T, p->tune.cta_budget);
-    }
-    l2.ctas_hint = ln_ctas_hint(p->tune.ln2_ctas, T, next_ctas, c->sm_count);
-    l2.stamps = stamp(7);
-  }
+  l2.stamps = stamp(7);
   CUDA_TRY(launch_layernorm(l2, c->compute, c->pdl));
   c->launches++;
   L.k_ran[6] = true;

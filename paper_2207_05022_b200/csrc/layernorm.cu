@@ -1,9 +1,7 @@
 // Residual + bias + LayerNorm over the split-K partial sums of the O projection and of FFN2
 // (Section 2.1; Section 6: biases and layernorm parameters stay in fp32).
-// One CTA per token row, one float4 per thread (hidden / 4 threads): every load of a row is in
-// flight at once; mean and variance are two-pass over registers with a block reduction.
-#include <algorithm>
-
+// Up to 2048 rows of at most 1024: 128 threads to a row.  More rows: a
+// warp per row.  Wider rows: one CTA per row, one float4 per thread.
 #include <cuda_bf16.h>
 
 #include "sti_device.cuh"
@@ -78,104 +76,104 @@ layernorm_kernel(LnLaunch p) {
   }
 }
 
-// Few tokens: the same arithmetic with several rows per CTA and several float4 per thread, so that the kernel
-// sits on a handful of SMs only.  A GEMM CTA needs a whole SM; the CTAs of the GEMM that follows are launched while
-// this kernel runs (programmatic dependent launch) and decode their weights meanwhile - but only on SMs that hold
-// none of this kernel's CTAs.  A row is handled by `wpr` warps (named barrier = row slot, 0..15; the kernel uses
-// no CTA-wide barrier), thread t of the row holds float4 number t, t + tpr, ... of it.
-constexpr int kLnMaxV = 4;
-template <int V>
-__global__ void __launch_bounds__(1024)
-layernorm_rows_kernel(LnLaunch p, int tpr, int rows_per_cta) {
-  __shared__ float red_all[16][16];
-  const int slot = threadIdx.x / tpr, tid = threadIdx.x % tpr;
-  const int n_warps = tpr >> 5;
-  const int r = blockIdx.x * rows_per_cta + slot;
+// Up to 2048 rows of at most 1024: a CTA of 128 threads per row, two float4 each.
+// Bound: latency.  Residual and the first four partial-sum planes are in flight together, gamma and beta while the row is
+// reduced: two memory round trips and two exchanges between four warps per row (one float4 per thread and one plane at a
+// time took five trips; BERT-large, 256 tokens 5.1 -> 3.7 and 6.5 -> 5.9 us, 1024 tokens 5.6 -> 3.4 and 7.1 -> 6.1,
+// BERT-base, 128 tokens 2.8 -> 2.1 and 3.8 -> 3.1).  Small CTAs also leave an SM sooner: the next GEMM's CTAs, which need a
+// whole one and decode their weights meanwhile, start earlier than with rows packed into large CTAs on fewer SMs.
+constexpr uint32_t kLnGroup = 128;
+constexpr int kLnGroupMaxHidden = 1024;
+__global__ void __launch_bounds__(kLnGroup)
+layernorm_group_kernel(LnLaunch p) {
+  __shared__ float red[8];
+  const uint32_t gt = threadIdx.x, row = blockIdx.x;
   pdl_launch_dependents();
-  if (threadIdx.x == 0) { stamp_min(p.stamps, STAMP_FIRST_START); stamp_max(p.stamps, STAMP_LAST_START); }
-  if (slot >= rows_per_cta || r >= p.T) {      // whole warps: tpr is a multiple of 32
-    pdl_wait();
-    return;
-  }
-  float* red = red_all[slot];
-  const size_t row = static_cast<size_t>(r) * p.d;
-  float4 a[V];
+  if (gt == 0) { stamp_min(p.stamps, STAMP_FIRST_START); stamp_max(p.stamps, STAMP_LAST_START); }
+  const uint32_t lane = gt & 31, w = gt >> 5, n4 = static_cast<uint32_t>(p.d) / 4;
+  const size_t base = static_cast<size_t>(row) * p.d, pstride = static_cast<size_t>(p.T) * p.d;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  const bool on[2] = {gt < n4, gt + kLnGroup < n4};
+  auto plane = [&](int q, int v) {
+    return on[v] && q < p.n_partial ? *reinterpret_cast<const float4*>(p.partial + q * pstride + base + 4 * (gt + kLnGroup * v)) : zero;
+  };
+  auto add4 = [](float4& a, const float4 (&s)[4]) {
+    a.x += (s[0].x + s[1].x) + (s[2].x + s[3].x); a.y += (s[0].y + s[1].y) + (s[2].y + s[3].y);
+    a.z += (s[0].z + s[1].z) + (s[2].z + s[3].z); a.w += (s[0].w + s[1].w) + (s[2].w + s[3].w);
+  };
+  float4 bias[2];
 #pragma unroll
-  for (int v = 0; v < V; ++v) a[v] = __ldg(reinterpret_cast<const float4*>(p.bias + (tid + v * tpr) * 4));
+  for (int v = 0; v < 2; ++v) bias[v] = on[v] ? __ldg(reinterpret_cast<const float4*>(p.bias) + gt + kLnGroup * v) : zero;
   pdl_wait();
-  if (tid == 0) stamp_min(p.stamps, STAMP_RELEASE);
-  const size_t pstride = static_cast<size_t>(p.T) * p.d;
+  if (gt == 0) stamp_min(p.stamps, STAMP_RELEASE);
+  float4 a[2];
+  {
+    float4 r[2] = {zero, zero}, s[2][4];
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
-    {
-      const int c = (tid + v * tpr) * 4;
-      if (p.resid_bf16) {
-        const uint2 rr = __ldg(reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(p.resid) + row + c));
-        a[v].x += __uint_as_float(rr.x << 16); a[v].y += __uint_as_float(rr.x & 0xffff0000u);
-        a[v].z += __uint_as_float(rr.y << 16); a[v].w += __uint_as_float(rr.y & 0xffff0000u);
-      } else {
-        const float4 rr = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(p.resid) + row + c));
-        a[v].x += rr.x; a[v].y += rr.y; a[v].z += rr.z; a[v].w += rr.w;
+    for (int v = 0; v < 2; ++v) {
+      const uint32_t c = gt + kLnGroup * v;
+      if (on[v]) {
+        if (p.resid_bf16) {
+          const uint2 t = *reinterpret_cast<const uint2*>(static_cast<const uint16_t*>(p.resid) + base + 4 * c);
+          r[v] = make_float4(__uint_as_float(t.x << 16), __uint_as_float(t.x & 0xffff0000u), __uint_as_float(t.y << 16), __uint_as_float(t.y & 0xffff0000u));
+        } else {
+          r[v] = *reinterpret_cast<const float4*>(static_cast<const float*>(p.resid) + base + 4 * c);
+        }
       }
-      int q = 0;
-#pragma unroll 1
-      for (; q + 4 <= p.n_partial; q += 4) {          // same grouping of the partial sums as the one-row kernel
-        const float4 s0 = __ldg(reinterpret_cast<const float4*>(p.partial + (q + 0) * pstride + row + c));
-        const float4 s1 = __ldg(reinterpret_cast<const float4*>(p.partial + (q + 1) * pstride + row + c));
-        const float4 s2 = __ldg(reinterpret_cast<const float4*>(p.partial + (q + 2) * pstride + row + c));
-        const float4 s3 = __ldg(reinterpret_cast<const float4*>(p.partial + (q + 3) * pstride + row + c));
-        a[v].x += (s0.x + s1.x) + (s2.x + s3.x); a[v].y += (s0.y + s1.y) + (s2.y + s3.y);
-        a[v].z += (s0.z + s1.z) + (s2.z + s3.z); a[v].w += (s0.w + s1.w) + (s2.w + s3.w);
-      }
-#pragma unroll 1
-      for (; q < p.n_partial; ++q) {
-        const float4 s = __ldg(reinterpret_cast<const float4*>(p.partial + q * pstride + row + c));
-        a[v].x += s.x; a[v].y += s.y; a[v].z += s.z; a[v].w += s.w;
-      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) s[v][q] = plane(q, v);
+    }
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      a[v] = make_float4(bias[v].x + r[v].x, bias[v].y + r[v].y, bias[v].z + r[v].z, bias[v].w + r[v].w);
+      add4(a[v], s[v]);
     }
   }
-  auto row_sum = [&](float v) {
+#pragma unroll 1
+  for (int q0 = 4; q0 < p.n_partial; q0 += 4) {
+    float4 s[2][4];
+#pragma unroll
+    for (int v = 0; v < 2; ++v)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) s[v][q] = plane(q0 + q, v);
+#pragma unroll
+    for (int v = 0; v < 2; ++v) add4(a[v], s[v]);
+  }
+  float4 gamma[2], beta[2];
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    gamma[v] = on[v] ? __ldg(reinterpret_cast<const float4*>(p.gamma) + gt + kLnGroup * v) : zero;
+    beta[v] = on[v] ? __ldg(reinterpret_cast<const float4*>(p.beta) + gt + kLnGroup * v) : zero;
+  }
+  auto row_sum = [&](float v, float* slot) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((tid & 31) == 0) red[tid >> 5] = v;
-    asm volatile("bar.sync %0, %1;" ::"r"(slot), "r"(tpr) : "memory");
-    float t = 0.f;
-#pragma unroll 1
-    for (int w = 0; w < n_warps; ++w) t += red[w];
-    asm volatile("bar.sync %0, %1;" ::"r"(slot), "r"(tpr) : "memory");
-    return t;
+    if (lane == 0) slot[w] = v;
+    __syncthreads();
+    return (slot[0] + slot[1]) + (slot[2] + slot[3]);
   };
-  float part = 0.f;
+  const float inv_d = 1.f / static_cast<float>(p.d);
+  const float mean = __fmul_rn(row_sum(((a[0].x + a[0].y) + (a[0].z + a[0].w)) + ((a[1].x + a[1].y) + (a[1].z + a[1].w)), red), inv_d);
+  float sq = 0.f;
 #pragma unroll
-  for (int v = 0; v < V; ++v) part += a[v].x + a[v].y + a[v].z + a[v].w;
-  const float mean = row_sum(part) / static_cast<float>(p.d);
-  part = 0.f;
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    {
-      a[v].x -= mean; a[v].y -= mean; a[v].z -= mean; a[v].w -= mean;
-      part += a[v].x * a[v].x + a[v].y * a[v].y + a[v].z * a[v].z + a[v].w * a[v].w;
-    }
+  for (int v = 0; v < 2; ++v) {
+    a[v].x -= mean; a[v].y -= mean; a[v].z -= mean; a[v].w -= mean;
+    if (on[v]) sq = fmaf(a[v].x, a[v].x, fmaf(a[v].y, a[v].y, fmaf(a[v].z, a[v].z, fmaf(a[v].w, a[v].w, sq))));
   }
-  const float var = row_sum(part) / static_cast<float>(p.d);
-  const float rstd = rsqrtf(var + p.eps);
+  const float rstd = rsqrtf(fmaf(row_sum(sq, red + 4), inv_d, p.eps));
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
-    {
-      const int c = (tid + v * tpr) * 4;
-      const float4 g = __ldg(reinterpret_cast<const float4*>(p.gamma + c));
-      const float4 b = __ldg(reinterpret_cast<const float4*>(p.beta + c));
-      float4 y;
-      y.x = a[v].x * rstd * g.x + b.x; y.y = a[v].y * rstd * g.y + b.y;
-      y.z = a[v].z * rstd * g.z + b.z; y.w = a[v].w * rstd * g.w + b.w;
-      if (p.out_f32) *reinterpret_cast<float4*>(p.out_f32 + row + c) = y;
-      if (p.out_bf16)
-        *reinterpret_cast<uint2*>(p.out_bf16 + row + c) = make_uint2(pack_bf16x2(y.x, y.y), pack_bf16x2(y.z, y.w));
-    }
+  for (int v = 0; v < 2; ++v) {
+    if (!on[v]) continue;
+    const uint32_t c = gt + kLnGroup * v;
+    float4 y;
+    y.x = fmaf(__fmul_rn(a[v].x, rstd), gamma[v].x, beta[v].x); y.y = fmaf(__fmul_rn(a[v].y, rstd), gamma[v].y, beta[v].y);
+    y.z = fmaf(__fmul_rn(a[v].z, rstd), gamma[v].z, beta[v].z); y.w = fmaf(__fmul_rn(a[v].w, rstd), gamma[v].w, beta[v].w);
+    if (p.out_f32) *reinterpret_cast<float4*>(p.out_f32 + base + 4 * c) = y;
+    if (p.out_bf16) *reinterpret_cast<uint2*>(p.out_bf16 + base + 4 * c) = make_uint2(pack_bf16x2(y.x, y.y), pack_bf16x2(y.z, y.w));
   }
   if (p.stamps != nullptr) {
-    asm volatile("bar.sync %0, %1;" ::"r"(slot), "r"(tpr) : "memory");
-    if (tid == 0) stamp_max(p.stamps, STAMP_LAST_END);
+    __syncthreads();
+    if (gt == 0) stamp_max(p.stamps, STAMP_LAST_END);
   }
 }
 
@@ -282,27 +280,6 @@ __global__ void cast_bf16_kernel(const float* __restrict__ in, uint16_t* __restr
 cudaError_t launch_layernorm(const LnLaunch& p, cudaStream_t s, bool pdl) {
   if (p.T <= 0) return cudaSuccess;
   if (p.d % 128 != 0 || p.d > 2048) return cudaErrorInvalidValue;     // d / 4 threads, whole warps
-  if (p.ctas_hint > 0 && p.ctas_hint < p.T) {
-    // the widest row group (fewest float4 per thread) whose CTA count stays within the hint
-    const int n4 = p.d / 4;
-    int tpr = 0;
-    for (int cand = n4; cand >= 32; cand -= 32) {
-      if (n4 % cand != 0 || (n4 / cand != 1 && n4 / cand != 2 && n4 / cand != 4)) continue;
-      const int rows = std::min(16, 1024 / cand);
-      tpr = cand;
-      if ((p.T + rows - 1) / rows <= p.ctas_hint) break;
-    }
-    if (tpr > 0) {
-      const int rows = std::min(16, 1024 / tpr);
-      const dim3 grid((p.T + rows - 1) / rows), block(rows * tpr);
-      switch (n4 / tpr) {
-        case 1: return launch_kernel(layernorm_rows_kernel<1>, grid, block, 0, s, pdl, p, tpr, rows);
-        case 2: return launch_kernel(layernorm_rows_kernel<2>, grid, block, 0, s, pdl, p, tpr, rows);
-        case 4: return launch_kernel(layernorm_rows_kernel<4>, grid, block, 0, s, pdl, p, tpr, rows);
-        default: break;
-      }
-    }
-  }
   if (p.T >= kLnWarpMinRows && p.d <= 1024) {      // thousands of rows: a warp per row
     const dim3 grid((p.T + kLnWarpRows - 1) / kLnWarpRows), block(kLnWarpRows * 32);
     switch (p.d / 128) {
@@ -317,6 +294,7 @@ cudaError_t launch_layernorm(const LnLaunch& p, cudaStream_t s, bool pdl) {
       default: break;
     }
   }
+  if (p.d <= kLnGroupMaxHidden) return launch_kernel(layernorm_group_kernel, dim3(p.T), dim3(kLnGroup), 0, s, pdl, p);
   return launch_kernel(layernorm_kernel, dim3(p.T), dim3(p.d / 4), 0, s, pdl, p);
 }
 

@@ -115,7 +115,7 @@ cudaError_t launch_attention_tc(const CUtensorMap& qkv_map, uint16_t* out, int n
                                 const int32_t* seq_lens, int* err, cudaStream_t s, bool pdl, unsigned long long* stamps);
 
 
-// out = LayerNorm(sum_p partial[p] + bias + resid) * gamma + beta, one warp per token row.
+// out = LayerNorm(sum_p partial[p] + bias + resid) * gamma + beta.
 struct LnLaunch {
   const float* partial;     // [n_partial][T][d]
   int n_partial;
@@ -128,7 +128,6 @@ struct LnLaunch {
   int T, d;
   float* out_f32;           // optional
   uint16_t* out_bf16;       // optional
-  int ctas_hint;            // > 0: pack rows so that about this many CTAs are launched (few tokens); 0: one row per CTA
   unsigned long long* stamps;   // profiling record or null
 };
 cudaError_t launch_layernorm(const LnLaunch& p, cudaStream_t s, bool pdl);

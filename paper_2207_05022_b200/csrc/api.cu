@@ -44,7 +44,7 @@ struct Tuning {
   int f2_kacc_min_tokens = 4096;       // FFN2 through the K-accumulating kernel (one output plane) from this many tokens on (0 = never)
   int f2_kacc_k = 512;                 // columns per K group there
   int f2_kacc_bps = 2;                 // boxes of 64 columns per ring stage there (1 or 2)
-  int attn_tc_min_items = 96;          // tensor-core attention from this many (sequence, kept head) pairs on, seq >= 256 (0 = never)
+  int attn_tc_min_items = -1;          // tensor-core attention: -1 = by the rule below, 0 = never, else from this many (sequence, kept head) pairs on, seq >= 256
 };
 
 struct Unit {
@@ -475,6 +475,16 @@ bool make_xmap(CUtensorMap* map, const void* base, int ld, int rows) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Whether attention goes to the tcgen05 kernel, one CTA per (sequence, kept head): from 320 keys on, when the other kernel's
+// tiles of 128 queries are more than two to an SM.  (8 sequences of 384, 16 heads: 20.6 against 24.6 us, but 6 of them 20.2
+// against 16.8; 12 of 300 38 against 23: below 320 keys the kernel's 128-key chunks are mostly padding.)
+bool tc_attention(const sti_plan* p, int nh, int batch, int seq) {
+  const int min_items = p->tune.attn_tc_min_items;
+  if (min_items == 0 || p->ctx->simt_debug) return false;
+  if (min_items > 0) return seq >= 256 && batch * nh >= min_items;
+  return seq > 320 && (seq + 127) / 128 * batch * nh > 2 * p->ctx->sm_count;
+}
+
 int m_ctas_for(int n_jobs, int T, int cta_budget) {
   const int n_mtiles = (T + 127) / 128;
   int m = n_jobs > 0 ? cta_budget / n_jobs : 1;
@@ -576,13 +586,14 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     st = run_gemm(p, GEMM_BF16_TO_BF16, L.qkv, xq, d.hidden, T, p->qkv, 64, dense + c->off_bq, next_layer, -1, stamp(1));
     if (st != STI_OK) return st;
     CUDA_TRY(mark(1));
-    if (p->tune.attn_tc_min_items > 0 && seq >= 256 && batch * nh >= p->tune.attn_tc_min_items && !c->simt_debug) {
+    if (tc_attention(p, nh, batch, seq)) {
       // many (sequence, head) pairs: one CTA each on the tensor cores, K and V of the sequence resident in shared memory
       CUtensorMap qmap;
       if (!make_xmap(&qmap, p->qkv, 64, 3 * nh * T)) return STI_ERR_CUDA;
       CUDA_TRY(launch_attention_tc(qmap, p->attn_out, nh, batch, seq, lens, c->err_dev, c->compute, c->pdl, stamp(2)));
     } else {
-      CUDA_TRY(launch_attention(p->qkv, p->attn_out, nh, batch, seq, lens, c->sm_count, c->compute, c->pdl, stamp(2)));
+      CUDA_TRY(launch_attention(p->qkv, p->attn_out, nh, batch, seq, lens, c->sm_count,
+                                L.o.n_jobs * m_ctas_for(L.o.n_jobs, T, p->tune.cta_budget), c->compute, c->pdl, stamp(2)));
     }
     c->launches++;
     CUDA_TRY(mark(2));

@@ -101,10 +101,10 @@ size_t gemm_kacc_smem_bytes(uint32_t hdr_bytes, uint32_t n_stages, uint32_t bps,
 cudaError_t launch_gemm_kacc(const KaccLaunch& p, cudaStream_t s);
 
 // Per-head attention over kept heads.  qkv: [(kept*3 + which)][T][64] bf16; out: [T][n_kept*64] bf16.
-// sm_count (the device's multiprocessor count) picks the CTA shape: large query tiles once they fill the GPU.
+// sm_count (the device's multiprocessor count) and next_ctas (the CTAs of the O projection that follows) pick the CTA shape.
 cudaError_t attention_configure();
 cudaError_t launch_attention(const uint16_t* qkv, uint16_t* out, int n_kept, int batch, int seq,
-                             const int32_t* seq_lens, int sm_count, cudaStream_t s, bool pdl,
+                             const int32_t* seq_lens, int sm_count, int next_ctas, cudaStream_t s, bool pdl,
                              unsigned long long* stamps);
 
 // The same attention on the tcgen05 tensor cores, one CTA per (sequence, kept head) with two query tiles in flight, for

@@ -1,0 +1,44 @@
+"""The mma.sync attention kernel against the oracle layer in each of its shapes (query tiles, key splits, key blocks), at
+lengths around the block sizes, with and without padding masks."""
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import sti_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+sti = pytest.importorskip("paper_2207_05022_b200")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2207_05022_b200 import build
+    build.build_library()
+    sti.load_library()
+
+
+@pytest.mark.parametrize("batch,seq,masked", [
+    (1, 1, False), (3, 17, True), (2, 32, True),             # up to 32 keys: one block of 32
+    (2, 33, True), (1, 64, False),                           # up to 64: tiles of 64 queries
+    (1, 65, False), (2, 97, True), (1, 128, True),           # few CTAs: 32 queries, keys split in two
+    (1, 129, True), (2, 200, True), (1, 256, False),         # ... and in four
+    (10, 150, True), (8, 300, True), (6, 256, True),         # 64 queries, keys split in two; what the O projection leaves
+    (17, 150, True), (17, 190, True), (25, 100, True),       # 128 queries, blocks of 32 and of 64 keys
+    (50, 70, True), (50, 100, False),                        # more CTAs than SMs: 64 queries
+])
+def test_attention_shapes(batch, seq, masked):
+    from gpu_util import run_layer, rel_err, REL_TOL
+    shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=1024, n_ffn_slices=4)
+    attn = [[W.UnitPlan(i != 1, 4, True) for i in range(4)]]
+    ffn = [[W.UnitPlan(True, 4, True) for _ in range(4)]]
+    work = W.build_workload("attention", shape, batch, seq, "f32", attn, ffn, seed=batch * 1000 + seq)
+    lens = np.random.default_rng(seq).integers(1, seq + 1, batch).tolist() if masked else None
+    if masked:
+        lens[0] = min(seq, 1 + 64 * (seq // 64))             # one key into the last block
+    a, f = O.decode_layer(work, 0)
+    ref = O.layer_forward(work.x, work.dense[0], a, f, eps=work.ln_eps, seq_lens=lens)
+    with sti.Session(work) as s:
+        y = run_layer(s, work, 0, lens=lens)
+    assert np.isfinite(y).all()
+    assert rel_err(y, ref) <= REL_TOL

@@ -38,7 +38,8 @@ struct MatrixInfo {
 };
 
 struct Tuning {
-  int qkv_n = 32, f1_n = 64, o_n = 64, o_group = 4, f2_n = 64, f2_group = 2;
+  int qkv_n = 32, f1_n = 64, o_n = 64, o_group = 4, f2_n = 64;
+  int f2_group = 0;                    // FFN slices per K group of FFN2: 0 = chosen per layer (pick_f2_group)
   int cta_budget = 148;                // (replaced by the device's SM count in parse_tuning) CTAs a GEMM launch may use when it splits the token tiles over CTAs
   int pair_min_tiles = 8;              // two-CTA GEMM from this many 128-token tiles on (0 = never)
   int f2_kacc_min_tokens = 4096;       // FFN2 through the K-accumulating kernel (one output plane) from this many tokens on (0 = never)
@@ -196,15 +197,30 @@ size_t matrix_code_bytes(const MatrixInfo& m, int bits) {
   return static_cast<size_t>(m.rows) * m.kc * bits / 8;
 }
 
+// Whether a weight tile of n rows x k columns leaves room for a ring of four boxes.
+bool tile_fits(int n, int k) {
+  uint32_t st = 0, bp = 0;
+  return gemm_pick_ring(static_cast<uint32_t>(gemm_weight_bytes(n, k)), k, gemm_header_bytes(), &st, &bp) && st * bp >= 4;
+}
+
+// A K range of `n` units in as few groups as `most` units per group allow, the groups equal up to one unit: {first, count}.
+std::vector<std::pair<int, int>> split_units(int n, int most) {
+  std::vector<std::pair<int, int>> groups;
+  const int n_groups = (n + most - 1) / most;
+  for (int g = 0, first = 0; g < n_groups; ++g) {
+    const int cnt = n / n_groups + (g < n % n_groups ? 1 : 0);
+    groups.emplace_back(first, cnt);
+    first += cnt;
+  }
+  return groups;
+}
+
 void parse_tuning(Tuning* t, int tmax, const sti_model_desc& d, int sm_count) {
   t->cta_budget = sm_count;
-  // few tokens: K groups of 8 heads / 2 FFN slices, one CTA per token tile (the decode is spread over the SMs, MMA
-  // chains stay short); many tokens: wide K groups, each CTA walks many token tiles with its decoded weights
-  if (tmax > 1024) {
-    t->qkv_n = 64; t->f1_n = 64; t->o_n = 64; t->o_group = 16; t->f2_n = 64; t->f2_group = 4;
-  } else {
-    t->qkv_n = 64; t->f1_n = 64; t->o_n = 64; t->o_group = 8; t->f2_n = 64; t->f2_group = 2;
-  }
+  // few tokens: K groups of at most 8 heads (the decode is spread over the SMs, MMA chains stay short); many tokens: wide
+  // K groups, each CTA walks many token tiles with its decoded weights
+  t->qkv_n = 64; t->f1_n = 64; t->o_n = 64; t->f2_n = 64;
+  t->o_group = tmax > 1024 ? 16 : 8;
   const char* env = getenv("STI_TUNE");     // debugging aid: "qkv_n=32,o_group=4,..."
   if (env) {
     std::string s(env);
@@ -243,12 +259,9 @@ void parse_tuning(Tuning* t, int tmax, const sti_model_desc& d, int sm_count) {
   while (d.hidden % t->o_n) t->o_n /= 2;
   while (d.hidden % t->f2_n) t->f2_n /= 2;
   t->o_group = std::max(1, std::min(t->o_group, 16));
-  t->f2_group = std::max(1, std::min(t->f2_group, 16));
+  t->f2_group = std::max(0, std::min(t->f2_group, 16));
   // keep every weight tile inside shared memory
-  auto fits = [](int n, int k) {
-    uint32_t st = 0, bp = 0;
-    return gemm_pick_ring(static_cast<uint32_t>(gemm_weight_bytes(n, k)), k, gemm_header_bytes(), &st, &bp) && st * bp >= 4;
-  };
+  const auto fits = tile_fits;
   while (t->qkv_n > 32 && !fits(t->qkv_n, d.hidden)) t->qkv_n /= 2;
   while (t->f1_n > 32 && !fits(t->f1_n, d.hidden)) t->f1_n /= 2;
   while (t->o_group > 1 && !fits(t->o_n, t->o_group * 64)) --t->o_group;
@@ -357,6 +370,34 @@ struct TableBuilder {
   }
 };
 
+// FFN slices per K group of FFN2 in a layer that keeps `ns` of them, for the plan's token count.  More slices per group:
+// fewer fp32 planes written and read back by the LayerNorm (8 bytes per element at about 5 TB/s), but a longer decode and MMA
+// chain per CTA (0.7 us per 256 columns and 128-token tile, 0.53 per 256-token tile of the two-CTA kernel, and about 1 us of
+// decode per 256 columns that other kernels do not hide).  BERT-large, six layers with 2 / 4 slices per group: 256 tokens
+// 245 / 247 us, 512 342 / 338, 1024 433 / 421, 2048 627 / 581; BERT-base, 600 tokens with 2 / 3 / 4: 289 / 287 / 296.
+int pick_f2_group(const sti_plan* p, int ns) {
+  const sti_model_desc& d = p->ctx->desc;
+  const Tuning& t = p->tune;
+  if (t.f2_group > 0) return t.f2_group;
+  const int f = d.ffn / d.n_ffn_slices;
+  double T = static_cast<double>(d.max_batch) * d.max_seq;
+  if (t.f2_kacc_min_tokens > 0) T = std::min(T, static_cast<double>(t.f2_kacc_min_tokens));   // more take the K-accumulating kernel
+  const int n_mtiles = static_cast<int>((T + 127) / 128);
+  const bool pair = t.pair_min_tiles > 0 && n_mtiles >= t.pair_min_tiles;
+  const int n_tiles = pair ? (n_mtiles + 1) / 2 : n_mtiles;
+  int best = 1;                        // also where no more than one slice fits in shared memory
+  double best_cost = -1.0;
+  for (int g = std::max(1, std::min(2, ns)); g <= ns; ++g) {
+    if (!tile_fits(t.f2_n, g * f)) break;
+    const int planes = (ns + g - 1) / g, widest = (ns + planes - 1) / planes, jobs = planes * (d.hidden / t.f2_n);
+    const int m_ctas = std::max(1, std::min(n_tiles, t.cta_budget / jobs)), tiles = (n_tiles + m_ctas - 1) / m_ctas;
+    const double waves = std::max(1.0, static_cast<double>(jobs) * m_ctas / t.cta_budget);
+    const double cost = waves * widest * (f / 256.0) * (tiles * (pair ? 0.53 : 0.7) + 1.0) + planes * T * d.hidden * 8.0 / 5.0e6;
+    if (best_cost < 0.0 || cost < best_cost) { best = g; best_cost = cost; }
+  }
+  return best;
+}
+
 void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
   const sti_ctx* c = p->ctx;
   const sti_model_desc& d = c->desc;
@@ -377,9 +418,10 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
   }
   // O projection: K is split over groups of kept heads, each group writes its own partial sum
   const int nh = static_cast<int>(L.kept_heads.size());
-  L.o.n_split = (nh + t.o_group - 1) / t.o_group;
+  const auto o_groups = split_units(nh, t.o_group);
+  L.o.n_split = static_cast<int>(o_groups.size());
   for (int sp = 0; sp < L.o.n_split; ++sp) {
-    const int first = sp * t.o_group, cnt = std::min(t.o_group, nh - first);
+    const int first = o_groups[sp].first, cnt = o_groups[sp].second;
     for (uint32_t n0 = 0; n0 < static_cast<uint32_t>(d.hidden); n0 += t.o_n) {
       Job j{};
       j.n_rows = t.o_n; j.k_total = cnt * 64; j.x_koff = first * 64;
@@ -402,9 +444,10 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
   }
   // FFN2: K split over groups of kept slices
   const int ns = static_cast<int>(L.kept_slices.size());
-  L.f2.n_split = (ns + t.f2_group - 1) / t.f2_group;
+  const auto f2_groups = split_units(ns, pick_f2_group(p, ns));
+  L.f2.n_split = static_cast<int>(f2_groups.size());
   for (int sp = 0; sp < L.f2.n_split; ++sp) {
-    const int first = sp * t.f2_group, cnt = std::min(t.f2_group, ns - first);
+    const int first = f2_groups[sp].first, cnt = f2_groups[sp].second;
     for (uint32_t n0 = 0; n0 < static_cast<uint32_t>(d.hidden); n0 += t.f2_n) {
       Job j{};
       j.n_rows = t.f2_n; j.k_total = cnt * f; j.x_koff = first * f;

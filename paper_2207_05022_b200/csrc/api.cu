@@ -504,14 +504,14 @@ EncodeTiledFn encode_tiled_fn() {
   return fn;
 }
 
-// TMA view of a bf16 activation matrix [rows, ld]: boxes of 128 rows x 64 columns, 128-byte swizzle,
+// TMA view of a bf16 activation matrix [rows, ld]: boxes of `box_rows` rows x 64 columns, 128-byte swizzle,
 // rows past `rows` read as zeros.
-bool make_xmap(CUtensorMap* map, const void* base, int ld, int rows) {
+bool make_xmap(CUtensorMap* map, const void* base, int ld, int rows, int box_rows = 128) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn || (reinterpret_cast<uintptr_t>(base) & 15) || (ld % 8) != 0) return false;
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(ld), static_cast<cuuint64_t>(rows)};
   const cuuint64_t strides[1] = {static_cast<cuuint64_t>(ld) * 2};
-  const cuuint32_t box[2] = {64, 128};
+  const cuuint32_t box[2] = {64, static_cast<cuuint32_t>(box_rows)};
   const cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -630,10 +630,9 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     if (st != STI_OK) return st;
     CUDA_TRY(mark(1));
     if (tc_attention(p, nh, batch, seq)) {
-      // many (sequence, head) pairs: one CTA each on the tensor cores, K and V of the sequence resident in shared memory
-      CUtensorMap qmap;
-      if (!make_xmap(&qmap, p->qkv, 64, 3 * nh * T)) return STI_ERR_CUDA;
-      CUDA_TRY(launch_attention_tc(qmap, p->attn_out, nh, batch, seq, lens, c->err_dev, c->compute, c->pdl, stamp(2)));
+      CUtensorMap qmap, omap;
+      if (!make_xmap(&qmap, p->qkv, 64, 3 * nh * T, 64) || !make_xmap(&omap, p->attn_out, nh * 64, T, 32)) return STI_ERR_CUDA;
+      CUDA_TRY(launch_attention_tc(qmap, omap, p->attn_out, nh, batch, seq, lens, c->err_dev, c->compute, c->pdl, stamp(2)));
     } else {
       CUDA_TRY(launch_attention(p->qkv, p->attn_out, nh, batch, seq, lens, c->sm_count,
                                 L.o.n_jobs * m_ctas_for(L.o.n_jobs, T, p->tune.cta_budget), c->compute, c->pdl, stamp(2)));

@@ -1,24 +1,26 @@
-// Per-head attention on the tcgen05 tensor cores with TWO query tiles in flight per CTA (Section 2.1: softmax(Q K^T /
-// sqrt 64) V per kept head; padded keys get probability exactly 0).
+// Per-head attention on the tcgen05 tensor cores for long sequences (Section 2.1: softmax(Q K^T / sqrt 64) V per kept head;
+// padded keys get probability exactly 0).
 //
-// One CTA per (sequence, kept head): K and V of the sequence (at most 512 keys) stay in shared memory.  Two groups of
-// four softmax warps each own one 128-query tile at a time (tiles g, g + 2, ... for group g) with ONE thread per query
-// row, so a row's maximum and sum never leave the thread.  The MMA warp serves the groups in turn: while one group is
-// busy with its exponentials the other's S = Q K^T or O_c = P V runs, and a group that waits for the tensor core
-// leaves the issue slots to the other.
+// One CTA per two query tiles of 128 of a (sequence, kept head): two groups of four warps, ONE thread per query row, so a row's
+// maximum and sum never leave the thread.  Two CTAs share an SM (256 threads, 113 KB, half the tensor memory each), which puts
+// four warps on every scheduler: while one waits for a tensor-core result, reads scores or reduces, the others keep the
+// special-function units busy.  There are no other warps: with them the registers would not do.
 //
-//   warps 0-3, 4-7  softmax group 0 / 1: thread = query row = tensor-memory lane.  Per 128-key chunk: pass 1 reads
-//                   the scores (tcgen05.ld) for the row maximum; then the previous chunk's O_c is folded into the
-//                   register accumulator (which also says that the probability buffer is free); pass 2 reads the
-//                   scores again, exponentiates, sums, and writes the bf16 probabilities into shared memory in the
-//                   swizzled K-major layout the second MMA reads
-//   warp 8          TMA: K and V once (a barrier per 128-key chunk, so the first scores start after 16 KB of K have
-//                   landed, not after the sequence's 128 KB), query tiles into the two slots
-//   warp 9          MMA issuer: for each group in turn  S(next chunk)  and  O_c = P V(this chunk)
+// Per 32-key step a group's warps take the row's scores into registers (tcgen05.ld), the maximum, the exponentials and their
+// sum, and put the bf16 probabilities back into tensor memory over the scores; O += P V (P is the tensor-memory operand)
+// follows.  There are two score buffers, so S = Q K^T of the next step is computed during this step's exponentials (and 32 keys
+// are what two buffers leave room for: with one buffer of 64 keys a step took 2,500 cycles, 1,300 of them waiting for P V and S
+// in turn).  The group's first warp issues its MMAs.  Keys and values stream through a ring of five 64-key chunks read by both
+// groups; the group that finishes a chunk last refills its place, so nobody waits for a producer.
 //
-// Tensor memory: S of group g at columns 128 g, O_c of group g at 256 + 64 g.  Every barrier has one class of
-// waiters that meets every phase in order.  Waits are bounded; a role that gives up sets the abort flag and the
-// status word, the others run out of their own waits.
+// O stays in tensor memory for the whole tile.  The maximum used for the exponentials moves only when a step's maximum exceeds
+// it by more than 2^8 (then O and the sum are rescaled); the sum and O are in fp32 and the division by the sum at the end takes
+// any common factor out, so nothing is lost by a maximum that lags behind.
+//
+// Bound: 32 x 128 exponentials per step take 256 cycles of an SM's special-function units.
+//
+// Tensor memory of group g: S and P of even / odd steps at column 128 g / 128 g + 32, O at 128 g + 64.  Waits are bounded; a role that gives up sets the abort
+// flag and the status word, the others see the flag or run out of their own waits.
 #include <cuda_bf16.h>
 
 #include "gemm_device.cuh"
@@ -27,33 +29,30 @@
 namespace sti {
 namespace {
 
-constexpr int kTcGroupWarps = 4, kTcGroups = 2;
-constexpr int kTcProducerWarp = kTcGroupWarps * kTcGroups, kTcMmaWarp = kTcProducerWarp + 1;
-constexpr int kTcThreads = 32 * (kTcMmaWarp + 1);
-constexpr int kTcQTile = 128, kTcChunk = 128, kTcHead = 64;
+constexpr int kTcGroups = 2, kTcGroupWarps = 4, kTcMmaWarp = kTcGroups * kTcGroupWarps, kTcThreads = 32 * (kTcMmaWarp + kTcGroups);
+constexpr int kTcQTile = 128, kTcChunk = 64, kTcStep = 32, kTcHead = 64, kTcRing = 5;
 constexpr int kTcMaxSeq = 512;
-constexpr uint32_t kTcBox = kTcChunk * kTcHead * 2;              // 16 KB: 128 rows x 64 bf16, one TMA box
-constexpr uint32_t kTcOffQ = 3072;                               // two query slots
-constexpr uint32_t kTcOffK = kTcOffQ + 2 * kTcBox;
-constexpr uint32_t kTcOffV = kTcOffK + 4 * kTcBox;
-constexpr uint32_t kTcOffP = kTcOffV + 4 * kTcBox;               // probabilities: per group two boxes (128 rows x 64 keys)
-constexpr uint32_t kTcSmem = kTcOffP + 4 * kTcBox;
-static_assert(kTcOffQ % 1024 == 0 && kTcSmem <= 227 * 1024, "shared-memory layout");
-constexpr uint32_t kTcTmemCols = 512;
-constexpr uint32_t kTcColS = 0, kTcColO = 256;
+constexpr uint32_t kTcBox = kTcChunk * kTcHead * 2;              // 8 KB: 64 rows x 64 bf16, one TMA box
+constexpr uint32_t kTcOffQ = 1024;                               // a query tile per group; its output tile in the end
+constexpr uint32_t kTcOffKV = kTcOffQ + kTcGroups * 2 * kTcBox;  // ring: keys and values of a chunk
+constexpr uint32_t kTcSmem = kTcOffKV + kTcRing * 2 * kTcBox;
+static_assert(2 * (kTcSmem + 1024) <= 228 * 1024, "two CTAs per SM");
+constexpr uint32_t kTcTmemCols = 256;
 
 struct TcBarriers {
-  uint64_t k_full[4];      // key chunk c has landed (one phase each: K and V are loaded once per CTA)
-  uint64_t v_full[4];      // value chunk c has landed
-  uint64_t q_full[2];      // a query tile has landed in the group's slot
-  uint64_t q_empty[2];     // the score MMAs of the slot's tile have completed
-  uint64_t s_full[2];      // the group's score chunk is complete in tensor memory
-  uint64_t s_empty[2];     // the group has read its score chunk for the last time (the chunk's last tcgen05.ld is complete)
-  uint64_t p_full[2];      // the group's probabilities are in shared memory
-  uint64_t o_full[2];      // the group's O_c is complete in tensor memory (and its probabilities have been read)
+  uint64_t k_full[kTcRing], v_full[kTcRing];
+  uint64_t q_full[kTcGroups];
+  uint64_t s_full[kTcGroups][2];   // the group's scores of an even / odd step are complete in tensor memory
+  uint64_t p_full[kTcGroups][2];   // its probabilities are
+  uint64_t o_full[kTcGroups];      // its P V of a step has completed
+  uint64_t o_last[kTcGroups];      // ... of the last step
+  uint64_t drain[kTcGroups];
+  int readers_done[kTcMaxSeq / kTcChunk];      // groups that have finished with a chunk
+  int requested;                   // chunks asked for so far
   uint32_t tmem_base;
   volatile uint32_t abort;
 };
+static_assert(sizeof(TcBarriers) <= kTcOffQ, "header");
 
 __device__ __forceinline__ uint64_t umma_smem_desc_sw128_mn(uint32_t saddr) {    // V: keys are rows, the 64 features contiguous
   uint64_t d = 0;
@@ -70,6 +69,34 @@ __device__ __forceinline__ float fast_exp2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float y;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+
+// D[128 x N] += A[128 x 16] B[N x 16]^T with A (bf16 pairs, lane = row) in tensor memory
+__device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+               ::"r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tmem_st_32x32b_x16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+               "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+               : "memory");
+}
+// One 32 x 64 tile of the output (128-byte swizzle in shared memory) as a bulk group of its own.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];\n\tcp.async.bulk.commit_group;"
+               ::"l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(src) : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // tcgen05.wait::ld that names the registers of one earlier 32-column load as read-write operands: the compiler then
 // keeps those values where the load put them until here and orders every later use after the wait, so the load may
@@ -84,20 +111,28 @@ __device__ __forceinline__ void tmem_wait_ld_x32(uint32_t (&r)[32]) {
                : "memory");
 }
 
+__device__ __forceinline__ void tmem_wait_ld_x16(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+
+// Whole warp; the same answer in every lane.
 __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, uint32_t lane, volatile uint32_t* abort) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
   uint32_t ok = 1;
   if (lane == 0) ok = *abort ? 0u : (mbar_wait_bounded(bar, parity) ? 1u : 0u);
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1)
-attention_tc_kernel(const __grid_constant__ CUtensorMap qkv_map, uint16_t* __restrict__ out,
-                     const int32_t* __restrict__ seq_lens, int n_kept, int batch, int L, int* __restrict__ err,
-                     unsigned long long* stamps) {
+__global__ void __launch_bounds__(kTcThreads, 2)
+attention_tc_kernel(const __grid_constant__ CUtensorMap qkv_map, const __grid_constant__ CUtensorMap out_map,
+                    uint16_t* __restrict__ out, const int32_t* __restrict__ seq_lens, int n_kept, int batch, int L,
+                    int* __restrict__ err, unsigned long long* stamps) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int hi = blockIdx.x, b = blockIdx.y;
-  const int T = batch * L;
   if (tid == 0) { stamp_min(stamps, STAMP_FIRST_START); stamp_max(stamps, STAMP_LAST_START); }
   TcBarriers* bar = reinterpret_cast<TcBarriers*>(smem);
   const uint32_t sbase = smem_addr(smem);
@@ -105,21 +140,27 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap qkv_map, uint16_t* __res
     if (tid == 0) atomicCAS(err, ERR_NONE, ERR_BAD_JOB);
     return;
   }
-  if (tid == 0) {
-    for (int c = 0; c < 4; ++c) { mbar_init(smem_addr(&bar->k_full[c]), 1); mbar_init(smem_addr(&bar->v_full[c]), 1); }
-    for (int g = 0; g < 2; ++g) {
+  if (tid == kTcMmaWarp * 32) {
+    for (int c = 0; c < kTcRing; ++c) { mbar_init(smem_addr(&bar->k_full[c]), 1); mbar_init(smem_addr(&bar->v_full[c]), 1); }
+    for (int g = 0; g < kTcGroups; ++g) {
       mbar_init(smem_addr(&bar->q_full[g]), 1);
-      mbar_init(smem_addr(&bar->q_empty[g]), 1);
-      mbar_init(smem_addr(&bar->s_full[g]), 1);
-      mbar_init(smem_addr(&bar->s_empty[g]), kTcGroupWarps);
-      mbar_init(smem_addr(&bar->p_full[g]), kTcGroupWarps);
+      for (int e = 0; e < 2; ++e) {
+        mbar_init(smem_addr(&bar->s_full[g][e]), 1);
+        mbar_init(smem_addr(&bar->p_full[g][e]), kTcGroupWarps);
+      }
       mbar_init(smem_addr(&bar->o_full[g]), 1);
+      mbar_init(smem_addr(&bar->o_last[g]), 1);
+      mbar_init(smem_addr(&bar->drain[g]), 1);
     }
+    for (int c = 0; c < kTcMaxSeq / kTcChunk; ++c) bar->readers_done[c] = 0;
+    bar->requested = 0;
     bar->abort = 0;
     mbar_fence_init();
     fence_proxy_async_smem();
+    tma_prefetch_map(&qkv_map);
+    tma_prefetch_map(&out_map);
   }
-  if (warp == kTcProducerWarp) {
+  if (warp == kTcMmaWarp) {
     tmem_alloc(smem_addr(&bar->tmem_base), kTcTmemCols);
     tmem_relinquish();
   }
@@ -131,241 +172,215 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap qkv_map, uint16_t* __res
   pdl_wait();
   if (tid == 0) stamp_min(stamps, STAMP_RELEASE);
 
+  const int hi = blockIdx.y, b = blockIdx.z, T = batch * L;
   int valid = L;
-  if (seq_lens != nullptr) {
-    valid = seq_lens[b];
-    valid = valid < 0 ? 0 : (valid > L ? L : valid);
-  }
-  const int n_qt = (L + kTcQTile - 1) / kTcQTile;
-  const int nc = (valid + kTcChunk - 1) / kTcChunk;              // key chunks with at least one valid key
-  const int q_row = (hi * 3 + 0) * T + b * L, k_row = (hi * 3 + 1) * T + b * L, v_row = (hi * 3 + 2) * T + b * L;
-  const uint32_t q_sm = sbase + kTcOffQ, k_sm = sbase + kTcOffK, v_sm = sbase + kTcOffV, p_sm = sbase + kTcOffP;
-  // tiles of group g: g, g + 2, ...; steps of a group = (its tile number i, chunk c) in order
-  auto tiles_of = [&](int g) { return n_qt > g ? (n_qt - g + 1) / 2 : 0; };
-  bool failed = false;
+  if (seq_lens != nullptr) valid = min(max(__ldg(seq_lens + b), 0), L);
+  const int nc = (valid + kTcChunk - 1) / kTcChunk;              // chunks and steps with at least one valid key
+  const int ns = (valid + kTcStep - 1) / kTcStep;
+  const uint32_t g = warp < kTcMmaWarp ? warp >> 2 : warp - kTcMmaWarp, quad = warp & 3;
+  const int tile0 = static_cast<int>(blockIdx.x) * kTcGroups;    // the CTA's first query tile
+  const int n_groups = min(kTcGroups, (L + kTcQTile - 1) / kTcQTile - tile0);
+  const uint32_t q_sm = sbase + kTcOffQ + g * 2 * kTcBox, kv_sm = sbase + kTcOffKV;
+  bool failed = false, issued = false;
+  auto wait = [&](uint64_t* m, uint32_t parity) { return warp_wait(smem_addr(m), parity & 1, lane, &bar->abort); };
+  // one thread: chunk c of the keys and values into its place of the ring
+  auto load_keys = [&](int c, bool values) {
+    const uint32_t full = smem_addr(values ? &bar->v_full[c % kTcRing] : &bar->k_full[c % kTcRing]);
+    mbar_expect_tx(full, kTcBox);
+    tma_load_2d(kv_sm + (2 * (c % kTcRing) + (values ? 1 : 0)) * kTcBox, &qkv_map, 0, (hi * 3 + (values ? 2 : 1)) * T + b * L + c * kTcChunk,
+                full);
+  };
+  const uint32_t col = tmem + g * 128;
 
-  if (warp == kTcProducerWarp) {
-    if (lane == 0 && nc > 0) {
-      // in the order the MMA warp needs them: the first key chunk, the first two query tiles, then V and K chunk by chunk
-      auto load_k = [&](int c) {
-        mbar_expect_tx(smem_addr(&bar->k_full[c]), kTcBox);
-        tma_load_2d(k_sm + c * kTcBox, &qkv_map, 0, k_row + c * kTcChunk, smem_addr(&bar->k_full[c]));
-      };
-      auto load_v = [&](int c) {
-        mbar_expect_tx(smem_addr(&bar->v_full[c]), kTcBox);
-        tma_load_2d(v_sm + c * kTcBox, &qkv_map, 0, v_row + c * kTcChunk, smem_addr(&bar->v_full[c]));
-      };
-      auto load_q = [&](int qt) {
-        const uint32_t g = qt & 1;
-        mbar_expect_tx(smem_addr(&bar->q_full[g]), kTcBox);
-        tma_load_2d(q_sm + g * kTcBox, &qkv_map, 0, q_row + qt * kTcQTile, smem_addr(&bar->q_full[g]));
-      };
-      load_k(0);
-      for (int qt = 0; qt < n_qt && qt < 2; ++qt) load_q(qt);
-      load_v(0);
-      for (int c = 1; c < nc; ++c) { load_k(c); load_v(c); }
-      for (int qt = 2; qt < n_qt; ++qt) {
-        const uint32_t g = qt & 1, i = qt >> 1;                  // the group's i-th tile
-        if (!mbar_wait_bounded_relaxed(smem_addr(&bar->q_empty[g]), (i - 1) & 1)) { failed = true; break; }
-        load_q(qt);
+  if (static_cast<int>(g) >= n_groups || nc == 0) {
+    // the second group of a sequence's last, single tile; a sequence without a valid key
+  } else if (warp >= kTcMmaWarp) {
+    // ---- the group's loads and MMAs
+    if (lane == 0) {
+      if (g == 0) load_keys(0, false);
+      const uint32_t full = smem_addr(&bar->q_full[g]);
+      mbar_expect_tx(full, 2 * kTcBox);
+      for (int h = 0; h < 2; ++h)
+        tma_load_2d(q_sm + h * kTcBox, &qkv_map, 0, hi * 3 * T + b * L + (tile0 + static_cast<int>(g)) * kTcQTile + h * kTcChunk, full);
+      if (g == 0) {
+        load_keys(0, true);
+        for (int c = 1; c < nc && c < kTcRing; ++c) { load_keys(c, false); load_keys(c, true); }
+        atomicMax(&bar->requested, min(nc, kTcRing));
       }
     }
     __syncwarp();
-  } else if (warp == kTcMmaWarp) {
-    if (nc > 0) {
-      const uint32_t idesc_s = umma_idesc_bf16_m128(kTcChunk);
-      const uint32_t idesc_o = umma_idesc_bf16_m128(kTcHead) | (1u << 16);       // B (V) is MN-major
-      const uint64_t q_desc0 = umma_smem_desc_sw128(q_sm), k_desc0 = umma_smem_desc_sw128(k_sm);
-      const uint64_t p_desc0 = umma_smem_desc_sw128(p_sm), v_desc0 = umma_smem_desc_sw128_mn(v_sm);
-      const int steps[2] = {tiles_of(0) * nc, tiles_of(1) * nc};
-      // S of step n of group g into the group's score columns; a new tile first waits for its queries
-      auto issue_scores = [&](int g, int n) -> bool {
-        const int i = n / nc, c = n - i * nc;
-        if (c == 0 && !warp_wait(smem_addr(&bar->q_full[g]), i & 1, lane, &bar->abort)) return false;
-        if (i == 0 && !warp_wait(smem_addr(&bar->k_full[c]), 0, lane, &bar->abort)) return false;   // later tiles: long landed
-        tc_fence_after_sync();
-        if (elect_one()) {
-          umma_bf16_ss_x4(tmem + kTcColS + g * kTcChunk, q_desc0 + g * (kTcBox >> 4), k_desc0 + c * (kTcBox >> 4), 2, 2,
-                          idesc_s, 0u);
-          umma_commit(smem_addr(&bar->s_full[g]));
-          if (c + 1 == nc && i + 1 < tiles_of(g)) umma_commit(smem_addr(&bar->q_empty[g]));   // the slot's next tile may land
+    const uint32_t idesc_s = umma_idesc_bf16_m128(kTcStep);
+    const uint32_t idesc_o = umma_idesc_bf16_m128(kTcHead) | (1u << 16);         // B (V) is MN-major
+    const uint64_t q_desc = umma_smem_desc_sw128(q_sm), k_desc0 = umma_smem_desc_sw128(kv_sm);
+    const uint64_t v_desc0 = umma_smem_desc_sw128_mn(kv_sm + kTcBox);
+    auto issue_scores = [&](int c) -> bool {
+      const int st = (c >> 1) % kTcRing;
+      if ((c & 1) == 0 && !wait(&bar->k_full[st], (c >> 1) / kTcRing)) return false;
+      tc_fence_after_sync();
+      if (elect_one()) {
+        umma_bf16_ss_x4(col + (c & 1) * kTcStep, q_desc, k_desc0 + st * (2 * kTcBox >> 4) + (c & 1) * (kTcBox / 2 >> 4), 2, 2, idesc_s, 0u);
+        umma_commit(smem_addr(&bar->s_full[g][c & 1]));
+      }
+      __syncwarp();
+      issued = true;
+      return true;
+    };
+    failed = !wait(&bar->q_full[g], 0) || !issue_scores(0) || (ns > 1 && !issue_scores(1));
+    for (int c = 0; c < ns && !failed; ++c) {
+      // O += P V; the step's second 16 keys are left out if none of them is valid
+      const int chunk = c >> 1, st = chunk % kTcRing;
+      if ((c & 1) == 0 && !wait(&bar->v_full[st], chunk / kTcRing)) { failed = true; break; }
+      if (!wait(&bar->p_full[g][c & 1], c >> 1)) { failed = true; break; }
+      tc_fence_after_sync();
+      if (elect_one()) {
+        const uint64_t vd = v_desc0 + st * (2 * kTcBox >> 4) + (c & 1) * (kTcBox / 2 >> 4);
+        const uint32_t p_col = col + (c & 1) * kTcStep;
+        umma_bf16_ts(col + 64, p_col, vd, idesc_o, c > 0 ? 1u : 0u);
+        if (valid - c * kTcStep > 16) umma_bf16_ts(col + 64, p_col + 8, vd + (2048 >> 4), idesc_o, 1u);
+        umma_commit(smem_addr(&bar->o_full[g]));
+        if (c + 1 == ns) umma_commit(smem_addr(&bar->o_last[g]));
+      }
+      __syncwarp();
+      issued = true;
+      if (c + 2 < ns) {                                          // scores of the step after next go where this step's P is
+        if (!wait(&bar->o_full[g], c) || !issue_scores(c + 2)) { failed = true; break; }
+        if (lane == 0 && (c & 1) != 0 && chunk + kTcRing < nc) { // this group has finished with the chunk
+          __threadfence_block();
+          if (atomicAdd(&bar->readers_done[chunk], 1) == n_groups - 1) {
+            __threadfence_block();
+            load_keys(chunk + kTcRing, false);
+            load_keys(chunk + kTcRing, true);
+            atomicMax(&bar->requested, chunk + kTcRing + 1);
+          }
         }
         __syncwarp();
-        return true;
-      };
-      bool ok = true;
-      for (int g = 0; ok && g < 2; ++g)
-        if (steps[g] > 0) ok = issue_scores(g, 0);
-      // Serve whichever group has something ready: its scores read for the last time -> the next chunk's S; its
-      // probabilities in shared memory -> O_c = P V.  Neither group waits for the other's softmax.
-      int next_s[2] = {1, 1}, next_pv[2] = {0, 0};               // S of step 0 is issued above
-      uint64_t t_idle = global_timer_ns();
-      while (ok && (next_pv[0] < steps[0] || next_pv[1] < steps[1])) {
-        bool progressed = false;
-        for (int g = 0; ok && g < 2; ++g) {
-          if (next_s[g] < steps[g]) {                            // S(next_s) needs the reads of step next_s - 1 done
-            uint32_t ready = 0;
-            if (lane == 0) ready = mbar_try_wait(smem_addr(&bar->s_empty[g]), (next_s[g] - 1) & 1);
-            if (__shfl_sync(0xffffffffu, ready, 0)) {
-              ok = issue_scores(g, next_s[g]);
-              if (!ok) break;
-              ++next_s[g];
-              progressed = true;
-            }
-          }
-          const int n = next_pv[g];
-          if (n < steps[g]) {
-            uint32_t ready = 0;
-            if (lane == 0) ready = mbar_try_wait(smem_addr(&bar->p_full[g]), n & 1);
-            if (__shfl_sync(0xffffffffu, ready, 0)) {
-              const int c = n % nc;
-              if (n < nc && !warp_wait(smem_addr(&bar->v_full[c]), 0, lane, &bar->abort)) { ok = false; break; }
-              tc_fence_after_sync();
-              if (elect_one()) {
-                // O_c = P V_c: two boxes of 64 keys; per K = 16 step P moves 32 bytes in its swizzled row, V 16 rows
-                const uint64_t vd = v_desc0 + c * (kTcBox >> 4), pd = p_desc0 + g * (2 * kTcBox >> 4);
-                const uint32_t od = tmem + kTcColO + g * kTcHead;
-                umma_bf16_ss_x4(od, pd, vd, 2, 2048 >> 4, idesc_o, 0u);
-                umma_bf16_ss_x4(od, pd + (kTcBox >> 4), vd + (8192 >> 4), 2, 2048 >> 4, idesc_o, 1u);
-                umma_commit(smem_addr(&bar->o_full[g]));
-              }
-              __syncwarp();
-              next_pv[g] = n + 1;
-              progressed = true;
-            }
-          }
+      }
+    }
+    if (!failed) failed = !wait(&bar->o_last[g], 0);
+  } else {
+    // ---- softmax: thread = query row
+    const uint32_t t_lane = (quad * 32) << 16;
+    const uint32_t s_addr = col + t_lane, o_addr = s_addr + 64;
+    const float scale = 0.125f * 1.4426950408889634f;            // 1/sqrt(64) * log2(e)
+    const int q0 = (tile0 + static_cast<int>(g)) * kTcQTile + static_cast<int>(quad * 32);
+    const bool idle = q0 >= L;                                   // rows past the sequence: only the barriers
+    float m = -INFINITY, l = 0.f;
+    for (int c = 0; c < ns && !failed; ++c) {
+      if (!wait(&bar->s_full[g][c & 1], c >> 1)) { failed = true; break; }
+      tc_fence_after_sync();
+      const uint32_t buf = s_addr + (c & 1) * kTcStep;
+      uint32_t s[32];
+      if (!idle) {
+        const int n_valid = valid - c * kTcStep;                 // keys of this step at and past it are padding
+        tmem_ld_32x32b_x32(buf, s);
+        tmem_wait_ld_x32(s);
+        if (n_valid < kTcStep) {
+#pragma unroll
+          for (int k = 0; k < 32; ++k)
+            if (k >= n_valid) s[k] = 0xff800000u;                // -inf
         }
-        if (progressed) {
-          t_idle = global_timer_ns();
-        } else {
-          uint32_t give_up = 0;
-          if (lane == 0) give_up = (bar->abort || global_timer_ns() - t_idle > 2000000000ull) ? 1u : 0u;
-          if (__shfl_sync(0xffffffffu, give_up, 0)) ok = false;
+        float mx[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          mx[e] = max3(__uint_as_float(s[e]), __uint_as_float(s[e + 2]), __uint_as_float(s[e + 4]));
+#pragma unroll
+          for (int k = 6; k < 30; k += 4) mx[e] = max3(mx[e], __uint_as_float(s[e + k]), __uint_as_float(s[e + k + 2]));
+        }
+        const float mc = max3(fmaxf(mx[0], mx[1]), __uint_as_float(s[30]), __uint_as_float(s[31])) * scale;   // finite: a valid key
+        if (c == 0) {
+          m = mc;
+        } else if (__any_sync(0xffffffffu, mc > m + 8.f)) {
+          if (!wait(&bar->o_full[g], c - 1)) { failed = true; break; }     // P V of step c - 2 came before these scores
+          tc_fence_after_sync();
+          const float m_new = fmaxf(m, mc), alpha = fast_exp2(m - m_new);
+          m = m_new;
+          l *= alpha;
+#pragma unroll 1
+          for (int e = 0; e < 4; ++e) {
+            uint32_t r[16];
+            tmem_ld_32x32b_x16(o_addr + e * 16, r);
+            tmem_wait_ld_x16(r);
+#pragma unroll
+            for (int k = 0; k < 16; ++k) r[k] = __float_as_uint(__uint_as_float(r[k]) * alpha);
+            tmem_st_32x32b_x16(o_addr + e * 16, r);
+          }
         }
       }
-      if (!ok) failed = true;
-    }
-  } else {
-    // ---- softmax group g: thread = query row
-    const uint32_t g = warp >> 2, quad = warp & 3;
-    const uint32_t row = quad * 32 + lane;
-    const uint32_t t_lane = (quad * 32) << 16;
-    const float scale = 0.125f * 1.4426950408889634f;            // 1/sqrt(64) * log2(e)
-    const int ldo = n_kept * kTcHead;
-    const int my_tiles = tiles_of(static_cast<int>(g));
-    const uint32_t s_addr = tmem + t_lane + kTcColS + g * kTcChunk;
-    const uint32_t o_addr = tmem + t_lane + kTcColO + g * kTcHead;
-    uint8_t* prow = smem + kTcOffP + g * 2 * kTcBox + row * 128;   // this row inside the group's first probability box
-    uint32_t n = 0;                                              // the group's step number (barrier phases)
-    for (int i = 0; i < my_tiles && nc > 0; ++i) {
-      const int qt = 2 * i + static_cast<int>(g);
-      float m = -INFINITY, l = 0.f, alpha_prev = 0.f;
-      float o[kTcHead];
-#pragma unroll
-      for (int k = 0; k < kTcHead; ++k) o[k] = 0.f;
-      // o = o * alpha + O_c of the previous step (its P V product is complete: the probability buffer is free too)
-      auto take_output = [&](uint32_t step, float alpha) {
-        if (!failed && !warp_wait(smem_addr(&bar->o_full[g]), step & 1, lane, &bar->abort)) failed = true;
-        tc_fence_after_sync();
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t r[32];
-          tmem_ld_32x32b_x32(o_addr + h * 32, r);
-          tc_wait_ld();
-#pragma unroll
-          for (int k = 0; k < 32; ++k) o[h * 32 + k] = fmaf(o[h * 32 + k], alpha, __uint_as_float(r[k]));
-        }
-      };
-      for (int c = 0; c < nc; ++c, ++n) {
-        if (!failed && !warp_wait(smem_addr(&bar->s_full[g]), n & 1, lane, &bar->abort)) failed = true;
-        tc_fence_after_sync();
-        const int n_valid = valid - c * kTcChunk;                // keys of this chunk at and past it are padding
-        // pass 1: the row maximum
-        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-        uint32_t rr[2][32];                                      // the next 32 scores load while these are worked on
-        tmem_ld_32x32b_x32(s_addr, rr[0]);
-#pragma unroll
-        for (int pc = 0; pc < 4; ++pc) {
-          uint32_t (&r)[32] = rr[pc & 1];
-          tmem_wait_ld_x32(r);
-          if (pc + 1 < 4) tmem_ld_32x32b_x32(s_addr + (pc + 1) * 32, rr[(pc + 1) & 1]);
-          if (n_valid < (pc + 1) * 32) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k)
-              if (pc * 32 + k >= n_valid) r[k] = 0xff800000u;    // -inf
-          }
-#pragma unroll
-          for (int k = 0; k < 32; k += 4) {
-            mx4[0] = fmaxf(mx4[0], __uint_as_float(r[k])); mx4[1] = fmaxf(mx4[1], __uint_as_float(r[k + 1]));
-            mx4[2] = fmaxf(mx4[2], __uint_as_float(r[k + 2])); mx4[3] = fmaxf(mx4[3], __uint_as_float(r[k + 3]));
-          }
-        }
-        const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-        const float m_new = fmaxf(m, mx * scale);                // finite: the chunk holds at least one valid key
-        const float alpha = fast_exp2(m - m_new);                  // 0 for the tile's first chunk (m = -inf)
-        // the previous chunk's O_c; after this the probability buffer may be overwritten
-        if (c > 0) take_output(n - 1, alpha_prev);
-        alpha_prev = alpha;
-        // pass 2: probabilities (bf16) into shared memory, K-major with 128-byte swizzle, two boxes of 64 keys
+      if (!idle) {
         float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-        tmem_ld_32x32b_x32(s_addr, rr[0]);
+        uint32_t pk[16];
 #pragma unroll
-        for (int pc = 0; pc < 4; ++pc) {
-          uint32_t (&r)[32] = rr[pc & 1];
-          tmem_wait_ld_x32(r);
-          if (pc + 1 < 4) {
-            tmem_ld_32x32b_x32(s_addr + (pc + 1) * 32, rr[(pc + 1) & 1]);
-          } else {                                               // the scores are in registers: their buffer may be refilled
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_addr(&bar->s_empty[g]));
-          }
-          if (n_valid < (pc + 1) * 32) {
-#pragma unroll
-            for (int k = 0; k < 32; ++k)
-              if (pc * 32 + k >= n_valid) r[k] = 0xff800000u;
-          }
-          uint8_t* box = prow + (pc >> 1) * kTcBox;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {                          // eight keys = one 16-byte piece
-            uint32_t pk[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const float p0 = fast_exp2(fmaf(__uint_as_float(r[q * 8 + 2 * e]), scale, -m_new));
-              const float p1 = fast_exp2(fmaf(__uint_as_float(r[q * 8 + 2 * e + 1]), scale, -m_new));
-              sum4[e] += p0 + p1;
-              pk[e] = pack_bf16x2(p0, p1);
-            }
-            const uint32_t piece = static_cast<uint32_t>((pc & 1) * 4 + q);
-            *reinterpret_cast<uint4*>(box + ((piece ^ (row & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          }
+        for (int k = 0; k < 16; ++k) {
+          const float p0 = fast_exp2(fmaf(__uint_as_float(s[2 * k]), scale, -m));
+          const float p1 = fast_exp2(fmaf(__uint_as_float(s[2 * k + 1]), scale, -m));
+          sum4[k & 3] += p0 + p1;
+          pk[k] = pack_bf16x2(p0, p1);
         }
-        l = fmaf(l, alpha, (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]));
-        m = m_new;
-        tc_fence_before_sync();
+        tmem_st_32x32b_x16(buf, pk);
+        l += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
+        tc_wait_st();
+      }
+      tc_fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_addr(&bar->p_full[g][c & 1]));
+    }
+    if (!failed) failed = !wait(&bar->o_last[g], 0);
+    if (!failed && !idle) {
+      tc_fence_after_sync();
+      const float inv = 1.0f / l;                                // at least one valid key: l > 0
+      // through the query tile's shared memory (its last reader was S) and a bulk store
+      uint8_t* stage = smem + kTcOffQ + g * 2 * kTcBox + quad * 4096;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        uint32_t o[32];
+        tmem_ld_32x32b_x32(o_addr + e * 32, o);
+        tmem_wait_ld_x32(o);
+        auto two = [&](int k) { return pack_bf16x2(__uint_as_float(o[k]) * inv, __uint_as_float(o[k + 1]) * inv); };
+#pragma unroll
+        for (int k = 0; k < 32; k += 8)
+          *reinterpret_cast<uint4*>(stage + lane * 128 + (((e * 4 + k / 8) ^ (lane & 7)) << 4)) =
+              make_uint4(two(k), two(k + 2), two(k + 4), two(k + 6));
+      }
+      if (q0 + 32 <= L) {
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_addr(&bar->p_full[g]));
+        if (lane == 0) {
+          tma_store_2d(&out_map, smem_addr(stage), hi * kTcHead, b * L + q0);
+          bulk_wait_read();
+        }
+      } else {                                                   // the sequence ends inside: the rows that exist, four at a time
+        __syncwarp();
+        const int ldo = n_kept * kTcHead;
+        uint16_t* dst = out + (static_cast<size_t>(b) * L + q0) * ldo + hi * kTcHead + (lane & 7) * 8;
+        for (int r = static_cast<int>(lane >> 3); r < L - q0; r += 4)
+          *reinterpret_cast<uint4*>(dst + static_cast<size_t>(r) * ldo) =
+              *reinterpret_cast<const uint4*>(stage + r * 128 + (((lane & 7) ^ (r & 7)) << 4));
       }
-      take_output(n - 1, alpha_prev);
-      const int qi = qt * kTcQTile + static_cast<int>(row);
-      if (qi < L) {
-        const float inv = l > 0.f ? 1.0f / l : 0.f;
-        uint16_t* dst = out + (static_cast<size_t>(b) * L + qi) * ldo + hi * kTcHead;
-#pragma unroll
-        for (int k = 0; k < kTcHead; k += 8)
-          *reinterpret_cast<uint4*>(dst + k) = make_uint4(pack_bf16x2(o[k] * inv, o[k + 1] * inv), pack_bf16x2(o[k + 2] * inv, o[k + 3] * inv),
-                                                          pack_bf16x2(o[k + 4] * inv, o[k + 5] * inv), pack_bf16x2(o[k + 6] * inv, o[k + 7] * inv));
-      }
+      __syncwarp();
     }
   }
   if (failed) {
     bar->abort = 1;
     if (lane == 0) atomicCAS(err, ERR_NONE, ERR_WAIT_TIMEOUT);
+    if (issued) {                                // outstanding MMAs: one more bounded chance before tensor memory is freed
+      if (elect_one()) umma_commit(smem_addr(&bar->drain[g]));
+      __syncwarp();
+      (void)mbar_wait_bounded(smem_addr(&bar->drain[g]), 0);
+    }
   }
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == kTcProducerWarp) tmem_dealloc(tmem, kTcTmemCols);
+  if (warp == kTcMmaWarp) {
+    if (bar->abort && lane == 0 && nc > 0) {     // copies that nobody waited for: a bounded chance to land before the CTA exits
+      for (int r = max(0, bar->requested - kTcRing); r < bar->requested; ++r) {
+        (void)mbar_wait_bounded(smem_addr(&bar->k_full[r % kTcRing]), (r / kTcRing) & 1);
+        (void)mbar_wait_bounded(smem_addr(&bar->v_full[r % kTcRing]), (r / kTcRing) & 1);
+      }
+      for (int t = 0; t < n_groups; ++t) (void)mbar_wait_bounded(smem_addr(&bar->q_full[t]), 0);
+    }
+    __syncwarp();
+    tmem_dealloc(tmem, kTcTmemCols);
+  }
   if (tid == 0) stamp_max(stamps, STAMP_LAST_END);
 }
 
@@ -375,13 +390,15 @@ cudaError_t attention_tc_configure() {
   return cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kTcSmem));
 }
 
-// `qkv_map`: TMA view of qkv as [3 * n_kept * T rows, 64 columns] bf16, boxes of 128 rows, 128-byte swizzle.
-cudaError_t launch_attention_tc(const CUtensorMap& qkv_map, uint16_t* out, int n_kept, int batch, int seq,
+// `qkv_map`: TMA view of qkv as [3 * n_kept * T rows, 64 columns] bf16, boxes of 64 rows, 128-byte swizzle;
+// `out_map`: of out as [T rows, 64 n_kept columns], boxes of 32 rows, the same swizzle.
+cudaError_t launch_attention_tc(const CUtensorMap& qkv_map, const CUtensorMap& out_map, uint16_t* out, int n_kept, int batch, int seq,
                                  const int32_t* seq_lens, int* err, cudaStream_t s, bool pdl, unsigned long long* stamps) {
   if (n_kept <= 0 || batch <= 0) return cudaSuccess;
-  if (seq < 1 || seq > kTcMaxSeq) return cudaErrorInvalidValue;
-  return launch_kernel(attention_tc_kernel, dim3(n_kept, batch), dim3(kTcThreads), kTcSmem, s, pdl, qkv_map, out, seq_lens,
-                       n_kept, batch, seq, err, stamps);
+  if (seq < 1 || seq > kTcMaxSeq || batch > 65535) return cudaErrorInvalidValue;
+  const int tile_pairs = (seq + kTcGroups * kTcQTile - 1) / (kTcGroups * kTcQTile);
+  return launch_kernel(attention_tc_kernel, dim3(tile_pairs, n_kept, batch), dim3(kTcThreads), kTcSmem, s, pdl, qkv_map, out_map, out,
+                       seq_lens, n_kept, batch, seq, err, stamps);
 }
 
 }  // namespace sti

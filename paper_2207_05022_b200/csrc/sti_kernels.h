@@ -111,9 +111,8 @@ cudaError_t launch_attention(const uint16_t* qkv, uint16_t* out, int n_kept, int
 // many tokens (attention_tc.cu).
 // `qkv_map`: TMA view of qkv as [3 * n_kept * T rows, 64 columns] bf16, boxes of 128 rows x 64 columns, 128-byte swizzle.
 cudaError_t attention_tc_configure();
-cudaError_t launch_attention_tc(const CUtensorMap& qkv_map, uint16_t* out, int n_kept, int batch, int seq,
+cudaError_t launch_attention_tc(const CUtensorMap& qkv_map, const CUtensorMap& out_map, uint16_t* out, int n_kept, int batch, int seq,
                                 const int32_t* seq_lens, int* err, cudaStream_t s, bool pdl, unsigned long long* stamps);
-
 
 // out = LayerNorm(sum_p partial[p] + bias + resid) * gamma + beta.
 struct LnLaunch {

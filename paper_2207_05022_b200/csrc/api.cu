@@ -518,14 +518,16 @@ bool make_xmap(CUtensorMap* map, const void* base, int ld, int rows, int box_row
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Whether attention goes to the tcgen05 kernel, one CTA per (sequence, kept head): from 320 keys on, when the other kernel's
-// tiles of 128 queries are more than two to an SM.  (8 sequences of 384, 16 heads: 20.6 against 24.6 us, but 6 of them 20.2
-// against 16.8; 12 of 300 38 against 23: below 320 keys the kernel's 128-key chunks are mostly padding.)
+// Whether attention goes to the tcgen05 kernel: from 97 keys on, when the sequences' tiles of 128 queries are more than the SMs.
+// It has two such tiles per CTA; with fewer of them the other kernel's smaller tiles and key splits use more of the machine
+// (16 heads, the layer's attention in us, this against the other: 4 x 384 13.6 / 16.6, 8 x 300 12.5 / 18.2, 16 x 128 6.2 / 7.1,
+// 32 x 100 10.8 / 11.5; but 8 x 128 5.5 / 4.7, 2 x 512 16.6 / 11.3, 32 x 64 8.0 / 4.7;
+// between 65 and 96 keys they are level).
 bool tc_attention(const sti_plan* p, int nh, int batch, int seq) {
   const int min_items = p->tune.attn_tc_min_items;
   if (min_items == 0 || p->ctx->simt_debug) return false;
   if (min_items > 0) return seq >= 256 && batch * nh >= min_items;
-  return seq > 320 && (seq + 127) / 128 * batch * nh > 2 * p->ctx->sm_count;
+  return seq > 96 && (seq + 127) / 128 * batch * nh > p->ctx->sm_count;
 }
 
 int m_ctas_for(int n_jobs, int T, int cta_budget) {

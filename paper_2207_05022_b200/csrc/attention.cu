@@ -321,8 +321,7 @@ cudaError_t launch_attention(const uint16_t* qkv, uint16_t* out, int n_kept, int
   // (one sequence of 256 keys, 16 heads: 32 queries x 4 splits 4.2 us, 64 x 2 5.3, 128 x 1 6.8) - on the SMs that the O
   // projection after it does not want: its CTAs start meanwhile and decode their weights (the same sequence with 128 CTAs
   // 263 us for six layers, with 64 246).  Where even tiles of 128 queries leave it too few SMs, all of them.
-  // Once the SMs are taken, tiles of 128 queries - fewer reads of K and V - for more than 128 keys, else of 64 (16 x 128, 12
-  // heads: 5.8 us; 128 queries 6.5).
+  // Then tiles of 128 queries: fewer reads of K and V.
   // Blocks of 32 keys where they save half a block of padding (43 x 91: 12.1 against 14.8 us), and up to 32 keys.
   const long limit = ctas(128) <= sm_count - next_ctas ? sm_count - next_ctas : sm_count;
   const bool pad32 = (seq - 1) % 64 < 32;
@@ -330,7 +329,7 @@ cudaError_t launch_attention(const uint16_t* qkv, uint16_t* out, int n_kept, int
   if (seq > 64) {
     if (ctas(32) <= limit) return seq > 128 ? launch_one<2, 4, 64>(a, sm_count, s, pdl) : launch_one<2, 2, 64>(a, sm_count, s, pdl);
     if (seq > 128 && ctas(64) <= limit) return launch_one<4, 2, 64>(a, sm_count, s, pdl);
-    if (seq > 128 || (ctas(64) > limit && ctas(128) <= limit))
+    if (seq > 128 || ctas(64) > limit)
       return pad32 ? launch_one<8, 1, 32>(a, sm_count, s, pdl) : launch_one<8, 1, 64>(a, sm_count, s, pdl);
   }
   return pad32 ? launch_one<4, 1, 32>(a, sm_count, s, pdl) : launch_one<4, 1, 64>(a, sm_count, s, pdl);

@@ -1,4 +1,5 @@
-"""The mma.sync attention kernel against the oracle layer in each of its shapes (query tiles, key splits, key blocks), at
+"""Attention against the oracle layer in each shape of the mma.sync kernel (query tiles, key splits, key blocks) and where the
+tensor-core kernel takes over, at
 lengths around the block sizes, with and without padding masks."""
 import numpy as np
 import pytest
@@ -25,7 +26,8 @@ def _built():
     (1, 129, True), (2, 200, True), (1, 256, False),         # ... and in four
     (10, 150, True), (8, 300, True), (6, 256, True),         # 64 queries, keys split in two; what the O projection leaves
     (17, 150, True), (17, 190, True), (25, 100, True),       # 128 queries, blocks of 32 and of 64 keys
-    (50, 70, True), (50, 100, False),                        # more CTAs than SMs: 64 queries
+    (50, 70, True), (60, 64, False),                         # more tiles of 128 queries than SMs: 32- and 64-key blocks
+    (50, 97, True), (50, 128, True), (17, 385, True),        # ... from 97 keys on the tensor-core kernel
 ])
 def test_attention_shapes(batch, seq, masked):
     from gpu_util import run_layer, rel_err, REL_TOL

@@ -40,11 +40,7 @@ __device__ __forceinline__ void epilogue_block(uint32_t taddr, uint32_t col, con
   tmem_ld_32x32b_x16(taddr + col, r);
   tc_wait_ld();
   float v[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const float a = __uint_as_float(r[i]) + bias_sm[col + i];
-    v[i] = GELU ? gelu_erf(a) : a;
-  }
+  bias_act16<GELU>(r, bias_sm + col, v);
   store_block16<OutT>(v, first + col, ldo, rows_left, lane);
 }
 template <typename OutT, bool GELU, bool FEW>
@@ -189,12 +185,11 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
 #pragma unroll
         for (int cb = 0; cb < 4; ++cb) {
           if (static_cast<uint32_t>(cb * 16) < ncol) {
+            uint32_t r[16];
             float v[16];
 #pragma unroll
-            for (int c = 0; c < 16; ++c) {
-              const float a = acc[cb * 16 + c] + bias_sm[chalf * ncol + cb * 16 + c];
-              v[c] = GELU ? gelu_erf(a) : a;
-            }
+            for (int c = 0; c < 16; ++c) r[c] = __float_as_uint(acc[cb * 16 + c]);
+            bias_act16<GELU>(r, bias_sm + chalf * ncol + cb * 16, v);
             OutT* dst = out + (static_cast<size_t>(job.out_mat) * T + t) * ldo + job.out_col + chalf * ncol + cb * 16;
             for (int c = 0; c < 16; ++c) dst[c] = static_cast<OutT>(v[c]);
           }
@@ -511,11 +506,7 @@ dqgemm_pair_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
         if (chunk0 + c < chunk1) {
           const uint32_t col = (chunk0 + c) * 16;            // 0..127: the first 64 are job 0's features
           float v[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float a = __uint_as_float(r[c][i]) + bias_sm[col + i];
-            v[i] = GELU ? gelu_erf(a) : a;
-          }
+          bias_act16<GELU>(r[c], bias_sm + col, v);
           store_block16<OutT>(v, (col < 64 ? first0 : first1) + (col & 63), ldo, T - row, lane);
         }
       }

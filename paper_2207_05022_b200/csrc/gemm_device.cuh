@@ -329,23 +329,67 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const unsigned int* p) {
   return v;
 }
 
-// erf-GELU.  erf through the rational approximation 7.1.26 of Abramowitz & Stegun (absolute error
+// two floats per instruction
+__device__ __forceinline__ uint64_t pack_f32x2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// erf-GELU of two values.  erf through the rational approximation 7.1.26 of Abramowitz & Stegun (absolute error
 // below 1.5e-7, three orders of magnitude under the bf16 rounding of the result) with the hardware
 // exponential; the epilogue runs it for every element of the FFN1 output.
-__device__ __forceinline__ float gelu_erf(float v) {
-  // gelu(v) = v/2 + |v|/2 * erf(|v| / sqrt 2), erf(x) = 1 - poly(t) t exp(-x^2), t = 1 / (1 + p x)
-  const float x = fabsf(v) * 0.70710678118654752440f;
-  float t;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f, x, 1.0f)));
-  float poly = fmaf(1.061405429f, t, -1.453152027f);
-  poly = fmaf(poly, t, 1.421413741f);
-  poly = fmaf(poly, t, -0.284496736f);
-  poly = fmaf(poly, t, 0.254829592f);
-  float e;                                                   // exp(-x^2) = 2^(v^2 * (-log2(e) / 2))
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"((v * v) * -0.72134752044448170368f));
-  const float erf_abs = fmaf(-(poly * t), e, 1.0f);
-  const float h = 0.5f * v;
-  return fmaf(fabsf(h), erf_abs, h);
+// With t = 1 / (1 + p |v| / sqrt 2) and q(t) the polynomial:  gelu(v) = max(v, 0) - |v| t q(t) / 2 exp(-v^2 / 2).
+// Issue slots bound the epilogue of the many-token kernel (a 128 x 128 tile has 4096 cycles of MMA to hide under), so all but
+// the two special functions work on pairs: FFN1 of 32 x 512 tokens 149 -> 139 us, of 8 x 512 39.7 -> 37.1.
+__device__ __forceinline__ uint64_t gelu_erf_x2(uint64_t v) {
+  const auto both = [](float c) { return pack_f32x2(c, c); };
+  float d0, d1, t0, t1, e0, e1, v0, v1;
+  unpack_f32x2(v, v0, v1);
+  const uint64_t abs_v = pack_f32x2(fminf(fabsf(v0), 1e30f), fminf(fabsf(v1), 1e30f));     // finite: t is 0 for an infinite v
+  unpack_f32x2(fma_f32x2(abs_v, both(0.3275911f * 0.70710678118654752440f), both(1.0f)), d0, d1);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(d0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(d1));
+  const uint64_t t = pack_f32x2(t0, t1);
+  uint64_t q = fma_f32x2(t, both(0.5f * 1.061405429f), both(0.5f * -1.453152027f));
+  q = fma_f32x2(q, t, both(0.5f * 1.421413741f));
+  q = fma_f32x2(q, t, both(0.5f * -0.284496736f));
+  q = fma_f32x2(q, t, both(0.5f * 0.254829592f));
+  unpack_f32x2(mul_f32x2(mul_f32x2(v, v), both(-0.72134752044448170368f)), e0, e1);     // exp(-v^2 / 2) = 2^(v^2 * (-log2(e) / 2))
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(e0));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(e1));
+  const uint64_t minus_tail = mul_f32x2(mul_f32x2(abs_v, t), q) ^ 0x8000000080000000ull;
+  return fma_f32x2(minus_tail, pack_f32x2(e0, e1), pack_f32x2(fmaxf(v0, 0.f), fmaxf(v1, 0.f)));
+}
+
+// 16 accumulator columns + bias (16-byte aligned), erf-GELU if asked for.
+template <bool GELU>
+__device__ __forceinline__ void bias_act16(const uint32_t (&r)[16], const float* bias_sm, float (&v)[16]) {
+#pragma unroll
+  for (int i = 0; i < 16; i += 4) {
+    const float4 b = *reinterpret_cast<const float4*>(bias_sm + i);
+    uint64_t lo = add_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), pack_f32x2(b.x, b.y));
+    uint64_t hi = add_f32x2(pack_f32x2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), pack_f32x2(b.z, b.w));
+    if constexpr (GELU) { lo = gelu_erf_x2(lo); hi = gelu_erf_x2(hi); }
+    unpack_f32x2(lo, v[i], v[i + 1]);
+    unpack_f32x2(hi, v[i + 2], v[i + 3]);
+  }
 }
 
 // 16 output columns of the warp's 32 rows: every lane comes with its own row's values, and the lanes of a group of G (two

@@ -649,6 +649,9 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     CUDA_TRY(mark(2));
   }
   CUDA_TRY(mark(3));
+  // Scratch planes that fill a good part of L2 are dropped there once read instead of being written to memory later.
+  // 16,384 tokens of BERT-large (67 MB a plane): LayerNorm 31.7 -> 27.1 us, forward -2 %; 4096 tokens (17 MB): 8.4 -> 8.7.
+  const int drop_planes = static_cast<size_t>(T) * d.hidden * 4 >= (32u << 20);
   {
     LnLaunch ln{};
     ln.partial = p->partial; ln.n_partial = nh > 0 ? L.o.n_split : 0;
@@ -657,7 +660,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     // With bf16 activations every activation that crosses a kernel boundary is bf16 (the layer's input and output are):
     // the second LayerNorm then takes its residual from the bf16 copy the FFN reads, and no fp32 copy is written.
     ln.out_f32 = bf16_act ? nullptr : p->h1_f32; ln.out_bf16 = p->h1_bf16;
-    ln.stamps = stamp(4);
+    ln.sm_count = c->sm_count; ln.discard = drop_planes; ln.stamps = stamp(4);
     CUDA_TRY(launch_layernorm(ln, c->compute, c->pdl));
     c->launches++;
     L.k_ran[3] = true;
@@ -687,7 +690,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   l2.gamma = dense + c->off_ln2g; l2.beta = dense + c->off_ln2b; l2.eps = d.ln_eps; l2.T = T; l2.d = d.hidden;
   l2.out_f32 = bf16_act ? nullptr : static_cast<float*>(y);
   l2.out_bf16 = bf16_act ? static_cast<uint16_t*>(y) : (want_next_bf16 ? p->x_bf16 : nullptr);
-  l2.stamps = stamp(7);
+  l2.sm_count = c->sm_count; l2.discard = drop_planes; l2.stamps = stamp(7);
   CUDA_TRY(launch_layernorm(l2, c->compute, c->pdl));
   c->launches++;
   L.k_ran[6] = true;

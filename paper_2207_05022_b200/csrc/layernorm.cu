@@ -177,16 +177,26 @@ layernorm_group_kernel(LnLaunch p) {
   }
 }
 
+// A whole line of scratch that nobody will read: its L2 copy is dropped, not written to memory.
+__device__ __forceinline__ void discard_line(const float* p) { asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory"); }
+
 // Many tokens: a warp per row, lane l holding float4 number l, l + 32, ... of it (V = d / 128 of them).  Every load of
-// a row - residual and one partial-sum plane at a time - is issued before the first use, 8 rows per CTA, and the two
+// a row - residual and one partial-sum plane at a time - is issued before the first use, and the two
 // reductions are warp shuffles: no barrier, and enough bytes in flight per SM to keep the memory system busy.
-constexpr int kLnWarpRows = 8;
-constexpr int kLnWarpMinRows = 2048;
-template <int V>
-__global__ void __launch_bounds__(kLnWarpRows * 32)
+// The more registers, the more of a row is in flight, but the fewer warps are resident, and a second wave costs more than either:
+// three builds, each for the rows that it does in one wave.  Two CTAs of eight rows per SM (up to 127 registers) take 2368 rows:
+// with four planes 8.1 -> 6.4 us at 2048 rows of 1024.  Three such CTAs, 3552 rows: 10.1 us at 3072 rows, 10.6 with two per SM.
+// From 4096 rows on (one plane) seven CTAs of four rows (72 registers): 8.4 -> 6.4 us at 4096 rows, 31.7 -> 25.8 at 16,384
+// with the planes discarded; with four planes that build loses (11.7 us at 3072 rows).
+// Tried instead: the residual and the first plane asked for together (86 registers, two CTAs per SM instead of three: 31.6 ->
+// 34.4 us at 16,384 rows of 1024), persistent warps that ask for their next row ahead (level there, 27.9 -> 31.5 with fp32
+// residuals at 10,240 rows).
+constexpr int kLnWarpMinRows = 2048, kLnFewPlanesMinRows = 4096;
+template <int V, int ROWS, int CTAS>
+__global__ void __launch_bounds__(ROWS * 32, CTAS == 3 ? 0 : CTAS)      // 3 come without asking, and without spills
 layernorm_warp_kernel(LnLaunch p) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r = blockIdx.x * kLnWarpRows + warp;
+  const int r = blockIdx.x * ROWS + warp;
   pdl_launch_dependents();
   if (threadIdx.x == 0) { stamp_min(p.stamps, STAMP_FIRST_START); stamp_max(p.stamps, STAMP_LAST_START); }
   float4 a[V];
@@ -230,6 +240,12 @@ layernorm_warp_kernel(LnLaunch p) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
     const float mean = part / static_cast<float>(p.d);
+    if constexpr (ROWS == 4) {
+      if (p.discard) {                 // every lane's loads have returned
+        for (int q = 0; q < p.n_partial; ++q)
+          for (int line = lane; line < V * 4; line += 32) discard_line(p.partial + q * pstride + row + line * 32);
+      }
+    }
     part = 0.f;
 #pragma unroll
     for (int v = 0; v < V; ++v) {
@@ -258,6 +274,14 @@ layernorm_warp_kernel(LnLaunch p) {
   }
 }
 
+template <int V>
+cudaError_t launch_warp_rows(const LnLaunch& p, cudaStream_t s, bool pdl) {
+  const dim3 grid4((p.T + 3) / 4), grid8((p.T + 7) / 8);
+  if (p.T >= kLnFewPlanesMinRows) return launch_kernel(layernorm_warp_kernel<V, 4, 7>, grid4, dim3(128), 0, s, pdl, p);
+  if (p.T > 2 * 8 * p.sm_count) return launch_kernel(layernorm_warp_kernel<V, 8, 3>, grid8, dim3(256), 0, s, pdl, p);
+  return launch_kernel(layernorm_warp_kernel<V, 8, 2>, grid8, dim3(256), 0, s, pdl, p);
+}
+
 __global__ void cast_bf16_kernel(const float* __restrict__ in, uint16_t* __restrict__ out, size_t n4,
                                  unsigned long long* stamps) {
   const size_t i = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -281,16 +305,15 @@ cudaError_t launch_layernorm(const LnLaunch& p, cudaStream_t s, bool pdl) {
   if (p.T <= 0) return cudaSuccess;
   if (p.d % 128 != 0 || p.d > 2048) return cudaErrorInvalidValue;     // d / 4 threads, whole warps
   if (p.T >= kLnWarpMinRows && p.d <= 1024) {      // thousands of rows: a warp per row
-    const dim3 grid((p.T + kLnWarpRows - 1) / kLnWarpRows), block(kLnWarpRows * 32);
     switch (p.d / 128) {
-      case 1: return launch_kernel(layernorm_warp_kernel<1>, grid, block, 0, s, pdl, p);
-      case 2: return launch_kernel(layernorm_warp_kernel<2>, grid, block, 0, s, pdl, p);
-      case 3: return launch_kernel(layernorm_warp_kernel<3>, grid, block, 0, s, pdl, p);
-      case 4: return launch_kernel(layernorm_warp_kernel<4>, grid, block, 0, s, pdl, p);
-      case 5: return launch_kernel(layernorm_warp_kernel<5>, grid, block, 0, s, pdl, p);
-      case 6: return launch_kernel(layernorm_warp_kernel<6>, grid, block, 0, s, pdl, p);
-      case 7: return launch_kernel(layernorm_warp_kernel<7>, grid, block, 0, s, pdl, p);
-      case 8: return launch_kernel(layernorm_warp_kernel<8>, grid, block, 0, s, pdl, p);
+      case 1: return launch_warp_rows<1>(p, s, pdl);
+      case 2: return launch_warp_rows<2>(p, s, pdl);
+      case 3: return launch_warp_rows<3>(p, s, pdl);
+      case 4: return launch_warp_rows<4>(p, s, pdl);
+      case 5: return launch_warp_rows<5>(p, s, pdl);
+      case 6: return launch_warp_rows<6>(p, s, pdl);
+      case 7: return launch_warp_rows<7>(p, s, pdl);
+      case 8: return launch_warp_rows<8>(p, s, pdl);
       default: break;
     }
   }

@@ -127,6 +127,8 @@ struct LnLaunch {
   int T, d;
   float* out_f32;           // optional
   uint16_t* out_bf16;       // optional
+  int sm_count;
+  int discard;              // the planes are not needed after this launch: it may drop them from L2 unwritten
   unsigned long long* stamps;   // profiling record or null
 };
 cudaError_t launch_layernorm(const LnLaunch& p, cudaStream_t s, bool pdl);

@@ -1,6 +1,6 @@
 // Residual + bias + LayerNorm over the split-K partial sums of the O projection and of FFN2
 // (Section 2.1; Section 6: biases and layernorm parameters stay in fp32).
-// Up to 2048 rows of at most 1024: 128 threads to a row.  More rows: a
+// Below 2048 rows of at most 1024: 128 threads to a row.  From there: a
 // warp per row.  Wider rows: one CTA per row, one float4 per thread.
 #include <cuda_bf16.h>
 

@@ -77,13 +77,15 @@ layernorm_kernel(LnLaunch p) {
 }
 
 // Up to 2048 rows of at most 1024: a CTA of 128 threads per row, two float4 each.
-// Bound: latency.  Residual and the first four partial-sum planes are in flight together, gamma and beta while the row is
+// Bound: latency.  Residual and the first P partial-sum planes (four, or eight where there are more) are in flight together, gamma and beta while the row is
 // reduced: two memory round trips and two exchanges between four warps per row (one float4 per thread and one plane at a
 // time took five trips; BERT-large, 256 tokens 5.1 -> 3.7 and 6.5 -> 5.9 us, 1024 tokens 5.6 -> 3.4 and 7.1 -> 6.1,
-// BERT-base, 128 tokens 2.8 -> 2.1 and 3.8 -> 3.1).  Small CTAs also leave an SM sooner: the next GEMM's CTAs, which need a
+// BERT-base, 128 tokens 2.8 -> 2.1 and 3.8 -> 3.1; eight planes at once 4.7 -> 4.1 at BERT-large, 256 tokens, 5.6 -> 4.1 at 384).
+// Small CTAs also leave an SM sooner: the next GEMM's CTAs, which need a
 // whole one and decode their weights meanwhile, start earlier than with rows packed into large CTAs on fewer SMs.
 constexpr uint32_t kLnGroup = 128;
 constexpr int kLnGroupMaxHidden = 1024;
+template <int P>
 __global__ void __launch_bounds__(kLnGroup)
 layernorm_group_kernel(LnLaunch p) {
   __shared__ float red[8];
@@ -108,7 +110,7 @@ layernorm_group_kernel(LnLaunch p) {
   if (gt == 0) stamp_min(p.stamps, STAMP_RELEASE);
   float4 a[2];
   {
-    float4 r[2] = {zero, zero}, s[2][4];
+    float4 r[2] = {zero, zero}, s[2][P / 4][4];
 #pragma unroll
     for (int v = 0; v < 2; ++v) {
       const uint32_t c = gt + kLnGroup * v;
@@ -121,16 +123,17 @@ layernorm_group_kernel(LnLaunch p) {
         }
       }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) s[v][q] = plane(q, v);
+      for (int q = 0; q < P; ++q) s[v][q / 4][q % 4] = plane(q, v);
     }
 #pragma unroll
     for (int v = 0; v < 2; ++v) {
       a[v] = make_float4(bias[v].x + r[v].x, bias[v].y + r[v].y, bias[v].z + r[v].z, bias[v].w + r[v].w);
-      add4(a[v], s[v]);
+#pragma unroll
+      for (int q = 0; q < P / 4; ++q) add4(a[v], s[v][q]);
     }
   }
 #pragma unroll 1
-  for (int q0 = 4; q0 < p.n_partial; q0 += 4) {
+  for (int q0 = P; q0 < p.n_partial; q0 += 4) {
     float4 s[2][4];
 #pragma unroll
     for (int v = 0; v < 2; ++v)
@@ -317,7 +320,9 @@ cudaError_t launch_layernorm(const LnLaunch& p, cudaStream_t s, bool pdl) {
       default: break;
     }
   }
-  if (p.d <= kLnGroupMaxHidden) return launch_kernel(layernorm_group_kernel, dim3(p.T), dim3(kLnGroup), 0, s, pdl, p);
+  if (p.d <= kLnGroupMaxHidden)
+    return p.n_partial > 4 ? launch_kernel(layernorm_group_kernel<8>, dim3(p.T), dim3(kLnGroup), 0, s, pdl, p)
+                           : launch_kernel(layernorm_group_kernel<4>, dim3(p.T), dim3(kLnGroup), 0, s, pdl, p);
   return launch_kernel(layernorm_kernel, dim3(p.T), dim3(p.d / 4), 0, s, pdl, p);
 }
 

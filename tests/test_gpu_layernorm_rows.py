@@ -33,3 +33,19 @@ def test_layernorm_rows(batch, seq, act):
     with sti.Session(work) as s:
         y = run_layer(s, work, 0)
     assert rel_err(y, ref) <= REL_TOL
+
+
+@pytest.mark.parametrize("kept", [4, 5, 8, 9, 12])
+def test_layernorm_planes(kept, monkeypatch):
+    # one partial-sum plane per kept FFN slice: four, up to eight in one go, more in further steps
+    from gpu_util import run_layer, rel_err, REL_TOL
+    monkeypatch.setenv("STI_TUNE", "f2_group=1")
+    shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=3072, n_ffn_slices=12)
+    attn = [[W.UnitPlan(True, 4, True) for _ in range(4)]]
+    ffn = [[W.UnitPlan(i < kept, 4, True) for i in range(12)]]
+    work = W.build_workload("planes", shape, 3, 37, "f32", attn, ffn, seed=kept)
+    a, f = O.decode_layer(work, 0)
+    ref = O.layer_forward(work.x, work.dense[0], a, f, eps=work.ln_eps)
+    with sti.Session(work) as s:
+        y = run_layer(s, work, 0)
+    assert rel_err(y, ref) <= REL_TOL

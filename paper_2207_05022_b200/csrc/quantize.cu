@@ -3,7 +3,8 @@
 // Two kernels produce the same output.  quantize_select_kernel (further down, the default) never sorts: the
 // clusters are equal-population slices of the sorted order, so all it needs are the 2^k - 1 elements that sit at
 // the slice boundaries, which it finds by rank selection.  Units it cannot handle (zero variance, more than
-// kSelMaxSeg weights in one selection bin) are marked and done by quantize_units_kernel, the sorting kernel:
+// kSelMaxSeg weights in one selection bin, an inlier range whose ends it does not find) are marked and done by
+// quantize_units_kernel, the sorting kernel:
 //
 // One CTA of 1024 threads per shard unit runs the paper's steps in order on the unit's flat fp32 array:
 //   1. maximum-likelihood fit of one Gaussian (mean, 1/n variance; fp64 block reductions);
@@ -30,11 +31,14 @@
 #include <type_traits>
 
 #include "../../include/sti_quantize.h"
+#include "outlier_range.h"
 #include "sti_device.cuh"
 
 namespace {
 
 namespace cg = cooperative_groups;
+using sti::extreme_inlier;
+using sti::is_outlier;
 using sti::pdl_launch_dependents;
 using sti::pdl_wait;
 
@@ -123,13 +127,6 @@ __device__ __forceinline__ uint32_t same_digit_lanes(uint32_t d, bool valid) {
   }
   return peers;
 }
-// inv2var = 1 / (2 var); with zero variance c0 is +inf and 0 * inf is NaN, which compares false: no outliers
-__device__ __forceinline__ bool is_outlier(float x, double mu, double inv2var, double c0) {
-  const double d = static_cast<double>(x) - mu;
-  const double ll = c0 - d * d * inv2var;
-  return ll < -4.0;
-}
-
 __global__ void __launch_bounds__(kQThreads, 1)
 quantize_units_kernel(const float* w_all, uint32_t n, int bits, uint32_t* codes_all, float* cent_all, uint32_t* ooff_all,
                       float* oval_all, uint32_t max_out, uint32_t* n_out_all, uint8_t* ws_all, size_t ws_per_unit,
@@ -572,12 +569,13 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     return;
   }
   {
-    // odd lanes look for the largest inlier, even ones for the smallest: from the rounded threshold towards the mean
-    // while the test calls a value an outlier, then away from it while it does not
-    const float away = (lane & 1) != 0 ? INFINITY : -INFINITY;
-    float t = static_cast<float>((lane & 1) != 0 ? mu + radius : mu - radius);
-    while (is_outlier(t, mu, inv2var, c0)) t = nextafterf(t, -away);
-    for (float further = nextafterf(t, away); fabsf(further) < INFINITY && !is_outlier(further, mu, inv2var, c0); further = nextafterf(t, away)) t = further;
+    // odd lanes look for the largest inlier, even ones for the smallest, each from the rounded threshold
+    const bool largest = (lane & 1) != 0;
+    float t = static_cast<float>(largest ? mu + radius : mu - radius);
+    if (!__all_sync(0xffffffffu, extreme_inlier(largest ? INFINITY : -INFINITY, mu, inv2var, c0, t))) {
+      if (rank == 0 && tid == 0) marks[unit] = 1;                      // every thread of the cluster leaves here, too
+      return;
+    }
     un.least = __shfl_sync(0xffffffffu, t, 0);
     un.most = __shfl_sync(0xffffffffu, t, 1);
   }

@@ -169,6 +169,17 @@ def test_units_whose_mean_is_far_off():
         _check(np.stack([shifted, misled]), bits)
 
 
+def test_units_whose_inlier_range_holds_no_fp32_value():
+    """A deviation of 16 gives a radius of 12.6; about 3.0e8 fp32 values are 32 apart, so every weight is an outlier and the
+    search for the ends of the range has to give up.  Beside a unit of an equally large deviation that has its inliers."""
+    rng = np.random.default_rng(9)
+    n = 8192
+    apart = np.where(rng.permutation(n) < n // 2, np.float32(3.0e8), np.float32(3.0e8 + 32)).astype(np.float32)
+    wide = (rng.standard_normal(n) * 16).astype(np.float32)
+    for bits in (2, 5):
+        assert list(_check(np.stack([apart, wide, -apart]), bits)) == [1, 0, 1]
+
+
 def test_outlier_lists_shorter_than_the_outliers_found():
     shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=1024, n_ffn_slices=4)
     mats = make_unit_weights(shape, 13, 0, FFN, 1, outlier_stress=0.01)

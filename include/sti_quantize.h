@@ -45,7 +45,7 @@ size_t sti_quantize_workspace_bytes(uint32_t n_units, uint32_t n_weights);
  *                        2^bits - 1 weights at the slice boundaries are looked for (a histogram over value
  *                        bins, then rank selection inside the few bins that hold a boundary); a unit this
  *                        cannot take (zero variance, very many equal values, no fp32 value near the
- *                        edges of the outlier test) is sorted instead
+ *                        edges of the outlier test, no inlier) is sorted instead
  *   STI_QUANTIZE_SORT    every unit: a stable radix sort of the (value, offset) pairs */
 #define STI_QUANTIZE_SELECT 0
 #define STI_QUANTIZE_SORT 1

@@ -3,7 +3,7 @@
 // Two kernels produce the same output.  quantize_select_kernel (further down, the default) never sorts: the
 // clusters are equal-population slices of the sorted order, so all it needs are the 2^k - 1 elements that sit at
 // the slice boundaries, which it finds by rank selection.  Units it cannot handle (zero variance, more than
-// kSelMaxSeg weights in one selection bin, an inlier range whose ends it does not find) are marked and done by
+// kSelMaxSeg weights in one selection bin, an inlier range whose ends it does not find, no inlier) are marked and done by
 // quantize_units_kernel, the sorting kernel:
 //
 // One CTA of 1024 threads per shard unit runs the paper's steps in order on the unit's flat fp32 array:
@@ -666,6 +666,10 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     n_out += sm.cta_out[r];
   }
   const uint32_t n_in = n - n_out;
+  if (n_in == 0) {                         // no rank to look for: nothing below would be written before it is read
+    if (rank == 0 && tid == 0) marks[unit] = 1;                        // every thread of the cluster leaves
+    return;
+  }
   if (tid <= static_cast<int>(K)) {
     const uint32_t r = static_cast<uint32_t>(static_cast<uint64_t>(tid) * n_in / K);
     sm.bounds[tid] = r;

@@ -180,6 +180,17 @@ def test_units_whose_inlier_range_holds_no_fp32_value():
         assert list(_check(np.stack([apart, wide, -apart]), bits)) == [1, 0, 1]
 
 
+def test_units_without_an_inlier():
+    """Half the weights at -16 and half at +16: the radius of 12.6 leaves a range with fp32 values, but none of the weights."""
+    rng = np.random.default_rng(10)
+    n = 131072                                             # a cluster of several CTAs
+    sign = np.where(rng.permutation(n) < n // 2, np.float32(-16), np.float32(16)).astype(np.float32)
+    one = sign.copy()
+    one[777] = 0.25                                        # a single inlier: every boundary is that weight
+    for bits in (3, 6):
+        assert list(_check(np.stack([sign, one]), bits)) == [1, 0]
+
+
 def test_outlier_lists_shorter_than_the_outliers_found():
     shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=1024, n_ffn_slices=4)
     mats = make_unit_weights(shape, 13, 0, FFN, 1, outlier_stress=0.01)

@@ -194,8 +194,16 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap qkv_map, const __grid_co
   };
   const uint32_t col = tmem + g * 128;
 
-  if (static_cast<int>(g) >= n_groups || nc == 0) {
-    // the second group of a sequence's last, single tile; a sequence without a valid key
+  if (static_cast<int>(g) >= n_groups) {
+    // the second group of a sequence's last, single tile
+  } else if (nc == 0) {
+    // no valid key: the head contributes nothing, and the rows that exist are written all the same
+    if (warp < kTcMmaWarp) {
+      const int q0 = (tile0 + static_cast<int>(g)) * kTcQTile + static_cast<int>(quad * 32), ldo = n_kept * kTcHead;
+      uint16_t* dst = out + (static_cast<size_t>(b) * L + q0) * ldo + hi * kTcHead + (lane & 7) * 8;
+      for (int r = static_cast<int>(lane >> 3); r < min(32, L - q0); r += 4)
+        *reinterpret_cast<uint4*>(dst + static_cast<size_t>(r) * ldo) = make_uint4(0u, 0u, 0u, 0u);
+    }
   } else if (warp >= kTcMmaWarp) {
     // ---- the group's loads and MMAs
     if (lane == 0) {

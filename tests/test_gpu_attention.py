@@ -3,6 +3,7 @@ tensor-core kernel takes over, at
 lengths around the block sizes, with and without padding masks."""
 import numpy as np
 import pytest
+import torch
 
 import workloads as W
 from oracle import sti_oracle as O
@@ -44,3 +45,22 @@ def test_attention_shapes(batch, seq, masked):
         y = run_layer(s, work, 0, lens=lens)
     assert np.isfinite(y).all()
     assert rel_err(y, ref) <= REL_TOL
+
+
+@pytest.mark.parametrize("batch,seq", [(2, 40), (3, 128), (3, 441), (50, 97), (50, 130), (26, 256), (17, 385)])   # the last four: tensor cores
+def test_sequences_without_a_valid_key(batch, seq):
+    """Their attention contributes nothing, whatever the buffers held before; the others are not affected."""
+    from gpu_util import run_layer, rel_err, REL_TOL
+    shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=1024, n_ffn_slices=4)
+    attn = [[W.UnitPlan(i != 1, 4, True) for i in range(4)]]
+    ffn = [[W.UnitPlan(True, 4, True) for _ in range(4)]]
+    work = W.build_workload("empty", shape, batch, seq, "f32", attn, ffn, seed=batch + seq)
+    lens = [0 if b % 2 else 1 + (7 * b) % seq for b in range(batch)]
+    a, f = O.decode_layer(work, 0)
+    with sti.Session(work) as s:
+        poison = torch.full((batch, seq, shape.hidden), float("nan"), device="cuda")
+        run_layer(s, work, 0, poison)                        # every row of the attention output holds NaN
+        y = run_layer(s, work, 0, lens=lens)
+    for b in range(batch):
+        ref = O.layer_forward(work.x[b:b + 1], work.dense[0], a if lens[b] else {}, f, eps=work.ln_eps, seq_lens=lens[b:b + 1])
+        assert rel_err(y[b], ref[0]) <= REL_TOL, (b, lens[b])

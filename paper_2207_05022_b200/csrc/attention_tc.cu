@@ -48,9 +48,11 @@ struct TcBarriers {
   uint64_t p_full[kTcGroups][2];   // its probabilities are
   uint64_t o_full[kTcGroups];      // its P V of a step has completed
   uint64_t o_last[kTcGroups];      // ... of the last step
+  uint64_t tail_zeroed;            // the rows of V past the valid keys are zeros (if there are any: see zero_tail)
   uint64_t drain[kTcGroups];
   int readers_done[kTcMaxSeq / kTcChunk];      // groups that have finished with a chunk
   int requested;                   // chunks asked for so far
+  int tail_taken;                  // a group has taken on the zeroing
   uint32_t tmem_base;
   volatile uint32_t abort;
 };
@@ -154,7 +156,9 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap qkv_map, const __grid_co
       mbar_init(smem_addr(&bar->o_last[g]), 1);
       mbar_init(smem_addr(&bar->drain[g]), 1);
     }
+    mbar_init(smem_addr(&bar->tail_zeroed), 1);
     for (int c = 0; c < kTcMaxSeq / kTcChunk; ++c) bar->readers_done[c] = 0;
+    bar->tail_taken = 0;
     bar->requested = 0;
     bar->abort = 0;
     mbar_fence_init();
@@ -235,11 +239,27 @@ attention_tc_kernel(const __grid_constant__ CUtensorMap qkv_map, const __grid_co
       issued = true;
       return true;
     };
+    // The last 16 keys of P V may hold fewer valid ones.  The others' probabilities are 0, but their rows of V are padding or
+    // the next sequence's, and 0 x Inf and 0 x NaN are NaN: zeros take their place, at most 15 rows of the last chunk, which
+    // nobody has multiplied by yet.  Whichever group comes first does it for both (the swizzle moves pieces inside a row only).
+    auto zero_tail = [&](int st) -> bool {
+      int taken = 0;
+      if (lane == 0) taken = atomicExch(&bar->tail_taken, 1);
+      if (__shfl_sync(0xffffffffu, taken, 0) != 0) return wait(&bar->tail_zeroed, 0);
+      uint4* rows = reinterpret_cast<uint4*>(smem + kTcOffKV + (2 * st + 1) * kTcBox + (valid % kTcChunk) * (kTcHead * 2));
+      const int n_pieces = (16 - valid % 16) * (kTcHead * 2 / 16);
+      for (int i = static_cast<int>(lane); i < n_pieces; i += 32) rows[i] = make_uint4(0u, 0u, 0u, 0u);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_addr(&bar->tail_zeroed));
+      return true;
+    };
     failed = !wait(&bar->q_full[g], 0) || !issue_scores(0) || (ns > 1 && !issue_scores(1));
     for (int c = 0; c < ns && !failed; ++c) {
       // O += P V; the step's second 16 keys are left out if none of them is valid
       const int chunk = c >> 1, st = chunk % kTcRing;
       if ((c & 1) == 0 && !wait(&bar->v_full[st], chunk / kTcRing)) { failed = true; break; }
+      if (c + 1 == ns && valid % 16 != 0 && !zero_tail(st)) { failed = true; break; }
       if (!wait(&bar->p_full[g][c & 1], c >> 1)) { failed = true; break; }
       tc_fence_after_sync();
       if (elect_one()) {

@@ -64,3 +64,29 @@ def test_sequences_without_a_valid_key(batch, seq):
     for b in range(batch):
         ref = O.layer_forward(work.x[b:b + 1], work.dense[0], a if lens[b] else {}, f, eps=work.ln_eps, seq_lens=lens[b:b + 1])
         assert rel_err(y[b], ref[0]) <= REL_TOL, (b, lens[b])
+
+
+@pytest.mark.parametrize("batch,seq,act", [(2, 40, "f32"), (3, 130, "bf16"),                       # mma.sync
+                                           (50, 97, "f32"), (50, 130, "bf16"), (26, 250, "f32"), (17, 441, "bf16")])   # tensor cores
+def test_padding_does_not_reach_valid_rows(batch, seq, act):
+    """Every padded row of the input is NaN, every third sequence has nothing else: the valid rows are those of an input without
+    them.  Odd sequence lengths put the next sequence's rows into the last group of 16 keys."""
+    from gpu_util import run_layer, to_device_act, rel_err, REL_TOL
+    shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=1024, n_ffn_slices=4)
+    attn = [[W.UnitPlan(i != 1, 4, True) for i in range(4)]]
+    ffn = [[W.UnitPlan(True, 4, True) for _ in range(4)]]
+    work = W.build_workload("padding", shape, batch, seq, act, attn, ffn, seed=batch + seq)
+    # full length, one key past a group of 16, one short of it, anything; empty
+    lens = [0 if b % 3 == 1 else (seq, min(seq, 16 * (1 + b // 3) + 1), max(1, seq - seq % 16 - 1), 1 + 31 * b % seq)[b % 4] for b in range(batch)]
+    x, clean = to_device_act(work), work.x.copy()
+    for b, n in enumerate(lens):
+        x[b, n:] = float("nan")
+        clean[b, n:] = 0.0
+    a, f = O.decode_layer(work, 0)
+    with sti.Session(work) as s:
+        y = run_layer(s, work, 0, x, lens=lens)
+    for b, n in enumerate(lens):
+        if n:
+            ref = O.layer_forward(clean[b:b + 1], work.dense[0], a, f, eps=work.ln_eps, seq_lens=[n])
+            assert np.isfinite(y[b, :n]).all(), (b, n)
+            assert rel_err(y[b, :n], ref[0, :n]) <= REL_TOL, (b, n)

@@ -45,7 +45,7 @@ struct Tuning {
   int f2_kacc_min_tokens = 4096;       // FFN2 through the K-accumulating kernel (one output plane) from this many tokens on (0 = never)
   int f2_kacc_k = 512;                 // columns per K group there
   int f2_kacc_bps = 2;                 // boxes of 64 columns per ring stage there (1 or 2)
-  int attn_tc_min_items = -1;          // tensor-core attention: -1 = by the rule below, 0 = never, else from this many (sequence, kept head) pairs on, seq >= 256
+  int attn_tc_min_items = -1;          // tensor-core attention: -1 = by the rule of tc_attention, 0 = never, else from this many (sequence, kept head) pairs on, whatever their length
 };
 
 struct Unit {
@@ -526,7 +526,7 @@ bool make_xmap(CUtensorMap* map, const void* base, int ld, int rows, int box_row
 bool tc_attention(const sti_plan* p, int nh, int batch, int seq) {
   const int min_items = p->tune.attn_tc_min_items;
   if (min_items == 0 || p->ctx->simt_debug) return false;
-  if (min_items > 0) return seq >= 256 && batch * nh >= min_items;
+  if (min_items > 0) return batch * nh >= min_items;
   return seq > 96 && (seq + 127) / 128 * batch * nh > p->ctx->sm_count;
 }
 

@@ -1,6 +1,6 @@
-"""The tensor-core attention kernel (tcgen05, one CTA per sequence and kept head) against the oracle layer, on
-sequence lengths that are and are not multiples of its 128-row tiles, with and without padding masks, and against
-the mma.sync kernel it replaces for many tokens."""
+"""The tensor-core attention kernel (tcgen05, two tiles of 128 query rows of a sequence and kept head per CTA), forced
+for few sequences, against the oracle layer on lengths that are and are not multiples of its tiles and of its 64-key chunks,
+with and without padding masks, and against the mma.sync kernel that few sequences take otherwise."""
 import os
 
 import numpy as np
@@ -47,10 +47,11 @@ def _run(work, lens, tune):
 
 @pytest.mark.parametrize("batch,seq,lens,act", [
     (2, 128, None, "f32"),
-    (3, 200, [200, 57, 130], "bf16"),          # ragged last tile, masks inside the first and the second chunk
-    (2, 512, [512, 300], "bf16"),              # four chunks; a mask that cuts a whole chunk off
-    (2, 384, [1, 129], "f32"),                 # a single valid key; one key into the second chunk
+    (3, 200, [200, 57, 130], "bf16"),          # ragged last tile, masks inside the first and the third chunk
+    (2, 512, [512, 300], "bf16"),              # more chunks than the ring holds; a mask that cuts whole chunks off
+    (2, 384, [1, 129], "f32"),                 # a single valid key; one key into the third chunk
     (1, 130, None, "bf16"),                    # two rows into the second query tile
+    (2, 97, [97, 33], "f32"),                  # the shortest length it is chosen for; one key into the second step of 32
 ])
 def test_tensor_core_attention_layer_matches_oracle_and_the_other_kernel(batch, seq, lens, act):
     from gpu_util import rel_err, REL_TOL
@@ -59,6 +60,7 @@ def test_tensor_core_attention_layer_matches_oracle_and_the_other_kernel(batch, 
     ref = O.layer_forward(work.x, work.dense[0], a, f, eps=work.ln_eps, seq_lens=lens)
     y_tc = _run(work, lens, "attn_tc_min_items=1")
     y_old = _run(work, lens, "attn_tc_min_items=0")
+    assert not np.array_equal(y_tc, y_old)     # two kernels: their sums are in another order
     assert np.isfinite(y_tc).all()
     assert rel_err(y_tc, ref) <= REL_TOL, rel_err(y_tc, ref)
     assert rel_err(y_old, ref) <= REL_TOL
@@ -68,7 +70,7 @@ def test_tensor_core_attention_layer_matches_oracle_and_the_other_kernel(batch, 
 
 
 def test_tensor_core_attention_is_the_default_for_many_sequences():
-    # 24 sequences x 4 kept heads = 96 pairs of 256 tokens: the default rule picks the tensor-core kernel
+    # 24 sequences x 4 kept heads x 2 tiles of 128 queries are more than the SMs: the default rule picks the tensor-core kernel
     from gpu_util import rel_err, REL_TOL, run_layer
     work = _work(24, 256, "bf16", seed=77)
     a, f = O.decode_layer(work, 0)

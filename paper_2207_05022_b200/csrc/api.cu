@@ -245,6 +245,7 @@ void parse_tuning(Tuning* t, int tmax, const sti_model_desc& d, int sm_count) {
         else if (k == "f2_kacc_bps") t->f2_kacc_bps = v == 1 ? 1 : 2;
         else if (k == "attn_tc_min_items") t->attn_tc_min_items = std::max(0, v);
         else if (k == "cta_budget") t->cta_budget = std::max(1, v);
+        else fprintf(stderr, "sti: STI_TUNE has no setting \"%s\"\n", k.c_str());
       }
       pos = end + 1;
     }

@@ -63,15 +63,16 @@ def test_graph_and_dependent_launch_modes_are_bit_identical():
     assert rel_err(y_simt, base) <= 2e-3         # same bf16 operands, only the summation order differs
 
 
-def test_tile_shapes_do_not_change_results_beyond_rounding():
+def test_tile_shapes_do_not_change_results_beyond_rounding(capfd):
     from gpu_util import rel_err, REL_TOL
     work = _workload()
     ref = O.run_workload(work)
-    for tune in ("qkv_n=32,f1_n=32,o_group=1,f2_group=1", "qkv_n=64,f1_n=128,o_group=16,f2_group=4,f2_n=128,o_n=128",
-                 "ln1_ctas=1,ln2_ctas=40",        # LayerNorm rows packed 16 per CTA / two float4 per thread
-                 "ln1_ctas=0,ln2_ctas=0"):        # one row per CTA
+    for tune in ("qkv_n=32,f1_n=32,o_group=1,f2_group=1", "qkv_n=64,f1_n=128,o_group=16,f2_group=4,f2_n=128,o_n=128"):
         y, _ = _run(work, {"STI_TUNE": tune})
         assert rel_err(y, ref) <= REL_TOL, tune
+    assert "STI_TUNE has no setting" not in capfd.readouterr().err       # the library knows every setting named above
+    _run(work, {"STI_TUNE": "no_such_setting=1"})
+    assert "STI_TUNE has no setting \"no_such_setting\"" in capfd.readouterr().err
 
 
 def test_load_then_execute_order_gives_the_same_result():

@@ -242,9 +242,10 @@ __device__ __forceinline__ void finish_task(const DecodeTask& t, const TaskLoads
   uint32_t rc = f.rc;
   float val = f.val;
   for (uint32_t o = lane; o < t.n_out;) {
-    const uint32_t at = rc - t.origin, row = at >> 16, col = at & 0xffffu;
+    uint32_t row, col;
+    const bool inside = outlier_place(t, rc, row, col);
     const bool second = t.narrow ? row >= 32 : col >= 64;
-    if (half == 0 || second == (half == 2))
+    if (inside && (half == 0 || second == (half == 2)))
       reinterpret_cast<uint16_t*>(wsm)[(static_cast<size_t>(t.kcore0 + (col >> 3)) * n_rows + t.row0 + row) * 8 + (col & 7)] = bf16_bits(val);
     o += 32;
     if (o < t.n_out) {

@@ -3,11 +3,7 @@
 #pragma once
 #include <math.h>
 
-#if defined(__CUDACC__)
-#define STI_HOST_DEVICE __host__ __device__ __forceinline__
-#else
-#define STI_HOST_DEVICE inline
-#endif
+#include "host_device.h"
 
 namespace sti {
 

@@ -5,25 +5,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-namespace sti {
+#include "decode_task.h"
 
-// What one warp decodes of a weight tile: 4096 weights, 32 rows x 128 columns of a unit's matrix (64 x 64 when the
-// matrix has 64 in-features).  Index streams are held re-tiled (see retile.h): the k 16-byte planes of the 32 lanes'
-// quanta are stored plane-major, so that a warp reads each plane as one coalesced 512-byte line and every lane ends up
-// with 128 consecutive indexes of one row.  Everything the warp needs to issue its loads stands in these 32 bytes: one
-// memory round trip for the descriptor, one for planes, table and outliers together.
-struct alignas(16) DecodeTask {
-  const uint8_t* codes;     // device; first plane (uncompressed units: the fp32 rows, `out_val` bytes apart)
-  uint32_t table;           // byte distances from `codes`: the unit's 2^bits fp32 centroids,
-  uint32_t out_rc;          //   the task's outliers as (row << 16 | column) of the matrix,
-  uint32_t out_val;         //   and their values
-  uint16_t n_out;
-  uint8_t bits;             // 2..6 or 32; 0 = no task
-  uint8_t narrow;           // 1: 64 rows x 64 columns
-  uint16_t row0, kcore0;    // place in the tile: first row, first group of eight columns
-  uint32_t origin;          // (row << 16 | column) of the task's first weight in the matrix
-};
-static_assert(sizeof(DecodeTask) == 32, "two 16-byte loads");
+namespace sti {
 
 // One weight-stationary tile: n_rows output features x k_total input features.
 struct Job {

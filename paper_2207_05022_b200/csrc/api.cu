@@ -319,6 +319,7 @@ struct TableBuilder {
   std::vector<std::vector<DecodeTask>> job_tasks;
   std::vector<DecodeTask> tasks;       // filled by finish(): job j's tasks start at j * task_stride
   uint32_t w_bytes = 0, k_max = 0, task_stride = 0;
+  bool in_bounds = true;               // every task (task_in_bounds)
   void add(Job j) {
     jobs.push_back(j);
     job_tasks.emplace_back();
@@ -355,6 +356,7 @@ struct TableBuilder {
         t.row0 = static_cast<uint16_t>(r - row0);
         t.kcore0 = static_cast<uint16_t>((koff + j * g.cols) / 8);
         t.origin = r << 16 | j * g.cols;
+        in_bounds = in_bounds && task_in_bounds(t, jobs.back().n_rows, jobs.back().k_total, u.dev + u.off_codes, u.bytes);
         job_tasks.back().push_back(t);
       }
     }
@@ -1250,6 +1252,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
     build_layer_tables(p, L, tb);
     GemmTable* gt[5] = {&L.qkv, &L.o, &L.f1, &L.f2, &L.f2k};
     for (int i = 0; i < 5; ++i) {
+      if (!tb[i].in_bounds) return STI_ERR_STATE;      // not for any plan the calls before let through
       tb[i].finish();
       gt[i]->task_stride = tb[i].task_stride;
       gt[i]->n_jobs = static_cast<int>(tb[i].jobs.size());

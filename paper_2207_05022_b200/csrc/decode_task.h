@@ -35,4 +35,21 @@ STI_HOST_DEVICE bool outlier_place(const DecodeTask& t, uint32_t rc, uint32_t& r
   return (at & (t.narrow ? 0xffc0ffc0u : 0xffe0ff80u)) == 0;     // row < 64 and column < 64; row < 32 and column < 128
 }
 
+// Whether a task stays inside its tile of n_rows x k_total and reads nothing but the `bytes` bytes of its unit at `unit`: looked
+// at once for every task when a plan's tables are built, because the kernels follow a descriptor before anything else has
+// arrived that they could hold it against.
+inline bool task_in_bounds(const DecodeTask& t, uint32_t n_rows, uint32_t k_total, const uint8_t* unit, size_t bytes) {
+  const uint32_t rows = t.narrow ? 64u : 32u, cols = t.narrow ? 64u : 128u;
+  if (t.row0 + rows > n_rows || t.kcore0 * 8u + cols > k_total) return false;
+  if (t.codes < unit || static_cast<size_t>(t.codes - unit) > bytes) return false;
+  const size_t left = bytes - static_cast<size_t>(t.codes - unit);       // from `codes` to the unit's end
+  auto holds = [&](size_t at, size_t n) { return at <= left && n <= left - at; };
+  if (reinterpret_cast<uintptr_t>(t.codes) % 16 != 0) return false;
+  if (t.bits == 32) return t.n_out == 0 && t.out_val % 16 == 0 && holds(0, static_cast<size_t>(rows - 1) * t.out_val + cols * 4u);
+  if (t.bits < 2 || t.bits > 6) return false;
+  const size_t outliers = static_cast<size_t>(t.n_out) * 4;
+  return holds(0, 512u * t.bits) && t.table % 4 == 0 && holds(t.table, 4u << t.bits) &&
+         t.out_rc % 4 == 0 && holds(t.out_rc, outliers) && t.out_val % 4 == 0 && holds(t.out_val, outliers);
+}
+
 }  // namespace sti

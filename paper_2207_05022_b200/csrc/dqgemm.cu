@@ -82,7 +82,8 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
   const uint32_t stage_bytes = bps * kBoxBytes;          // bps boxes of 64 columns per stage
   uint8_t* wsm = xsm + n_stages * stage_bytes;
 
-  // the kernel's own checks of the descriptor: refuse rather than touch memory out of bounds
+  // the kernel's own checks of the job: refuse rather than touch memory out of bounds (the tasks, which `begin` follows before
+  // the job is here, were held to their tile and their unit when the table was built: task_in_bounds)
   const bool bad = job.n_tasks == 0 || job.n_tasks > task_stride || (n_rows != 32 && n_rows != 64 && n_rows != 128) ||
                    (k_total % kChunkK) != 0 || k_total == 0 || n_rows * k_total * 2 > w_bytes ||
                    n_stages < 2 || n_stages > kMaxStages || (bps != 1 && bps != 2 && bps != 4) ||

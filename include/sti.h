@@ -115,7 +115,8 @@ typedef struct {
 
 /* Section 3.1 (the system model: a library the app links; one model per context).
  * Creates streams and scratch sized for max_batch*max_seq tokens on `device`.
- * `compute_stream` is a cudaStream_t to borrow, or NULL to create one. */
+ * `compute_stream` is a cudaStream_t to borrow, or NULL to create one.  The forwards capture graphs of their own on it,
+ * so it must not be under capture by the caller. */
 sti_status sti_ctx_create(const sti_model_desc* desc, int device, void* compute_stream, sti_ctx** out);
 
 /* Section 6: biases and LayerNorm parameters are not quantized; they stay in memory as fp32.
@@ -146,7 +147,9 @@ sti_status sti_plan_finalize(sti_plan* plan);
 /* Section 2.1 / 4.2: one layer over its kept units.  x_dev, y_dev: device, [batch, seq, hidden]
  * contiguous in act_dtype, caller-owned; x_dev == y_dev allowed.  seq_lens_dev: device int32
  * [batch] of valid lengths (padded keys get probability 0) or NULL.  A streamed layer is
- * copied first (not overlapped).  Asynchronous. */
+ * copied first (not overlapped).  Asynchronous.  Host time per call: one graph launch (about 4 us), or seven kernel
+ * launches (about 20 us) for a resident layer of at most 512 tokens whose stream still works on this thread's layer
+ * call before, which then takes 2 to 4 us less on the device. */
 sti_status sti_layer_forward(sti_plan* plan, int layer, const void* x_dev, void* y_dev,
                              int batch, int seq, const int32_t* seq_lens_dev);
 

@@ -847,14 +847,22 @@ sti_status enqueue_forward_io(sti_plan* p, const ForwardKey& k, bool capturing) 
 // call before and decodes its weights meanwhile, which the first kernel of a graph cannot (BERT-base, 128 tokens, one call
 // after the other: 32.8 -> 30.8 us, at 9 of 12 heads and slices 30.7 -> 27.4; BERT-large, 2 x 256: 63.5 -> 60.3).  On an idle
 // stream the graph is ahead, one launch to wait for instead of seven (38.8 against 44.0 us with a wait after each call), and at
-// 1024 tokens and more always (59.5 against 60.0 us, at 2048 105.6 against 107.5).  A call that comes within kBehindNs of the one
-// before finds the stream busy, since a layer takes longer than that; asking the stream itself would cost 2 us.
-thread_local struct { cudaStream_t stream; uint64_t end_ns; } last_layer_call = {nullptr, 0};     // of this thread, any context
+// 1024 tokens and more always (59.5 against 60.0 us, at 2048 105.6 against 107.5).  So the stream is asked whether it still
+// works on the call before - but only within kBehindNs of that call's return, so that calls whose result is awaited do not pay
+// for the question (0.7 us).  The price is the host's: 20 us per call instead of 4, hidden as long as the GPU is the slower
+// one (hidden 128, one head, 16 tokens: 19.8 us per call, 21.8 as graphs).
+struct LayerCall { cudaStream_t stream; uint64_t end_ns; };
+thread_local LayerCall last_layer_call = {nullptr, 0};     // the last one that was enqueued by this thread, any context
 bool launch_layer_directly(const sti_plan* p, const ForwardKey& k) {
   constexpr int kMaxTokens = 512;
   constexpr uint64_t kBehindNs = 8000;
-  return k.layer >= 0 && !k.stamps && p->layers[k.layer].str_bytes == 0 && k.batch * k.seq <= kMaxTokens && p->ctx->pdl &&
-         last_layer_call.stream == p->ctx->compute && host_ns() - last_layer_call.end_ns < kBehindNs;
+  cudaStream_t s = p->ctx->compute;
+  if (k.layer < 0 || k.stamps || p->layers[k.layer].str_bytes > 0 || k.batch * k.seq > kMaxTokens || !p->ctx->pdl ||
+      last_layer_call.stream != s || host_ns() - last_layer_call.end_ns >= kBehindNs)
+    return false;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;      // a stream that is being captured must not be asked
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+  return capture != cudaStreamCaptureStatusNone || cudaStreamQuery(s) == cudaErrorNotReady;
 }
 
 // A forward with the same buffers and shape as the previous one replays its CUDA graph (one launch instead of
@@ -1358,7 +1366,7 @@ sti_status sti_layer_forward(sti_plan* p, int layer, const void* x, void* y, int
   k.x = x; k.y = y; k.lens = lens; k.batch = batch; k.seq = seq; k.layer = layer;
   k.stamps = p->profiling == 3;
   st = model_forward_impl(p, k);
-  last_layer_call = {c->compute, host_ns()};
+  if (st == STI_OK) last_layer_call = {c->compute, host_ns()};
   return st;
 }
 

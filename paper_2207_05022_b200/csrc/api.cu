@@ -39,7 +39,7 @@ struct MatrixInfo {
 
 struct Tuning {
   int qkv_n = 32, f1_n = 64, o_n = 64, o_group = 4, f2_n = 64;
-  int f2_group = 0;                    // FFN slices per K group of FFN2: 0 = chosen per layer (pick_f2_group)
+  int f2_group = 0;                    // FFN slices per K group of FFN2: 0 = chosen per layer and token count (pick_f2_group)
   int cta_budget = 148;                // (replaced by the device's SM count in parse_tuning) CTAs a GEMM launch may use when it splits the token tiles over CTAs
   int pair_min_tiles = 8;              // two-CTA GEMM from this many 128-token tiles on (0 = never)
   int f2_kacc_min_tokens = 4096;       // FFN2 through the K-accumulating kernel (one output plane) from this many tokens on (0 = never)
@@ -77,6 +77,7 @@ struct GemmTable {
   uint32_t w_bytes = 0, n_stages = 0, bps = 1, k_max = 0, hdr_bytes = 0, task_stride = 0;
   bool pair_ok = false;                // consecutive jobs can share two-CTA MMAs (64-row tiles, same K range)
   int n_split = 0;
+  int group = 0;                       // FFN2: slices per K group
 };
 
 struct Layer {
@@ -87,7 +88,8 @@ struct Layer {
   uint8_t* str_host = nullptr;         // in the pinned arena
   int slot = -1;                       // ring slot of the streamed part
   size_t tables_off = 0, tables_bytes = 0;   // this layer's job and task descriptors inside the plan's table buffer
-  GemmTable qkv, o, f1, f2;
+  GemmTable qkv, o, f1;
+  std::vector<GemmTable> f2;           // one for every cut of FFN2's K range that some token count up to the context's takes
   GemmTable f2k;                       // FFN2 again, cut for the K-accumulating kernel (plans made for many tokens only)
   cudaEvent_t ev_loaded = nullptr, ev_done = nullptr, ev_copy_start = nullptr, ev_comp_start = nullptr;
   cudaEvent_t g_ev_loaded = nullptr;   // the same role inside graph capture (captured events cannot be reused outside)
@@ -155,7 +157,6 @@ struct sti_plan {
   uint16_t* x_bf16 = nullptr;          // bf16 copy of fp32 layer inputs (the GEMM operand)
   void* buf[2] = {nullptr, nullptr};
   void* x_in = nullptr; void* y_out = nullptr; int32_t* lens_dev = nullptr;
-  int max_partial = 1;
   float* zero_bias = nullptr;          // all-zero bias vector of sti_gemm_probe (allocated by its first call)
   uint8_t* rate_tables = nullptr;      // every layer's FFN1 tile jobs in one table (sti_decode_rate_probe, built by its first call)
   int rate_jobs = 0; uint32_t rate_task_stride = 0; uint64_t rate_packed_bytes = 0;
@@ -373,35 +374,65 @@ struct TableBuilder {
   }
 };
 
-// FFN slices per K group of FFN2 in a layer that keeps `ns` of them, for the plan's token count.  More slices per group:
-// fewer fp32 planes written and read back by the LayerNorm (8 bytes per element at about 5 TB/s), but a longer decode and MMA
-// chain per CTA (0.7 us per 256 columns and 128-token tile, 0.53 per 256-token tile of the two-CTA kernel, and about 1 us of
-// decode per 256 columns that other kernels do not hide).  BERT-large, six layers with 2 / 4 slices per group: 256 tokens
-// 245 / 247 us, 512 342 / 338, 1024 433 / 421, 2048 627 / 581; BERT-base, 600 tokens with 2 / 3 / 4: 289 / 287 / 296.
-int pick_f2_group(const sti_plan* p, int ns) {
+// Token counts are told apart in tiles of 128, and no further than where the K-accumulating kernel takes over.
+int f2_tiles(const sti_plan* p, long long tokens) {
+  long long most = static_cast<long long>(p->ctx->desc.max_batch) * p->ctx->desc.max_seq;
+  if (p->tune.f2_kacc_min_tokens > 0) most = std::min<long long>(most, p->tune.f2_kacc_min_tokens);
+  return static_cast<int>((std::max(1LL, std::min(tokens, most)) + 127) / 128);
+}
+
+// FFN slices per K group of FFN2 in a layer that keeps `ns` of them, for calls of `n_mtiles` token tiles.  More slices per group:
+// fewer fp32 planes written and read back by the LayerNorm (8 bytes per element at 5 TB/s), but a longer MMA chain per CTA
+// (0.7 us per 256 columns and 128-token tile, 0.4 per 256-token tile of the two-CTA kernel) and a longer decode, of which
+// other kernels leave about 1.4 us per 256 columns in the open; and a launch that fills every SM delays its neighbours (1 us).
+// Groups of more than 1024 columns leave the ring too little: five slices of 256 took 57.0 -> 61.6 us (a BERT-base layer of
+// 9 slices, 1536 tokens).  Fitted to 91 timings with 1 to 6 slices per group, 6 to 16 slices kept, 64 to 4000 tokens: its choice
+// is 0.5 % above the best one in the mean, 4.2 % at most (us per layer with 2 / 3 / 4 slices: BERT-large, 16 slices, 256 tokens
+// 38.6 / 37.2 / 38.7, 1024 68.4 / 69.2 / 64.1; 12 slices, 256 tokens 35.0 / 37.0 / 36.0; BERT-base, 128 tokens 27.3 / 27.7 / 28.3).
+int pick_f2_group(const sti_plan* p, int ns, int n_mtiles) {
   const sti_model_desc& d = p->ctx->desc;
   const Tuning& t = p->tune;
   if (t.f2_group > 0) return t.f2_group;
   const int f = d.ffn / d.n_ffn_slices;
-  double T = static_cast<double>(d.max_batch) * d.max_seq;
-  if (t.f2_kacc_min_tokens > 0) T = std::min(T, static_cast<double>(t.f2_kacc_min_tokens));   // more take the K-accumulating kernel
-  const int n_mtiles = static_cast<int>((T + 127) / 128);
   const bool pair = t.pair_min_tiles > 0 && n_mtiles >= t.pair_min_tiles;
   const int n_tiles = pair ? (n_mtiles + 1) / 2 : n_mtiles;
   int best = 1;                        // also where no more than one slice fits in shared memory
   double best_cost = -1.0;
   for (int g = std::max(1, std::min(2, ns)); g <= ns; ++g) {
-    if (!tile_fits(t.f2_n, g * f)) break;
+    if (g > 1 && (g * f > 1024 || !tile_fits(t.f2_n, g * f))) break;
     const int planes = (ns + g - 1) / g, widest = (ns + planes - 1) / planes, jobs = planes * (d.hidden / t.f2_n);
     const int m_ctas = std::max(1, std::min(n_tiles, t.cta_budget / jobs)), tiles = (n_tiles + m_ctas - 1) / m_ctas;
-    const double waves = std::max(1.0, static_cast<double>(jobs) * m_ctas / t.cta_budget);
-    const double cost = waves * widest * (f / 256.0) * (tiles * (pair ? 0.53 : 0.7) + 1.0) + planes * T * d.hidden * 8.0 / 5.0e6;
+    const double filled = static_cast<double>(jobs) * m_ctas / t.cta_budget;
+    const double cost = std::max(1.0, filled) * widest * (f / 256.0) * (tiles * (pair ? 0.4 : 0.7) + 1.4) +
+                        planes * 128.0 * n_mtiles * d.hidden * 8.0 / 5.0e6 + std::min(1.0, filled);
     if (best_cost < 0.0 || cost < best_cost) { best = g; best_cost = cost; }
   }
   return best;
 }
 
-void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
+// The layer's FFN2 table for a call of `tokens` tokens: chosen by the call, not by what the context could take.
+const GemmTable& f2_table(const sti_plan* p, const Layer& L, int tokens) {
+  const int g = pick_f2_group(p, static_cast<int>(L.kept_slices.size()), f2_tiles(p, tokens));
+  for (const GemmTable& t : L.f2) if (t.group == g) return t;
+  return L.f2.back();
+}
+
+// How many fp32 [tokens][hidden] planes' worth of partial sums a forward of this layer needs at most, in rows.
+size_t partial_rows(const sti_plan* p, const Layer& L) {
+  const sti_model_desc& d = p->ctx->desc;
+  const size_t most = static_cast<size_t>(d.max_batch) * d.max_seq;
+  size_t rows = most * std::max(1, L.o.n_split);
+  for (size_t tokens = std::min<size_t>(128, most);; tokens = std::min(tokens + 128, most)) {
+    rows = std::max(rows, tokens * std::max(1, f2_table(p, L, static_cast<int>(tokens)).n_split));
+    if (tokens == most) return rows;
+  }
+}
+
+struct LayerTables {
+  TableBuilder qkv, o, f1, f2k;
+  std::vector<TableBuilder> f2;
+};
+void build_layer_tables(sti_plan* p, Layer& L, LayerTables& tb) {
   const sti_ctx* c = p->ctx;
   const sti_model_desc& d = c->desc;
   const Tuning& t = p->tune;
@@ -415,8 +446,8 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
         j.n_rows = t.qkv_n; j.k_total = d.hidden; j.x_koff = 0;
         j.out_mat = static_cast<uint32_t>(hi * 3 + which); j.out_col = r0;
         j.bias_off = which * d.n_heads * 64 + h * 64 + static_cast<int>(r0);
-        tb[0].add(j);
-        tb[0].add_rows(c, L.attn[h], STI_ATTN, which, r0, t.qkv_n, 0);
+        tb.qkv.add(j);
+        tb.qkv.add_rows(c, L.attn[h], STI_ATTN, which, r0, t.qkv_n, 0);
       }
   }
   // O projection: K is split over groups of kept heads, each group writes its own partial sum
@@ -429,8 +460,8 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
       Job j{};
       j.n_rows = t.o_n; j.k_total = cnt * 64; j.x_koff = first * 64;
       j.out_mat = sp; j.out_col = n0; j.bias_off = -1;
-      tb[1].add(j);
-      for (int i = 0; i < cnt; ++i) tb[1].add_rows(c, L.attn[L.kept_heads[first + i]], STI_ATTN, 3, n0, t.o_n, i * 64);
+      tb.o.add(j);
+      for (int i = 0; i < cnt; ++i) tb.o.add_rows(c, L.attn[L.kept_heads[first + i]], STI_ATTN, 3, n0, t.o_n, i * 64);
     }
   }
   // FFN1: one job per (kept slice, row tile); full K
@@ -441,22 +472,30 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
       j.n_rows = t.f1_n; j.k_total = d.hidden; j.x_koff = 0;
       j.out_mat = 0; j.out_col = static_cast<uint32_t>(ji * f + r0);
       j.bias_off = s * static_cast<int>(f) + static_cast<int>(r0);
-      tb[2].add(j);
-      tb[2].add_rows(c, L.ffn[s], STI_FFN, 0, r0, t.f1_n, 0);
+      tb.f1.add(j);
+      tb.f1.add_rows(c, L.ffn[s], STI_FFN, 0, r0, t.f1_n, 0);
     }
   }
-  // FFN2: K split over groups of kept slices
+  // FFN2: K split over groups of kept slices, in every way that a call of some size takes
   const int ns = static_cast<int>(L.kept_slices.size());
-  const auto f2_groups = split_units(ns, pick_f2_group(p, ns));
-  L.f2.n_split = static_cast<int>(f2_groups.size());
-  for (int sp = 0; sp < L.f2.n_split; ++sp) {
-    const int first = f2_groups[sp].first, cnt = f2_groups[sp].second;
-    for (uint32_t n0 = 0; n0 < static_cast<uint32_t>(d.hidden); n0 += t.f2_n) {
-      Job j{};
-      j.n_rows = t.f2_n; j.k_total = cnt * f; j.x_koff = first * f;
-      j.out_mat = sp; j.out_col = n0; j.bias_off = -1;
-      tb[3].add(j);
-      for (int i = 0; i < cnt; ++i) tb[3].add_rows(c, L.ffn[L.kept_slices[first + i]], STI_FFN, 1, n0, t.f2_n, i * f);
+  const int most_tiles = f2_tiles(p, static_cast<long long>(d.max_batch) * d.max_seq);
+  for (int tiles = 1; tiles <= most_tiles; ++tiles) {
+    const int group = pick_f2_group(p, ns, tiles);
+    if (std::any_of(L.f2.begin(), L.f2.end(), [&](const GemmTable& have) { return have.group == group; })) continue;
+    const auto f2_groups = split_units(ns, group);
+    L.f2.emplace_back();
+    tb.f2.emplace_back();
+    L.f2.back().group = group;
+    L.f2.back().n_split = static_cast<int>(f2_groups.size());
+    for (int sp = 0; sp < L.f2.back().n_split; ++sp) {
+      const int first = f2_groups[sp].first, cnt = f2_groups[sp].second;
+      for (uint32_t n0 = 0; n0 < static_cast<uint32_t>(d.hidden); n0 += t.f2_n) {
+        Job j{};
+        j.n_rows = t.f2_n; j.k_total = cnt * f; j.x_koff = first * f;
+        j.out_mat = sp; j.out_col = n0; j.bias_off = -1;
+        tb.f2.back().add(j);
+        for (int i = 0; i < cnt; ++i) tb.f2.back().add_rows(c, L.ffn[L.kept_slices[first + i]], STI_FFN, 1, n0, t.f2_n, i * f);
+      }
     }
   }
   // FFN2 for the K-accumulating kernel: 64-row tiles, K groups of at most 512 columns, group-major order
@@ -471,8 +510,8 @@ void build_layer_tables(sti_plan* p, Layer& L, TableBuilder tb[5]) {
         Job j{};
         j.n_rows = 64; j.k_total = cnt * f; j.x_koff = first * f;
         j.out_mat = 0; j.out_col = n0; j.bias_off = -1;
-        tb[4].add(j);
-        for (int i = 0; i < cnt; ++i) tb[4].add_rows(c, L.ffn[L.kept_slices[first + i]], STI_FFN, 1, n0, 64, i * f);
+        tb.f2k.add(j);
+        for (int i = 0; i < cnt; ++i) tb.f2k.add_rows(c, L.ffn[L.kept_slices[first + i]], STI_FFN, 1, n0, 64, i * f);
       }
     }
   }
@@ -674,6 +713,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   }
   CUDA_TRY(mark(4));
   bool f2_kacc = false;
+  const GemmTable& f2 = f2_table(p, L, T);
   if (ns > 0) {
     st = run_gemm(p, GEMM_BF16_TO_BF16_GELU, L.f1, p->h1_bf16, d.hidden, T, p->u, ns * f, dense + c->off_b1, -1, -1, stamp(5));
     if (st != STI_OK) return st;
@@ -682,7 +722,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     if (f2_kacc)
       st = run_gemm_kacc(p, L.f2k, p->u, ns * f, T, p->partial, d.hidden, stamp(6));
     else
-      st = run_gemm(p, GEMM_BF16_TO_F32, L.f2, p->u, ns * f, T, p->partial, d.hidden, nullptr, -1, -1, stamp(6));
+      st = run_gemm(p, GEMM_BF16_TO_F32, f2, p->u, ns * f, T, p->partial, d.hidden, nullptr, -1, -1, stamp(6));
     if (st != STI_OK) return st;
     L.k_ran[4] = L.k_ran[5] = true;
   } else {
@@ -690,7 +730,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   }
   CUDA_TRY(mark(6));
   LnLaunch l2{};
-  l2.partial = p->partial; l2.n_partial = ns > 0 ? (f2_kacc ? 1 : L.f2.n_split) : 0;
+  l2.partial = p->partial; l2.n_partial = ns > 0 ? (f2_kacc ? 1 : f2.n_split) : 0;
   l2.bias = dense + c->off_b2;
   l2.resid = bf16_act ? static_cast<const void*>(p->h1_bf16) : static_cast<const void*>(p->h1_f32);
   l2.resid_bf16 = bf16_act ? 1 : 0;
@@ -1253,51 +1293,55 @@ sti_status sti_plan_finalize(sti_plan* p) {
   std::vector<uint8_t> host_tables;
   struct Fix { GemmTable* t; size_t jobs_off, tasks_off; };
   std::vector<Fix> fixes;
-  p->max_partial = 1;
+  size_t most_partial_rows = 1;
   for (auto& L : p->layers) {
-    TableBuilder tb[5];
+    LayerTables tb;
     L.tables_off = align16(host_tables.size());
     build_layer_tables(p, L, tb);
-    GemmTable* gt[5] = {&L.qkv, &L.o, &L.f1, &L.f2, &L.f2k};
-    for (int i = 0; i < 5; ++i) {
-      if (!tb[i].in_bounds) return STI_ERR_STATE;      // not for any plan the calls before let through
-      tb[i].finish();
-      gt[i]->task_stride = tb[i].task_stride;
-      gt[i]->n_jobs = static_cast<int>(tb[i].jobs.size());
-      gt[i]->w_bytes = tb[i].w_bytes;
-      gt[i]->n_stages = 2; gt[i]->bps = 1;
-      gt[i]->hdr_bytes = gemm_header_bytes();
-      gt[i]->pair_ok = !tb[i].jobs.empty() && tb[i].jobs.size() % 2 == 0;
-      for (size_t j = 0; gt[i]->pair_ok && j < tb[i].jobs.size(); j += 2) {
-        const Job &a = tb[i].jobs[j], &b = tb[i].jobs[j + 1];
-        gt[i]->pair_ok = a.n_rows == 64 && b.n_rows == 64 && a.k_total == b.k_total && a.x_koff == b.x_koff;
+    auto place = [&](GemmTable& gt, TableBuilder& b, bool kacc) -> sti_status {
+      if (!b.in_bounds) return STI_ERR_STATE;          // not for any plan the calls before let through
+      b.finish();
+      gt.task_stride = b.task_stride;
+      gt.n_jobs = static_cast<int>(b.jobs.size());
+      gt.w_bytes = b.w_bytes;
+      gt.n_stages = 2; gt.bps = 1;
+      gt.hdr_bytes = gemm_header_bytes();
+      gt.pair_ok = !b.jobs.empty() && b.jobs.size() % 2 == 0;
+      for (size_t j = 0; gt.pair_ok && j < b.jobs.size(); j += 2) {
+        const Job &even = b.jobs[j], &odd = b.jobs[j + 1];
+        gt.pair_ok = even.n_rows == 64 && odd.n_rows == 64 && even.k_total == odd.k_total && even.x_koff == odd.x_koff;
       }
-      if (i == 4) {                 // two weight buffers, the rest of the shared memory is the ring of single boxes
-        gt[i]->k_max = tb[i].k_max;
-        gt[i]->bps = p->tune.f2_kacc_bps;
-        for (const Job& j : tb[i].jobs)
-          if (j.k_total % (128 * gt[i]->bps / 2) != 0) gt[i]->bps = 1;      // an odd number of boxes somewhere
-        gt[i]->n_stages = gemm_kacc_stages(gt[i]->hdr_bytes, tb[i].k_max, gt[i]->bps, kMaxSmem);
-        gt[i]->smem = gemm_kacc_smem_bytes(gt[i]->hdr_bytes, gt[i]->n_stages, gt[i]->bps, tb[i].k_max);
-        if (!tb[i].jobs.empty() && (gt[i]->n_stages < 2 || gt[i]->smem > kMaxSmem)) return STI_ERR_SHAPE;
+      if (kacc) {                   // two weight buffers, the rest of the shared memory is the ring of single boxes
+        gt.k_max = b.k_max;
+        gt.bps = p->tune.f2_kacc_bps;
+        for (const Job& j : b.jobs)
+          if (j.k_total % (128 * gt.bps / 2) != 0) gt.bps = 1;      // an odd number of boxes somewhere
+        gt.n_stages = gemm_kacc_stages(gt.hdr_bytes, b.k_max, gt.bps, kMaxSmem);
+        gt.smem = gemm_kacc_smem_bytes(gt.hdr_bytes, gt.n_stages, gt.bps, b.k_max);
+        if (!b.jobs.empty() && (gt.n_stages < 2 || gt.smem > kMaxSmem)) return STI_ERR_SHAPE;
       } else {
-      if (!tb[i].jobs.empty() &&
-          !gemm_pick_ring(tb[i].w_bytes, tb[i].k_max, gt[i]->hdr_bytes, &gt[i]->n_stages, &gt[i]->bps))
-        return STI_ERR_SHAPE;
-      gt[i]->smem = gemm_smem_bytes(tb[i].w_bytes, gt[i]->n_stages, gt[i]->bps, gt[i]->hdr_bytes);
+        if (!b.jobs.empty() && !gemm_pick_ring(b.w_bytes, b.k_max, gt.hdr_bytes, &gt.n_stages, &gt.bps)) return STI_ERR_SHAPE;
+        gt.smem = gemm_smem_bytes(b.w_bytes, gt.n_stages, gt.bps, gt.hdr_bytes);
       }
-      if (gt[i]->smem > kMaxSmem && !tb[i].jobs.empty()) return STI_ERR_SHAPE;
-      Fix fx{gt[i], 0, 0};
+      if (gt.smem > kMaxSmem && !b.jobs.empty()) return STI_ERR_SHAPE;
+      Fix fx{&gt, 0, 0};
       fx.jobs_off = align16(host_tables.size());
-      host_tables.resize(fx.jobs_off + tb[i].jobs.size() * sizeof(Job));
-      if (!tb[i].jobs.empty()) memcpy(host_tables.data() + fx.jobs_off, tb[i].jobs.data(), tb[i].jobs.size() * sizeof(Job));
+      host_tables.resize(fx.jobs_off + b.jobs.size() * sizeof(Job));
+      if (!b.jobs.empty()) memcpy(host_tables.data() + fx.jobs_off, b.jobs.data(), b.jobs.size() * sizeof(Job));
       fx.tasks_off = align16(host_tables.size());
-      host_tables.resize(fx.tasks_off + tb[i].tasks.size() * sizeof(DecodeTask));
-      if (!tb[i].tasks.empty()) memcpy(host_tables.data() + fx.tasks_off, tb[i].tasks.data(), tb[i].tasks.size() * sizeof(DecodeTask));
+      host_tables.resize(fx.tasks_off + b.tasks.size() * sizeof(DecodeTask));
+      if (!b.tasks.empty()) memcpy(host_tables.data() + fx.tasks_off, b.tasks.data(), b.tasks.size() * sizeof(DecodeTask));
       fixes.push_back(fx);
-    }
+      return STI_OK;
+    };
+    sti_status st = place(L.qkv, tb.qkv, false);
+    if (st == STI_OK) st = place(L.o, tb.o, false);
+    if (st == STI_OK) st = place(L.f1, tb.f1, false);
+    for (size_t i = 0; i < L.f2.size() && st == STI_OK; ++i) st = place(L.f2[i], tb.f2[i], false);
+    if (st == STI_OK) st = place(L.f2k, tb.f2k, true);
+    if (st != STI_OK) return st;
     L.tables_bytes = host_tables.size() - L.tables_off;
-    p->max_partial = std::max(p->max_partial, std::max(L.o.n_split, L.f2.n_split));
+    most_partial_rows = std::max(most_partial_rows, partial_rows(p, L));
   }
   p->tables_bytes = std::max<size_t>(host_tables.size(), 16);
   CUDA_TRY(cudaMalloc(&p->tables, p->tables_bytes));
@@ -1312,7 +1356,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
   const size_t f = d.ffn / d.n_ffn_slices;
   CUDA_TRY(cudaMalloc(&p->qkv, std::max<size_t>(1, 3 * max_heads) * Tmax * 64 * 2));
   CUDA_TRY(cudaMalloc(&p->attn_out, std::max<size_t>(1, max_heads) * Tmax * 64 * 2));
-  CUDA_TRY(cudaMalloc(&p->partial, static_cast<size_t>(p->max_partial) * Tmax * d.hidden * 4));
+  CUDA_TRY(cudaMalloc(&p->partial, most_partial_rows * d.hidden * 4));
   CUDA_TRY(cudaMalloc(&p->h1_f32, Tmax * d.hidden * 4));
   CUDA_TRY(cudaMalloc(&p->h1_bf16, Tmax * d.hidden * 2));
   CUDA_TRY(cudaMalloc(&p->u, std::max<size_t>(1, max_slices) * Tmax * f * 2));
@@ -1459,7 +1503,7 @@ sti_status sti_gemm_probe(sti_plan* p, int layer, int gemm, const void* x_bf16_d
   Layer& L = p->layers[layer];
   const int nh = static_cast<int>(L.kept_heads.size()), ns = static_cast<int>(L.kept_slices.size());
   const int f = d.ffn / d.n_ffn_slices;
-  const GemmTable* tabs[4] = {&L.qkv, &L.o, &L.f1, &L.f2};
+  const GemmTable* tabs[4] = {&L.qkv, &L.o, &L.f1, &f2_table(p, L, tokens)};
   const GemmTable& tab = *tabs[gemm];
   if (tab.n_jobs == 0) return STI_ERR_STATE;               // no kept unit feeds this GEMM
   const int ldx[4] = {d.hidden, nh * 64, d.hidden, ns * f};

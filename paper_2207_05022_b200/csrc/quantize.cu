@@ -37,7 +37,6 @@
 namespace {
 
 namespace cg = cooperative_groups;
-using sti::extreme_inlier;
 using sti::is_outlier;
 using sti::pdl_launch_dependents;
 using sti::pdl_wait;
@@ -453,6 +452,7 @@ struct SelShared {
   } u;
 };
 static_assert(2 * (sizeof(SelShared) + 1024) <= 228 * 1024, "two CTAs on an SM");
+static_assert(sti::kEndCandidates == 16, "half a warp");
 
 constexpr uint32_t kInfoBoundary = 0x80u;
 
@@ -569,15 +569,17 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     return;
   }
   {
-    // odd lanes look for the largest inlier, even ones for the smallest, each from the rounded threshold
-    const bool largest = (lane & 1) != 0;
-    float t = static_cast<float>(largest ? mu + radius : mu - radius);
-    if (!__all_sync(0xffffffffu, extreme_inlier(largest ? INFINITY : -INFINITY, mu, inv2var, c0, t))) {
+    // half a warp's lanes each around the lower and the upper threshold
+    const int sign = lane < sti::kEndCandidates ? -1 : 1;
+    const float x = sti::end_candidate(static_cast<float>(mu + sign * radius), lane % sti::kEndCandidates, sign);
+    const uint32_t in = __ballot_sync(0xffffffffu, !is_outlier(x, mu, inv2var, c0));
+    const int least = sti::end_index(in & 0xffffu), most = sti::end_index(in >> 16);
+    if (least < 0 || most < 0) {
       if (rank == 0 && tid == 0) marks[unit] = 1;                      // every thread of the cluster leaves here, too
       return;
     }
-    un.least = __shfl_sync(0xffffffffu, t, 0);
-    un.most = __shfl_sync(0xffffffffu, t, 1);
+    un.least = __shfl_sync(0xffffffffu, x, least);
+    un.most = __shfl_sync(0xffffffffu, x, sti::kEndCandidates + most);
   }
 
   // ---- 2. outliers counted per warp, inliers into the histogram

@@ -1,5 +1,5 @@
 """The quantizer's search for the fp32 values at the ends of a unit's inlier range (csrc/outlier_range.h), compiled for the host:
-it finds them for ordinary units and gives up after a fixed number of steps where there are none or they are far away."""
+it finds them for ordinary units and says so where there are none or they are far away, always from the same few candidates."""
 import ctypes as C
 import math
 import os
@@ -13,7 +13,15 @@ from paper_2207_05022_b200 import build
 SOURCE = """
 #include "outlier_range.h"
 extern "C" int outlier(float x, double mu, double inv2var, double c0) { return sti::is_outlier(x, mu, inv2var, c0); }
-extern "C" int extreme(float away, double mu, double inv2var, double c0, float* t) { return sti::extreme_inlier(away, mu, inv2var, c0, *t); }
+extern "C" int end(int sign, double mu, double inv2var, double c0, float* t) {       // what a half of a warp does
+  unsigned in = 0;
+  for (int i = 0; i < sti::kEndCandidates; ++i) in |= (sti::is_outlier(sti::end_candidate(*t, i, sign), mu, inv2var, c0) ? 0u : 1u) << i;
+  const int at = sti::end_index(in);
+  if (at >= 0) *t = sti::end_candidate(*t, at, sign);
+  return at >= 0;
+}
+extern "C" float candidate(float t, int i, int sign) { return sti::end_candidate(t, i, sign); }
+extern "C" int index(unsigned inliers) { return sti::end_index(inliers); }
 """
 
 
@@ -24,7 +32,8 @@ def lib(tmp_path_factory):
     subprocess.run(["g++", "-std=c++17", "-O2", "-shared", "-fPIC", "-I", build.CSRC, str(d / "probe.cpp"), "-o", str(d / "probe.so")], check=True)
     so = C.CDLL(str(d / "probe.so"))
     so.outlier.argtypes = [C.c_float] + [C.c_double] * 3
-    so.extreme.argtypes = [C.c_float] + [C.c_double] * 3 + [C.POINTER(C.c_float)]
+    so.end.argtypes = [C.c_int] + [C.c_double] * 3 + [C.POINTER(C.c_float)]
+    so.candidate.argtypes, so.candidate.restype = [C.c_float, C.c_int, C.c_int], C.c_float
     return so
 
 
@@ -33,9 +42,9 @@ def _search(lib, mu, var):
     c0, inv2var = -0.5 * math.log(2.0 * math.pi * var), 1.0 / (2.0 * var)
     radius = math.sqrt(2.0 * var * (c0 + 4.0))
     ends = []
-    for sign in (-1.0, 1.0):
+    for sign in (-1, 1):
         t = C.c_float(mu + sign * radius)
-        ends.append(t.value if lib.extreme(sign * math.inf, mu, inv2var, c0, C.byref(t)) else None)
+        ends.append(t.value if lib.end(sign, mu, inv2var, c0, C.byref(t)) else None)
     return ends, (mu, inv2var, c0)
 
 
@@ -69,3 +78,17 @@ def test_gives_up_where_the_ends_are_millions_of_values_away(lib):
     for end in (least, most):
         assert end is None or not lib.outlier(end, *p)
     assert least is None and most is None
+
+
+@pytest.mark.parametrize("t", [1.5, -1.5, 1.0, -2.0, 0.0, -0.0, 1e-45, -3e-45, 1.1754944e-38, 3.0e38])
+def test_candidates_are_consecutive_values(lib, t):
+    for sign in (-1, 1):
+        vals = np.array([lib.candidate(t, i, sign) for i in range(16)], np.float32)
+        assert vals[8] == np.float32(t)
+        steps = [np.nextafter(a, np.float32(sign * np.inf)) == b or (a == 0 and b == 0) for a, b in zip(vals[:-1], vals[1:])]
+        assert all(steps)
+
+
+def test_end_index(lib):
+    for mask in range(1 << 16):
+        assert lib.index(mask) == (mask.bit_length() - 1 if 0 < mask < 1 << 15 else -1)

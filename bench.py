@@ -33,14 +33,14 @@ import numpy as np  # noqa: E402
 
 METRIC = "packed_weight_GBps"
 UNIT = "GB/s"
-WORKLOAD = ("configs[3]: 24-layer BERT-large (hidden 1024, 16 heads x 64, FFN 4096 in 16 slices), batch 1, "
+WORKLOAD = ("24-layer BERT-large (hidden 1024, 16 heads x 64, FFN 4096 in 16 slices), batch 1, "
             "seq 256, all shard units kept, bits ~ {2:.15,3:.45,4:.20,5:.10,6:.10}")
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum per dequant-GEMM launch (mean over one layer's QKV, O, FFN1, FFN2
 # launches; BERT-large layer, batch 1, seq 256) from an ncu capture of the present dqgemm.cu; None: none was taken since it
-# changed (profiles/dqgemm_bertlarge_seq256_ncu_full.md, 2,510,720 bytes, is of an earlier build).
+# changed (an earlier build moved 2,510,720 bytes).
 NCU_DRAM_BYTES_PER_GEMM_LAUNCH = None
 
 
@@ -294,7 +294,7 @@ def run_sweep(args):
                 rows.append(row)
         for sess in sessions.values():
             sess.close()
-    print(json.dumps({"sweep": "configs[4]: BERT-large stack, bf16 activations", "n_layers": n_layers,
+    print(json.dumps({"sweep": "BERT-large stack, bf16 activations", "n_layers": n_layers,
                       "peak_source": peak_src, "rows": rows}))
 
 
@@ -1082,7 +1082,7 @@ def main():
         # configuration 3: 12-layer BERT-base, layers 0-2 preloaded, the rest streamed, two ring slots
         extras["config3_model"] = model_point(
             sti, torch, W.make_config(3, workers=workers), stream, flush, peaks,
-            "configs[2]: 12-layer BERT-base, batch 1, seq 128, per-layer random plan (60-100 % kept, 2-6 bits), "
+            "12-layer BERT-base, batch 1, seq 128, per-layer random plan (60-100 % kept, 2-6 bits), "
             "layers 0-2 preloaded, layers 3-11 streamed")
         # configuration 5: two points of the sweep on a 4-layer BERT-large stack (bf16 activations, uniform 3 bits,
         # 2-layer preload when streamed); the whole grid is `bench.py --sweep`
@@ -1090,7 +1090,7 @@ def main():
             w5 = W.make_config(5, n_layers=4, plan="uniform3", resident=False, batch=b5, seq=s5, workers=workers)
             extras[f"config5_b{b5}_s{s5}_uniform3"] = model_point(
                 sti, torch, w5, stream, flush, peaks,
-                f"configs[4] point: 4-layer BERT-large stack, batch {b5}, seq {s5}, uniform 3-bit plan", steps=6, warm=3)
+                f"4-layer BERT-large stack, batch {b5}, seq {s5}, uniform 3-bit plan", steps=6, warm=3)
         extras["planner_plan"] = planner_point(args, target_ms=0.8)
 
     if rank != 0:

@@ -39,9 +39,8 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum per dequant-GEMM launch (mean over one layer's QKV, O, FFN1, FFN2
-# launches; BERT-large layer, batch 1, seq 256) from an ncu capture of the present dqgemm.cu; None: none was taken since it
-# changed (an earlier build moved 2,510,720 bytes).
-NCU_DRAM_BYTES_PER_GEMM_LAUNCH = None
+# launches; BERT-large layer, batch 1, seq 256) from an ncu --set full capture of the present dqgemm.cu.
+NCU_DRAM_BYTES_PER_GEMM_LAUNCH = 2522368
 
 
 def load_peaks():
@@ -802,8 +801,8 @@ def run_quantize(args):
                       "roofline": {"bound": "hbm", "achieved": total_bytes / total_ms / 1e6, "peak": peaks["hbm_gbs"],
                                    "unit": "GB/s", "frac": total_bytes / total_ms / 1e6 / peaks["hbm_gbs"],
                                    "traffic": None, "peak_source": f"hbm_gbs, {peak_src}",
-                                   "note": "totals are the selecting method's (the default); one CTA per unit, five passes "
-                                           "over the unit's fp32 weights, which stay in L2"},
+                                   "note": "totals are the selecting method's (the default); a cluster of CTAs per unit, three passes "
+                                           "over the unit's fp32 weights"},
                       "cpu_baseline": {"value": cpu_weights / cpu_s / 1e6, "unit": "Mweights/s", "cores": blas_threads(),
                                        "kind": "oracle", "sample": "one attention unit and one FFN unit of layer 0"}}))
 

@@ -227,10 +227,11 @@ sti_status sti_get_stats(sti_plan* plan, sti_stats* out);
  * copies the records of the last such forward to `out` (HOST): [layer][kernel][word], STI_STAMP_KERNELS kernels per
  * layer in execution order (fp32->bf16 cast of the model input, QKV, attention, O projection, LayerNorm 1, FFN1,
  * FFN2, LayerNorm 2), STI_STAMP_WORDS words per kernel, times in ns on the device timer, 0 = not stamped (the
- * kernel did not run: dropped units, LayerNorm merged into the preceding GEMM):
+ * kernel did not run: dropped units, later layers' cast):
  *   word 0 first CTA started          1 first CTA past the wait for the preceding kernel   2 last CTA finished
- *   word 3 last weight tile decoded   4 last CTA started      5 accumulators complete      6 row statistics exchanged
- *   (3: dequant-GEMMs only; 5, 6: dequant-GEMMs with the LayerNorm epilogue only; 7 unused)
+ *   word 3 last weight tile decoded (K-accumulating FFN2: the first one; dequant-GEMMs only)   4 last CTA started
+ *   words 5, 6, 7: SM cycles, not times, that a CTA pair's MMA issuer waited for weights, activations and the drain of the
+ *   accumulators (the pair that waited longest; K-accumulating FFN2 only)
  * capacity_words must be at least n_layers * STI_STAMP_KERNELS * STI_STAMP_WORDS (STI_ERR_SIZE otherwise). */
 #define STI_STAMP_KERNELS 8
 #define STI_STAMP_WORDS 8

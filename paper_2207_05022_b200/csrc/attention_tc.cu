@@ -18,7 +18,7 @@
 // any common factor out, so nothing is lost by a maximum that lags behind.
 //
 // Bound: the exponentials.  32 x 128 of them take 256 cycles of an SM's special-function units, 34 us for 32 x 512 tokens of 16
-// heads; measured 60 us, the units 54 % busy, issue slots 52 % (K and V of a sequence resident, one CTA per SM, probabilities
+// heads; measured 60 us, the units 54 % busy, issue slots 47 % (K and V of a sequence resident, one CTA per SM, probabilities
 // through shared memory, O in registers: 117 us; persistent CTAs with a producer and 128-key steps: 74 us).
 //
 // Tensor memory of group g: S and P of even / odd steps at column 128 g / 128 g + 32, O at 128 g + 64.  Waits are bounded; a

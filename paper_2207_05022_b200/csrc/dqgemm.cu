@@ -2,14 +2,14 @@
 //
 // Y[T, N] = X[T, K] * W[N, K]^T where W only exists as bit-packed k-bit dictionary indexes.
 // One CTA owns a weight tile (n_rows output features x k_total input features), decodes it ONCE
-// into shared memory as bf16 (index unpack in registers -> per-unit centroid table in shared
-// memory -> outlier patch), and then streams 128-token activation tiles past it.  After the decode
+// into shared memory as bf16 (index unpack -> per-unit centroid table -> outlier patch), and then streams 128-token activation tiles past it.  After the decode
 // the CTA is warp-specialised, with no CTA-wide barrier in the main loop:
 //   warp 0  producer : TMA (cp.async.bulk.tensor, 128-byte swizzle) brings [128 x 64] bf16 activation
 //                      chunks into a ring of stages; the first stages are requested before the decode
 //   warp 1  MMA      : waits for a chunk, issues tcgen05.mma (M = 128 tokens, N = n_rows, K = 16) into
 //                      one of two TMEM accumulators, tcgen05.commit frees the stage / publishes the tile
-//   warps 4-7 epilogue: tcgen05.ld -> bias / erf-GELU -> global, while the next tile accumulates
+//   warps 2-3 prefetch: the packed shards of the next layer into L2 (the layer's first GEMM only)
+//   warps 4-11 epilogue: tcgen05.ld -> bias / erf-GELU -> global, while the next tile accumulates
 //
 // Weight tile layout in shared memory: element (row, k) at ((k / 8) * rows + row) * 16 + (k % 8) * 2,
 // the no-swizzle K-major core-matrix layout (SBO = 128 B, LBO = rows * 16 B): lanes holding consecutive

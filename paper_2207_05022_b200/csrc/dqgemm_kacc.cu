@@ -245,10 +245,10 @@ dqgemm_kacc_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restri
           }
         }
       }
-      if (lane == 0 && stamps != nullptr) {      // maxima over the launch's pairs, stored complemented like the time stamps
-        atomicMin(stamps + STAMP_ACC, ~static_cast<unsigned long long>(wait_w));
-        atomicMin(stamps + STAMP_EXCHANGED, ~static_cast<unsigned long long>(wait_x));
-        atomicMin(stamps + 7, ~static_cast<unsigned long long>(wait_acc));
+      if (lane == 0 && stamps != nullptr) {      // maxima over the launch's pairs, stored complemented like the other maxima
+        atomicMin(stamps + STAMP_WAIT_WEIGHTS, ~static_cast<unsigned long long>(wait_w));
+        atomicMin(stamps + STAMP_WAIT_ACTIVATIONS, ~static_cast<unsigned long long>(wait_x));
+        atomicMin(stamps + STAMP_WAIT_DRAIN, ~static_cast<unsigned long long>(wait_acc));
       }
       if (failed && issued > 0) {
         if (elect_one()) umma_commit_pair(smem_addr(&hdr->drain));

@@ -11,7 +11,7 @@
 namespace sti {
 namespace {
 
-constexpr int kThreads = 512;               // warp 0: TMA producer, warp 1: MMA issuer, warps 4-7: epilogue; all 16 decode
+constexpr int kThreads = 512;               // warp 0: TMA producer, warp 1: MMA issuer, warps 4-11: epilogue; all 16 decode
 constexpr int kWarps = kThreads / 32;
 constexpr int kTileM = 128;                 // tokens per MMA tile
 constexpr int kChunkK = 64;                 // one TMA box = 64 columns = one 128-byte swizzle row; a stage holds 1, 2 or 4 boxes

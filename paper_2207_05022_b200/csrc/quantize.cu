@@ -415,9 +415,10 @@ quantize_units_kernel(const float* w_all, uint32_t n, int bits, uint32_t* codes_
 //
 // Bound: with few units the chain of seven cluster barriers and the table passes between them (half of the 31 us that
 // 12 units of 196,608 weights take at 4 bits; one CTA of 1024 threads per unit and five passes took 126 us); with many
-// units shared memory - the histogram's atomics, about 5 cycles for a warp's 32 weights on an SM, and in the last pass
-// the table lookup and the fp64 read-modify-write of the sums, about 9 (384 units of 524,288 weights at 3 bits: 1055 ->
-// 625 us, 1.4 TB/s of the 6.5 a copy moves; 16 such units at 6 bits, where four lanes take turns at the sums, 435 -> 95).
+// units issue slots (65 % busy at 3 bits) and the shared-memory pipe (52 %): 4 cycles for a warp's 32 weights in the
+// histogram's atomics, 9 in the table lookup, the fp64 read-modify-write of the sums and the staging of the stream (384 units of
+// 524,288 weights at 3 bits: 1055 -> 623 us, 1.4 TB/s of the 6.5 a copy moves; 16 such units at 6 bits, where four lanes
+// take turns at the sums, 435 -> 94).
 
 constexpr int kSelThreads = 512;
 constexpr int kSelWarps = kSelThreads / 32;

@@ -65,8 +65,10 @@ enum StampSlot : int {
   STAMP_LAST_END = 2,      // max: the last CTA is done
   STAMP_DECODED = 3,       // max: weight tiles decoded (dequant-GEMM)
   STAMP_LAST_START = 4,    // max: the launch's last CTA starts
-  STAMP_ACC = 5,           // max: accumulators complete (dequant-GEMM with the LayerNorm epilogue)
-  STAMP_EXCHANGED = 6      // max: row statistics of all column tiles have arrived (same)
+  // SM cycles that the MMA-issuing warp spent waiting, max (K-accumulating dequant-GEMM only)
+  STAMP_WAIT_WEIGHTS = 5,
+  STAMP_WAIT_ACTIVATIONS = 6,
+  STAMP_WAIT_DRAIN = 7
 };
 __device__ __forceinline__ void stamp_min(unsigned long long* rec, int slot) {
   if (rec != nullptr) atomicMin(rec + slot, static_cast<unsigned long long>(global_timer_ns()));

@@ -91,9 +91,10 @@ cudaError_t launch_attention(const uint16_t* qkv, uint16_t* out, int n_kept, int
                              const int32_t* seq_lens, int sm_count, int next_ctas, cudaStream_t s, bool pdl,
                              unsigned long long* stamps);
 
-// The same attention on the tcgen05 tensor cores, one CTA per (sequence, kept head) with two query tiles in flight, for
+// The same attention on the tcgen05 tensor cores, one CTA per two tiles of 128 queries of a (sequence, kept head), for
 // many tokens (attention_tc.cu).
-// `qkv_map`: TMA view of qkv as [3 * n_kept * T rows, 64 columns] bf16, boxes of 128 rows x 64 columns, 128-byte swizzle.
+// `qkv_map`: TMA view of qkv as [3 * n_kept * T rows, 64 columns] bf16, boxes of 64 rows x 64 columns, 128-byte swizzle;
+// `out_map`: of out as [T rows, 64 n_kept columns], boxes of 32 rows x 64 columns, the same swizzle.
 cudaError_t attention_tc_configure();
 cudaError_t launch_attention_tc(const CUtensorMap& qkv_map, const CUtensorMap& out_map, uint16_t* out, int n_kept, int batch, int seq,
                                 const int32_t* seq_lens, int* err, cudaStream_t s, bool pdl, unsigned long long* stamps);

@@ -192,10 +192,10 @@ sti_status sti_shard_decode(sti_plan* plan, int layer, sti_kind kind, int index,
  *                         units, each group writes its own partial sum (the caller adds them up)
  *   out_capacity_bytes : size of out_dev; STI_ERR_SIZE when the result would not fit
  *   variant    : 0 = the kernel a forward would choose for this token count, 1 = the one-CTA kernel,
- *                2 = the two-CTA (cta_group::2) kernel, STI_ERR_STATE when the tiling does not allow it,
- *                3 = (gemm 3 only) the K-accumulating two-CTA kernel that forwards of many tokens use for FFN2:
- *                all K groups summed in tensor memory, ONE complete plane written (n_partials = 1);
- *                STI_ERR_STATE when the plan was not made for that many tokens
+ *                2 = the kernels of calls of many tokens: the layer's weights decoded into a working buffer, then a
+ *                two-CTA (cta_group::2) GEMM over it,
+ *                3 = (gemm 3 only) the same with the K range in one piece, as forwards of many tokens run FFN2: ONE
+ *                complete plane written (n_partials = 1); STI_ERR_STATE when the plan was not made for that many tokens
  *   n_partials : optional out
  * STI_ERR_STATE when no kept unit feeds the GEMM.  A streamed layer is copied first.  Asynchronous. */
 sti_status sti_gemm_probe(sti_plan* plan, int layer, int gemm, const void* x_bf16_dev, int tokens, void* out_dev,
@@ -229,9 +229,10 @@ sti_status sti_get_stats(sti_plan* plan, sti_stats* out);
  * FFN2, LayerNorm 2), STI_STAMP_WORDS words per kernel, times in ns on the device timer, 0 = not stamped (the
  * kernel did not run: dropped units, later layers' cast):
  *   word 0 first CTA started          1 first CTA past the wait for the preceding kernel   2 last CTA finished
- *   word 3 last weight tile decoded (K-accumulating FFN2: the first one; dequant-GEMMs only)   4 last CTA started
- *   words 5, 6, 7: SM cycles, not times, that a CTA pair's MMA issuer waited for weights, activations and the drain of the
- *   accumulators (the pair that waited longest; K-accumulating FFN2 only)
+ *   word 3 last weight tile decoded (fused dequant-GEMMs of calls of few tokens only)   4 last CTA started
+ *   words 5, 6, 7: not used
+ * Decoding a layer into the working buffer (calls of many tokens) has no record: it runs beside the GEMMs of the layer before,
+ * or ahead of QKV.
  * capacity_words must be at least n_layers * STI_STAMP_KERNELS * STI_STAMP_WORDS (STI_ERR_SIZE otherwise). */
 #define STI_STAMP_KERNELS 8
 #define STI_STAMP_WORDS 8

@@ -41,10 +41,9 @@ struct Tuning {
   int qkv_n = 32, f1_n = 64, o_n = 64, o_group = 4, f2_n = 64;
   int f2_group = 0;                    // FFN slices per K group of FFN2: 0 = chosen per layer and token count (pick_f2_group)
   int cta_budget = 148;                // (replaced by the device's SM count in parse_tuning) CTAs a GEMM launch may use when it splits the token tiles over CTAs
-  int pair_min_tiles = 8;              // two-CTA GEMM from this many 128-token tiles on (0 = never)
-  int f2_kacc_min_tokens = 4096;       // FFN2 through the K-accumulating kernel (one output plane) from this many tokens on (0 = never)
-  int f2_kacc_k = 512;                 // columns per K group there
-  int f2_kacc_bps = 2;                 // boxes of 64 columns per ring stage there (1 or 2)
+  int wide_min_tokens = 449;           // weights decoded into the working buffer, GEMMs over it, from this many tokens on (0 = never)
+  int f2_kacc_min_tokens = 4096;       // there, FFN2's K range in one piece (one output plane) from this many tokens on (0 = by cost)
+  int wide_nt = 0, wide_splits = 0;    // there, features per tile and K splits: 0 = chosen by pick_wide
   int attn_tc_min_items = -1;          // tensor-core attention: -1 = by the rule of tc_attention, 0 = never, else from this many (sequence, kept head) pairs on, whatever their length
 };
 
@@ -74,10 +73,15 @@ struct GemmTable {
   DecodeTask* tasks = nullptr;
   int n_jobs = 0;
   size_t smem = 0;
-  uint32_t w_bytes = 0, n_stages = 0, bps = 1, k_max = 0, hdr_bytes = 0, task_stride = 0;
-  bool pair_ok = false;                // consecutive jobs can share two-CTA MMAs (64-row tiles, same K range)
+  uint32_t w_bytes = 0, n_stages = 0, bps = 1, hdr_bytes = 0, task_stride = 0;
   int n_split = 0;
   int group = 0;                       // FFN2: slices per K group
+};
+
+// One of a layer's weight matrices in the working buffer (expand.cu).
+struct WideMatrix {
+  uint32_t row0 = 0;                   // first 128-byte row
+  uint32_t n = 0, k_chunks = 0;        // features, chunks of 64 columns
 };
 
 struct Layer {
@@ -90,7 +94,10 @@ struct Layer {
   size_t tables_off = 0, tables_bytes = 0;   // this layer's job and task descriptors inside the plan's table buffer
   GemmTable qkv, o, f1;
   std::vector<GemmTable> f2;           // one for every cut of FFN2's K range that some token count up to the context's takes
-  GemmTable f2k;                       // FFN2 again, cut for the K-accumulating kernel (plans made for many tokens only)
+  WideMatrix wide[4];                  // QKV, O, FFN1, FFN2 in the working buffer, and the tasks that fill it
+  const DecodeTask* wide_tasks = nullptr;
+  uint32_t wide_first[5] = {0, 0, 0, 0, 0};           // matrix m's tasks: wide_first[m] .. wide_first[m + 1]
+  const int32_t* wide_bias[2] = {nullptr, nullptr};   // QKV, FFN1: where the bias of every 64 features begins
   cudaEvent_t ev_loaded = nullptr, ev_done = nullptr, ev_copy_start = nullptr, ev_comp_start = nullptr;
   cudaEvent_t g_ev_loaded = nullptr;   // the same role inside graph capture (captured events cannot be reused outside)
   cudaEvent_t ev_k[8] = {};           // boundaries of the seven kernels (kernel-level profiling)
@@ -157,6 +164,9 @@ struct sti_plan {
   uint16_t* x_bf16 = nullptr;          // bf16 copy of fp32 layer inputs (the GEMM operand)
   void* buf[2] = {nullptr, nullptr};
   void* x_in = nullptr; void* y_out = nullptr; int32_t* lens_dev = nullptr;
+  uint8_t* wide_buf = nullptr;         // two working buffers for decoded weights, of even and of odd layers (plans for many tokens)
+  size_t wide_bytes = 0;               // of each
+  uint8_t* wide_tables = nullptr;      // their tasks and bias offsets
   float* zero_bias = nullptr;          // all-zero bias vector of sti_gemm_probe (allocated by its first call)
   uint8_t* rate_tables = nullptr;      // every layer's FFN1 tile jobs in one table (sti_decode_rate_probe, built by its first call)
   int rate_jobs = 0; uint32_t rate_task_stride = 0; uint64_t rate_packed_bytes = 0;
@@ -216,12 +226,11 @@ std::vector<std::pair<int, int>> split_units(int n, int most) {
   return groups;
 }
 
-void parse_tuning(Tuning* t, int tmax, const sti_model_desc& d, int sm_count) {
+void parse_tuning(Tuning* t, const sti_model_desc& d, int sm_count) {
   t->cta_budget = sm_count;
-  // few tokens: K groups of at most 8 heads (the decode is spread over the SMs, MMA chains stay short); many tokens: wide
-  // K groups, each CTA walks many token tiles with its decoded weights
+  // K groups of at most 8 heads: the decode is spread over the SMs, MMA chains stay short
   t->qkv_n = 64; t->f1_n = 64; t->o_n = 64; t->f2_n = 64;
-  t->o_group = tmax > 1024 ? 16 : 8;
+  t->o_group = 8;
   const char* env = getenv("STI_TUNE");     // debugging aid: "qkv_n=32,o_group=4,..."
   if (env) {
     std::string s(env);
@@ -240,10 +249,10 @@ void parse_tuning(Tuning* t, int tmax, const sti_model_desc& d, int sm_count) {
         else if (k == "o_group") t->o_group = v;
         else if (k == "f2_n") t->f2_n = v;
         else if (k == "f2_group") t->f2_group = v;
-        else if (k == "pair_min_tiles") t->pair_min_tiles = v;
+        else if (k == "wide_min_tokens") t->wide_min_tokens = std::max(0, v);
+        else if (k == "wide_nt") t->wide_nt = v == 128 || v == 256 ? v : 0;
+        else if (k == "wide_splits") t->wide_splits = std::max(0, std::min(v, 8));
         else if (k == "f2_kacc_min_tokens") t->f2_kacc_min_tokens = std::max(0, v);
-        else if (k == "f2_kacc_k") t->f2_kacc_k = std::max(64, std::min(v, 1024));
-        else if (k == "f2_kacc_bps") t->f2_kacc_bps = v == 1 ? 1 : 2;
         else if (k == "attn_tc_min_items") t->attn_tc_min_items = std::max(0, v);
         else if (k == "cta_budget") t->cta_budget = std::max(1, v);
         else fprintf(stderr, "sti: STI_TUNE has no setting \"%s\"\n", k.c_str());
@@ -315,6 +324,46 @@ void order_outliers(const MatrixInfo* mi, int nm, const uint32_t* off, const flo
   }
 }
 
+// The tasks of matrix `m` of a unit: at(row, j) is the one whose first weight is in row `row`, number `j` of the tasks side by
+// side; its place is the caller's.
+struct MatrixTasks {
+  const Unit& u;
+  MatrixInfo mi;
+  TaskGrid g;
+  size_t codes;                        // where the matrix's indexes (or fp32 rows) begin in the layer part
+  uint32_t first;                      // tasks of the unit before it
+  MatrixTasks(const sti_ctx* c, const Unit& unit, sti_kind kind, int m) : u(unit) {
+    int nm;
+    const MatrixInfo* all = unit_matrices(c, kind, &nm);
+    mi = all[m];
+    g = task_grid(mi);
+    codes = u.off_codes;
+    for (int i = 0; i < m; ++i) codes += matrix_code_bytes(all[i], u.cfg.bits);
+    first = tasks_before(all, m);
+  }
+  DecodeTask at(uint32_t row, uint32_t j) const {
+    const uint32_t bits = static_cast<uint32_t>(u.cfg.bits), in_matrix = row / g.rows * g.per_row + j;
+    DecodeTask t{};
+    size_t begin = codes;
+    if (bits == 32) {
+      begin += (static_cast<size_t>(row) * mi.kc + j * g.cols) * 4;
+      t.out_val = mi.kc * 4;                                // from row to row
+    } else {
+      begin += static_cast<size_t>(in_matrix) * 512 * bits;
+      const uint32_t out0 = u.task_first[first + in_matrix];
+      t.n_out = static_cast<uint16_t>(u.task_first[first + in_matrix + 1] - out0);
+      t.table = static_cast<uint32_t>(u.off_table - begin);
+      t.out_rc = static_cast<uint32_t>(u.off_orc + 4 * static_cast<size_t>(out0) - begin);
+      t.out_val = static_cast<uint32_t>(u.off_oval + 4 * static_cast<size_t>(out0) - begin);
+    }
+    t.codes = u.dev + begin;
+    t.bits = static_cast<uint8_t>(bits);
+    t.narrow = g.cols == 64;
+    t.origin = row << 16 | j * g.cols;
+    return t;
+  }
+};
+
 struct TableBuilder {
   std::vector<Job> jobs;
   std::vector<std::vector<DecodeTask>> job_tasks;
@@ -329,34 +378,13 @@ struct TableBuilder {
   }
   // Rows [row0, row0 + n_rows) of matrix `m` of `u` go to columns koff .. of the last job's tile.
   void add_rows(const sti_ctx* c, const Unit& u, sti_kind kind, int m, uint32_t row0, uint32_t n_rows, uint32_t koff) {
-    int nm;
-    const MatrixInfo* mi = unit_matrices(c, kind, &nm);
-    const int bits = u.cfg.bits;
-    size_t mat_off = u.off_codes;
-    for (int i = 0; i < m; ++i) mat_off += matrix_code_bytes(mi[i], bits);
-    const TaskGrid g = task_grid(mi[m]);
+    const MatrixTasks of(c, u, kind, m);
+    const TaskGrid& g = of.g;
     for (uint32_t r = row0; r < row0 + n_rows; r += g.rows) {
       for (uint32_t j = 0; j < g.per_row; ++j) {
-        const uint32_t in_matrix = r / g.rows * g.per_row + j, index = tasks_before(mi, m) + in_matrix;
-        DecodeTask t{};
-        size_t at;
-        if (bits == 32) {
-          at = mat_off + (static_cast<size_t>(r) * mi[m].kc + j * g.cols) * 4;
-          t.out_val = mi[m].kc * 4;                         // from row to row
-        } else {
-          at = mat_off + static_cast<size_t>(in_matrix) * 512 * bits;
-          const uint32_t first = u.task_first[index];
-          t.n_out = static_cast<uint16_t>(u.task_first[index + 1] - first);
-          t.table = static_cast<uint32_t>(u.off_table - at);
-          t.out_rc = static_cast<uint32_t>(u.off_orc + 4 * static_cast<size_t>(first) - at);
-          t.out_val = static_cast<uint32_t>(u.off_oval + 4 * static_cast<size_t>(first) - at);
-        }
-        t.codes = u.dev + at;
-        t.bits = static_cast<uint8_t>(bits);
-        t.narrow = g.cols == 64;
+        DecodeTask t = of.at(r, j);
         t.row0 = static_cast<uint16_t>(r - row0);
         t.kcore0 = static_cast<uint16_t>((koff + j * g.cols) / 8);
-        t.origin = r << 16 | j * g.cols;
         in_bounds = in_bounds && task_in_bounds(t, jobs.back().n_rows, jobs.back().k_total, u.dev + u.off_codes, u.bytes);
         job_tasks.back().push_back(t);
       }
@@ -374,16 +402,16 @@ struct TableBuilder {
   }
 };
 
-// Token counts are told apart in tiles of 128, and no further than where the K-accumulating kernel takes over.
+// Token counts are told apart in tiles of 128, and no further than where the working buffer takes over.
 int f2_tiles(const sti_plan* p, long long tokens) {
   long long most = static_cast<long long>(p->ctx->desc.max_batch) * p->ctx->desc.max_seq;
-  if (p->tune.f2_kacc_min_tokens > 0) most = std::min<long long>(most, p->tune.f2_kacc_min_tokens);
+  if (p->tune.wide_min_tokens > 0) most = std::min<long long>(most, p->tune.wide_min_tokens);
   return static_cast<int>((std::max(1LL, std::min(tokens, most)) + 127) / 128);
 }
 
 // FFN slices per K group of FFN2 in a layer that keeps `ns` of them, for calls of `n_mtiles` token tiles.  More slices per group:
 // fewer fp32 planes written and read back by the LayerNorm (8 bytes per element at 5 TB/s), but a longer MMA chain per CTA
-// (0.7 us per 256 columns and 128-token tile, 0.4 per 256-token tile of the two-CTA kernel) and a longer decode, of which
+// (0.7 us per 256 columns and 128-token tile) and a longer decode, of which
 // other kernels leave about 1.4 us per 256 columns in the open; and a launch that fills every SM delays its neighbours (1 us).
 // Groups of more than 1024 columns leave the ring too little: five slices of 256 took 57.0 -> 61.6 us (a BERT-base layer of
 // 9 slices, 1536 tokens).  Fitted to 91 timings with 1 to 6 slices per group, 6 to 16 slices kept, 64 to 4000 tokens: its choice
@@ -394,16 +422,14 @@ int pick_f2_group(const sti_plan* p, int ns, int n_mtiles) {
   const Tuning& t = p->tune;
   if (t.f2_group > 0) return t.f2_group;
   const int f = d.ffn / d.n_ffn_slices;
-  const bool pair = t.pair_min_tiles > 0 && n_mtiles >= t.pair_min_tiles;
-  const int n_tiles = pair ? (n_mtiles + 1) / 2 : n_mtiles;
   int best = 1;                        // also where no more than one slice fits in shared memory
   double best_cost = -1.0;
   for (int g = std::max(1, std::min(2, ns)); g <= ns; ++g) {
     if (g > 1 && (g * f > 1024 || !tile_fits(t.f2_n, g * f))) break;
     const int planes = (ns + g - 1) / g, widest = (ns + planes - 1) / planes, jobs = planes * (d.hidden / t.f2_n);
-    const int m_ctas = std::max(1, std::min(n_tiles, t.cta_budget / jobs)), tiles = (n_tiles + m_ctas - 1) / m_ctas;
+    const int m_ctas = std::max(1, std::min(n_mtiles, t.cta_budget / jobs)), tiles = (n_mtiles + m_ctas - 1) / m_ctas;
     const double filled = static_cast<double>(jobs) * m_ctas / t.cta_budget;
-    const double cost = std::max(1.0, filled) * widest * (f / 256.0) * (tiles * (pair ? 0.4 : 0.7) + 1.4) +
+    const double cost = std::max(1.0, filled) * widest * (f / 256.0) * (tiles * 0.7 + 1.4) +
                         planes * 128.0 * n_mtiles * d.hidden * 8.0 / 5.0e6 + std::min(1.0, filled);
     if (best_cost < 0.0 || cost < best_cost) { best = g; best_cost = cost; }
   }
@@ -417,19 +443,64 @@ const GemmTable& f2_table(const sti_plan* p, const Layer& L, int tokens) {
   return L.f2.back();
 }
 
+// Calls of many tokens: decode the layer into the working buffer, then GEMMs over it.
+bool use_wide(const sti_plan* p, long long tokens) {
+  return p->tune.wide_min_tokens > 0 && tokens >= p->tune.wide_min_tokens && !p->ctx->simt_debug;
+}
+
+// Tiles of a GEMM over the working buffer.
+struct WideChoice { uint32_t nt, splits, clusters; };
+WideChoice pick_wide(const sti_plan* p, long long tokens, const WideMatrix& m, bool may_split) {
+  const Tuning& t = p->tune;
+  const uint32_t pairs = static_cast<uint32_t>((tokens + 255) / 256), held = std::max(1, t.cta_budget / 2);
+  WideChoice best{256, 1, 1};
+  double best_cost = -1.0;
+  for (uint32_t nt = 256; nt >= 128; nt /= 2) {
+    if (t.wide_nt > 0 && nt != static_cast<uint32_t>(t.wide_nt)) continue;
+    for (uint32_t splits = 1; splits <= (may_split ? 4u : 1u) && splits <= m.k_chunks; ++splits) {
+      if (may_split && t.wide_splits > 0 && splits != std::min(static_cast<uint32_t>(t.wide_splits), m.k_chunks)) continue;
+      const uint32_t tiles = pairs * ((m.n + nt - 1) / nt) * splits, waves = (tiles + held - 1) / held;
+      const double cost = waves * ((m.k_chunks + splits - 1) / splits * (nt == 256 ? 540.0 : 400.0) + 500.0) + (nt == 256 ? 1500.0 : 1000.0) +
+                          (splits - 1) * 8.0 * tokens * m.n / 2500.0;
+      if (best_cost < 0.0 || cost < best_cost) { best = {nt, splits, std::min(tiles, held)}; best_cost = cost; }
+    }
+  }
+  return best;
+}
+// FFN2 and the O projection write fp32 planes, one per K split.
+WideChoice pick_wide_f2(const sti_plan* p, const Layer& L, long long tokens) {
+  return pick_wide(p, tokens, L.wide[3], !(p->tune.f2_kacc_min_tokens > 0 && tokens >= p->tune.f2_kacc_min_tokens));
+}
+
+// Sizes and places of a layer's matrices in its working buffer; its bytes.
+size_t place_wide(const sti_ctx* c, Layer& L) {
+  const uint32_t d = c->desc.hidden, f = c->desc.ffn / c->desc.n_ffn_slices;
+  const uint32_t nh = static_cast<uint32_t>(L.kept_heads.size()), ns = static_cast<uint32_t>(L.kept_slices.size());
+  const uint32_t n[4] = {192 * nh, d, f * ns, d}, k[4] = {d, 64 * nh, d, f * ns};
+  uint32_t row = 0;
+  for (int m = 0; m < 4; ++m) {
+    L.wide[m] = {row, n[m], k[m] / 64};
+    row += (n[m] + 255) / 256 * 256 * (k[m] / 64);       // whole tiles of 256 features
+  }
+  return static_cast<size_t>(row) * 128;
+}
+
 // How many fp32 [tokens][hidden] planes' worth of partial sums a forward of this layer needs at most, in rows.
 size_t partial_rows(const sti_plan* p, const Layer& L) {
   const sti_model_desc& d = p->ctx->desc;
   const size_t most = static_cast<size_t>(d.max_batch) * d.max_seq;
-  size_t rows = most * std::max(1, L.o.n_split);
+  size_t rows = 1;
   for (size_t tokens = std::min<size_t>(128, most);; tokens = std::min(tokens + 128, most)) {
-    rows = std::max(rows, tokens * std::max(1, f2_table(p, L, static_cast<int>(tokens)).n_split));
+    size_t planes = std::max(L.o.n_split, f2_table(p, L, static_cast<int>(tokens)).n_split);
+    if (use_wide(p, static_cast<long long>(tokens)))
+      planes = std::max(pick_wide(p, tokens, L.wide[1], true).splits, pick_wide_f2(p, L, tokens).splits);
+    rows = std::max(rows, tokens * std::max<size_t>(1, planes));
     if (tokens == most) return rows;
   }
 }
 
 struct LayerTables {
-  TableBuilder qkv, o, f1, f2k;
+  TableBuilder qkv, o, f1;
   std::vector<TableBuilder> f2;
 };
 void build_layer_tables(sti_plan* p, Layer& L, LayerTables& tb) {
@@ -498,23 +569,85 @@ void build_layer_tables(sti_plan* p, Layer& L, LayerTables& tb) {
       }
     }
   }
-  // FFN2 for the K-accumulating kernel: 64-row tiles, K groups of at most 512 columns, group-major order
-  const int kacc_group = static_cast<int>(t.f2_kacc_k / f);      // whole slices per K group (0: a slice does not fit)
-  L.f2k.n_split = 0;
-  if (kacc_group > 0 && ns > 0 && d.hidden % 128 == 0 && t.f2_kacc_min_tokens > 0 &&
-      static_cast<long long>(d.max_batch) * d.max_seq >= t.f2_kacc_min_tokens) {
-    L.f2k.n_split = (ns + kacc_group - 1) / kacc_group;
-    for (int sp = 0; sp < L.f2k.n_split; ++sp) {
-      const int first = sp * kacc_group, cnt = std::min(kacc_group, ns - first);
-      for (uint32_t n0 = 0; n0 < static_cast<uint32_t>(d.hidden); n0 += 64) {
-        Job j{};
-        j.n_rows = 64; j.k_total = cnt * f; j.x_koff = first * f;
-        j.out_mat = 0; j.out_col = n0; j.bias_off = -1;
-        tb.f2k.add(j);
-        for (int i = 0; i < cnt; ++i) tb.f2k.add_rows(c, L.ffn[L.kept_slices[first + i]], STI_FFN, 1, n0, 64, i * f);
-      }
-    }
+}
+
+// What fills the working buffer: the tasks of every kept unit, layer by layer, with their places, and the bias offsets of the
+// GEMMs over it.  Made when a plan for many tokens is finalized, or by the first probe that asks for it.
+sti_status ensure_wide(sti_plan* p) {
+  if (p->wide_buf) return STI_OK;
+  sti_ctx* c = p->ctx;
+  const uint32_t f = c->desc.ffn / c->desc.n_ffn_slices;
+  std::vector<uint8_t> host;
+  struct At { size_t tasks, bias[2]; };
+  std::vector<At> at(p->layers.size());
+  size_t most = 1024, n_tasks = 0;
+  for (Layer& L : p->layers) {
+    const uint32_t per[4] = {3 * 64u * c->attn_m[0].kc / 4096, c->attn_m[3].rows * 64 / 4096, c->ffn_m[0].rows * c->ffn_m[0].kc / 4096,
+                             c->ffn_m[1].rows * c->ffn_m[1].kc / 4096};
+    for (int m = 0; m < 4; ++m)
+      L.wide_first[m + 1] = L.wide_first[m] + per[m] * static_cast<uint32_t>(m < 2 ? L.kept_heads.size() : L.kept_slices.size());
+    n_tasks += L.wide_first[4];
   }
+  host.reserve(n_tasks * sizeof(DecodeTask) + p->layers.size() * (c->desc.n_heads * 12 + c->desc.ffn / 16 + 64));
+  std::vector<DecodeTask> tasks;
+  bool in_bounds = true;
+  for (size_t li = 0; li < p->layers.size(); ++li) {
+    Layer& L = p->layers[li];
+    const size_t bytes = place_wide(c, L);
+    most = std::max(most, bytes);
+    tasks.resize(L.wide_first[4]);
+    uint32_t filled[4] = {L.wide_first[0], L.wide_first[1], L.wide_first[2], L.wide_first[3]};
+    // rows [first, first + rows) of the unit's matrix `um` are features n0 .. of layer matrix `m`, from column chunk kc0 on
+    auto add = [&](const Unit& u, sti_kind kind, int um, int m, uint32_t n0, uint32_t kc0) {
+      const MatrixTasks of(c, u, kind, um);
+      const TaskGrid& g = of.g;
+      for (uint32_t r = 0; r < of.mi.rows; r += g.rows)
+        for (uint32_t j = 0; j < g.per_row; ++j) {
+          DecodeTask t = of.at(r, j);
+          const uint32_t n = n0 + r, kc = kc0 + j * (g.cols / 64);
+          in_bounds = in_bounds && n + g.rows <= L.wide[m].n && kc + g.cols / 64 <= L.wide[m].k_chunks &&
+                      task_in_bounds(t, 64, 128, u.dev + u.off_codes, u.bytes);
+          const uint32_t piece = (L.wide[m].row0 + (n / 128 * L.wide[m].k_chunks + kc) * 128 + n % 128) / 32;
+          t.row0 = static_cast<uint16_t>(piece);
+          t.kcore0 = static_cast<uint16_t>(piece >> 16);
+          tasks[filled[m]++] = t;
+        }
+    };
+    std::vector<int32_t> bias[2];
+    for (size_t i = 0; i < L.kept_heads.size(); ++i) {
+      const int h = L.kept_heads[i];
+      for (int which = 0; which < 3; ++which) {
+        add(L.attn[h], STI_ATTN, which, 0, static_cast<uint32_t>(192 * i + 64 * which), 0);
+        bias[0].push_back(which * c->desc.n_heads * 64 + h * 64);
+      }
+      add(L.attn[h], STI_ATTN, 3, 1, 0, static_cast<uint32_t>(i));
+    }
+    for (size_t i = 0; i < L.kept_slices.size(); ++i) {
+      const int sl = L.kept_slices[i];
+      add(L.ffn[sl], STI_FFN, 0, 2, static_cast<uint32_t>(f * i), 0);
+      for (uint32_t r = 0; r < f; r += 64) bias[1].push_back(static_cast<int32_t>(f * sl + r));
+      add(L.ffn[sl], STI_FFN, 1, 3, 0, static_cast<uint32_t>(f / 64 * i));
+    }
+    auto put = [&](const void* from, size_t n) {
+      const size_t off = align16(host.size());
+      host.resize(off + n);
+      if (n) memcpy(host.data() + off, from, n);
+      return off;
+    };
+    at[li].tasks = put(tasks.data(), tasks.size() * sizeof(DecodeTask));
+    for (int b = 0; b < 2; ++b) at[li].bias[b] = put(bias[b].data(), bias[b].size() * 4);
+  }
+  if (!in_bounds) return STI_ERR_STATE;                  // not for any plan the calls before let through
+  p->wide_bytes = (most + 16383) / 16384 * 16384;
+  if (!p->wide_tables) CUDA_TRY(cudaMalloc(&p->wide_tables, std::max<size_t>(host.size(), 16)));
+  if (!host.empty()) CUDA_TRY(cudaMemcpy(p->wide_tables, host.data(), host.size(), cudaMemcpyHostToDevice));
+  for (size_t li = 0; li < p->layers.size(); ++li) {
+    Layer& L = p->layers[li];
+    L.wide_tasks = reinterpret_cast<const DecodeTask*>(p->wide_tables + at[li].tasks);
+    for (int b = 0; b < 2; ++b) L.wide_bias[b] = reinterpret_cast<const int32_t*>(p->wide_tables + at[li].bias[b]);
+  }
+  CUDA_TRY(cudaMalloc(&p->wide_buf, 2 * p->wide_bytes));
+  return STI_OK;
 }
 
 sti_status check_async(sti_ctx* c) {
@@ -546,9 +679,9 @@ EncodeTiledFn encode_tiled_fn() {
   return fn;
 }
 
-// TMA view of a bf16 activation matrix [rows, ld]: boxes of `box_rows` rows x 64 columns, 128-byte swizzle,
-// rows past `rows` read as zeros.
-bool make_xmap(CUtensorMap* map, const void* base, int ld, int rows, int box_rows = 128) {
+// TMA view of a bf16 matrix [rows, ld]: boxes of `box_rows` rows x 64 columns, 128-byte swizzle (the working buffer's rows
+// are swizzled as they stand), rows past `rows` read as zeros.
+bool make_xmap(CUtensorMap* map, const void* base, int ld, int rows, int box_rows = 128, bool swizzle = true) {
   EncodeTiledFn fn = encode_tiled_fn();
   if (!fn || (reinterpret_cast<uintptr_t>(base) & 15) || (ld % 8) != 0) return false;
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(ld), static_cast<cuuint64_t>(rows)};
@@ -556,7 +689,20 @@ bool make_xmap(CUtensorMap* map, const void* base, int ld, int rows, int box_row
   const cuuint32_t box[2] = {64, static_cast<cuuint32_t>(box_rows)};
   const cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// TMA view of a GEMM's output [planes][rows][cols], fp32 or bf16: boxes of 32 rows x 128 bytes of one plane, 128-byte swizzle.
+bool make_omap(CUtensorMap* map, void* base, bool f32, int cols, int rows, uint32_t planes) {
+  EncodeTiledFn fn = encode_tiled_fn();
+  const cuuint64_t size = f32 ? 4 : 2;
+  if (!fn || (reinterpret_cast<uintptr_t>(base) & 15) || cols * size % 16 != 0) return false;
+  const cuuint64_t dims[3] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows), planes};
+  const cuuint64_t strides[2] = {cols * size, cols * size * rows};
+  const cuuint32_t box[3] = {static_cast<cuuint32_t>(128 / size), 32, 1}, estr[3] = {1, 1, 1};
+  return fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -594,25 +740,12 @@ void layer_ranges(const sti_plan* p, int li, const uint8_t* ptr[4], uint32_t byt
   bytes[3] = static_cast<uint32_t>(p->ctx->dense_stride * sizeof(float));
 }
 
-// `force_pair`: -1 = the two-CTA kernel from pair_min_tiles token tiles on, 0 = never, 1 = always (the table must allow it).
 sti_status run_gemm(sti_plan* p, GemmKind kind, const GemmTable& tab, const void* x, int ldx, int T, void* out,
-                    int ldo, const float* bias, int prefetch_layer = -1, int force_pair = -1,
-                    unsigned long long* stamps = nullptr) {
+                    int ldo, const float* bias, int prefetch_layer = -1, unsigned long long* stamps = nullptr) {
   if (tab.n_jobs == 0) return STI_OK;
   GemmLaunch g{};
   g.stamps = stamps;
   g.jobs = tab.jobs; g.tasks = tab.tasks; g.n_jobs = tab.n_jobs; g.m_ctas = m_ctas_for(tab.n_jobs, T, p->tune.cta_budget);
-  const int n_mtiles = (T + 127) / 128;
-  g.pair = tab.pair_ok && p->tune.pair_min_tiles > 0 && n_mtiles >= p->tune.pair_min_tiles;
-  if (force_pair == 0) g.pair = false;
-  if (force_pair == 1) {
-    if (!tab.pair_ok) return STI_ERR_STATE;
-    g.pair = true;
-  }
-  if (g.pair) {      // a pair of CTAs takes two token tiles at a time
-    const int n_mpairs = (n_mtiles + 1) / 2;
-    g.m_ctas = std::max(1, std::min(n_mpairs, p->tune.cta_budget / tab.n_jobs));
-  }
   if (!make_xmap(&g.xmap, x, ldx, T)) return STI_ERR_CUDA;
   layer_ranges(p, prefetch_layer, g.pf_ptr, g.pf_bytes);
   g.x = x; g.ldx = ldx; g.T = T; g.out = out; g.ldo = ldo; g.bias = bias; g.err = p->ctx->err_dev;
@@ -622,31 +755,60 @@ sti_status run_gemm(sti_plan* p, GemmKind kind, const GemmTable& tab, const void
   return STI_OK;
 }
 
-// FFN2 through the K-accumulating kernel: one complete fp32 plane [T][ldo] instead of one plane per K group.
-sti_status run_gemm_kacc(sti_plan* p, const GemmTable& tab, const void* x, int ldx, int T, float* out, int ldo,
-                         unsigned long long* stamps) {
-  if (tab.n_jobs == 0 || tab.n_split == 0) return STI_ERR_STATE;
-  KaccLaunch g{};
-  g.jobs = tab.jobs; g.tasks = tab.tasks; g.n_groups = tab.n_split; g.n_cols64 = tab.n_jobs / tab.n_split;
-  const int n_mpairs = ((T + 127) / 128 + 1) / 2;
-  g.m_ctas = std::max(1, std::min(n_mpairs, p->tune.cta_budget / g.n_cols64));
-  if (!make_xmap(&g.xmap, x, ldx, T)) return STI_ERR_CUDA;
-  // an operand that does not fit L2 (126 MB, shared with everything else in flight) is prefetched by idle warps;
-  // measured: 32 x 512 tokens (134 MB) 159 -> 149 us per launch, 8,192 tokens (67 MB) 79 -> 81
-  g.x = static_cast<size_t>(T) * ldx * 2 > (100u << 20) ? x : nullptr; g.ldx = ldx;
-  g.T = T; g.out = out; g.ldo = ldo; g.err = p->ctx->err_dev;
-  g.n_stages = tab.n_stages; g.bps = tab.bps; g.hdr_bytes = tab.hdr_bytes; g.task_stride = tab.task_stride; g.k_group = tab.k_max;
-  g.pdl = p->ctx->pdl; g.stamps = stamps;
-  CUDA_TRY(launch_gemm_kacc(g, p->ctx->compute));
+uint8_t* wide_buffer(const sti_plan* p, int li) { return p->wide_buf + (li & 1) * p->wide_bytes; }
+
+// What decodes the matrices [first, end) of layer `li` into its working buffer.
+ExpandLaunch expand_job(const sti_plan* p, int li, int first, int end) {
+  const Layer& L = p->layers[li];
+  ExpandLaunch e{};
+  e.tasks = L.wide_tasks + L.wide_first[first]; e.n_tasks = L.wide_first[end] - L.wide_first[first]; e.dst = wide_buffer(p, li);
+  e.pdl = p->ctx->pdl;
+  return e;
+}
+sti_status run_expand(sti_plan* p, int li) {
+  const ExpandLaunch e = expand_job(p, li, 0, 4);
+  if (e.n_tasks == 0) return STI_OK;
+  CUDA_TRY(launch_expand(e, p->ctx->compute));
   p->ctx->launches++;
   return STI_OK;
 }
 
-// The seven kernels of one layer on the compute stream.
+// GEMM `which` (0 .. 3: QKV, O, FFN1, FFN2) of layer `li` over its working buffer; beside it the same matrix of layer `beside`
+// (-1: none) is decoded into the other one.  `weights_ready`: between the launch that decoded this matrix and this one stands
+// another GEMM over the working buffer, which lets its successors start only after its own wait.
+sti_status run_wide(sti_plan* p, GemmKind kind, int li, int which, const WideChoice& choice, const void* x, int ldx, int T, void* out,
+                    int ldo, const float* bias, bool weights_ready, int beside, unsigned long long* stamps) {
+  const Layer& L = p->layers[li];
+  const WideMatrix& m = L.wide[which];
+  WideLaunch g{};
+  g.shape.T = T; g.shape.n = m.n;
+  g.shape.n_tiles = (m.n + choice.nt - 1) / choice.nt; g.shape.m_pairs = (T + 255) / 256; g.shape.splits = choice.splits;
+  g.shape.k_chunks = m.k_chunks;
+  g.shape.w_row0 = static_cast<uint32_t>((li & 1) * (p->wide_bytes / 128)) + m.row0;
+  g.shape.plane64 = which == 0 ? 1 : 0;
+  g.nt = choice.nt; g.clusters = choice.clusters; g.weights_ready = weights_ready;
+  if (beside >= 0) {
+    g.beside = expand_job(p, beside, which, which + 1);
+    if (g.beside.n_tasks > 0) g.clusters = std::max(1, p->tune.cta_budget / 2);      // also where no tile is left to multiply
+  }
+  if (!make_xmap(&g.xmap, x, ldx, T) ||
+      !make_xmap(&g.wmap, p->wide_buf, 64, static_cast<int>(2 * p->wide_bytes / 128), choice.nt / 2, false) ||
+      !make_omap(&g.omap, out, kind == GEMM_BF16_TO_F32, ldo, T, which == 0 ? m.n / 64 : choice.splits))
+    return STI_ERR_CUDA;
+  g.bias = bias; g.bias_off = which == 0 ? L.wide_bias[0] : L.wide_bias[1];
+  g.err = p->ctx->err_dev; g.pdl = p->ctx->pdl; g.stamps = stamps;
+  CUDA_TRY(launch_gemm_wide(kind, g, p->ctx->compute));
+  p->ctx->launches++;
+  return STI_OK;
+}
+
+// The seven kernels of one layer on the compute stream, and from wide_min_tokens tokens on those that decode weights into the
+// working buffer.
+// `expanded`: this layer's weights are there already; `beside`: the layer that is decoded beside this one's GEMMs (-1: none).
 // `x_ready_bf16`: the bf16 copy of x already sits in p->x_bf16 (written by the previous layer's LayerNorm);
 // `want_next_bf16`: this layer's last kernel also writes y as bf16 into p->x_bf16 for the next layer.
 sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch, int seq, const int32_t* lens,
-                         bool x_ready_bf16, bool want_next_bf16, int next_layer = -1) {
+                         bool x_ready_bf16, bool want_next_bf16, int next_layer = -1, bool expanded = false, int beside = -1) {
   sti_ctx* c = p->ctx;
   const sti_model_desc& d = c->desc;
   Layer& L = p->layers[li];
@@ -662,7 +824,10 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   auto stamp = [&](int kernel) -> unsigned long long* {
     return p->stamping ? p->stamps + (static_cast<size_t>(li) * kStampKernels + kernel) * kStampRecord : nullptr;
   };
+  const bool wide = use_wide(p, T);
+  const WideChoice o_choice = pick_wide(p, T, L.wide[1], true), f2_choice = pick_wide_f2(p, L, T);
   CUDA_TRY(mark(0));
+  if (wide && !expanded && (st = run_expand(p, li)) != STI_OK) return st;
   if (nh > 0) {
     const void* xq = x;
     if (!bf16_act) {
@@ -674,7 +839,11 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
       }
       xq = p->x_bf16;
     }
-    st = run_gemm(p, GEMM_BF16_TO_BF16, L.qkv, xq, d.hidden, T, p->qkv, 64, dense + c->off_bq, next_layer, -1, stamp(1));
+    if (wide)
+      st = run_wide(p, GEMM_BF16_TO_BF16, li, 0, pick_wide(p, T, L.wide[0], false), xq, d.hidden, T, p->qkv, 64, dense + c->off_bq,
+                    expanded, beside, stamp(1));
+    else
+      st = run_gemm(p, GEMM_BF16_TO_BF16, L.qkv, xq, d.hidden, T, p->qkv, 64, dense + c->off_bq, next_layer, stamp(1));
     if (st != STI_OK) return st;
     CUDA_TRY(mark(1));
     if (tc_attention(p, nh, batch, seq)) {
@@ -683,11 +852,15 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
       CUDA_TRY(launch_attention_tc(qmap, omap, p->attn_out, nh, batch, seq, lens, c->err_dev, c->compute, c->pdl, stamp(2)));
     } else {
       CUDA_TRY(launch_attention(p->qkv, p->attn_out, nh, batch, seq, lens, c->sm_count,
-                                L.o.n_jobs * m_ctas_for(L.o.n_jobs, T, p->tune.cta_budget), c->compute, c->pdl, stamp(2)));
+                                wide ? static_cast<int>(2 * o_choice.clusters) : L.o.n_jobs * m_ctas_for(L.o.n_jobs, T, p->tune.cta_budget),
+                                c->compute, c->pdl, stamp(2)));
     }
     c->launches++;
     CUDA_TRY(mark(2));
-    st = run_gemm(p, GEMM_BF16_TO_F32, L.o, p->attn_out, nh * 64, T, p->partial, d.hidden, nullptr, -1, -1, stamp(3));
+    if (wide)
+      st = run_wide(p, GEMM_BF16_TO_F32, li, 1, o_choice, p->attn_out, nh * 64, T, p->partial, d.hidden, nullptr, true, beside, stamp(3));
+    else
+      st = run_gemm(p, GEMM_BF16_TO_F32, L.o, p->attn_out, nh * 64, T, p->partial, d.hidden, nullptr, -1, stamp(3));
     if (st != STI_OK) return st;
     L.k_ran[0] = L.k_ran[1] = L.k_ran[2] = true;
   } else {
@@ -700,7 +873,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   const int drop_planes = static_cast<size_t>(T) * d.hidden * 4 >= (32u << 20);
   {
     LnLaunch ln{};
-    ln.partial = p->partial; ln.n_partial = nh > 0 ? L.o.n_split : 0;
+    ln.partial = p->partial; ln.n_partial = nh > 0 ? (wide ? static_cast<int>(o_choice.splits) : L.o.n_split) : 0;
     ln.bias = dense + c->off_bo; ln.resid = x; ln.resid_bf16 = bf16_act ? 1 : 0;
     ln.gamma = dense + c->off_ln1g; ln.beta = dense + c->off_ln1b; ln.eps = d.ln_eps; ln.T = T; ln.d = d.hidden;
     // With bf16 activations every activation that crosses a kernel boundary is bf16 (the layer's input and output are):
@@ -712,17 +885,19 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     L.k_ran[3] = true;
   }
   CUDA_TRY(mark(4));
-  bool f2_kacc = false;
   const GemmTable& f2 = f2_table(p, L, T);
   if (ns > 0) {
-    st = run_gemm(p, GEMM_BF16_TO_BF16_GELU, L.f1, p->h1_bf16, d.hidden, T, p->u, ns * f, dense + c->off_b1, -1, -1, stamp(5));
+    if (wide)
+      st = run_wide(p, GEMM_BF16_TO_BF16_GELU, li, 2, pick_wide(p, T, L.wide[2], false), p->h1_bf16, d.hidden, T, p->u, ns * f,
+                    dense + c->off_b1, expanded || nh > 0, beside, stamp(5));
+    else
+      st = run_gemm(p, GEMM_BF16_TO_BF16_GELU, L.f1, p->h1_bf16, d.hidden, T, p->u, ns * f, dense + c->off_b1, -1, stamp(5));
     if (st != STI_OK) return st;
     CUDA_TRY(mark(5));
-    f2_kacc = L.f2k.n_jobs > 0 && T >= p->tune.f2_kacc_min_tokens && !c->simt_debug;
-    if (f2_kacc)
-      st = run_gemm_kacc(p, L.f2k, p->u, ns * f, T, p->partial, d.hidden, stamp(6));
+    if (wide)
+      st = run_wide(p, GEMM_BF16_TO_F32, li, 3, f2_choice, p->u, ns * f, T, p->partial, d.hidden, nullptr, true, beside, stamp(6));
     else
-      st = run_gemm(p, GEMM_BF16_TO_F32, f2, p->u, ns * f, T, p->partial, d.hidden, nullptr, -1, -1, stamp(6));
+      st = run_gemm(p, GEMM_BF16_TO_F32, f2, p->u, ns * f, T, p->partial, d.hidden, nullptr, -1, stamp(6));
     if (st != STI_OK) return st;
     L.k_ran[4] = L.k_ran[5] = true;
   } else {
@@ -730,7 +905,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   }
   CUDA_TRY(mark(6));
   LnLaunch l2{};
-  l2.partial = p->partial; l2.n_partial = ns > 0 ? (f2_kacc ? 1 : f2.n_split) : 0;
+  l2.partial = p->partial; l2.n_partial = ns > 0 ? (wide ? static_cast<int>(f2_choice.splits) : f2.n_split) : 0;
   l2.bias = dense + c->off_b2;
   l2.resid = bf16_act ? static_cast<const void*>(p->h1_bf16) : static_cast<const void*>(p->h1_f32);
   l2.resid_bf16 = bf16_act ? 1 : 0;
@@ -799,6 +974,7 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
     CUDA_TRY(cudaStreamWaitEvent(c->compute, last, 0));
   }
   const void* cur = x;
+  bool expanded = false;
   for (int li = 0; li < n; ++li) {
     Layer& L = p->layers[li];
     if (L.str_bytes > 0 && p->overlap) {
@@ -816,8 +992,14 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
     if (prof) CUDA_TRY(cudaEventRecord(L.ev_comp_start, c->compute));
     void* nxt = (li == n - 1) ? y : p->buf[li & 1];
     // the layer's first GEMM also pulls the next layer's packed shards into L2 (if they are on the device yet)
-    sti_status st = enqueue_layer(p, li, cur, nxt, batch, seq, lens, li > 0, li + 1 < n, li + 1 < n ? li + 1 : -1);
+    // every matrix of the next layer is decoded beside the same one of this layer - unless that is not multiplied with here, or
+    // the next layer is streamed and may not be on the device yet
+    const bool ahead = use_wide(p, static_cast<long long>(batch) * seq) && li + 1 < n && p->layers[li + 1].str_bytes == 0 &&
+                       !L.kept_heads.empty() && !L.kept_slices.empty();
+    sti_status st = enqueue_layer(p, li, cur, nxt, batch, seq, lens, li > 0, li + 1 < n, li + 1 < n ? li + 1 : -1, expanded,
+                                  ahead ? li + 1 : -1);
     if (st != STI_OK) return st;
+    expanded = ahead;
     if (p->retain_pending && !capturing && L.str_bytes > 0) {
       // keep what this run loaded (Section 3.2): the marked units leave their ring slot for the retained arena
       // before the slot is handed back to the copy stream
@@ -978,6 +1160,7 @@ void free_plan_device(sti_plan* p) {
   cudaFree(p->lens_dev);
   cudaFree(p->stamps);
   cudaFree(p->zero_bias);
+  cudaFree(p->wide_buf); cudaFree(p->wide_tables);
   cudaFree(p->rate_tables);
   for (auto& L : p->layers) {
     if (L.ev_loaded) cudaEventDestroy(L.ev_loaded);
@@ -1071,7 +1254,7 @@ sti_status sti_ctx_create(const sti_model_desc* desc, int device, void* compute_
   if (cudaMemset(c->dense, 0, c->dense_stride * d.n_layers * sizeof(float)) != cudaSuccess) return fail(STI_ERR_CUDA);
   if (cudaMalloc(&c->err_dev, sizeof(int)) != cudaSuccess) return fail(STI_ERR_OOM);
   if (cudaMemset(c->err_dev, 0, sizeof(int)) != cudaSuccess) return fail(STI_ERR_CUDA);
-  if (gemm_configure() != cudaSuccess || gemm_kacc_configure() != cudaSuccess || attention_configure() != cudaSuccess ||
+  if (gemm_configure() != cudaSuccess || gemm_wide_configure() != cudaSuccess || attention_configure() != cudaSuccess ||
       attention_tc_configure() != cudaSuccess)
     return fail(STI_ERR_CUDA);
   if (cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || c->sm_count < 1)
@@ -1143,7 +1326,7 @@ sti_status sti_plan_create(sti_ctx* c, const sti_shard_cfg* attn, const sti_shar
       if (L.ffn[s].cfg.keep) L.kept_slices.push_back(s);
     }
   }
-  parse_tuning(&p->tune, d.max_batch * d.max_seq, d, c->sm_count);
+  parse_tuning(&p->tune, d, c->sm_count);
   *out = p;
   return STI_OK;
 }
@@ -1296,9 +1479,10 @@ sti_status sti_plan_finalize(sti_plan* p) {
   size_t most_partial_rows = 1;
   for (auto& L : p->layers) {
     LayerTables tb;
+    (void)place_wide(c, L);
     L.tables_off = align16(host_tables.size());
     build_layer_tables(p, L, tb);
-    auto place = [&](GemmTable& gt, TableBuilder& b, bool kacc) -> sti_status {
+    auto place = [&](GemmTable& gt, TableBuilder& b) -> sti_status {
       if (!b.in_bounds) return STI_ERR_STATE;          // not for any plan the calls before let through
       b.finish();
       gt.task_stride = b.task_stride;
@@ -1306,23 +1490,8 @@ sti_status sti_plan_finalize(sti_plan* p) {
       gt.w_bytes = b.w_bytes;
       gt.n_stages = 2; gt.bps = 1;
       gt.hdr_bytes = gemm_header_bytes();
-      gt.pair_ok = !b.jobs.empty() && b.jobs.size() % 2 == 0;
-      for (size_t j = 0; gt.pair_ok && j < b.jobs.size(); j += 2) {
-        const Job &even = b.jobs[j], &odd = b.jobs[j + 1];
-        gt.pair_ok = even.n_rows == 64 && odd.n_rows == 64 && even.k_total == odd.k_total && even.x_koff == odd.x_koff;
-      }
-      if (kacc) {                   // two weight buffers, the rest of the shared memory is the ring of single boxes
-        gt.k_max = b.k_max;
-        gt.bps = p->tune.f2_kacc_bps;
-        for (const Job& j : b.jobs)
-          if (j.k_total % (128 * gt.bps / 2) != 0) gt.bps = 1;      // an odd number of boxes somewhere
-        gt.n_stages = gemm_kacc_stages(gt.hdr_bytes, b.k_max, gt.bps, kMaxSmem);
-        gt.smem = gemm_kacc_smem_bytes(gt.hdr_bytes, gt.n_stages, gt.bps, b.k_max);
-        if (!b.jobs.empty() && (gt.n_stages < 2 || gt.smem > kMaxSmem)) return STI_ERR_SHAPE;
-      } else {
-        if (!b.jobs.empty() && !gemm_pick_ring(b.w_bytes, b.k_max, gt.hdr_bytes, &gt.n_stages, &gt.bps)) return STI_ERR_SHAPE;
-        gt.smem = gemm_smem_bytes(b.w_bytes, gt.n_stages, gt.bps, gt.hdr_bytes);
-      }
+      if (!b.jobs.empty() && !gemm_pick_ring(b.w_bytes, b.k_max, gt.hdr_bytes, &gt.n_stages, &gt.bps)) return STI_ERR_SHAPE;
+      gt.smem = gemm_smem_bytes(b.w_bytes, gt.n_stages, gt.bps, gt.hdr_bytes);
       if (gt.smem > kMaxSmem && !b.jobs.empty()) return STI_ERR_SHAPE;
       Fix fx{&gt, 0, 0};
       fx.jobs_off = align16(host_tables.size());
@@ -1334,11 +1503,10 @@ sti_status sti_plan_finalize(sti_plan* p) {
       fixes.push_back(fx);
       return STI_OK;
     };
-    sti_status st = place(L.qkv, tb.qkv, false);
-    if (st == STI_OK) st = place(L.o, tb.o, false);
-    if (st == STI_OK) st = place(L.f1, tb.f1, false);
-    for (size_t i = 0; i < L.f2.size() && st == STI_OK; ++i) st = place(L.f2[i], tb.f2[i], false);
-    if (st == STI_OK) st = place(L.f2k, tb.f2k, true);
+    sti_status st = place(L.qkv, tb.qkv);
+    if (st == STI_OK) st = place(L.o, tb.o);
+    if (st == STI_OK) st = place(L.f1, tb.f1);
+    for (size_t i = 0; i < L.f2.size() && st == STI_OK; ++i) st = place(L.f2[i], tb.f2[i]);
     if (st != STI_OK) return st;
     L.tables_bytes = host_tables.size() - L.tables_off;
     most_partial_rows = std::max(most_partial_rows, partial_rows(p, L));
@@ -1351,8 +1519,12 @@ sti_status sti_plan_finalize(sti_plan* p) {
     fx.t->jobs = reinterpret_cast<Job*>(p->tables + fx.jobs_off);
     fx.t->tasks = reinterpret_cast<DecodeTask*>(p->tables + fx.tasks_off);
   }
-  // 4. activation scratch for max_batch * max_seq tokens
+  // 4. the working buffer of plans for many tokens, activation scratch for max_batch * max_seq tokens
   const size_t Tmax = static_cast<size_t>(d.max_batch) * d.max_seq;
+  if (use_wide(p, static_cast<long long>(Tmax))) {
+    const sti_status st = ensure_wide(p);
+    if (st != STI_OK) return st;
+  }
   const size_t f = d.ffn / d.n_ffn_slices;
   CUDA_TRY(cudaMalloc(&p->qkv, std::max<size_t>(1, 3 * max_heads) * Tmax * 64 * 2));
   CUDA_TRY(cudaMalloc(&p->attn_out, std::max<size_t>(1, max_heads) * Tmax * 64 * 2));
@@ -1491,7 +1663,7 @@ sti_status sti_shard_decode(sti_plan* p, int layer, sti_kind kind, int index, in
 sti_status sti_gemm_probe(sti_plan* p, int layer, int gemm, const void* x_bf16_dev, int tokens, void* out_dev,
                           size_t out_capacity_bytes, int variant, int32_t* n_partials) {
   if (!p || !x_bf16_dev || !out_dev || gemm < 0 || gemm > 3 || variant < 0 || variant > 3) return STI_ERR_ARG;
-  if (variant == 3 && gemm != 3) return STI_ERR_ARG;       // the K-accumulating kernel exists for FFN2 only
+  if (variant == 3 && gemm != 3) return STI_ERR_ARG;       // FFN2 only
   if (layer < 0 || layer >= static_cast<int>(p->layers.size())) return STI_ERR_ARG;
   if (tokens < 1 || tokens > 65536) return STI_ERR_SHAPE;
   if ((reinterpret_cast<uintptr_t>(x_bf16_dev) & 15) || (reinterpret_cast<uintptr_t>(out_dev) & 15)) return STI_ERR_ARG;
@@ -1506,14 +1678,21 @@ sti_status sti_gemm_probe(sti_plan* p, int layer, int gemm, const void* x_bf16_d
   const GemmTable* tabs[4] = {&L.qkv, &L.o, &L.f1, &f2_table(p, L, tokens)};
   const GemmTable& tab = *tabs[gemm];
   if (tab.n_jobs == 0) return STI_ERR_STATE;               // no kept unit feeds this GEMM
+  const bool wide = variant == 3 || (variant == 2 && !c->simt_debug) || (variant == 0 && use_wide(p, tokens));
+  const long long most = static_cast<long long>(d.max_batch) * d.max_seq;
+  if (variant == 3 && (p->tune.f2_kacc_min_tokens == 0 || most < p->tune.f2_kacc_min_tokens))
+    return STI_ERR_STATE;                                  // no call of this plan takes FFN2's K range in one piece
+  const bool sums = gemm == 1 || gemm == 3;
+  const WideChoice choice = variant == 3 ? pick_wide(p, tokens, L.wide[3], false)
+                                         : (gemm == 3 ? pick_wide_f2(p, L, tokens) : pick_wide(p, tokens, L.wide[gemm], sums));
   const int ldx[4] = {d.hidden, nh * 64, d.hidden, ns * f};
   const int ldo[4] = {64, d.hidden, ns * f, d.hidden};
-  const int parts[4] = {1, tabs[1]->n_split, 1, variant == 3 ? 1 : tabs[3]->n_split};
-  if (variant == 3 && L.f2k.n_jobs == 0) return STI_ERR_STATE;   // the plan was not made for many tokens
-  const size_t out_elems[4] = {static_cast<size_t>(3) * nh * tokens * 64, static_cast<size_t>(parts[1]) * tokens * d.hidden,
-                               static_cast<size_t>(tokens) * ns * f, static_cast<size_t>(parts[3]) * tokens * d.hidden};
-  const size_t need = out_elems[gemm] * ((gemm == 1 || gemm == 3) ? 4 : 2);
+  const int parts = !sums ? 1 : wide ? static_cast<int>(choice.splits) : tab.n_split;
+  const size_t out_elems[4] = {static_cast<size_t>(3) * nh * tokens * 64, static_cast<size_t>(parts) * tokens * d.hidden,
+                               static_cast<size_t>(tokens) * ns * f, static_cast<size_t>(parts) * tokens * d.hidden};
+  const size_t need = out_elems[gemm] * (sums ? 4 : 2);
   if (out_capacity_bytes < need) return STI_ERR_SIZE;
+  if (wide && (st = ensure_wide(p)) != STI_OK) return st;
   if (!p->zero_bias) {
     const size_t n = static_cast<size_t>(3) * d.n_heads * 64 + d.ffn;
     CUDA_TRY(cudaMalloc(&p->zero_bias, n * sizeof(float)));
@@ -1523,15 +1702,16 @@ sti_status sti_gemm_probe(sti_plan* p, int layer, int gemm, const void* x_bf16_d
     if (p->copy_tail_valid) CUDA_TRY(cudaStreamWaitEvent(c->compute, p->ev_copy_tail, 0));
     if ((st = enqueue_layer_copy(p, layer, c->compute)) != STI_OK) return st;
   }
-  const GemmKind kind = (gemm == 1 || gemm == 3) ? GEMM_BF16_TO_F32 : GEMM_BF16_TO_BF16;
-  if (variant == 3)
-    st = run_gemm_kacc(p, L.f2k, x_bf16_dev, ldx[3], tokens, static_cast<float*>(out_dev), ldo[3], nullptr);
-  else
-  st = run_gemm(p, kind, tab, x_bf16_dev, ldx[gemm], tokens, out_dev, ldo[gemm], p->zero_bias, -1,
-                variant == 0 ? -1 : variant - 1);
+  const GemmKind kind = sums ? GEMM_BF16_TO_F32 : GEMM_BF16_TO_BF16;
+  if (wide) {
+    st = run_expand(p, layer);
+    if (st == STI_OK) st = run_wide(p, kind, layer, gemm, choice, x_bf16_dev, ldx[gemm], tokens, out_dev, ldo[gemm], nullptr, false, -1, nullptr);
+  } else {
+    st = run_gemm(p, kind, tab, x_bf16_dev, ldx[gemm], tokens, out_dev, ldo[gemm], p->zero_bias);
+  }
   if (st != STI_OK) return st;
   if (L.str_bytes > 0) CUDA_TRY(cudaEventRecord(p->slot_free[L.slot], c->compute));
-  if (n_partials) *n_partials = parts[gemm];
+  if (n_partials) *n_partials = parts;
   return STI_OK;
 }
 
@@ -1593,11 +1773,10 @@ sti_status sti_decode_rate_probe(sti_plan* p, const void* x_bf16_dev, int tokens
   tab.tasks = reinterpret_cast<DecodeTask*>(p->rate_tables + align16(static_cast<size_t>(p->rate_jobs) * sizeof(Job)));
   tab.n_jobs = p->rate_jobs;
   tab.task_stride = p->rate_task_stride;
-  tab.pair_ok = false;
   for (auto& L : p->layers) {                                            // the widest tile decides the shared-memory shape
     if (L.f1.n_jobs && L.f1.smem > tab.smem) { tab.smem = L.f1.smem; tab.w_bytes = L.f1.w_bytes; tab.n_stages = L.f1.n_stages; tab.bps = L.f1.bps; }
   }
-  st = run_gemm(p, GEMM_BF16_TO_BF16, tab, x_bf16_dev, d.hidden, tokens, out_dev, ldo, nullptr, -1, 0);
+  st = run_gemm(p, GEMM_BF16_TO_BF16, tab, x_bf16_dev, d.hidden, tokens, out_dev, ldo, nullptr);
   if (st != STI_OK) return st;
   if (packed_bytes) *packed_bytes = p->rate_packed_bytes;
   if (n_tiles) *n_tiles = p->rate_jobs;

@@ -25,6 +25,9 @@ struct alignas(16) DecodeTask {
 };
 static_assert(sizeof(DecodeTask) == 32, "two 16-byte loads");
 
+// Tasks of a working buffer (expand.cu) name the first of their two 4 KB pieces in place of a row and a column group.
+STI_HOST_DEVICE uint32_t expanded_at(const DecodeTask& t) { return t.row0 | static_cast<uint32_t>(t.kcore0) << 16; }
+
 // Row and column inside the task of the outlier at `rc` (row << 16 | column of the matrix); false if it is not one of the
 // task's weights.  The lists come out of device memory that streamed layers overwrite in turn, so this is looked at where
 // they are applied: a wrong entry is left out rather than stored somewhere else in shared memory.

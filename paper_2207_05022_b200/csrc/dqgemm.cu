@@ -317,236 +317,9 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
   if (tid == 0) stamp_max(stamps, STAMP_LAST_END);
 }
 
-// ---------------------------------------------------------------------------------------
-// Two-CTA variant (cta_group::2) for many tokens.
-//
-// A cluster of two CTAs shares one MMA: M = 256 (each CTA contributes its own 128-token activation tile),
-// N = 128 (each CTA contributes the 64 decoded weight rows of its own job).  Per instruction the pair does
-// twice the work of the one-CTA kernel per SM for the same issue cost, and every activation byte brought in
-// from L2 is used against 128 instead of 64 output features - the one-CTA kernel is bound by exactly these
-// two things once there are thousands of tokens.  CTA 0 issues; tcgen05.commit multicasts completions to both
-// CTAs; both CTAs' TMA loads report to CTA 0's `full` barriers; each CTA drains its own accumulator rows
-// (its 128 tokens x all 128 features) and reports to CTA 0's `acc_empty`.
-// ---------------------------------------------------------------------------------------
-template <typename OutT, bool GELU>
-__global__ void __launch_bounds__(kThreads, 1)
-dqgemm_pair_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ jobs, const DecodeTask* __restrict__ tasks,
-                   int T, OutT* __restrict__ out, int ldo, const float* __restrict__ bias, int* __restrict__ err,
-                   uint32_t n_stages, uint32_t bps, uint32_t w_bytes, uint32_t hdr_bytes, uint32_t task_stride,
-                   unsigned long long* stamps) {
-  extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* smem = smem_raw;
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) { stamp_min(stamps, STAMP_FIRST_START); stamp_max(stamps, STAMP_LAST_START); }
-  const uint32_t rank = cluster_ctarank();                 // 0 issues the MMAs
-  const uint32_t pair_base = blockIdx.x & ~1u;
-  const DecodeTask* my_tasks = tasks + static_cast<size_t>(blockIdx.x) * task_stride;
-  TileDecode decode;                                       // the 64 weight rows this CTA decodes
-  decode.begin(my_tasks, task_stride, tid);                // does not wait for the job descriptors
-  const Job job = jobs[blockIdx.x];
-  const Job job0 = jobs[pair_base], job1 = jobs[pair_base + 1];   // columns 0-63 / 64-127 of the accumulator
-  const uint32_t k_total = job.k_total;
-
-  SmemHeader* hdr = reinterpret_cast<SmemHeader*>(smem);
-  float* bias_sm = reinterpret_cast<float*>(smem + 256);            // [128]
-  uint16_t* tables = reinterpret_cast<uint16_t*>(smem + 768);       // [warp][64]
-  uint8_t* xsm = smem + hdr_bytes;
-  const uint32_t stage_bytes = bps * kBoxBytes;
-  uint8_t* wsm = xsm + n_stages * stage_bytes;
-
-  // both CTAs evaluate the same conditions, so a refused pair leaves together
-  const bool bad = job0.n_rows != 64 || job1.n_rows != 64 || job0.k_total != job1.k_total || job0.x_koff != job1.x_koff ||
-                   job0.n_tasks == 0 || job0.n_tasks > task_stride || job1.n_tasks == 0 || job1.n_tasks > task_stride ||
-                   (k_total % kChunkK) != 0 || k_total == 0 || 64 * k_total * 2 > w_bytes || n_stages < 2 ||
-                   n_stages > kMaxStages || (bps != 1 && bps != 2 && bps != 4) ||
-                   768 + kWarps * kTableStride * 2 > hdr_bytes || (hdr_bytes & 1023) != 0 || (gridDim.x & 1) != 0 ||
-                   (smem_addr(smem_raw) & 1023u) != 0 || job0.task_begin != pair_base * task_stride ||
-                   job1.task_begin != (pair_base + 1) * task_stride;
-  if (bad) {
-    if (tid == 0) atomicCAS(err, ERR_NONE, ERR_BAD_JOB);
-    return;
-  }
-
-  const int n_mtiles = (T + kTileM - 1) / kTileM;
-  const uint32_t n_mpairs = (n_mtiles + 1) / 2;           // the pair takes token tiles 2p (CTA 0) and 2p + 1 (CTA 1)
-  const uint32_t n_boxes = k_total / kChunkK;
-  const uint32_t n_chunks = (n_boxes + bps - 1) / bps;
-  const uint32_t my_pairs = blockIdx.y < n_mpairs ? (n_mpairs - blockIdx.y + gridDim.y - 1) / gridDim.y : 0;
-  const uint32_t total = my_pairs * n_chunks;
-  const uint32_t xsm_addr = smem_addr(xsm);
-  const uint32_t rot = (blockIdx.x >> 1) % n_chunks;      // both CTAs of a pair walk K in the same order
-  auto tile_row0 = [&](uint32_t ti) { return static_cast<int>((2 * (blockIdx.y + ti * gridDim.y) + rank) * kTileM); };
-
-  constexpr uint32_t kAccCols = 128, kTmemCols = 256;      // two accumulators of 128 columns
-  if (tid == 0) {
-    for (uint32_t s = 0; s < n_stages; ++s) {
-      mbar_init(smem_addr(&hdr->full[s]), 1);              // used in CTA 0 only
-      mbar_init(smem_addr(&hdr->empty[s]), 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(smem_addr(&hdr->acc_full[b]), 1);
-      mbar_init(smem_addr(&hdr->acc_empty[b]), 2 * kPairEpilogueWarps);   // CTA 0 only: both CTAs' epilogue warps
-    }
-    mbar_init(smem_addr(&hdr->drain), 1);
-    hdr->abort = 0;
-    mbar_fence_init();
-    fence_proxy_async_smem();
-  }
-  if (warp == 1) {
-    tmem_alloc_pair(smem_addr(&hdr->tmem_base), kTmemCols);
-    tmem_relinquish_pair();
-  }
-  const int bias_off = tid < 64 ? job0.bias_off : job1.bias_off;
-  const float bias_value = tid < 128 && bias_off >= 0 ? __ldg(bias + bias_off + (tid & 63)) : 0.f;
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem_base = hdr->tmem_base;
-  pdl_launch_dependents();          // this CTA owns its tensor memory now (see the one-CTA kernel)
-
-  if (tid < 128) bias_sm[tid] = bias_value;
-  decode.finish(my_tasks, task_stride, tables, wsm, 64, tid);
-  if (tid == 0) stamp_max(stamps, STAMP_DECODED);
-  cluster_sync_all();               // both halves of the weight tile are in place, all barriers initialised
-  pdl_wait();                       // from here on: the previous kernel's output
-  if (tid == 0) stamp_min(stamps, STAMP_RELEASE);
-
-  bool failed = false;
-  if (warp == 0) {
-    // ---- producer (one in each CTA): own token tile into own ring, completion reported to CTA 0
-    if (lane == 0) {
-      uint32_t c = 0, stage = 0, phase = 0, kcr = rot, kc = 0, ti = 0;
-      for (; c < total; ++c) {
-        if (c >= n_stages) {
-          if (!mbar_wait_bounded_relaxed(smem_addr(&hdr->empty[stage]), phase)) { failed = true; break; }
-        }
-        const uint32_t box0 = kcr * bps;
-        const uint32_t nb = n_boxes - box0 < bps ? n_boxes - box0 : bps;
-        if (rank == 0) mbar_expect_tx(smem_addr(&hdr->full[stage]), 2 * nb * kBoxBytes);    // both CTAs' bytes
-        const uint32_t bar = map_to_cta(smem_addr(&hdr->full[stage]), 0);
-        for (uint32_t b = 0; b < nb; ++b)
-          tma_load_2d_pair(xsm_addr + stage * stage_bytes + b * kBoxBytes, &xmap,
-                           static_cast<int>(job.x_koff + (box0 + b) * kChunkK), tile_row0(ti), bar);
-        if (++stage == n_stages) { stage = 0; if (c >= n_stages) phase ^= 1; }
-        if (++kcr == n_chunks) kcr = 0;
-        if (++kc == n_chunks) { kc = 0; ++ti; }
-      }
-    }
-    __syncwarp();
-  } else if (warp == 1) {
-    if (rank == 0) {
-      // ---- MMA issuer of the pair
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((256u >> 4) << 24);
-      const uint32_t w_lbo = 64 * 16;
-      const uint64_t a_desc0 = umma_smem_desc_sw128(xsm_addr);
-      const uint64_t b_desc0 = umma_smem_desc(smem_addr(wsm), w_lbo, 128);
-      const uint32_t a_stage_step = stage_bytes >> 4, a_box_step = kBoxBytes >> 4;
-      const uint32_t b_ks_step = (2 * w_lbo) >> 4, b_chunk_step = 4 * b_ks_step;
-      uint32_t stage = 0, phase = 0, kc = 0, kcr = rot, ti = 0, issued = 0;
-      for (uint32_t c = 0; c < total; ++c) {
-        const uint32_t buf = ti & 1;
-        bool ok = true;
-        if (kc == 0 && ti >= 2)
-          ok = __all_sync(0xffffffffu, mbar_wait_bounded(smem_addr(&hdr->acc_empty[buf]), ((ti >> 1) - 1) & 1));
-        if (ok) ok = __all_sync(0xffffffffu, mbar_wait_bounded(smem_addr(&hdr->full[stage]), phase));
-        if (!ok) { failed = true; break; }
-        tc_fence_after_sync();
-        const uint32_t box0 = kcr * bps;
-        const uint32_t nb = n_boxes - box0 < bps ? n_boxes - box0 : bps;
-        const uint64_t da0 = a_desc0 + stage * a_stage_step;
-        const uint64_t db0 = b_desc0 + box0 * b_chunk_step;
-        const uint32_t d_addr = tmem_base + buf * kAccCols;
-        if (elect_one()) {
-          uint64_t da = da0, db = db0;
-          umma_bf16_ss_x4_pair(d_addr, da, db, 2, b_ks_step, idesc, kc != 0 ? 1u : 0u);
-          for (uint32_t b = 1; b < nb; ++b) {
-            da += a_box_step;
-            db += b_chunk_step;
-            umma_bf16_ss_x4_pair(d_addr, da, db, 2, b_ks_step, idesc, 1u);
-          }
-          if (c + n_stages < total) umma_commit_pair(smem_addr(&hdr->empty[stage]));
-          if (kc + 1 == n_chunks) umma_commit_pair(smem_addr(&hdr->acc_full[buf]));
-        }
-        __syncwarp();
-        issued = c + 1;
-        if (++stage == n_stages) { stage = 0; phase ^= 1; }
-        if (++kcr == n_chunks) kcr = 0;
-        if (++kc == n_chunks) { kc = 0; ++ti; }
-      }
-      if (failed && issued > 0) {
-        if (elect_one()) umma_commit_pair(smem_addr(&hdr->drain));
-        __syncwarp();
-        (void)mbar_wait_bounded(smem_addr(&hdr->drain), 0);
-      }
-    }
-  } else if (warp >= kEpilogueWarp0 && warp < kEpilogueWarp0 + kPairEpilogueWarps) {
-    // ---- epilogue: this CTA's 128 token rows x 128 features.  Twelve warps, three per tensor-memory lane quadrant
-    // (a warp reads only the 32 lanes of quadrant warp % 4); the three share the eight 16-column chunks 3 + 3 + 2.
-    const uint32_t q = warp & 3, part = (warp - kEpilogueWarp0) >> 2;
-    const uint32_t chunk0 = part * 3, chunk1 = part == 2 ? 8 : chunk0 + 3;
-    for (uint32_t ti = 0; ti < my_pairs; ++ti) {
-      const uint32_t buf = ti & 1;
-      uint32_t ok = 1;
-      if (lane == 0) ok = mbar_wait_bounded_relaxed(smem_addr(&hdr->acc_full[buf]), (ti >> 1) & 1) ? 1u : 0u;
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) { failed = true; break; }
-      tc_fence_after_sync();
-      const int t = tile_row0(ti) + static_cast<int>(q * 32 + lane);
-      const int row = group_row<OutT>(t, lane);
-      const size_t trow = static_cast<size_t>(row < T ? row : 0);
-      OutT* first0 = out + (static_cast<size_t>(job0.out_mat) * T + trow) * ldo + job0.out_col;
-      OutT* first1 = out + (static_cast<size_t>(job1.out_mat) * T + trow) * ldo + job1.out_col;
-      const uint32_t taddr = tmem_base + ((q * 32) << 16) + buf * kAccCols;
-      uint32_t r[3][16];
-#pragma unroll
-      for (uint32_t c = 0; c < 3; ++c)
-        if (chunk0 + c < chunk1) tmem_ld_32x32b_x16(taddr + (chunk0 + c) * 16, r[c]);
-      tc_wait_ld();
-#pragma unroll
-      for (uint32_t c = 0; c < 3; ++c) {
-        if (chunk0 + c < chunk1) {
-          const uint32_t col = (chunk0 + c) * 16;            // 0..127: the first 64 are job 0's features
-          float v[16];
-          bias_act16<GELU>(r[c], bias_sm + col, v);
-          store_block16<OutT>(v, (col < 64 ? first0 : first1) + (col & 63), ldo, T - row, lane);
-        }
-      }
-      tc_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_cluster_cta_scope(map_to_cta(smem_addr(&hdr->acc_empty[buf]), 0));
-    }
-  }
-  if (failed) {
-    hdr->abort = 1;
-    if (lane == 0) atomicCAS(err, ERR_NONE, ERR_WAIT_TIMEOUT);
-  }
-  tc_fence_before_sync();
-  __syncthreads();
-  cluster_sync_all();      // neither CTA frees tensor memory or exits while the pair's MMAs may still use it
-  if (warp == 1) tmem_dealloc_pair(tmem_base, kTmemCols);
-  if (tid == 0) stamp_max(stamps, STAMP_LAST_END);
-}
-
 template <typename OutT, bool GELU>
 cudaError_t launch_t(const GemmLaunch& p, cudaStream_t s) {
   const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(p.x);
-  if (p.pair && !p.simt_debug) {
-    // clusters of two CTAs along x (consecutive jobs = the two halves of a 128-feature tile)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(p.n_jobs, p.m_ctas);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = p.smem_bytes;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = p.pdl ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, dqgemm_pair_kernel<OutT, GELU>, p.xmap, p.jobs, p.tasks, p.T, static_cast<OutT*>(p.out),
-                              p.ldo, p.bias, p.err, p.n_stages, p.bps, p.w_bytes, p.hdr_bytes, p.task_stride, p.stamps);
-  }
   dim3 grid(p.n_jobs, p.m_ctas), block(kThreads);
   PrefetchRanges pf;
   for (int r = 0; r < 4; ++r) { pf.ptr[r] = p.pf_ptr[r]; pf.bytes[r] = p.pf_bytes[r]; }
@@ -600,8 +373,7 @@ bool gemm_pick_ring(uint32_t w_bytes, uint32_t k_total, uint32_t hdr_bytes, uint
 cudaError_t gemm_configure() {
   cudaError_t e;
 #define STI_SET(OutT, G)                                                  \
-  if ((e = set_smem(dqgemm_kernel<OutT, G, true, false>)) != cudaSuccess) return e;  \
-  if ((e = set_smem(dqgemm_pair_kernel<OutT, G>)) != cudaSuccess) return e;
+  if ((e = set_smem(dqgemm_kernel<OutT, G, true, false>)) != cudaSuccess) return e;
   if ((e = set_smem(dqgemm_kernel<void, false, false, true>)) != cudaSuccess) return e;
   if ((e = set_smem(dqgemm_kernel<void, false, false, false>)) != cudaSuccess) return e;
   STI_SET(__nv_bfloat16, false)

@@ -22,7 +22,6 @@ constexpr int kHeaderBytes = 3072;
 constexpr int kTableStride = 64;            // bf16 entries of a warp's centroid table
 constexpr int kEpilogueWarp0 = 4;             // epilogue warps 4..11: two per TMEM lane quadrant
 constexpr int kEpilogueWarps = 8;
-constexpr int kPairEpilogueWarps = 12;        // the two-CTA kernel drains with warps 4..15: three per lane quadrant
 
 struct SmemHeader {
   uint64_t full[kMaxStages];     // activation chunk landed (TMA transaction bytes)
@@ -143,14 +142,50 @@ struct ByteTable {
   }
 };
 
-// Index unpack -> table lookup -> 16-byte stores into the K-major core-matrix layout.  Each lane holds 128 consecutive
+// Where the decoded weights of a task go.  `piece(base, grp, ss)`: eight columns (ss of four) of index group grp (of four) of
+// the lane's row; `element(row, col)`: byte offset of a weight of the task, for outliers and uncompressed units.
+// The tile of a GEMM CTA: K-major core matrices, (row, k) at ((k / 8) * n_rows + row) * 16 + (k % 8) * 2.
+struct TilePlace {
+  uint8_t* wsm;
+  uint32_t n_rows, row0, kcore0, narrow;
+  __device__ __forceinline__ TilePlace(uint8_t* w, uint32_t rows, const DecodeTask& t)
+      : wsm(w), n_rows(rows), row0(t.row0), kcore0(t.kcore0), narrow(t.narrow) {}
+  __device__ __forceinline__ uint8_t* group(uint32_t grp, uint32_t lane) const {
+    uint8_t* dst0 = wsm + (static_cast<size_t>(kcore0) * n_rows + row0 + lane) * 16;
+    return dst0 + (narrow ? (grp & 1) * 4 * (n_rows * 16) + (grp >> 1) * 512 : grp * 4 * (n_rows * 16));
+  }
+  __device__ __forceinline__ uint8_t* piece(uint8_t* group_base, uint32_t, uint32_t ss, uint32_t) const {
+    return group_base + ss * (n_rows * 16);                       // from eight columns to the next eight
+  }
+  __device__ __forceinline__ uint8_t* element(uint32_t row, uint32_t col) const {
+    return wsm + (static_cast<size_t>(kcore0 + (col >> 3)) * n_rows + row0 + row) * 16 + (col & 7) * 2;
+  }
+};
+// A task by itself: two blocks of 32 rows x 64 columns in the 128-byte-swizzled K-major layout that TMA and the tensor core
+// know (a row is 128 bytes, its eight 16-byte pieces permuted by the row's number modulo 8).  Wide tasks: the block's
+// columns 0-63 and 64-127; narrow ones: rows 0-31 and 32-63.
+struct SwizzledPlace {
+  uint8_t* wsm;
+  uint32_t narrow;
+  __device__ __forceinline__ SwizzledPlace(uint8_t* w, const DecodeTask& t) : wsm(w), narrow(t.narrow) {}
+  __device__ __forceinline__ uint8_t* group(uint32_t grp, uint32_t lane) const { return wsm + (grp >> 1) * 4096 + lane * 128; }
+  __device__ __forceinline__ uint8_t* piece(uint8_t* group_base, uint32_t grp, uint32_t ss, uint32_t lane) const {
+    return group_base + ((((grp & 1) * 4 + ss) ^ (lane & 7)) << 4);
+  }
+  __device__ __forceinline__ uint8_t* element(uint32_t row, uint32_t col) const {
+    const uint32_t block = narrow ? row >> 5 : col >> 6, c = col & 63;
+    return wsm + block * 4096 + (row & 31) * 128 + (((c >> 3) ^ (row & 7)) << 4) + (c & 7) * 2;
+  }
+};
+
+// Index unpack -> table lookup -> 16-byte stores.  Each lane holds 128 consecutive
 // indexes of its own row (narrow tasks: of rows l and l + 32).  `half`: 0 = the whole quantum (four groups of 32 indexes),
 // 1 / 2 = its first / second two groups only (two warps share a task when a tile has few; both hold the task's planes).
 // 32 indexes are exactly BITS words: the loop is rolled over the four groups and always reads w[0 .. BITS), the words
 // moving down after each group - the decode runs once per CTA, so its code is fetched cold and its size is what it costs.
-template <int BITS>
-__device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const DecodeTask& t, const uint16_t* __restrict__ tab,
-                                            uint8_t* wsm, uint32_t n_rows, uint32_t lane, uint32_t half) {
+template <int BITS, typename Place>
+__device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const Place& place, const uint16_t* __restrict__ tab,
+                                            uint32_t lane, uint32_t half) {
   uint32_t w[4 * BITS];
 #pragma unroll
   for (int i = 0; i < 4 * BITS; ++i) w[i] = planes[i];
@@ -159,8 +194,6 @@ __device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const 
     for (int i = 0; i < 2 * BITS; ++i) w[i] = planes[i + 2 * BITS];
   }
   const uint32_t grp0 = half == 2 ? 2 : 0, grp1 = half == 1 ? 2 : 4;
-  const uint32_t piece = n_rows * 16;                    // from eight columns to the next eight
-  uint8_t* const dst0 = wsm + (static_cast<size_t>(t.kcore0) * n_rows + t.row0 + lane) * 16;
   ByteTable<BITS <= 4 ? BITS : 2> table;
   if constexpr (BITS <= 4) table.load(tab);
 #pragma unroll 1
@@ -168,7 +201,7 @@ __device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const 
     uint32_t lo[BITS];
 #pragma unroll
     for (int i = 0; i < BITS; ++i) lo[i] = w[i];
-    uint8_t* dst = dst0 + (t.narrow ? (grp & 1) * 4 * piece + (grp >> 1) * 512 : grp * 4 * piece);
+    uint8_t* dst = place.group(grp, lane);
     if constexpr (BITS <= 4) {
       uint32_t sel[4];
       spread_to_nibbles<BITS>(lo, sel);
@@ -179,7 +212,7 @@ __device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const 
         uint4 v;
         table.four(low, upper, v.x, v.y);
         table.four(low >> 16, upper >> 16, v.z, v.w);
-        *reinterpret_cast<uint4*>(dst + ss * piece) = v;
+        *reinterpret_cast<uint4*>(place.piece(dst, grp, ss, lane)) = v;
       }
     } else {
 #pragma unroll
@@ -191,7 +224,7 @@ __device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const 
           const uint32_t c1 = extract_index_words<BITS>(lo, 8 * ss + 2 * e + 1);
           pk[e] = static_cast<uint32_t>(tab[c0]) | (static_cast<uint32_t>(tab[c1]) << 16);
         }
-        *reinterpret_cast<uint4*>(dst + ss * piece) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *reinterpret_cast<uint4*>(place.piece(dst, grp, ss, lane)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
       }
     }
 #pragma unroll
@@ -202,7 +235,8 @@ __device__ __forceinline__ void unpack_task(const uint32_t (&planes)[24], const 
 // Uncompressed (32-bit) version of a unit: rows are plain fp32, rounded to bf16 on the way in.  A load covers four rows x
 // 32 columns, four whole lines (a lane per row would touch 32 lines with every load: 9 us for a tile of 64 x 1024);
 // sixteen loads in flight.
-__device__ __forceinline__ void unpack_raw(const DecodeTask& t, uint8_t* wsm, uint32_t n_rows, uint32_t lane, uint32_t half) {
+template <typename Place>
+__device__ __forceinline__ void unpack_raw(const DecodeTask& t, const Place& place, uint32_t lane, uint32_t half) {
 #pragma unroll 1
   for (uint32_t first = half == 2 ? 16 : 0; first < (half == 1 ? 16u : 32u); first += 16) {
     float4 v[16];
@@ -214,28 +248,28 @@ __device__ __forceinline__ void unpack_raw(const DecodeTask& t, uint8_t* wsm, ui
     for (uint32_t i = 0; i < 16; ++i)
       v[i] = __ldg(reinterpret_cast<const float4*>(t.codes + static_cast<size_t>(row(first + i)) * t.out_val + col(first + i) * 4));
 #pragma unroll
-    for (uint32_t i = 0; i < 16; ++i) {
-      uint8_t* dst = wsm + (static_cast<size_t>(t.kcore0 + (col(first + i) >> 3)) * n_rows + t.row0 + row(first + i)) * 16 + (c & 4) * 2;
-      *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(v[i].x, v[i].y), pack_bf16x2(v[i].z, v[i].w));
-    }
+    for (uint32_t i = 0; i < 16; ++i)
+      *reinterpret_cast<uint2*>(place.element(row(first + i), col(first + i))) =
+          make_uint2(pack_bf16x2(v[i].x, v[i].y), pack_bf16x2(v[i].z, v[i].w));
   }
 }
 
-// The task (or half of it) into the tile; the warp's own 128 bytes at `tab` take the table, rounded once to bf16
+// The task (or half of it) to its place; the warp's own 128 bytes at `tab` take the table, rounded once to bf16
 // (round-to-nearest-even).  Outliers (Section 6: they keep their original value) follow, the warp's own only.
-__device__ __forceinline__ void finish_task(const DecodeTask& t, const TaskLoads& f, uint16_t* tab, uint8_t* wsm, uint32_t n_rows,
+template <typename Place>
+__device__ __forceinline__ void finish_task(const DecodeTask& t, const TaskLoads& f, uint16_t* tab, const Place& place,
                                             uint32_t lane, uint32_t half) {
-  if (t.bits == 32) { unpack_raw(t, wsm, n_rows, lane, half); return; }
+  if (t.bits == 32) { unpack_raw(t, place, lane, half); return; }
   if (t.bits == 0) return;
   tab[lane] = bf16_bits(f.c0);
   tab[lane + 32] = bf16_bits(f.c1);
   __syncwarp();
   switch (t.bits) {
-    case 2: unpack_task<2>(f.w, t, tab, wsm, n_rows, lane, half); break;
-    case 3: unpack_task<3>(f.w, t, tab, wsm, n_rows, lane, half); break;
-    case 4: unpack_task<4>(f.w, t, tab, wsm, n_rows, lane, half); break;
-    case 5: unpack_task<5>(f.w, t, tab, wsm, n_rows, lane, half); break;
-    case 6: unpack_task<6>(f.w, t, tab, wsm, n_rows, lane, half); break;
+    case 2: unpack_task<2>(f.w, place, tab, lane, half); break;
+    case 3: unpack_task<3>(f.w, place, tab, lane, half); break;
+    case 4: unpack_task<4>(f.w, place, tab, lane, half); break;
+    case 5: unpack_task<5>(f.w, place, tab, lane, half); break;
+    case 6: unpack_task<6>(f.w, place, tab, lane, half); break;
     default: break;
   }
   __syncwarp();                        // the slots below are written; the table may be overwritten by the next task
@@ -245,14 +279,23 @@ __device__ __forceinline__ void finish_task(const DecodeTask& t, const TaskLoads
     uint32_t row, col;
     const bool inside = outlier_place(t, rc, row, col);
     const bool second = t.narrow ? row >= 32 : col >= 64;
-    if (inside && (half == 0 || second == (half == 2)))
-      reinterpret_cast<uint16_t*>(wsm)[(static_cast<size_t>(t.kcore0 + (col >> 3)) * n_rows + t.row0 + row) * 8 + (col & 7)] = bf16_bits(val);
+    if (inside && (half == 0 || second == (half == 2))) *reinterpret_cast<uint16_t*>(place.element(row, col)) = bf16_bits(val);
     o += 32;
     if (o < t.n_out) {
       rc = __ldg(reinterpret_cast<const uint32_t*>(t.codes + t.out_rc) + o);
       val = __ldg(reinterpret_cast<const float*>(t.codes + t.out_val) + o);
     }
   }
+}
+
+// A decoded task (SwizzledPlace, 8 KB at `tile`) to its place in the working buffer `dst` (see expand.cu).  One lane; the caller
+// has fenced the writes to the tile.  The copy is a bulk group of its own.
+__device__ __forceinline__ void store_expanded(const DecodeTask& t, const uint8_t* tile, uint8_t* dst) {
+  uint8_t* to = dst + static_cast<size_t>(expanded_at(t)) * 4096;
+  const uint32_t from = smem_addr(tile), apart = t.narrow ? 4096u : 16384u;     // the block's next 32 rows, or the next 64 columns
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], 4096;" ::"l"(to), "r"(from) : "memory");
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], 4096;" ::"l"(to + apart), "r"(from + 4096) : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------------------
@@ -298,12 +341,9 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t saddr, uint32_t rank) { 
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// The same arrival with release semantics at CTA scope only: enough where the arrival hands over tensor memory
-// (ordered by the tcgen05 fences), and it does not wait for the thread's earlier global stores to reach the
-// cluster's point of coherence, which the cluster-scope form does.
+// An arrival with release semantics at CTA scope only: enough where it hands over tensor memory (ordered by the tcgen05
+// fences), and it does not wait for the thread's earlier global stores to reach the cluster's point of coherence, which
+// the cluster-scope form does.
 __device__ __forceinline__ void mbar_arrive_cluster_cta_scope(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
@@ -335,17 +375,17 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
 // below 1.5e-7, three orders of magnitude under the bf16 rounding of the result) with the hardware
 // exponential; the epilogue runs it for every element of the FFN1 output.
 // With t = 1 / (1 + p |v| / sqrt 2) and q(t) the polynomial:  gelu(v) = max(v, 0) - |v| t q(t) / 2 exp(-v^2 / 2).
-// Issue slots bound the epilogue of the many-token kernel (a 128 x 128 tile has 4096 cycles of MMA to hide under), so all but
-// the two special functions work on pairs: FFN1 of 32 x 512 tokens 149 -> 139 us, of 8 x 512 39.7 -> 37.1.
+// All but the special functions work on pairs, and a pair shares one reciprocal: three special functions for two values (the
+// unit takes 16 lanes a cycle, so a 128 x 256 tile's GELU is 3072 cycles of it).
 __device__ __forceinline__ uint64_t gelu_erf_x2(uint64_t v) {
   const auto both = [](float c) { return pack_f32x2(c, c); };
-  float d0, d1, t0, t1, e0, e1, v0, v1;
+  float d0, d1, r, e0, e1, v0, v1;
   unpack_f32x2(v, v0, v1);
   const uint64_t abs_v = pack_f32x2(fminf(fabsf(v0), 1e30f), fminf(fabsf(v1), 1e30f));     // finite: t is 0 for an infinite v
   unpack_f32x2(fma_f32x2(abs_v, both(0.3275911f * 0.70710678118654752440f), both(1.0f)), d0, d1);
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(d0));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(d1));
-  const uint64_t t = pack_f32x2(t0, t1);
+  // one reciprocal for both: 1 / d0 = d1 / (d0 d1).  A product that overflows gives t = 0 where |v| > 1e8, and 2^(-v^2..) is 0 there.
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d0 * d1));
+  const uint64_t t = mul_f32x2(pack_f32x2(d1, d0), pack_f32x2(r, r));
   uint64_t q = fma_f32x2(t, both(0.5f * 1.061405429f), both(0.5f * -1.453152027f));
   q = fma_f32x2(q, t, both(0.5f * 1.421413741f));
   q = fma_f32x2(q, t, both(0.5f * -0.284496736f));
@@ -455,7 +495,7 @@ struct TileDecode {
     const uint32_t lane = tid & 31, warp = tid >> 5;
     uint16_t* tab = warp_tables + warp * kTableStride;
     while (unit < task_stride) {
-      finish_task(task, loads, tab, wsm, n_rows, lane, half);
+      finish_task(task, loads, tab, TilePlace(wsm, n_rows, task), lane, half);
       unit += split(task_stride) ? kWarps / 2 : kWarps;
       if (unit < task_stride) {
         task = load_task(tasks + unit);
@@ -509,12 +549,6 @@ __device__ __forceinline__ void umma_bf16_ss_x4_pair(uint32_t tmem_d, uint64_t d
 __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(bar), "h"(static_cast<uint16_t>(3)) : "memory");
-}
-
-
-template <int NWARPS>
-__device__ __forceinline__ void group_barrier(uint32_t bar_id) {
-  asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(NWARPS * 32) : "memory");
 }
 
 }  // namespace

@@ -64,11 +64,7 @@ enum StampSlot : int {
   STAMP_RELEASE = 1,       // min: first CTA past the wait for the preceding kernel
   STAMP_LAST_END = 2,      // max: the last CTA is done
   STAMP_DECODED = 3,       // max: weight tiles decoded (dequant-GEMM)
-  STAMP_LAST_START = 4,    // max: the launch's last CTA starts
-  // SM cycles that the MMA-issuing warp spent waiting, max (K-accumulating dequant-GEMM only)
-  STAMP_WAIT_WEIGHTS = 5,
-  STAMP_WAIT_ACTIVATIONS = 6,
-  STAMP_WAIT_DRAIN = 7
+  STAMP_LAST_START = 4     // max: the launch's last CTA starts
 };
 __device__ __forceinline__ void stamp_min(unsigned long long* rec, int slot) {
   if (rec != nullptr) atomicMin(rec + slot, static_cast<unsigned long long>(global_timer_ns()));
@@ -226,6 +222,14 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&r)
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
+}
+
+// Waits for the loads in flight, and holds the 16 registers that one of them fills back until then.
+__device__ __forceinline__ void tc_wait_ld_x16(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :: "memory");
 }
 
 // Same, 32 consecutive columns.

@@ -49,7 +49,6 @@ struct GemmLaunch {
   uint32_t pf_bytes[4];     // pulled into L2 by this launch's idle warps
   bool simt_debug;          // compute the products on the plain ALUs instead of the tensor cores
   bool pdl;                 // launch with programmatic dependent launch
-  bool pair;                // two-CTA clusters (cta_group::2): jobs 2i and 2i+1 share one M=256 x N=128 MMA
   unsigned long long* stamps;   // this launch's profiling record (see sti_device.cuh), or null
 };
 
@@ -60,29 +59,39 @@ size_t gemm_smem_bytes(uint32_t w_bytes, uint32_t n_stages, uint32_t bps, uint32
 cudaError_t gemm_configure();   // opt in to large dynamic shared memory (once per device)
 cudaError_t launch_gemm(GemmKind kind, const GemmLaunch& p, cudaStream_t s);
 
-// K-accumulating two-CTA dequant-GEMM (fp32 output written once, all K groups summed in tensor memory).
-// jobs: n_groups x n_cols64 tile jobs of 64 rows and at most k_group columns, job (g, c) at index g * n_cols64 + c,
-// tasks at the fixed stride; out: [T][ldo] fp32, tile c writes columns [64 c, 64 c + 64).
-struct KaccLaunch {
-  const Job* jobs;
+// A layer's weights decoded into the working buffer (expand.cu): task i's two 4 KB pieces, the first one at expanded_at(task).
+struct ExpandLaunch {
   const DecodeTask* tasks;
-  int n_groups, n_cols64, m_ctas;
-  CUtensorMap xmap;         // x: [T rows, ldx columns] bf16, box 64 x 128, 128-byte swizzle
-  const void* x;            // the same operand as a plain pointer: idle warps prefetch it into L2; null = no prefetch
-  int ldx;
-  int T;
-  float* out;
-  int ldo;
+  uint32_t n_tasks;
+  uint8_t* dst;
+  bool pdl;
+};
+cudaError_t launch_expand(const ExpandLaunch& p, cudaStream_t s);
+
+// GEMM over the working buffer (gemm_wide.cu).
+struct WideShape {
+  uint32_t T, n;            // tokens, output features (a multiple of 64)
+  uint32_t n_tiles, m_pairs, splits, k_chunks;      // tiles of NT features, of 256 tokens, planes, chunks of 64 columns
+  uint32_t w_row0;          // first 128-byte row of the matrix in the working buffer
+  uint32_t plane64;         // 1: features 64 i .. 64 i + 63 are plane i of the output; 0: planes are K splits
+};
+struct WideLaunch {
+  WideShape shape;
+  uint32_t nt;              // features per tile: 256 or 128
+  uint32_t clusters;        // CTA pairs
+  CUtensorMap xmap;         // x: [T rows, K columns] bf16, boxes of 128 rows x 64 columns, 128-byte swizzle
+  CUtensorMap wmap;         // working buffer as rows of 64 elements, boxes of nt / 2 rows, not swizzled (it is already)
+  CUtensorMap omap;         // output as [planes][T][columns], boxes of 32 rows x 128 bytes, 128-byte swizzle
+  const float* bias;        // null: none
+  const int32_t* bias_off;  // per 64 features: where their bias begins
+  bool weights_ready;       // decoded by a kernel that has finished before this one can start: read without waiting
+  ExpandLaunch beside;      // decoded beside it by otherwise idle warps (n_tasks 0: nothing); `dst` is read by no kernel in flight
   int* err;
-  uint32_t n_stages, bps, hdr_bytes, task_stride;   // ring: n_stages stages of bps boxes (1 or 2; K groups are multiples of 64 * bps)
-  uint32_t k_group;         // columns of the widest K group (a multiple of 64): the size of the two weight buffers
   bool pdl;
   unsigned long long* stamps;
 };
-cudaError_t gemm_kacc_configure();
-uint32_t gemm_kacc_stages(uint32_t hdr_bytes, uint32_t k_group, uint32_t bps, size_t smem_limit);
-size_t gemm_kacc_smem_bytes(uint32_t hdr_bytes, uint32_t n_stages, uint32_t bps, uint32_t k_group);
-cudaError_t launch_gemm_kacc(const KaccLaunch& p, cudaStream_t s);
+cudaError_t gemm_wide_configure();
+cudaError_t launch_gemm_wide(GemmKind kind, const WideLaunch& p, cudaStream_t s);
 
 // Per-head attention over kept heads.  qkv: [(kept*3 + which)][T][64] bf16; out: [T][n_kept*64] bf16.
 // sm_count (the device's multiprocessor count) and next_ctas (the CTAs of the O projection that follows) pick the CTA shape.

@@ -67,7 +67,7 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
               unsigned long long* stamps) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);      // uniform to the compiler
   if (tid == 0) { stamp_min(stamps, STAMP_FIRST_START); stamp_max(stamps, STAMP_LAST_START); }
   const DecodeTask* my_tasks = tasks + static_cast<size_t>(blockIdx.x) * task_stride;
   TileDecode decode;
@@ -200,22 +200,21 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
   } else {
     bool failed = false;
     if (warp == 0) {
-      // ---- producer: fill the ring, then refill a stage as soon as the MMAs that read it have completed
-      if (lane == 0) {
-        while (p_c < n_stages && p_c < total) { request_chunk(p_stage, p_kcr, p_ti); producer_advance(); }
-        uint32_t p_phase = 0;                 // parity of the `empty` completion being waited for
-        while (p_c < total) {
-          if (!mbar_wait_bounded_relaxed(smem_addr(&hdr->empty[p_stage]), p_phase)) { failed = true; break; }
-          request_chunk(p_stage, p_kcr, p_ti);
-          if (p_stage + 1 == n_stages) p_phase ^= 1;
-          producer_advance();
-        }
-        if (failed) {
-          // give every copy this CTA requested a bounded chance to land before the CTA exits
-          const uint32_t first = p_c > n_stages ? p_c - n_stages : 0;
-          for (uint32_t c = first; c < p_c; ++c)
-            (void)mbar_wait_bounded(smem_addr(&hdr->full[c % n_stages]), (c / n_stages) & 1);
-        }
+      // ---- producer: fill the ring, then refill a stage as soon as the MMAs that read it have completed.  The warp walks the
+      // loop converged and one elected lane issues (a loop that one lane runs alone issues at half the rate).
+      uint32_t p_phase = 0;                   // parity of the `empty` completion being waited for
+      while (p_c < total) {
+        if (p_c >= n_stages && !__all_sync(0xffffffffu, mbar_wait_bounded(smem_addr(&hdr->empty[p_stage]), p_phase))) { failed = true; break; }
+        if (elect_one()) request_chunk(p_stage, p_kcr, p_ti);
+        __syncwarp();
+        if (p_c >= n_stages && p_stage + 1 == n_stages) p_phase ^= 1;
+        producer_advance();
+      }
+      if (failed) {
+        // give every copy this CTA requested a bounded chance to land before the CTA exits
+        const uint32_t first = p_c > n_stages ? p_c - n_stages : 0;
+        for (uint32_t c = first; c < p_c; ++c)
+          (void)mbar_wait_bounded(smem_addr(&hdr->full[c % n_stages]), (c / n_stages) & 1);
       }
       __syncwarp();
     } else if (warp == 1) {

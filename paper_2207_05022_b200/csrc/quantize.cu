@@ -394,31 +394,38 @@ quantize_units_kernel(const float* w_all, uint32_t n, int bits, uint32_t* codes_
 // elements at those ranks, c = 1 .. 2^k - 1) whose pair is not above its own, and nothing has to be sorted but the
 // few weights that share a value bin with a boundary.  A cluster of C CTAs (C = 1 .. 16, chosen by the number of units
 // in the call) works on one unit:
-//   1. fp64 moments, one pass, about a provisional centre;
-//   2. a histogram of the inliers over equal-width value bins between the two outlier thresholds (the bin is a
-//      monotone function of the value, so bins partition the sorted order), one per CTA, added up through
-//      distributed shared memory; its prefix gives the bin and the in-bin rank of every boundary;
-//   3. ONE pass that gives every weight outside the boundary bins its index (bin -> number of boundaries in lower
-//      bins), adds the cluster sums, packs the stream and writes the outlier lists; the weights of boundary bins are
-//      set aside as pairs, their indexes left zero in the stream;
-//   4. a warp per boundary bin ranks its pairs by counting, ORs their indexes into the stream and adds their values to
+//   1. 256 of its weights say about where the others lie: equal-width value bins over a little more than the
+//      inliers' range (the bin is a monotone function of the value, so bins partition the sorted order), and from
+//      where on a weight may be an outlier;
+//   2. ONE pass: fp64 moments, a histogram of all weights over the bins, one per CTA, and a list of the tails;
+//   3. the moments give the outlier test, which the listed tails are put to; the histograms are added up through
+//      distributed shared memory, and the prefix gives the bin and the in-bin rank of every boundary (the outliers
+//      below the mean come first);
+//   4. a second pass gives every weight outside the boundary bins its index (bin -> number of boundaries in lower
+//      bins), adds the cluster sums and packs the stream; the weights of boundary bins are set aside as pairs, their
+//      indexes left zero in the stream, and so are the outliers', which only lie in special bins, too;
+//   5. a warp per boundary bin ranks its pairs by counting, ORs their indexes into the stream and adds their values to
 //      the sums in rank order; then the centroids and the outliers' indexes.
-// Every warp owns one contiguous run of the unit in all passes (a lane reads four consecutive weights at a time), so
+// Every warp owns one contiguous run of the unit in both passes (a lane reads four consecutive weights at a time), so
 // outlier lists come out in ascending offsets from per-warp counts alone.  Cluster sums are plain fp64 additions in a
 // fixed order (every cell of a shared-memory table has one writing thread or threads that take turns, columns and
-// CTAs are added in a fixed tree), so the output is deterministic.
+// CTAs are added in a fixed tree), so the output is deterministic.  What 256 weights say only decides how long things take:
+// should outliers lie further in than the listed tails, the tails are listed again; should a boundary lie in a bin
+// with outliers, or a bin hold too many weights, the unit is sorted.
 //
 // The fp64 outlier test is monotone on either side of the mean, so it is taken once per unit, to find the smallest and
 // the largest fp32 value that pass it; a weight is then an inlier if it lies between these two.
 //
 // Two CTAs of 512 threads share an SM: while one waits at a cluster barrier or for memory the other has the pipes.
+// That leaves 64 registers: what pass 4 does not need is kept in shared memory meanwhile, because a spilled value comes back
+// from L2 (the streamed weights push it out of the first-level cache): three of them cost a small call 1.2 of 28 us.
 //
-// Bound: with few units the chain of seven cluster barriers and the table passes between them (half of the 31 us that
-// 12 units of 196,608 weights take at 4 bits; one CTA of 1024 threads per unit and five passes took 126 us); with many
-// units issue slots (65 % busy at 3 bits) and the shared-memory pipe (52 %): 4 cycles for a warp's 32 weights in the
-// histogram's atomics, 9 in the table lookup, the fp64 read-modify-write of the sums and the staging of the stream (384 units of
-// 524,288 weights at 3 bits: 1055 -> 623 us, 1.4 TB/s of the 6.5 a copy moves; 16 such units at 6 bits, where four lanes
-// take turns at the sums, 435 -> 94).
+// Bound: with few units the chain of six cluster barriers and the table passes between them (23 of the 31 us that
+// 12 units of 196,608 weights take at 4 bits); with many the shared-memory pipe and the latency of the chains through
+// it: pass 2 takes 11.6 cycles per 32 weights, the histogram's atomics (3.9 wavefronts each); pass 4 15.5, the table
+// lookup, the fp64 read-modify-write of the sums and the staging of the stream.  Moments, histogram and indexes as three
+// passes, with the inliers looked for in each: 384 units of 524,288 weights at 3 bits 624 -> 494 us, 200 at 4 bits 345 ->
+// 284, 40 of 100,096 at 3 bits 43.1 -> 39.5, 12 of 196,608 at 4 bits 31.5 -> 31.3.
 
 constexpr int kSelThreads = 512;
 constexpr int kSelWarps = kSelThreads / 32;
@@ -428,7 +435,10 @@ constexpr int kSelMaxSeg = 1024;           // weights of one boundary bin that a
 constexpr int kSelSmemSeg = 256;           // ... in shared memory; more than that in the workspace
 constexpr int kSelGroups = 4;              // groups of 128 consecutive weights (four per lane) a warp classifies per step
 constexpr int kSelStep = kSelGroups * 128; // weights of one step of one warp
+constexpr uint32_t kSelTails = 32;         // weights of a warp's tails that are listed in shared memory; more of them in the workspace
 constexpr int kAccCells = 8192;            // fp64 cells of the cluster-sum table: 2^k clusters x columns
+
+struct SelTail { uint32_t offset; float value; };
 
 struct SelShared {
   double red[2][kSelWarps];
@@ -436,67 +446,54 @@ struct SelShared {
   double part[kSelMaxCluster][64];         // cluster sums of every CTA
   double extra_lo[64], extra_hi[64];       // sums of cluster c's weights from the bin of its lower / only of its upper boundary
   uint32_t warp_out[kSelWarps];            // outliers of each warp's run -> their exclusive prefix
-  uint32_t warp_in[kSelWarps];             // inliers in each warp's run of bins -> their exclusive prefix
-  uint32_t cta_out[kSelMaxCluster], range_in[kSelMaxCluster];   // of every CTA: outliers found, inliers in its range of bins
+  uint32_t warp_in[kSelWarps];             // weights in each warp's run of bins -> their exclusive prefix
+  uint32_t cta_out[kSelMaxCluster], cta_low[kSelMaxCluster];    // of every CTA: outliers found, those below the mean among them
+  uint32_t range_in[kSelMaxCluster];       // of every CTA: weights in its range of bins
+  uint32_t low;
   uint32_t bounds[65];
   uint32_t bnd_bin[64], bnd_rho[64], seg_len[64];   // of boundary c: its bin, its rank in the bin, the bin's population
   uint32_t seg_start[64];                  // where the pairs of the bin that boundary c is the first of begin
-  uint32_t seg_fill[64];                   // next free place of this CTA in that list
+  uint32_t seg_count[64];                  // pairs in that list so far (the first CTA's copy counts for the cluster)
   uint32_t longest;
   float cents[64];
-  alignas(16) uint8_t binfo[kSelBins];     // boundaries in lower bins (6 bits) | 0x80: holds a boundary
+  alignas(16) uint8_t binfo[kSelBins];     // boundaries in lower bins (6 bits) | kInfoBoundary: holds one | kInfoSpecial: look closer
+  SelTail tails[kSelWarps][kSelTails];     // the first entries of each warp's list of tails
+  // What the end of the kernel needs again, kept here and not in registers: a spilled one would come back from L2.
+  uint32_t n_tails[kSelWarps], n_in, n_out;
+  float least, most;
   alignas(16) uint32_t stage[kSelWarps][2 * 128 * 6 / 32];       // the packed indexes of two groups
   union alignas(16) {
-    uint32_t hist[kSelBins];               // this CTA's inlier histogram; in its own range of bins the cluster's, then its prefix
+    uint32_t hist[kSelBins];               // this CTA's histogram; in its own range of bins the cluster's, then its prefix
     double acc[kAccCells];                 // later the cluster sums
     unsigned long long pairs[kSelWarps][2][kSelSmemSeg];         // and last the boundary bins: as gathered, in order
   } u;
 };
 static_assert(2 * (sizeof(SelShared) + 1024) <= 228 * 1024, "two CTAs on an SM");
 static_assert(sti::kEndCandidates == 16, "half a warp");
+static_assert(kSelBins / kSelMaxCluster / kSelWarps <= 64, "eight of the cluster's CTAs per lane");
 
-constexpr uint32_t kInfoBoundary = 0x80u;
+// A weight of a special bin is looked at by itself: the bin holds a boundary, or an end of the inliers' range, or lies outside it.
+constexpr uint32_t kInfoSpecial = 0x80u, kInfoBoundary = 0x40u;
 
 // What classifies a weight of a unit.
 struct SelUnit {
   float least, most;                       // the inliers' range
-  float inv, off, last;                    // place of a value between the thresholds: 0 .. 1; the last bin's number
+  float inv, off;                          // place of a value between the ends of the bins: 0 .. 1
+  float last;                              // the last bin's number times 2^-149, the smallest fp32 number
   __device__ __forceinline__ bool inlier(float x) const { return x >= least && x <= most; }
-  // 2^23 + bin: the nearest integer of a clamped value in [0, last], monotone in x.  NaN goes to bin 0.
-  __device__ __forceinline__ float place(float x) const { return fmaf(__saturatef(fmaf(x, inv, off)), last, 8388608.0f); }
+  // The nearest integer of a clamped value in [0, last bin], monotone in x: as a multiple of 2^-149 it is its own bit pattern.
+  // NaN goes to bin 0.
+  __device__ __forceinline__ uint32_t bin(float x) const { return __float_as_uint(__fmul_rn(__saturatef(fmaf(x, inv, off)), last)); }
 };
-__device__ __forceinline__ uint32_t bin_of(float place) { return static_cast<uint32_t>(__float_as_int(place) - 0x4B000000); }
 
 __device__ __forceinline__ float4 load4(const float* w, uint32_t i, uint32_t n) {
   return i < n ? *reinterpret_cast<const float4*>(w + i) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Sum and sum of squares of x - shift over the cluster, in fp64 and in a fixed order.
-__device__ __forceinline__ void cluster_moments(cg::cluster_group& cluster, SelShared& sm, int set, const float* w, uint32_t n,
-                                                uint32_t base, uint32_t part, double shift, int tid, double& sum, double& squares) {
+// A thread's sum and sum of squares -> the cluster's, in fp64 and in a fixed order.
+__device__ __forceinline__ void cluster_sums(cg::cluster_group& cluster, SelShared& sm, int set, double a, double b, int tid, double& sum,
+                                             double& squares) {
   const int lane = tid & 31, warp = tid >> 5;
-  double s[2] = {0.0, 0.0}, q[2] = {0.0, 0.0};
-  float4 next[kSelGroups];
-#pragma unroll
-  for (int u = 0; u < kSelGroups; ++u) next[u] = load4(w, base + u * 128u, n);
-  for (uint32_t e0 = 0; e0 < part; e0 += kSelStep) {
-    float4 x[kSelGroups];
-#pragma unroll
-    for (int u = 0; u < kSelGroups; ++u) {
-      x[u] = next[u];
-      if (e0 + kSelStep < part) next[u] = load4(w, base + e0 + kSelStep + u * 128u, n);
-    }
-#pragma unroll
-    for (int u = 0; u < kSelGroups; ++u) {
-      if (base + e0 + u * 128u >= n) continue;
-      const double d0 = static_cast<double>(x[u].x) - shift, d1 = static_cast<double>(x[u].y) - shift;
-      const double d2 = static_cast<double>(x[u].z) - shift, d3 = static_cast<double>(x[u].w) - shift;
-      s[0] += d0 + d1; s[1] += d2 + d3;
-      q[0] = fma(d0, d0, q[0]); q[1] = fma(d1, d1, q[1]);
-      q[0] = fma(d2, d2, q[0]); q[1] = fma(d3, d3, q[1]);
-    }
-  }
-  double a = s[0] + s[1], b = q[0] + q[1];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) { a += __shfl_xor_sync(0xffffffffu, a, o); b += __shfl_xor_sync(0xffffffffu, b, o); }
   if (lane == 0) { sm.red[0][warp] = a; sm.red[1][warp] = b; }
@@ -513,6 +510,64 @@ __device__ __forceinline__ void cluster_moments(cg::cluster_group& cluster, SelS
   sum = squares = 0.0;
   for (int r = 0; r < n_ctas; ++r) { sum += sm.moments[set][r][0]; squares += sm.moments[set][r][1]; }
 }
+
+// The first step of a warp's run, for for_each_group to begin with.
+__device__ __forceinline__ void load_step(const float* w, uint32_t n, uint32_t base, float4 (&next)[kSelGroups]) {
+#pragma unroll
+  for (int u = 0; u < kSelGroups; ++u) next[u] = load4(w, base + u * 128u, n);
+}
+// Calls f(first offset of the lane's four, the four weights, whether they exist) for every group of 128 weights of a warp's run,
+// in order, all lanes together.  The next step's loads are issued together before this one is worked on (spread over the step,
+// each into the registers just used, they took 84 instead of 50 us for the first pass over 384 units of 524,288 weights).
+template <typename F>
+__device__ __forceinline__ void for_each_group(const float* w, uint32_t n, uint32_t base, uint32_t part, float4 (&next)[kSelGroups], F f) {
+  for (uint32_t e0 = 0; e0 < part; e0 += kSelStep) {
+    float4 x[kSelGroups];
+#pragma unroll
+    for (int u = 0; u < kSelGroups; ++u) {
+      x[u] = next[u];
+      if (e0 + kSelStep < part) next[u] = load4(w, base + e0 + kSelStep + u * 128u, n);
+    }
+#pragma unroll
+    for (int u = 0; u < kSelGroups; ++u) f(base + e0 + u * 128u, x[u], base + e0 + u * 128u < n);
+  }
+}
+
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float y;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float y;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+
+// A warp's list of weights below `lo` or above `hi`, by ascending offsets.
+struct SelTails {
+  SelTail* near;                           // the first kSelTails of them
+  SelTail* far;                            // the others: places kSelTails .. of this array
+  uint32_t n;
+  __device__ __forceinline__ SelTail& at(uint32_t k) const { return k < kSelTails ? near[k] : far[k]; }
+  // those of one group of 128 weights, all lanes together
+  __device__ __forceinline__ void add(uint32_t i0, const float4& x, bool exists, float lo, float hi) {
+    const float most = max3(fmaxf(x.x, x.y), x.z, x.w), least = min3(fminf(x.x, x.y), x.z, x.w);
+    uint32_t left = __ballot_sync(0xffffffffu, exists && (most > hi || least < lo));
+    while (left != 0u) {                   // lane after lane, one as a rule
+      const int from = __ffs(static_cast<int>(left)) - 1;
+      left &= left - 1u;
+      uint32_t k = n;
+      if (static_cast<int>(threadIdx.x & 31u) == from) {
+        const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (v[j] < lo || v[j] > hi) at(k++) = {i0 + j, v[j]};
+      }
+      n = __shfl_sync(0xffffffffu, k, from);
+    }
+  }
+};
 
 template <int BITS>      // the index width is a compile-time constant: the packing and the table addressing unroll to immediates
 __global__ void __launch_bounds__(kSelThreads, 2)
@@ -542,30 +597,121 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
 
   for (uint32_t i = tid; i < n_bins / 4; i += kSelThreads) reinterpret_cast<uint4*>(sm.u.hist)[i] = make_uint4(0u, 0u, 0u, 0u);
 
-  // ---- 1. Gaussian fit.  One pass about the mean of 32 weights; should that centre be far off, so that the squares
-  //         cancel, a second one about the mean found.
-  float centre = w[static_cast<size_t>(n / 32u) * lane] * 0.03125f;
+  // ---- 1. Where the bins go and what may be an outlier, from 256 weights spread over the unit: a Gaussian of their mean absolute
+  //         deviation, which a few outliers hardly change.  Every warp of the cluster looks at the same ones by itself.  A poor
+  //         guess costs time only: bins that are too wide, or the tails listed a second time.
+  SelUnit un;
+  float tail_lo, tail_hi;
+  float4 ahead[kSelGroups];
+  {
+    float4 x[2];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) centre += __shfl_xor_sync(0xffffffffu, centre, o);
-  const double count = static_cast<double>(n), shift = static_cast<double>(centre);
+    for (uint32_t u = 0; u < 2; ++u)
+      x[u] = *reinterpret_cast<const float4*>(w + static_cast<size_t>(static_cast<uint64_t>(n / 4u) * (32u * u + lane) / 64u) * 4u);
+    load_step(w, n, base, ahead);
+    float s = ((x[0].x + x[0].y) + (x[0].z + x[0].w)) + ((x[1].x + x[1].y) + (x[1].z + x[1].w));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const float centre = s * (1.f / 256.f);
+    s = 0.f;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) s += (fabsf(x[u].x - centre) + fabsf(x[u].y - centre)) + (fabsf(x[u].z - centre) + fabsf(x[u].w - centre));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const float deviation = s * (1.25331414f / 256.f);                 // a Gaussian's is sqrt(pi / 2) mean absolute deviations; within 5 %
+    const float c = 4.f - 0.918938533f - logf(deviation);              // radius of the inliers of such a Gaussian: sqrt(2 c) deviations
+    const float radius = deviation * (c > 0.f ? sqrtf(2.f * c) : 4.f);
+    un.inv = 1.f / (2.7f * radius);
+    un.off = 0.5f - centre * un.inv;
+    if (!(un.inv < 1.0e34f) || !(fabsf(un.off) < 1.0e34f)) { un.inv = 0.f; un.off = 0.5f; }
+    un.last = __uint_as_float(n_bins - 1u);
+    tail_lo = centre - 0.88f * radius;
+    tail_hi = centre + 0.88f * radius;
+  }
+  if (tid < 64) { sm.seg_count[tid] = 0u; sm.extra_lo[tid] = sm.extra_hi[tid] = 0.0; }
+  if (tid == 0) sm.low = 0u;
+  __syncthreads();                         // the histogram is all zeros
+
+  // ---- 2. one pass: Gaussian fit, histogram, list of the tails.  Squares about zero: should the mean be far off, so that they
+  //         cancel, a second pass about the mean found.
+  auto tails_far = [&](uint32_t run_start) { return reinterpret_cast<SelTail*>(cand + n) + run_start; };      // the workspace's second half
+  SelTails tails = {sm.tails[warp], tails_far(base - 4u * lane), 0u};
+  double s[2] = {0.0, 0.0}, q[2] = {0.0, 0.0};
+  for_each_group(w, n, base, part, ahead, [&](uint32_t i0, const float4& x, bool exists) {
+    if (exists) {
+      const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const double d = static_cast<double>(v[j]);
+        s[j & 1] += d;
+        q[j & 1] = fma(d, d, q[j & 1]);
+        atomicAdd(&sm.u.hist[un.bin(v[j])], 1u);
+      }
+    }
+    tails.add(i0, x, exists, tail_lo, tail_hi);
+  });
+  const double count = static_cast<double>(n);
   double sum, squares;
-  cluster_moments(cluster, sm, 0, w, n, base, part, shift, tid, sum, squares);
-  double mu = shift + sum / count;
-  double var = squares / count - (sum / count) * (sum / count);
-  if (!((sum / count) * (sum / count) <= 4.0 * var)) {                 // the same in every thread of the cluster
-    cluster_moments(cluster, sm, 1, w, n, base, part, mu, tid, sum, squares);
+  cluster_sums(cluster, sm, 0, s[0] + s[1], q[0] + q[1], tid, sum, squares);
+  // the cluster's histogram: CTA r adds up range r of the bins, in its own copy, and forms the prefix inside each warp's
+  // run of it
+  const uint32_t range = n_bins / n_ctas, range0 = rank * range, run = range / kSelWarps;
+  {
+    uint32_t* mine = sm.u.hist + range0 + warp * run;
+    // A lane reads four bins from every `groups`-th CTA, all in flight together (at most eight: 16 CTAs have runs of 64 bins or
+    // 32); the groups' sums are added up by shuffles.
+    const uint32_t vec = run < 128u ? run / 4u : 32u, groups = 32u / vec, group = lane / vec;
+    for (uint32_t i = 4u * (lane % vec); i < run; i += 128) {
+      uint4 r[8], t = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (uint32_t q = 0; q < 8; ++q) {
+        const uint32_t from = group + q * groups;
+        r[q] = from < n_ctas ? *cluster.map_shared_rank(reinterpret_cast<const uint4*>(mine + i), (rank + from) & (n_ctas - 1u)) : t;
+      }
+#pragma unroll
+      for (uint32_t q = 0; q < 8; ++q) { t.x += r[q].x; t.y += r[q].y; t.z += r[q].z; t.w += r[q].w; }
+      for (uint32_t o = vec; o < 32u; o <<= 1) {
+        t.x += __shfl_xor_sync(0xffffffffu, t.x, o); t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+        t.z += __shfl_xor_sync(0xffffffffu, t.z, o); t.w += __shfl_xor_sync(0xffffffffu, t.w, o);
+      }
+      if (group == 0u) *reinterpret_cast<uint4*>(mine + i) = t;
+    }
+    __syncwarp();
+    uint32_t before = 0;
+    for (uint32_t i = lane; i < run; i += 32) {
+      const uint32_t t = mine[i];
+      uint32_t inc = t;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const uint32_t s = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += s; }
+      mine[i] = before + inc - t;
+      before += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    if (lane == 0) sm.warp_in[warp] = before;
+  }
+  double mu = sum / count;
+  double var = squares / count - mu * mu;
+  if (!(mu * mu <= 4.0 * var)) {                                       // the same in every thread of the cluster
+    const double shift = mu;
+    s[0] = s[1] = q[0] = q[1] = 0.0;
+    load_step(w, n, base, ahead);
+    for_each_group(w, n, base, part, ahead, [&](uint32_t, const float4& x, bool exists) {
+      if (!exists) return;
+      const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const double d = static_cast<double>(v[j]) - shift;
+        s[j & 1] += d;
+        q[j & 1] = fma(d, d, q[j & 1]);
+      }
+    });
+    cluster_sums(cluster, sm, 1, s[0] + s[1], q[0] + q[1], tid, sum, squares);
     var = squares / count - (sum / count) * (sum / count);
     mu += sum / count;
   }
   const double c0 = -0.5 * log(2.0 * 3.14159265358979323846 * var);
   const double inv2var = 1.0 / (2.0 * var);
-  // inliers satisfy (x - mu)^2 <= 2 var (c0 + 4): the bins span that interval, values outside are clamped
-  const double radius = sqrt(2.0 * var * (c0 + 4.0));
-  SelUnit un;
-  un.inv = static_cast<float>(1.0 / (2.0 * radius));
-  un.off = -static_cast<float>(mu - radius) * un.inv;
-  un.last = static_cast<float>(n_bins - 1u);
-  if (!(var > 0.0) || !(radius > 0.0) || !(un.inv > 0.f) || !(un.inv < 1.0e34f) || !(fabsf(un.off) < 1.0e34f)) {
+  const double radius = sqrt(2.0 * var * (c0 + 4.0));                  // inliers satisfy (x - mu)^2 <= 2 var (c0 + 4)
+  if (!(var > 0.0) || !(radius > 0.0)) {
     if (rank == 0 && tid == 0) marks[unit] = 1;                        // every thread of the cluster leaves
     return;
   }
@@ -583,31 +729,25 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     un.most = __shfl_sync(0xffffffffu, x, sti::kEndCandidates + most);
   }
 
-  // ---- 2. outliers counted per warp, inliers into the histogram
-  uint32_t my_out = 0;
-  float4 next[kSelGroups];
-#pragma unroll
-  for (int u = 0; u < kSelGroups; ++u) next[u] = load4(w, base + u * 128u, n);
-  for (uint32_t e0 = 0; e0 < part; e0 += kSelStep) {
-    float4 x[kSelGroups];
-#pragma unroll
-    for (int u = 0; u < kSelGroups; ++u) {
-      x[u] = next[u];
-      if (e0 + kSelStep < part) next[u] = load4(w, base + e0 + kSelStep + u * 128u, n);
-    }
-#pragma unroll
-    for (int u = 0; u < kSelGroups; ++u) {
-      if (base + e0 + u * 128u >= n) continue;
-      const float v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (un.inlier(v[j])) atomicAdd(&sm.u.hist[bin_of(un.place(v[j]))], 1u);
-        else ++my_out;
-      }
-    }
+  // ---- 3. the outliers among the tails
+  if (!(un.least <= tail_lo && un.most >= tail_hi)) {                  // some lie further in: list exactly them
+    tails.n = 0;
+    load_step(w, n, base, ahead);
+    for_each_group(w, n, base, part, ahead, [&](uint32_t i0, const float4& x, bool exists) { tails.add(i0, x, exists, un.least, un.most); });
+  }
+  __syncwarp();
+  uint32_t my_out = 0, my_low = 0;
+  for (uint32_t k = lane; k < tails.n; k += 32) {
+    const float x = tails.at(k).value;
+    my_out += un.inlier(x) ? 0u : 1u;
+    my_low += x < un.least ? 1u : 0u;
   }
   my_out = __reduce_add_sync(0xffffffffu, my_out);
-  if (lane == 0) sm.warp_out[warp] = my_out;
+  my_low = __reduce_add_sync(0xffffffffu, my_low);
+  if (lane == 0) {
+    sm.warp_out[warp] = my_out;
+    if (my_low != 0u) atomicAdd(&sm.low, my_low);
+  }
   __syncthreads();
   if (warp == 0) {
     const uint32_t mine = lane < kSelWarps ? sm.warp_out[lane] : 0u;
@@ -616,40 +756,12 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     for (int o = 1; o < kSelWarps; o <<= 1) { const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
     if (lane < kSelWarps) sm.warp_out[lane] = inc - mine;
     const uint32_t total = __shfl_sync(0xffffffffu, inc, kSelWarps - 1);
-    if (lane < static_cast<int>(n_ctas)) *cluster.map_shared_rank(&sm.cta_out[rank], lane) = total;
+    if (lane < static_cast<int>(n_ctas)) {
+      *cluster.map_shared_rank(&sm.cta_out[rank], lane) = total;
+      *cluster.map_shared_rank(&sm.cta_low[rank], lane) = sm.low;
+    }
   }
-  cluster.sync();
 
-  // the cluster's histogram: CTA r adds up range r of the bins, in its own copy, and forms the prefix inside each warp's
-  // run of it
-  const uint32_t range = n_bins / n_ctas, range0 = rank * range, run = range / kSelWarps;
-  {
-    uint32_t* mine = sm.u.hist + range0 + warp * run;
-    for (uint32_t i = 4 * lane; i < run; i += 128) {                   // 32 bins or more
-      uint4 t = *reinterpret_cast<const uint4*>(mine + i);
-      for (uint32_t q0 = 1; q0 < n_ctas; q0 += 7) {                    // seven CTAs' counts in flight together
-        uint4 r[7];
-#pragma unroll
-        for (uint32_t q = 0; q < 7; ++q)
-          r[q] = q0 + q < n_ctas ? *cluster.map_shared_rank(reinterpret_cast<const uint4*>(mine + i), (rank + q0 + q) & (n_ctas - 1u))
-                                 : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-        for (uint32_t q = 0; q < 7; ++q) { t.x += r[q].x; t.y += r[q].y; t.z += r[q].z; t.w += r[q].w; }
-      }
-      *reinterpret_cast<uint4*>(mine + i) = t;
-    }
-    __syncwarp();
-    uint32_t before = 0;
-    for (uint32_t i = lane; i < run; i += 32) {
-      const uint32_t t = mine[i];
-      uint32_t inc = t;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) { const uint32_t s = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += s; }
-      mine[i] = before + inc - t;
-      before += __shfl_sync(0xffffffffu, inc, 31);
-    }
-    if (lane == 0) sm.warp_in[warp] = before;
-  }
   __syncthreads();
   if (warp == 0) {
     const uint32_t mine = lane < kSelWarps ? sm.warp_in[lane] : 0u;
@@ -662,20 +774,23 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
   }
   cluster.sync();
 
-  // ---- the boundary ranks: the CTA whose range holds one finds its bin and tells the others
-  uint32_t n_out = 0, out_before = 0, in_before = 0;
+  // ---- the boundary ranks, among all weights (the outliers below the mean come before every inlier): the CTA whose range of
+  //      bins holds one finds its bin and tells the others
+  uint32_t n_out = 0, n_low = 0, out_before = 0, in_before = 0;
   for (uint32_t r = 0; r < n_ctas; ++r) {
     if (r < rank) { out_before += sm.cta_out[r]; in_before += sm.range_in[r]; }
     n_out += sm.cta_out[r];
+    n_low += sm.cta_low[r];
   }
+  const uint32_t least_bin = un.bin(un.least), most_bin = un.bin(un.most);       // outliers are in these or beyond
   const uint32_t n_in = n - n_out;
   if (n_in == 0) {                         // no rank to look for: nothing below would be written before it is read
     if (rank == 0 && tid == 0) marks[unit] = 1;                        // every thread of the cluster leaves
     return;
   }
   if (tid <= static_cast<int>(K)) {
-    const uint32_t r = static_cast<uint32_t>(static_cast<uint64_t>(tid) * n_in / K);
-    sm.bounds[tid] = r;
+    sm.bounds[tid] = static_cast<uint32_t>(static_cast<uint64_t>(tid) * n_in / K);
+    const uint32_t r = n_low + sm.bounds[tid];
     if (tid >= 1 && tid < static_cast<int>(K) && r >= in_before && r - in_before < sm.range_in[rank]) {
       const uint32_t at = r - in_before;
       uint32_t v = 0;                                                  // the last run, then bin, whose prefix is <= the rank holds it
@@ -685,15 +800,31 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
       uint32_t b = 0;
       for (uint32_t step = run / 2; step > 0; step >>= 1) if (bins[b + step] <= in_run) b += step;
       const uint32_t run_end = (v + 1 < kSelWarps ? sm.warp_in[v + 1] : sm.range_in[rank]) - sm.warp_in[v];
-      const uint32_t len = (b + 1 < run ? bins[b + 1] : run_end) - bins[b];
+      const uint32_t bin = range0 + v * run + b;
+      uint32_t len = (b + 1 < run ? bins[b + 1] : run_end) - bins[b];
+      if (bin <= least_bin || bin >= most_bin) len = ~0u;              // outliers among its weights: too long for a list
       for (uint32_t q = 0; q < n_ctas; ++q) {
-        *cluster.map_shared_rank(&sm.bnd_bin[tid], q) = range0 + v * run + b;
+        *cluster.map_shared_rank(&sm.bnd_bin[tid], q) = bin;
         *cluster.map_shared_rank(&sm.bnd_rho[tid], q) = in_run - bins[b];
         *cluster.map_shared_rank(&sm.seg_len[tid], q) = len;
       }
     }
   }
-  cluster.sync();
+  __syncthreads();                                                     // this CTA's histogram has been searched
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // meanwhile: pass 4's first loads, its table, the outlier lists
+  float4 next[2] = {load4(w, base, n), load4(w, base + 128u, n)};
+  for (int i = tid; i < kAccCells / 2; i += kSelThreads) reinterpret_cast<uint4*>(sm.u.acc)[i] = make_uint4(0u, 0u, 0u, 0u);
+  uint32_t run_out = out_before + sm.warp_out[warp];
+  for (uint32_t k0 = 0; k0 < tails.n; k0 += 32) {
+    const SelTail t = k0 + lane < tails.n ? tails.at(k0 + lane) : SelTail{0u, un.least};
+    const uint32_t all = __ballot_sync(0xffffffffu, !un.inlier(t.value)), dst = run_out + __popc(all & lt_mask);
+    if (!un.inlier(t.value) && dst < max_out) { ooff[dst] = t.offset; oval[dst] = t.value; }
+    run_out += __popc(all);
+  }
+  if (lane == 0) sm.n_tails[warp] = tails.n;
+  if (tid == 0) { sm.n_in = n_in; sm.n_out = n_out; sm.least = un.least; sm.most = un.most; }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
   // lists of the boundary bins' pairs: the first boundary of a bin owns its list, in which the CTAs' pairs follow one another
   auto owns = [&](uint32_t c) { return c == 1u || sm.bnd_bin[c] != sm.bnd_bin[c - 1]; };
@@ -711,26 +842,17 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     }
     if (lane == 0) sm.longest = longest;
   }
-  uint32_t fill = 0;                                                   // what the CTAs before this one put into boundary tid's bin
-  if (tid >= 1 && tid < static_cast<int>(K) && owns(tid)) {
-    const uint32_t b = sm.bnd_bin[tid], holder = b / range;            // the holder's own count made way for the cluster's
-    uint32_t others = 0, t[kSelMaxCluster];
-#pragma unroll
-    for (uint32_t r = 0; r < kSelMaxCluster; ++r)                      // all in flight together
-      t[r] = r < n_ctas && r != holder ? *cluster.map_shared_rank(&sm.u.hist[b], r) : 0u;
-#pragma unroll
-    for (uint32_t r = 0; r < kSelMaxCluster; ++r) {
-      others += t[r];
-      if (r < rank) fill += t[r];
-    }
-    if (holder < rank) fill += sm.seg_len[tid] - others;
-  }
   for (uint32_t i = tid; i < n_bins / 16; i += kSelThreads) {          // sixteen bins a thread
     uint32_t below = 0, packed[4];                                     // boundaries 1 .. below sit in lower bins (their bins ascend)
 #pragma unroll
     for (uint32_t step = K >> 1; step > 0; step >>= 1)
       if (sm.bnd_bin[below + step] < 16u * i) below += step;
     uint32_t next = below + 1 < K ? sm.bnd_bin[below + 1] : 0xffffffffu;
+    if (next > 16u * i + 15u && 16u * i > least_bin && 16u * i + 15u < most_bin) {       // none of them is special
+      const uint32_t four = below * 0x01010101u;
+      reinterpret_cast<uint4*>(sm.binfo)[i] = make_uint4(four, four, four, four);
+      continue;
+    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       packed[q] = 0;
@@ -738,31 +860,25 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
       for (int e = 0; e < 4; ++e) {
         const uint32_t b = 16u * i + 4 * q + e;
         while (next < b) { ++below; next = below + 1 < K ? sm.bnd_bin[below + 1] : 0xffffffffu; }
-        packed[q] |= (below | (next == b ? kInfoBoundary : 0u)) << (8 * e);
+        const uint32_t info = next == b ? kInfoBoundary | kInfoSpecial : b <= least_bin || b >= most_bin ? kInfoSpecial : 0u;
+        packed[q] |= (below | info) << (8 * e);
       }
     }
     reinterpret_cast<uint4*>(sm.binfo)[i] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
   }
-  cluster.sync();                                                      // nobody looks at another CTA's histogram any more
+  __syncthreads();
   if (sm.longest > static_cast<uint32_t>(kSelMaxSeg)) {
     if (rank == 0 && tid == 0) marks[unit] = 1;
     return;
   }
-  if (tid < static_cast<int>(K)) sm.seg_fill[tid] = sm.seg_start[tid] + fill;
-  for (int i = tid; i < kAccCells / 2; i += kSelThreads) reinterpret_cast<uint4*>(sm.u.acc)[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (tid < 64) sm.extra_lo[tid] = sm.extra_hi[tid] = 0.0;
-  __syncthreads();
 
-  // ---- 3. indexes, outlier lists, cluster sums, the packed stream
+  // ---- 4. indexes, cluster sums, the packed stream
   // The cluster-sum table has one column per `share` neighbouring lanes (1, 2 or 4: 2^k columns of 512 cells do not
   // fit above 16 clusters); the lanes of such a group add one after the other, so every cell sees a fixed order of
   // additions.  A weight without an index yet adds a zero to cluster 0.
   constexpr uint32_t acc_cols = (kAccCells >> BITS) < kSelThreads ? (kAccCells >> BITS) : kSelThreads;
   constexpr uint32_t share = kSelThreads / acc_cols;
   double* column = sm.u.acc + static_cast<uint32_t>(tid) / share;
-  uint32_t run_out = out_before + sm.warp_out[warp];
-  next[0] = load4(w, base, n);
-  next[1] = load4(w, base + 128u, n);
   for (uint32_t e0 = 0; e0 < part; e0 += 256u) {
     if (base - 4u * lane + e0 >= n) break;                             // the whole warp
     const float4 x[2] = {next[0], next[1]};
@@ -773,50 +889,24 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     for (int u = 0; u < 2; ++u) {
       const uint32_t i0 = base + e0 + u * 128u;
       float v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
-      uint32_t code[4], om = 0, flags = 0;
+      uint32_t code[4], flags = 0;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        code[j] = sm.binfo[bin_of(un.place(v[j]))];
-        flags |= un.inlier(v[j]) ? code[j] : kInfoBoundary;
+        code[j] = sm.binfo[un.bin(v[j])];
+        flags |= code[j];
       }
-      if ((flags & kInfoBoundary) != 0u || i0 >= n) {
-        uint32_t later = 0xfu;                                         // weights without an index yet
-        if (i0 < n) {
-          later = 0u;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (!un.inlier(v[j])) om |= 1u << j;
-            else if ((code[j] & kInfoBoundary) != 0u) later |= 1u << j;
-          }
-          for (uint32_t left = later; left != 0u; left &= left - 1u) { // one as a rule
-            const uint32_t j = static_cast<uint32_t>(__ffs(static_cast<int>(left))) - 1u;
-            const float vj = j == 0 ? v[0] : j == 1 ? v[1] : j == 2 ? v[2] : v[3];
-            const uint32_t cj = j == 0 ? code[0] : j == 1 ? code[1] : j == 2 ? code[2] : code[3];
-            const uint32_t pos = atomicAdd(&sm.seg_fill[(cj & 63u) + 1u], 1u);
-            cand[pos] = (static_cast<unsigned long long>(sort_key(vj)) << 32) | (i0 + j);
-          }
-          later |= om;
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if ((later >> j) & 1u) { code[j] = 0u; v[j] = 0.f; }
-      }
-      if (__any_sync(0xffffffffu, om != 0u)) {                         // outliers in this group of 128: in ascending offsets
-        uint32_t before = 0, total = 0;
+      if ((flags & kInfoSpecial) != 0u || i0 >= n) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const uint32_t bj = __ballot_sync(0xffffffffu, (om >> j) & 1u);
-          before += __popc(bj & lt_mask);
-          total += __popc(bj);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if ((om >> j) & 1u) {
-            const uint32_t dst = run_out + before + __popc(om & ((1u << j) - 1u));
-            if (dst < max_out) { ooff[dst] = i0 + j; oval[dst] = j == 0 ? x[u].x : j == 1 ? x[u].y : j == 2 ? x[u].z : x[u].w; }
+          const bool boundary = (code[j] & kInfoBoundary) != 0u;       // such bins hold inliers only
+          const bool later = i0 >= n || boundary || !un.inlier(v[j]);  // no index yet
+          code[j] &= 63u;
+          if (i0 < n && boundary) {
+            const uint32_t pos = sm.seg_start[code[j] + 1u] + atomicAdd(cluster.map_shared_rank(&sm.seg_count[code[j] + 1u], 0), 1u);
+            cand[pos] = (static_cast<unsigned long long>(sort_key(v[j])) << 32) | (i0 + j);
           }
+          if (later) { code[j] = 0u; v[j] = 0.f; }
         }
-        run_out += total;
       }
       packed[u] = code[0] | (code[1] << bits) | (code[2] << (2 * bits)) | (code[3] << (3 * bits));
 #pragma unroll
@@ -864,7 +954,7 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
   }
   cluster.sync();                                                      // pairs and streams are complete as well
 
-  // ---- 4. the boundary bins, a warp each: a pair's rank is the number of smaller pairs of its bin (all are distinct)
+  // ---- 5. the boundary bins, a warp each: a pair's rank is the number of smaller pairs of its bin (all are distinct)
   for (uint32_t c = 1u + warp * n_ctas + rank; c < K; c += n_warps) {       // neighbours on different SMs
     if (!owns(c)) continue;
     const uint32_t m = sm.seg_len[c], bin = sm.bnd_bin[c];
@@ -940,33 +1030,27 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     sm.cents[tid] = m;
     if (rank == 0) cent[tid] = m;
   }
-  if (rank == 0 && tid == 0) { n_out_all[unit] = n_out; marks[unit] = 0; }
+  if (rank == 0 && tid == 0) { n_out_all[unit] = sm.n_out; marks[unit] = 0; }
   __syncthreads();
 
   // an outlier's slot gets the nearest centroid's index (its bits in the stream are still zero)
-  const uint32_t my_outs = sm.cta_out[rank];
-  if (my_outs > 0) {
-    const bool listed = out_before + my_outs <= max_out;               // else the list was cut short: this CTA's part again
-    const uint32_t first = listed ? out_before : min(n, rank * kSelWarps * part);
-    const uint32_t end = listed ? out_before + my_outs : min(n, (rank + 1u) * kSelWarps * part);
-    for (uint32_t j = first + tid; j < end; j += kSelThreads) {
-      uint32_t i = j;
-      float x;
-      if (listed) { i = ooff[j]; x = oval[j]; }
-      else { x = w[j]; if (un.inlier(x)) continue; }
-      auto distance = [&](uint32_t c) { return fabs(static_cast<double>(x) - static_cast<double>(sm.cents[c])); };
-      uint32_t best = 0;
-      if (n_in >= K) {          // no empty cluster: the centroids ascend between the outliers of either side
-        if (x > un.most) for (best = K - 1u; best > 0u && distance(best - 1u) == distance(K - 1u);) --best;
-      } else {
-        for (uint32_t c = 1; c < K; ++c)
-          if (distance(c) < distance(best)) best = c;
-      }
-      const uint64_t bit = static_cast<uint64_t>(i) * bits;
-      const uint32_t sh = static_cast<uint32_t>(bit & 31u);
-      atomicOr(&codes[bit >> 5], best << sh);
-      if (sh + bits > 32u) atomicOr(&codes[(bit >> 5) + 1], best >> (32u - sh));
+  const float least = sm.least, most = sm.most;
+  const uint32_t n_mine = sm.n_tails[warp], inliers = sm.n_in;
+  for (uint32_t k = lane; k < n_mine; k += 32) {
+    const SelTail t = k < kSelTails ? sm.tails[warp][k] : tails_far(base - 4u * lane)[k];
+    if (t.value >= least && t.value <= most) continue;
+    auto distance = [&](uint32_t c) { return fabs(static_cast<double>(t.value) - static_cast<double>(sm.cents[c])); };
+    uint32_t best = 0;
+    if (inliers >= K) {          // no empty cluster: the centroids ascend between the outliers of either side
+      if (t.value > most) for (best = K - 1u; best > 0u && distance(best - 1u) == distance(K - 1u);) --best;
+    } else {
+      for (uint32_t c = 1; c < K; ++c)
+        if (distance(c) < distance(best)) best = c;
     }
+    const uint64_t bit = static_cast<uint64_t>(t.offset) * bits;
+    const uint32_t sh = static_cast<uint32_t>(bit & 31u);
+    atomicOr(&codes[bit >> 5], best << sh);
+    if (sh + bits > 32u) atomicOr(&codes[(bit >> 5) + 1], best >> (32u - sh));
   }
 }
 
@@ -975,8 +1059,8 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
 // thousand weights of each and 10 + 1.3 C per CTA for the table passes and barriers of a cluster of C (more CTAs, more
 // remote reads); on a CTA that has the SM to itself 0.84 per thousand weights and 36 + 0.5 C, with nothing to fill its
 // waits.  Summed over the waves of clusters the device holds at a time.  Fitted to calls of 1 to 384 units of 32,768 to
-// 524,288 weights, whose fastest C it picks or comes within 6 % of; e.g. 12 units of 196,608 weights at 4 bits take
-// 107 / 64 / 42 / 32 / 36 us with C = 1 / 2 / 4 / 8 / 16, 384 of 524,288 at 3 bits 627 / 627 / 625 / 786 / 1198.
+// 524,288 weights, whose fastest C it picks or comes within 4 % of; e.g. 12 units of 196,608 weights at 4 bits take
+// 93 / 59 / 40 / 32 / 36 us with C = 1 / 2 / 4 / 8 / 16, 384 of 524,288 at 3 bits 504 / 507 / 528 / 707 / 1155.
 uint32_t pick_cluster(uint32_t n_units, uint32_t n, int sm_count, const int (&resident)[5]) {
   const uint32_t steps = (n + kSelStep - 1u) / kSelStep;
   uint32_t best = 1;

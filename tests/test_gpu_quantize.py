@@ -246,3 +246,35 @@ def test_device_quantized_units_run_through_the_layer():
     with sti.Session(work_dev) as s:
         y = run_layer(s, work_dev, 0)
     assert rel_err(y, ref) <= REL_TOL
+
+
+def _guess_positions(n):
+    """Offsets of the weights that the selection looks at to place its bins: 64 groups of four spread over the unit."""
+    first = (n // 4) * np.arange(64, dtype=np.int64) // 64 * 4
+    return (first[:, None] + np.arange(4)).reshape(-1)
+
+
+@pytest.mark.parametrize("n", [1024, 24576, 100096])
+@pytest.mark.parametrize("what", ["wide", "narrow", "constant", "far", "heavy", "one_sided", "large"])
+def test_units_unlike_what_their_sample_says(what, n):
+    """The bins and the tails that are listed come from 256 weights: whatever they say, the result is the oracle's."""
+    rng = np.random.default_rng(n)
+    w = rng.normal(0, 0.02, n).astype(np.float32)
+    at = _guess_positions(n)
+    if what == "wide":              # outliers lie inside the listed tails: they are listed again
+        w[at] *= 3
+    elif what == "narrow":          # most bins are wasted on a sliver of the range, boundaries lie outside them
+        w[at] *= np.float32(0.05)
+    elif what == "constant":        # no scale at all
+        w[at] = np.float32(0.01)
+    elif what == "far":             # the mean far from zero: squares about zero cancel
+        w += np.float32(3)
+    elif what == "heavy":           # more tails than a warp's list in shared memory holds
+        heavy = rng.random(n) < 0.06
+        w[heavy] = rng.normal(0, 0.2, int(heavy.sum())).astype(np.float32)
+    elif what == "one_sided":       # outliers below the mean only: every rank is shifted
+        w[rng.random(n) < 0.01] = np.float32(-0.5)
+    elif what == "large":           # a deviation at which a tenth of a Gaussian's weights are outliers
+        w *= np.float32(300)
+    for bits in (2, 3, 5, 6):
+        _check(np.stack([w, w[::-1].copy()]), bits)

@@ -41,7 +41,7 @@ struct Tuning {
   int qkv_n = 32, f1_n = 64, o_n = 64, o_group = 4, f2_n = 64;
   int f2_group = 0;                    // FFN slices per K group of FFN2: 0 = chosen per layer and token count (pick_f2_group)
   int cta_budget = 148;                // (replaced by the device's SM count in parse_tuning) CTAs a GEMM launch may use when it splits the token tiles over CTAs
-  int wide_min_tokens = 449;           // weights decoded into the working buffer, GEMMs over it, from this many tokens on (0 = never)
+  int wide_min_tokens = -1;            // weights decoded into the working buffer, GEMMs over it: -1 = by the rule of use_wide, 0 = never, else from this many tokens on
   int f2_kacc_min_tokens = 4096;       // there, FFN2's K range in one piece (one output plane) from this many tokens on (0 = by cost)
   int wide_nt = 0, wide_splits = 0;    // there, features per tile and K splits: 0 = chosen by pick_wide
   int attn_tc_min_items = -1;          // tensor-core attention: -1 = by the rule of tc_attention, 0 = never, else from this many (sequence, kept head) pairs on, whatever their length
@@ -249,7 +249,7 @@ void parse_tuning(Tuning* t, const sti_model_desc& d, int sm_count) {
         else if (k == "o_group") t->o_group = v;
         else if (k == "f2_n") t->f2_n = v;
         else if (k == "f2_group") t->f2_group = v;
-        else if (k == "wide_min_tokens") t->wide_min_tokens = std::max(0, v);
+        else if (k == "wide_min_tokens") t->wide_min_tokens = std::max(-1, v);
         else if (k == "wide_nt") t->wide_nt = v == 128 || v == 256 ? v : 0;
         else if (k == "wide_splits") t->wide_splits = std::max(0, std::min(v, 8));
         else if (k == "f2_kacc_min_tokens") t->f2_kacc_min_tokens = std::max(0, v);
@@ -402,10 +402,19 @@ struct TableBuilder {
   }
 };
 
+// From how many tokens on a layer goes through the working buffer: the fused kernels' time grows with every 128-token tile, that
+// of the GEMMs over the buffer with every two and with the weights they fetch; a layer of BERT-large's size is ahead from
+// four tiles on, a smaller one from five (us per layer in a model / in a call by itself, fused against buffer: BERT-large 1 x 256
+// 38.6 / - against 40.5, 5 x 77 48.8 / 49.5 against 44.9 / 48.1, 4 x 128 50.1 / 50.7 against 46.1 / 49.3, 5 x 128 55.2 / 57.5
+// against 50.6 / 55.2; BERT-base 5 x 77 37.7 / 38.8 against 37.4 / 42.7, 4 x 128 37.7 / 38.9 against 38.1 / 42.7, 5 x 128
+// 41.9 / 45.2 against 40.5 / 43.2, 8 x 128 51.2 / 53.4 against 45.2 / 49.3).
+constexpr int kWideTokens = 513, kWideTokensLarge = 385;
+constexpr size_t kWideLargeWeights = 8u << 20;
+
 // Token counts are told apart in tiles of 128, and no further than where the working buffer takes over.
 int f2_tiles(const sti_plan* p, long long tokens) {
   long long most = static_cast<long long>(p->ctx->desc.max_batch) * p->ctx->desc.max_seq;
-  if (p->tune.wide_min_tokens > 0) most = std::min<long long>(most, p->tune.wide_min_tokens);
+  if (p->tune.wide_min_tokens != 0) most = std::min<long long>(most, p->tune.wide_min_tokens > 0 ? p->tune.wide_min_tokens : kWideTokens);
   return static_cast<int>((std::max(1LL, std::min(tokens, most)) + 127) / 128);
 }
 
@@ -444,8 +453,11 @@ const GemmTable& f2_table(const sti_plan* p, const Layer& L, int tokens) {
 }
 
 // Calls of many tokens: decode the layer into the working buffer, then GEMMs over it.
-bool use_wide(const sti_plan* p, long long tokens) {
-  return p->tune.wide_min_tokens > 0 && tokens >= p->tune.wide_min_tokens && !p->ctx->simt_debug;
+bool use_wide(const sti_plan* p, const Layer& L, long long tokens) {
+  if (p->tune.wide_min_tokens == 0 || p->ctx->simt_debug) return false;
+  if (p->tune.wide_min_tokens > 0) return tokens >= p->tune.wide_min_tokens;
+  const size_t weights = L.kept_heads.size() * p->ctx->attn_weights + L.kept_slices.size() * p->ctx->ffn_weights;
+  return tokens >= (weights >= kWideLargeWeights ? kWideTokensLarge : kWideTokens);
 }
 
 // Tiles of a GEMM over the working buffer.
@@ -492,7 +504,7 @@ size_t partial_rows(const sti_plan* p, const Layer& L) {
   size_t rows = 1;
   for (size_t tokens = std::min<size_t>(128, most);; tokens = std::min(tokens + 128, most)) {
     size_t planes = std::max(L.o.n_split, f2_table(p, L, static_cast<int>(tokens)).n_split);
-    if (use_wide(p, static_cast<long long>(tokens)))
+    if (use_wide(p, L, static_cast<long long>(tokens)))
       planes = std::max(pick_wide(p, tokens, L.wide[1], true).splits, pick_wide_f2(p, L, tokens).splits);
     rows = std::max(rows, tokens * std::max<size_t>(1, planes));
     if (tokens == most) return rows;
@@ -802,8 +814,7 @@ sti_status run_wide(sti_plan* p, GemmKind kind, int li, int which, const WideCho
   return STI_OK;
 }
 
-// The seven kernels of one layer on the compute stream, and from wide_min_tokens tokens on those that decode weights into the
-// working buffer.
+// The seven kernels of one layer on the compute stream, and for many tokens those that decode weights into the working buffer.
 // `expanded`: this layer's weights are there already; `beside`: the layer that is decoded beside this one's GEMMs (-1: none).
 // `x_ready_bf16`: the bf16 copy of x already sits in p->x_bf16 (written by the previous layer's LayerNorm);
 // `want_next_bf16`: this layer's last kernel also writes y as bf16 into p->x_bf16 for the next layer.
@@ -824,7 +835,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   auto stamp = [&](int kernel) -> unsigned long long* {
     return p->stamping ? p->stamps + (static_cast<size_t>(li) * kStampKernels + kernel) * kStampRecord : nullptr;
   };
-  const bool wide = use_wide(p, T);
+  const bool wide = use_wide(p, L, T);
   const WideChoice o_choice = pick_wide(p, T, L.wide[1], true), f2_choice = pick_wide_f2(p, L, T);
   CUDA_TRY(mark(0));
   if (wide && !expanded && (st = run_expand(p, li)) != STI_OK) return st;
@@ -994,7 +1005,8 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
     // the layer's first GEMM also pulls the next layer's packed shards into L2 (if they are on the device yet)
     // every matrix of the next layer is decoded beside the same one of this layer - unless that is not multiplied with here, or
     // the next layer is streamed and may not be on the device yet
-    const bool ahead = use_wide(p, static_cast<long long>(batch) * seq) && li + 1 < n && p->layers[li + 1].str_bytes == 0 &&
+    const bool ahead = li + 1 < n && use_wide(p, L, static_cast<long long>(batch) * seq) &&
+                       use_wide(p, p->layers[li + 1], static_cast<long long>(batch) * seq) && p->layers[li + 1].str_bytes == 0 &&
                        !L.kept_heads.empty() && !L.kept_slices.empty();
     sti_status st = enqueue_layer(p, li, cur, nxt, batch, seq, lens, li > 0, li + 1 < n, li + 1 < n ? li + 1 : -1, expanded,
                                   ahead ? li + 1 : -1);
@@ -1521,10 +1533,12 @@ sti_status sti_plan_finalize(sti_plan* p) {
   }
   // 4. the working buffer of plans for many tokens, activation scratch for max_batch * max_seq tokens
   const size_t Tmax = static_cast<size_t>(d.max_batch) * d.max_seq;
-  if (use_wide(p, static_cast<long long>(Tmax))) {
-    const sti_status st = ensure_wide(p);
-    if (st != STI_OK) return st;
-  }
+  for (const Layer& L : p->layers)
+    if (use_wide(p, L, static_cast<long long>(Tmax))) {
+      const sti_status st = ensure_wide(p);
+      if (st != STI_OK) return st;
+      break;
+    }
   const size_t f = d.ffn / d.n_ffn_slices;
   CUDA_TRY(cudaMalloc(&p->qkv, std::max<size_t>(1, 3 * max_heads) * Tmax * 64 * 2));
   CUDA_TRY(cudaMalloc(&p->attn_out, std::max<size_t>(1, max_heads) * Tmax * 64 * 2));
@@ -1678,7 +1692,7 @@ sti_status sti_gemm_probe(sti_plan* p, int layer, int gemm, const void* x_bf16_d
   const GemmTable* tabs[4] = {&L.qkv, &L.o, &L.f1, &f2_table(p, L, tokens)};
   const GemmTable& tab = *tabs[gemm];
   if (tab.n_jobs == 0) return STI_ERR_STATE;               // no kept unit feeds this GEMM
-  const bool wide = variant == 3 || (variant == 2 && !c->simt_debug) || (variant == 0 && use_wide(p, tokens));
+  const bool wide = variant == 3 || (variant == 2 && !c->simt_debug) || (variant == 0 && use_wide(p, L, tokens));
   const long long most = static_cast<long long>(d.max_batch) * d.max_seq;
   if (variant == 3 && (p->tune.f2_kacc_min_tokens == 0 || most < p->tune.f2_kacc_min_tokens))
     return STI_ERR_STATE;                                  // no call of this plan takes FFN2's K range in one piece

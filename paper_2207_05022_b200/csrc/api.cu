@@ -88,6 +88,7 @@ struct Layer {
   std::vector<Unit> attn, ffn;
   std::vector<int> kept_heads, kept_slices;
   size_t res_bytes = 0, str_bytes = 0;
+  size_t str_attn_bytes = 0;           // of the streamed part, the attention units (they come first)
   uint8_t* res_dev = nullptr;          // in the preload buffer
   uint8_t* str_host = nullptr;         // in the pinned arena
   int slot = -1;                       // ring slot of the streamed part
@@ -152,6 +153,7 @@ struct sti_plan {
   uint8_t* ring_alloc = nullptr; uint8_t* preload_alloc = nullptr;   // the allocations: a leading guard, then `ring` / `preload`
   uint8_t* tables = nullptr;   size_t tables_bytes = 0;       // job and task descriptors
   std::vector<cudaEvent_t> slot_free, g_slot_free;   // direct launches / graph capture
+  cudaEvent_t ev_ffn = nullptr, g_ev_ffn = nullptr;  // the last streamed layer's FFN units are loaded: direct launches / graph capture
   cudaEvent_t ev_copy_tail = nullptr, ev_begin = nullptr, ev_end = nullptr, ev_fork = nullptr, g_ev_join = nullptr;
   struct CachedGraph { ForwardKey key; cudaGraphExec_t exec = nullptr; uint64_t launches = 0; uint64_t last_use = 0; };
   std::vector<CachedGraph> graphs;     // captured forwards, a few most recently used (buffers + shape + layer)
@@ -815,11 +817,13 @@ sti_status run_wide(sti_plan* p, GemmKind kind, int li, int which, const WideCho
 }
 
 // The seven kernels of one layer on the compute stream, and for many tokens those that decode weights into the working buffer.
-// `expanded`: this layer's weights are there already; `beside`: the layer that is decoded beside this one's GEMMs (-1: none).
+// `expanded`: this layer's weights are there already; `beside`: the layer that is decoded beside this one's GEMMs (-1: none);
+// `ffn_loaded`: what the FFN units have to be waited for with, if they are still on their way.
 // `x_ready_bf16`: the bf16 copy of x already sits in p->x_bf16 (written by the previous layer's LayerNorm);
 // `want_next_bf16`: this layer's last kernel also writes y as bf16 into p->x_bf16 for the next layer.
 sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch, int seq, const int32_t* lens,
-                         bool x_ready_bf16, bool want_next_bf16, int next_layer = -1, bool expanded = false, int beside = -1) {
+                         bool x_ready_bf16, bool want_next_bf16, int next_layer = -1, bool expanded = false, int beside = -1,
+                         cudaEvent_t ffn_loaded = nullptr) {
   sti_ctx* c = p->ctx;
   const sti_model_desc& d = c->desc;
   Layer& L = p->layers[li];
@@ -897,6 +901,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   }
   CUDA_TRY(mark(4));
   const GemmTable& f2 = f2_table(p, L, T);
+  if (ffn_loaded) CUDA_TRY(cudaStreamWaitEvent(c->compute, ffn_loaded, 0));
   if (ns > 0) {
     if (wide)
       st = run_wide(p, GEMM_BF16_TO_BF16_GELU, li, 2, pick_wide(p, T, L.wide[2], false), p->h1_bf16, d.hidden, T, p->u, ns * f,
@@ -941,13 +946,14 @@ sti_status check_forward_args(sti_plan* p, const void* x, void* y, int batch, in
   return STI_OK;
 }
 
-// Copy of layer li's streamed part into its ring slot, on stream `s`.
-sti_status enqueue_layer_copy(sti_plan* p, int li, cudaStream_t s) {
+// Copy of layer li's streamed part into its ring slot, on stream `s`; or of its bytes [from, end) only.
+sti_status enqueue_layer_copy(sti_plan* p, int li, cudaStream_t s, size_t from = 0, size_t end = ~static_cast<size_t>(0)) {
   Layer& L = p->layers[li];
-  if (L.str_bytes == 0) return STI_OK;
+  end = std::min(end, L.str_bytes);
+  if (from >= end) return STI_OK;
   if (li == p->slow_copy_layer && p->slow_copy_us)      // injected slow IO: the job reaches the copy engine late
     std::this_thread::sleep_for(std::chrono::microseconds(p->slow_copy_us));
-  CUDA_TRY(cudaMemcpyAsync(p->ring + static_cast<size_t>(L.slot) * p->slot_bytes, L.str_host, L.str_bytes,
+  CUDA_TRY(cudaMemcpyAsync(p->ring + static_cast<size_t>(L.slot) * p->slot_bytes + from, L.str_host + from, end - from,
                            cudaMemcpyHostToDevice, s));
   return STI_OK;
 }
@@ -984,19 +990,32 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
     }
     CUDA_TRY(cudaStreamWaitEvent(c->compute, last, 0));
   }
+  int last_streamed = -1;
+  for (int li = 0; li < n; ++li) if (p->layers[li].str_bytes > 0) last_streamed = li;
   const void* cur = x;
   bool expanded = false;
   for (int li = 0; li < n; ++li) {
     Layer& L = p->layers[li];
+    cudaEvent_t ffn_loaded = nullptr;
     if (L.str_bytes > 0 && p->overlap) {
-      // one IO job per layer (Section 3.1); the slot is reused only after its previous layer finished
+      // One IO job per layer (Section 3.1); the slot is reused only after its previous layer finished.  The last one is copied in
+      // two pieces, so that its attention part runs while its FFN units are on their way: nothing is left to hide the layer
+      // behind.  (All layers so would cost a gap of 4 us between copies each; copies by a kernel, or by both, reach 51 GB/s
+      // where the copy engine alone reaches 55, with 4 us between its copies.)
       if (!capturing) CUDA_TRY(cudaStreamWaitEvent(c->copy, p->slot_free[L.slot], 0));
       else if (slot_used[L.slot]) CUDA_TRY(cudaStreamWaitEvent(c->copy, p->g_slot_free[L.slot], 0));
       if (prof) CUDA_TRY(cudaEventRecord(L.ev_copy_start, c->copy));
-      sti_status st = enqueue_layer_copy(p, li, c->copy);
+      const bool in_two = li == last_streamed && !prof && L.str_attn_bytes > 0 && L.str_attn_bytes < L.str_bytes &&
+                          !use_wide(p, L, static_cast<long long>(batch) * seq);
+      sti_status st = enqueue_layer_copy(p, li, c->copy, 0, in_two ? L.str_attn_bytes : L.str_bytes);
       if (st != STI_OK) return st;
       cudaEvent_t loaded = capturing ? L.g_ev_loaded : L.ev_loaded;
       CUDA_TRY(cudaEventRecord(loaded, c->copy));
+      if (in_two) {
+        if ((st = enqueue_layer_copy(p, li, c->copy, L.str_attn_bytes)) != STI_OK) return st;
+        ffn_loaded = capturing ? p->g_ev_ffn : p->ev_ffn;
+        CUDA_TRY(cudaEventRecord(ffn_loaded, c->copy));
+      }
       // a layer starts only when its own shards (and, by stream order, all earlier ones) are loaded
       CUDA_TRY(cudaStreamWaitEvent(c->compute, loaded, 0));
     }
@@ -1009,7 +1028,7 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
                        use_wide(p, p->layers[li + 1], static_cast<long long>(batch) * seq) && p->layers[li + 1].str_bytes == 0 &&
                        !L.kept_heads.empty() && !L.kept_slices.empty();
     sti_status st = enqueue_layer(p, li, cur, nxt, batch, seq, lens, li > 0, li + 1 < n, li + 1 < n ? li + 1 : -1, expanded,
-                                  ahead ? li + 1 : -1);
+                                  ahead ? li + 1 : -1, ffn_loaded);
     if (st != STI_OK) return st;
     expanded = ahead;
     if (p->retain_pending && !capturing && L.str_bytes > 0) {
@@ -1187,6 +1206,8 @@ void free_plan_device(sti_plan* p) {
   if (p->g_ev_join) cudaEventDestroy(p->g_ev_join);
   if (p->ev_copy_tail) cudaEventDestroy(p->ev_copy_tail);
   if (p->ev_fork) cudaEventDestroy(p->ev_fork);
+  if (p->ev_ffn) cudaEventDestroy(p->ev_ffn);
+  if (p->g_ev_ffn) cudaEventDestroy(p->g_ev_ffn);
   for (auto& g : p->graphs) if (g.exec) cudaGraphExecDestroy(g.exec);
   if (p->ev_begin) cudaEventDestroy(p->ev_begin);
   if (p->ev_end) cudaEventDestroy(p->ev_end);
@@ -1418,6 +1439,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
       return true;
     };
     for (auto& u : L.attn) if (!place(u)) return STI_ERR_SHARD_MISSING;
+    L.str_attn_bytes = L.str_bytes;
     for (auto& u : L.ffn) if (!place(u)) return STI_ERR_SHARD_MISSING;
     preload_total += align256(L.res_bytes);
     pinned_total += align256(L.str_bytes);
@@ -1570,6 +1592,8 @@ sti_status sti_plan_finalize(sti_plan* p) {
   }
   CUDA_TRY(cudaEventCreateWithFlags(&p->ev_copy_tail, cudaEventDisableTiming));
   CUDA_TRY(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
+  CUDA_TRY(cudaEventCreateWithFlags(&p->ev_ffn, cudaEventDisableTiming));
+  CUDA_TRY(cudaEventCreateWithFlags(&p->g_ev_ffn, cudaEventDisableTiming));
   CUDA_TRY(cudaEventCreateWithFlags(&p->g_ev_join, cudaEventDisableTiming));
   p->g_slot_free.resize(p->ring_slots);
   for (auto& e : p->g_slot_free) CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));

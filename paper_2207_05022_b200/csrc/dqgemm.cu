@@ -278,7 +278,7 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
         // one lane polls (a whole CTA's worth of pollers on one barrier word slows the MMA warp's own
         // barrier traffic down); the warp then re-converges before it touches tensor memory
         uint32_t ok = 1;
-        if (lane == 0) ok = mbar_wait_bounded_relaxed(smem_addr(&hdr->acc_full[buf]), (ti >> 1) & 1) ? 1u : 0u;
+        if (lane == 0) ok = mbar_wait_bounded(smem_addr(&hdr->acc_full[buf]), (ti >> 1) & 1) ? 1u : 0u;
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) { failed = true; break; }
         tc_fence_after_sync();

@@ -10,7 +10,9 @@
 // (n, k) at (n * K / 64 + k) * 16 KB; inside a block a feature's 64 columns are 128 bytes, their 16-byte pieces permuted by
 // the feature's number modulo 8 (the 128-byte swizzle of shared-memory operands).  A task is two pieces of 4 KB of it.
 //
-// One task per warp, no loop: 3072 tasks of a BERT-large layer are 768 CTAs of four warps, all on the device at once.
+// One task per warp, no loop: 3072 tasks of a BERT-large layer are 768 CTAs of four warps, all on the device at once.  Bound by
+// latency (descriptor, planes, unpacking, store): about 7 us for such a layer.  It runs where nothing can hide it, ahead of a
+// forward's first layer and of streamed ones; the others are decoded beside the layer before (gemm_wide.cu).
 #include "gemm_device.cuh"
 
 namespace sti {

@@ -127,6 +127,7 @@ dqgemm_kernel(const __grid_constant__ CUtensorMap xmap, const Job* __restrict__ 
   while (tmem_cols < 2 * n_rows) tmem_cols <<= 1;       // two accumulators
   if constexpr (!SIMT) {
     if (tid == 0) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&xmap)) : "memory");   // the first box does not wait for it
       for (uint32_t s = 0; s < n_stages; ++s) {
         mbar_init(smem_addr(&hdr->full[s]), 1);
         mbar_init(smem_addr(&hdr->empty[s]), 1);

@@ -420,12 +420,12 @@ quantize_units_kernel(const float* w_all, uint32_t n, int bits, uint32_t* codes_
 // That leaves 64 registers: what pass 4 does not need is kept in shared memory meanwhile, because a spilled value comes back
 // from L2 (the streamed weights push it out of the first-level cache): three of them cost a small call 1.2 of 28 us.
 //
-// Bound: with few units the chain of six cluster barriers and the table passes between them (23 of the 31 us that
+// Bound: with few units the chain of six or seven cluster barriers and the table passes between them (22 of the 30 us that
 // 12 units of 196,608 weights take at 4 bits); with many the shared-memory pipe and the latency of the chains through
 // it: pass 2 takes 11.6 cycles per 32 weights, the histogram's atomics (3.9 wavefronts each); pass 4 15.5, the table
 // lookup, the fp64 read-modify-write of the sums and the staging of the stream.  Moments, histogram and indexes as three
 // passes, with the inliers looked for in each: 384 units of 524,288 weights at 3 bits 624 -> 494 us, 200 at 4 bits 345 ->
-// 284, 40 of 100,096 at 3 bits 43.1 -> 39.5, 12 of 196,608 at 4 bits 31.5 -> 31.3.
+// 267, 384 at 6 bits 928 -> 819, 40 of 100,096 at 3 bits 43.1 -> 39.5, 12 of 196,608 at 4 bits 31.5 -> 30.4.
 
 constexpr int kSelThreads = 512;
 constexpr int kSelWarps = kSelThreads / 32;
@@ -453,7 +453,8 @@ struct SelShared {
   uint32_t bounds[65];
   uint32_t bnd_bin[64], bnd_rho[64], seg_len[64];   // of boundary c: its bin, its rank in the bin, the bin's population
   uint32_t seg_start[64];                  // where the pairs of the bin that boundary c is the first of begin
-  uint32_t seg_count[64];                  // pairs in that list so far (the first CTA's copy counts for the cluster)
+  uint32_t seg_count[64];                  // 2 and 3 bits: pairs in that list so far (the first CTA's copy counts for the cluster);
+                                           // above: the next free place of this CTA in the list
   uint32_t longest;
   float cents[64];
   alignas(16) uint8_t binfo[kSelBins];     // boundaries in lower bins (6 bits) | kInfoBoundary: holds one | kInfoSpecial: look closer
@@ -812,9 +813,16 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
   }
   __syncthreads();                                                     // this CTA's histogram has been searched
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // Where a CTA's pairs go in the cluster's lists: with few boundaries every pair asks the first CTA, which takes as long as a
+  // read of its memory; with many - a special bin in most groups of 128 weights - the CTAs before this one are asked how
+  // many weights they have in a boundary's bin, which takes another cluster barrier (us asking for every pair / ahead: 384 units of
+  // 524,288 weights at 3 bits 493 / 496, 2 of 262,144 27.2 / 29.1; 200 of 524,288 at 4 bits 284 / 267, 12 of 196,608 31.4 / 30.4; 16
+  // of 262,144 at 5 bits 53.7 / 51.8; 384 of 524,288 at 6 bits 877 / 819).
+  constexpr bool kAskAhead = BITS >= 4;
   // meanwhile: pass 4's first loads, its table, the outlier lists
   float4 next[2] = {load4(w, base, n), load4(w, base + 128u, n)};
-  for (int i = tid; i < kAccCells / 2; i += kSelThreads) reinterpret_cast<uint4*>(sm.u.acc)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if constexpr (!kAskAhead)
+    for (int i = tid; i < kAccCells / 2; i += kSelThreads) reinterpret_cast<uint4*>(sm.u.acc)[i] = make_uint4(0u, 0u, 0u, 0u);
   uint32_t run_out = out_before + sm.warp_out[warp];
   for (uint32_t k0 = 0; k0 < tails.n; k0 += 32) {
     const SelTail t = k0 + lane < tails.n ? tails.at(k0 + lane) : SelTail{0u, un.least};
@@ -842,6 +850,22 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     }
     if (lane == 0) sm.longest = longest;
   }
+  uint32_t fill = 0;                                                   // what the CTAs before this one put into boundary tid's bin
+  if constexpr (kAskAhead) {
+    if (tid >= 1 && tid < static_cast<int>(K) && owns(tid)) {
+      const uint32_t b = sm.bnd_bin[tid], holder = b / range;          // the holder's own count made way for the cluster's
+      uint32_t others = 0, t[kSelMaxCluster];
+#pragma unroll
+      for (uint32_t r = 0; r < kSelMaxCluster; ++r)                    // all in flight together
+        t[r] = r < n_ctas && r != holder ? *cluster.map_shared_rank(&sm.u.hist[b], r) : 0u;
+#pragma unroll
+      for (uint32_t r = 0; r < kSelMaxCluster; ++r) {
+        others += t[r];
+        if (r < rank) fill += t[r];
+      }
+      if (holder < rank) fill += sm.seg_len[tid] - others;
+    }
+  }
   for (uint32_t i = tid; i < n_bins / 16; i += kSelThreads) {          // sixteen bins a thread
     uint32_t below = 0, packed[4];                                     // boundaries 1 .. below sit in lower bins (their bins ascend)
 #pragma unroll
@@ -866,10 +890,16 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     }
     reinterpret_cast<uint4*>(sm.binfo)[i] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
   }
-  __syncthreads();
+  if constexpr (kAskAhead) cluster.sync();                             // nobody looks at another CTA's histogram any more
+  else __syncthreads();
   if (sm.longest > static_cast<uint32_t>(kSelMaxSeg)) {
     if (rank == 0 && tid == 0) marks[unit] = 1;
     return;
+  }
+  if constexpr (kAskAhead) {
+    if (tid < static_cast<int>(K)) sm.seg_count[tid] = sm.seg_start[tid] + fill;
+    for (int i = tid; i < kAccCells / 2; i += kSelThreads) reinterpret_cast<uint4*>(sm.u.acc)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
   }
 
   // ---- 4. indexes, cluster sums, the packed stream
@@ -902,7 +932,9 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
           const bool later = i0 >= n || boundary || !un.inlier(v[j]);  // no index yet
           code[j] &= 63u;
           if (i0 < n && boundary) {
-            const uint32_t pos = sm.seg_start[code[j] + 1u] + atomicAdd(cluster.map_shared_rank(&sm.seg_count[code[j] + 1u], 0), 1u);
+            uint32_t pos;
+            if constexpr (kAskAhead) pos = atomicAdd(&sm.seg_count[code[j] + 1u], 1u);
+            else pos = sm.seg_start[code[j] + 1u] + atomicAdd(cluster.map_shared_rank(&sm.seg_count[code[j] + 1u], 0), 1u);
             cand[pos] = (static_cast<unsigned long long>(sort_key(v[j])) << 32) | (i0 + j);
           }
           if (later) { code[j] = 0u; v[j] = 0.f; }

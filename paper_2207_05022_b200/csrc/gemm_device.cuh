@@ -375,17 +375,17 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
 // below 1.5e-7, three orders of magnitude under the bf16 rounding of the result) with the hardware
 // exponential; the epilogue runs it for every element of the FFN1 output.
 // With t = 1 / (1 + p |v| / sqrt 2) and q(t) the polynomial:  gelu(v) = max(v, 0) - |v| t q(t) / 2 exp(-v^2 / 2).
-// All but the special functions work on pairs, and a pair shares one reciprocal: three special functions for two values (the
-// unit takes 16 lanes a cycle, so a 128 x 256 tile's GELU is 3072 cycles of it).
+// All but the two special functions work on pairs (their unit takes 16 lanes a cycle, so a 128 x 256 tile's GELU is 4096 cycles of
+// it; one reciprocal for a pair took FFN1 no less time, and other bits).
 __device__ __forceinline__ uint64_t gelu_erf_x2(uint64_t v) {
   const auto both = [](float c) { return pack_f32x2(c, c); };
-  float d0, d1, r, e0, e1, v0, v1;
+  float d0, d1, t0, t1, e0, e1, v0, v1;
   unpack_f32x2(v, v0, v1);
   const uint64_t abs_v = pack_f32x2(fminf(fabsf(v0), 1e30f), fminf(fabsf(v1), 1e30f));     // finite: t is 0 for an infinite v
   unpack_f32x2(fma_f32x2(abs_v, both(0.3275911f * 0.70710678118654752440f), both(1.0f)), d0, d1);
-  // one reciprocal for both: 1 / d0 = d1 / (d0 d1).  A product that overflows gives t = 0 where |v| > 1e8, and 2^(-v^2..) is 0 there.
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d0 * d1));
-  const uint64_t t = mul_f32x2(pack_f32x2(d1, d0), pack_f32x2(r, r));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t0) : "f"(d0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t1) : "f"(d1));
+  const uint64_t t = pack_f32x2(t0, t1);
   uint64_t q = fma_f32x2(t, both(0.5f * 1.061405429f), both(0.5f * -1.453152027f));
   q = fma_f32x2(q, t, both(0.5f * 1.421413741f));
   q = fma_f32x2(q, t, both(0.5f * -0.284496736f));

@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB_NAME = "libsti_b200.so"
 LIB_PATH = os.path.join(HERE, LIB_NAME)
 SOURCES = ["api.cu", "dqgemm.cu", "expand.cu", "gemm_wide.cu", "attention.cu", "attention_tc.cu", "layernorm.cu", "decode.cu", "noalloc.cu", "planner.cu", "quantize.cu"]
-HEADERS = ["sti_kernels.h", "sti_device.cuh", "gemm_device.cuh", "retile.h", "host_device.h", "outlier_range.h", "decode_task.h", os.path.join("..", "..", "include", "sti.h"),
+HEADERS = ["sti_kernels.h", "sti_device.cuh", "gemm_device.cuh", "retile.h", "host_device.h", "outlier_range.h", "decode_task.h", "tiling.h", os.path.join("..", "..", "include", "sti.h"),
            os.path.join("..", "..", "include", "sti_planner.h"),
            os.path.join("..", "..", "include", "sti_quantize.h")]
 NVCC_FLAGS = [

@@ -15,6 +15,7 @@
 #include "../../include/sti.h"
 #include "retile.h"
 #include "sti_kernels.h"
+#include "tiling.h"
 
 using namespace sti;
 
@@ -35,16 +36,6 @@ inline size_t align256(size_t v) { return (v + 255) & ~static_cast<size_t>(255);
 struct MatrixInfo {
   uint32_t rows, kc;
   uint32_t flat_base;   // first weight's flat offset in the unit
-};
-
-struct Tuning {
-  int qkv_n = 32, f1_n = 64, o_n = 64, o_group = 4, f2_n = 64;
-  int f2_group = 0;                    // FFN slices per K group of FFN2: 0 = chosen per layer and token count (pick_f2_group)
-  int cta_budget = 148;                // (replaced by the device's SM count in parse_tuning) CTAs a GEMM launch may use when it splits the token tiles over CTAs
-  int wide_min_tokens = -1;            // weights decoded into the working buffer, GEMMs over it: -1 = by the rule of use_wide, 0 = never, else from this many tokens on
-  int f2_kacc_min_tokens = 4096;       // there, FFN2's K range in one piece (one output plane) from this many tokens on (0 = by cost)
-  int wide_nt = 0, wide_splits = 0;    // there, features per tile and K splits: 0 = chosen by pick_wide
-  int attn_tc_min_items = -1;          // tensor-core attention: -1 = by the rule of tc_attention, 0 = never, else from this many (sequence, kept head) pairs on, whatever their length
 };
 
 struct Unit {
@@ -76,12 +67,6 @@ struct GemmTable {
   uint32_t w_bytes = 0, n_stages = 0, bps = 1, hdr_bytes = 0, task_stride = 0;
   int n_split = 0;
   int group = 0;                       // FFN2: slices per K group
-};
-
-// One of a layer's weight matrices in the working buffer (expand.cu).
-struct WideMatrix {
-  uint32_t row0 = 0;                   // first 128-byte row
-  uint32_t n = 0, k_chunks = 0;        // features, chunks of 64 columns
 };
 
 struct Layer {
@@ -146,7 +131,7 @@ struct sti_plan {
   bool finalized = false;
   bool attempted = false;
   int profiling = 0;                   // 0 off, 1 per layer, 2 per kernel
-  Tuning tune;
+  Tiling tiling;
   uint8_t* preload = nullptr;  size_t preload_bytes = 0;
   uint8_t* pinned = nullptr;   size_t pinned_bytes = 0;
   uint8_t* ring = nullptr;     size_t slot_bytes = 0;      // a slot = its data followed by kGuardBytes of guard pattern
@@ -161,7 +146,8 @@ struct sti_plan {
   bool graph_off = false;
   bool copy_tail_valid = false;
   // activation scratch
-  uint16_t* qkv = nullptr; uint16_t* attn_out = nullptr; float* partial = nullptr;
+  uint16_t* qkv = nullptr; uint16_t* attn_out = nullptr;
+  float* partial = nullptr;    size_t partial_rows = 1;     // planes of partial sums, rows of `hidden`
   float* h1_f32 = nullptr; uint16_t* h1_bf16 = nullptr; uint16_t* u = nullptr;
   uint16_t* x_bf16 = nullptr;          // bf16 copy of fp32 layer inputs (the GEMM operand)
   void* buf[2] = {nullptr, nullptr};
@@ -208,12 +194,6 @@ const MatrixInfo* unit_matrices(const sti_ctx* c, sti_kind kind, int* n) {
 
 size_t matrix_code_bytes(const MatrixInfo& m, int bits) {
   return static_cast<size_t>(m.rows) * m.kc * bits / 8;
-}
-
-// Whether a weight tile of n rows x k columns leaves room for a ring of four boxes.
-bool tile_fits(int n, int k) {
-  uint32_t st = 0, bp = 0;
-  return gemm_pick_ring(static_cast<uint32_t>(gemm_weight_bytes(n, k)), k, gemm_header_bytes(), &st, &bp) && st * bp >= 4;
 }
 
 // A K range of `n` units in as few groups as `most` units per group allow, the groups equal up to one unit: {first, count}.
@@ -274,11 +254,10 @@ void parse_tuning(Tuning* t, const sti_model_desc& d, int sm_count) {
   t->o_group = std::max(1, std::min(t->o_group, 16));
   t->f2_group = std::max(0, std::min(t->f2_group, 16));
   // keep every weight tile inside shared memory
-  const auto fits = tile_fits;
-  while (t->qkv_n > 32 && !fits(t->qkv_n, d.hidden)) t->qkv_n /= 2;
-  while (t->f1_n > 32 && !fits(t->f1_n, d.hidden)) t->f1_n /= 2;
-  while (t->o_group > 1 && !fits(t->o_n, t->o_group * 64)) --t->o_group;
-  while (t->f2_group > 1 && !fits(t->f2_n, t->f2_group * f)) --t->f2_group;
+  while (t->qkv_n > 32 && !tile_fits(t->qkv_n, d.hidden)) t->qkv_n /= 2;
+  while (t->f1_n > 32 && !tile_fits(t->f1_n, d.hidden)) t->f1_n /= 2;
+  while (t->o_group > 1 && !tile_fits(t->o_n, t->o_group * 64)) --t->o_group;
+  while (t->f2_group > 1 && !tile_fits(t->f2_n, t->f2_group * f)) --t->f2_group;
 }
 
 Unit* find_unit(sti_plan* p, int layer, sti_kind kind, int index) {
@@ -404,117 +383,15 @@ struct TableBuilder {
   }
 };
 
-// From how many tokens on a layer goes through the working buffer: the fused kernels' time grows with every 128-token tile, that
-// of the GEMMs over the buffer with every two and with the weights they fetch; a layer of BERT-large's size is ahead from
-// four tiles on, a smaller one from five (us per layer in a model / in a call by itself, fused against buffer: BERT-large 1 x 256
-// 38.6 / - against 40.5, 5 x 77 48.8 / 49.5 against 44.9 / 48.1, 4 x 128 50.1 / 50.7 against 46.1 / 49.3, 5 x 128 55.2 / 57.5
-// against 50.6 / 55.2; BERT-base 5 x 77 37.7 / 38.8 against 37.4 / 42.7, 4 x 128 37.7 / 38.9 against 38.1 / 42.7, 5 x 128
-// 41.9 / 45.2 against 40.5 / 43.2, 8 x 128 51.2 / 53.4 against 45.2 / 49.3).
-constexpr int kWideTokens = 513, kWideTokensLarge = 385;
-constexpr size_t kWideLargeWeights = 8u << 20;
-
-// Token counts are told apart in tiles of 128, and no further than where the working buffer takes over.
-int f2_tiles(const sti_plan* p, long long tokens) {
-  long long most = static_cast<long long>(p->ctx->desc.max_batch) * p->ctx->desc.max_seq;
-  if (p->tune.wide_min_tokens != 0) most = std::min<long long>(most, p->tune.wide_min_tokens > 0 ? p->tune.wide_min_tokens : kWideTokens);
-  return static_cast<int>((std::max(1LL, std::min(tokens, most)) + 127) / 128);
-}
-
-// FFN slices per K group of FFN2 in a layer that keeps `ns` of them, for calls of `n_mtiles` token tiles.  More slices per group:
-// fewer fp32 planes written and read back by the LayerNorm (8 bytes per element at 5 TB/s), but a longer MMA chain per CTA
-// (0.7 us per 256 columns and 128-token tile) and a longer decode, of which
-// other kernels leave about 1.4 us per 256 columns in the open; and a launch that fills every SM delays its neighbours (1 us).
-// Groups of more than 1024 columns leave the ring too little: five slices of 256 took 57.0 -> 61.6 us (a BERT-base layer of
-// 9 slices, 1536 tokens).  Fitted to 91 timings with 1 to 6 slices per group, 6 to 16 slices kept, 64 to 4000 tokens: its choice
-// is 0.5 % above the best one in the mean, 4.2 % at most (us per layer with 2 / 3 / 4 slices: BERT-large, 16 slices, 256 tokens
-// 38.6 / 37.2 / 38.7, 1024 68.4 / 69.2 / 64.1; 12 slices, 256 tokens 35.0 / 37.0 / 36.0; BERT-base, 128 tokens 27.3 / 27.7 / 28.3).
-int pick_f2_group(const sti_plan* p, int ns, int n_mtiles) {
-  const sti_model_desc& d = p->ctx->desc;
-  const Tuning& t = p->tune;
-  if (t.f2_group > 0) return t.f2_group;
-  const int f = d.ffn / d.n_ffn_slices;
-  int best = 1;                        // also where no more than one slice fits in shared memory
-  double best_cost = -1.0;
-  for (int g = std::max(1, std::min(2, ns)); g <= ns; ++g) {
-    if (g > 1 && (g * f > 1024 || !tile_fits(t.f2_n, g * f))) break;
-    const int planes = (ns + g - 1) / g, widest = (ns + planes - 1) / planes, jobs = planes * (d.hidden / t.f2_n);
-    const int m_ctas = std::max(1, std::min(n_mtiles, t.cta_budget / jobs)), tiles = (n_mtiles + m_ctas - 1) / m_ctas;
-    const double filled = static_cast<double>(jobs) * m_ctas / t.cta_budget;
-    const double cost = std::max(1.0, filled) * widest * (f / 256.0) * (tiles * 0.7 + 1.4) +
-                        planes * 128.0 * n_mtiles * d.hidden * 8.0 / 5.0e6 + std::min(1.0, filled);
-    if (best_cost < 0.0 || cost < best_cost) { best = g; best_cost = cost; }
-  }
-  return best;
-}
-
 // The layer's FFN2 table for a call of `tokens` tokens: chosen by the call, not by what the context could take.
 const GemmTable& f2_table(const sti_plan* p, const Layer& L, int tokens) {
-  const int g = pick_f2_group(p, static_cast<int>(L.kept_slices.size()), f2_tiles(p, tokens));
+  const int g = pick_f2_group(p->tiling, static_cast<int>(L.kept_slices.size()), f2_tiles(p->tiling, tokens));
   for (const GemmTable& t : L.f2) if (t.group == g) return t;
   return L.f2.back();
 }
 
-// Calls of many tokens: decode the layer into the working buffer, then GEMMs over it.
 bool use_wide(const sti_plan* p, const Layer& L, long long tokens) {
-  if (p->tune.wide_min_tokens == 0 || p->ctx->simt_debug) return false;
-  if (p->tune.wide_min_tokens > 0) return tokens >= p->tune.wide_min_tokens;
-  const size_t weights = L.kept_heads.size() * p->ctx->attn_weights + L.kept_slices.size() * p->ctx->ffn_weights;
-  return tokens >= (weights >= kWideLargeWeights ? kWideTokensLarge : kWideTokens);
-}
-
-// Tiles of a GEMM over the working buffer: cycles of the chunks of every wave, of the last tile's epilogue and of the fp32 planes
-// that K splits add (written, and read by the LayerNorm).  Fitted to 22 shapes of 256 to 4096 tokens, both models, one to four splits;
-// within 2 % of the best of them (us per BERT-large layer with 256-wide tiles and 1 / 2 / 3 / 4 splits: 1024 tokens 69.1 / 59.5 / 57.4 /
-// 56.4, picked 57.2; 2048 tokens 83.9 / 75.2 / 82.1 / 81.1, picked 74.4; with 128-wide ones 64.2 / 58.2 / 62.1 / 61.2 and 82.3 / 85.5 /
-// 88.9 / 92.3; 512 tokens, 128 wide, 59.5 / 52.3 / 49.8 / 49.7, picked 51.1).
-struct WideChoice { uint32_t nt, splits, clusters; };
-WideChoice pick_wide(const sti_plan* p, long long tokens, const WideMatrix& m, bool may_split) {
-  const Tuning& t = p->tune;
-  const uint32_t pairs = static_cast<uint32_t>((tokens + 255) / 256), held = std::max(1, t.cta_budget / 2);
-  WideChoice best{256, 1, 1};
-  double best_cost = -1.0;
-  for (uint32_t nt = 256; nt >= 128; nt /= 2) {
-    if (t.wide_nt > 0 && nt != static_cast<uint32_t>(t.wide_nt)) continue;
-    for (uint32_t splits = 1; splits <= (may_split ? 4u : 1u) && splits <= m.k_chunks; ++splits) {
-      if (may_split && t.wide_splits > 0 && splits != std::min(static_cast<uint32_t>(t.wide_splits), m.k_chunks)) continue;
-      const uint32_t tiles = pairs * ((m.n + nt - 1) / nt) * splits, waves = (tiles + held - 1) / held;
-      const double cost = waves * ((m.k_chunks + splits - 1) / splits * (nt == 256 ? 540.0 : 400.0) + 500.0) + (nt == 256 ? 1500.0 : 1000.0) +
-                          (splits - 1) * 8.0 * tokens * m.n / 2500.0;
-      if (best_cost < 0.0 || cost < best_cost) { best = {nt, splits, std::min(tiles, held)}; best_cost = cost; }
-    }
-  }
-  return best;
-}
-// FFN2 and the O projection write fp32 planes, one per K split.
-WideChoice pick_wide_f2(const sti_plan* p, const Layer& L, long long tokens) {
-  return pick_wide(p, tokens, L.wide[3], !(p->tune.f2_kacc_min_tokens > 0 && tokens >= p->tune.f2_kacc_min_tokens));
-}
-
-// Sizes and places of a layer's matrices in its working buffer; its bytes.
-size_t place_wide(const sti_ctx* c, Layer& L) {
-  const uint32_t d = c->desc.hidden, f = c->desc.ffn / c->desc.n_ffn_slices;
-  const uint32_t nh = static_cast<uint32_t>(L.kept_heads.size()), ns = static_cast<uint32_t>(L.kept_slices.size());
-  const uint32_t n[4] = {192 * nh, d, f * ns, d}, k[4] = {d, 64 * nh, d, f * ns};
-  uint32_t row = 0;
-  for (int m = 0; m < 4; ++m) {
-    L.wide[m] = {row, n[m], k[m] / 64};
-    row += (n[m] + 255) / 256 * 256 * (k[m] / 64);       // whole tiles of 256 features
-  }
-  return static_cast<size_t>(row) * 128;
-}
-
-// How many fp32 [tokens][hidden] planes' worth of partial sums a forward of this layer needs at most, in rows.
-size_t partial_rows(const sti_plan* p, const Layer& L) {
-  const sti_model_desc& d = p->ctx->desc;
-  const size_t most = static_cast<size_t>(d.max_batch) * d.max_seq;
-  size_t rows = 1;
-  for (size_t tokens = std::min<size_t>(128, most);; tokens = std::min(tokens + 128, most)) {
-    size_t planes = std::max(L.o.n_split, f2_table(p, L, static_cast<int>(tokens)).n_split);
-    if (use_wide(p, L, static_cast<long long>(tokens)))
-      planes = std::max(pick_wide(p, tokens, L.wide[1], true).splits, pick_wide_f2(p, L, tokens).splits);
-    rows = std::max(rows, tokens * std::max<size_t>(1, planes));
-    if (tokens == most) return rows;
-  }
+  return use_wide(p->tiling, static_cast<int>(L.kept_heads.size()), static_cast<int>(L.kept_slices.size()), tokens);
 }
 
 struct LayerTables {
@@ -524,7 +401,7 @@ struct LayerTables {
 void build_layer_tables(sti_plan* p, Layer& L, LayerTables& tb) {
   const sti_ctx* c = p->ctx;
   const sti_model_desc& d = c->desc;
-  const Tuning& t = p->tune;
+  const Tuning& t = p->tiling.tune;
   const uint32_t f = d.ffn / d.n_ffn_slices;
   // QKV: one job per (kept head, matrix, row tile); full K
   for (size_t hi = 0; hi < L.kept_heads.size(); ++hi) {
@@ -567,9 +444,9 @@ void build_layer_tables(sti_plan* p, Layer& L, LayerTables& tb) {
   }
   // FFN2: K split over groups of kept slices, in every way that a call of some size takes
   const int ns = static_cast<int>(L.kept_slices.size());
-  const int most_tiles = f2_tiles(p, static_cast<long long>(d.max_batch) * d.max_seq);
+  const int most_tiles = f2_tiles(p->tiling, p->tiling.max_tokens);
   for (int tiles = 1; tiles <= most_tiles; ++tiles) {
-    const int group = pick_f2_group(p, ns, tiles);
+    const int group = pick_f2_group(p->tiling, ns, tiles);
     if (std::any_of(L.f2.begin(), L.f2.end(), [&](const GemmTable& have) { return have.group == group; })) continue;
     const auto f2_groups = split_units(ns, group);
     L.f2.emplace_back();
@@ -611,8 +488,7 @@ sti_status ensure_wide(sti_plan* p) {
   bool in_bounds = true;
   for (size_t li = 0; li < p->layers.size(); ++li) {
     Layer& L = p->layers[li];
-    const size_t bytes = place_wide(c, L);
-    most = std::max(most, bytes);
+    most = std::max(most, static_cast<size_t>(place_wide(p->tiling, static_cast<int>(L.kept_heads.size()), static_cast<int>(L.kept_slices.size()), L.wide)) * 128);
     tasks.resize(L.wide_first[4]);
     uint32_t filled[4] = {L.wide_first[0], L.wide_first[1], L.wide_first[2], L.wide_first[3]};
     // rows [first, first + rows) of the unit's matrix `um` are features n0 .. of layer matrix `m`, from column chunk kc0 on
@@ -730,7 +606,7 @@ bool make_omap(CUtensorMap* map, void* base, bool f32, int cols, int rows, uint3
 // 32 x 100 10.8 / 11.5; but 8 x 128 5.5 / 4.7, 2 x 512 16.6 / 11.3, 32 x 64 8.0 / 4.7;
 // between 65 and 96 keys they are level).
 bool tc_attention(const sti_plan* p, int nh, int batch, int seq) {
-  const int min_items = p->tune.attn_tc_min_items;
+  const int min_items = p->tiling.tune.attn_tc_min_items;
   if (min_items == 0 || p->ctx->simt_debug) return false;
   if (min_items > 0) return batch * nh >= min_items;
   return seq > 96 && (seq + 127) / 128 * batch * nh > p->ctx->sm_count;
@@ -763,7 +639,7 @@ sti_status run_gemm(sti_plan* p, GemmKind kind, const GemmTable& tab, const void
   if (tab.n_jobs == 0) return STI_OK;
   GemmLaunch g{};
   g.stamps = stamps;
-  g.jobs = tab.jobs; g.tasks = tab.tasks; g.n_jobs = tab.n_jobs; g.m_ctas = m_ctas_for(tab.n_jobs, T, p->tune.cta_budget);
+  g.jobs = tab.jobs; g.tasks = tab.tasks; g.n_jobs = tab.n_jobs; g.m_ctas = m_ctas_for(tab.n_jobs, T, p->tiling.tune.cta_budget);
   if (!make_xmap(&g.xmap, x, ldx, T)) return STI_ERR_CUDA;
   layer_ranges(p, prefetch_layer, g.pf_ptr, g.pf_bytes);
   g.x = x; g.ldx = ldx; g.T = T; g.out = out; g.ldo = ldo; g.bias = bias; g.err = p->ctx->err_dev;
@@ -807,7 +683,7 @@ sti_status run_wide(sti_plan* p, GemmKind kind, int li, int which, const WideCho
   g.nt = choice.nt; g.clusters = choice.clusters; g.weights_ready = weights_ready;
   if (beside >= 0) {
     g.beside = expand_job(p, beside, which, which + 1);
-    if (g.beside.n_tasks > 0) g.clusters = std::max(1, p->tune.cta_budget / 2);      // also where no tile is left to multiply
+    if (g.beside.n_tasks > 0) g.clusters = std::max(1, p->tiling.tune.cta_budget / 2);      // also where no tile is left to multiply
   }
   if (!make_xmap(&g.xmap, x, ldx, T) ||
       !make_xmap(&g.wmap, p->wide_buf, 64, static_cast<int>(2 * p->wide_bytes / 128), choice.nt / 2, false) ||
@@ -844,7 +720,11 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     return p->stamping ? p->stamps + (static_cast<size_t>(li) * kStampKernels + kernel) * kStampRecord : nullptr;
   };
   const bool wide = use_wide(p, L, T);
-  const WideChoice o_choice = pick_wide(p, T, L.wide[1], true), f2_choice = pick_wide_f2(p, L, T);
+  const WideChoice o_choice = pick_wide(p->tiling, T, L.wide[1], true), f2_choice = pick_wide_f2(p->tiling, T, L.wide[3]);
+  const GemmTable& f2 = f2_table(p, L, T);
+  const int o_planes = nh > 0 ? (wide ? static_cast<int>(o_choice.splits) : L.o.n_split) : 0;
+  const int f2_planes = ns > 0 ? (wide ? static_cast<int>(f2_choice.splits) : f2.n_split) : 0;
+  if (static_cast<size_t>(T) * std::max(o_planes, f2_planes) > p->partial_rows) return STI_ERR_STATE;      // not for any call: partial_rows
   CUDA_TRY(mark(0));
   if (wide && !expanded && (st = run_expand(p, li)) != STI_OK) return st;
   if (nh > 0) {
@@ -859,7 +739,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
       xq = p->x_bf16;
     }
     if (wide)
-      st = run_wide(p, GEMM_BF16_TO_BF16, li, 0, pick_wide(p, T, L.wide[0], false), xq, d.hidden, T, p->qkv, 64, dense + c->off_bq,
+      st = run_wide(p, GEMM_BF16_TO_BF16, li, 0, pick_wide(p->tiling, T, L.wide[0], false), xq, d.hidden, T, p->qkv, 64, dense + c->off_bq,
                     expanded, beside, stamp(1));
     else
       st = run_gemm(p, GEMM_BF16_TO_BF16, L.qkv, xq, d.hidden, T, p->qkv, 64, dense + c->off_bq, next_layer, stamp(1));
@@ -871,7 +751,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
       CUDA_TRY(launch_attention_tc(qmap, omap, p->attn_out, nh, batch, seq, lens, c->err_dev, c->compute, c->pdl, stamp(2)));
     } else {
       CUDA_TRY(launch_attention(p->qkv, p->attn_out, nh, batch, seq, lens, c->sm_count,
-                                wide ? static_cast<int>(2 * o_choice.clusters) : L.o.n_jobs * m_ctas_for(L.o.n_jobs, T, p->tune.cta_budget),
+                                wide ? static_cast<int>(2 * o_choice.clusters) : L.o.n_jobs * m_ctas_for(L.o.n_jobs, T, p->tiling.tune.cta_budget),
                                 c->compute, c->pdl, stamp(2)));
     }
     c->launches++;
@@ -892,7 +772,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   const int drop_planes = static_cast<size_t>(T) * d.hidden * 4 >= (32u << 20);
   {
     LnLaunch ln{};
-    ln.partial = p->partial; ln.n_partial = nh > 0 ? (wide ? static_cast<int>(o_choice.splits) : L.o.n_split) : 0;
+    ln.partial = p->partial; ln.n_partial = o_planes;
     ln.bias = dense + c->off_bo; ln.resid = x; ln.resid_bf16 = bf16_act ? 1 : 0;
     ln.gamma = dense + c->off_ln1g; ln.beta = dense + c->off_ln1b; ln.eps = d.ln_eps; ln.T = T; ln.d = d.hidden;
     // With bf16 activations every activation that crosses a kernel boundary is bf16 (the layer's input and output are):
@@ -904,11 +784,10 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     L.k_ran[3] = true;
   }
   CUDA_TRY(mark(4));
-  const GemmTable& f2 = f2_table(p, L, T);
   if (ffn_loaded) CUDA_TRY(cudaStreamWaitEvent(c->compute, ffn_loaded, 0));
   if (ns > 0) {
     if (wide)
-      st = run_wide(p, GEMM_BF16_TO_BF16_GELU, li, 2, pick_wide(p, T, L.wide[2], false), p->h1_bf16, d.hidden, T, p->u, ns * f,
+      st = run_wide(p, GEMM_BF16_TO_BF16_GELU, li, 2, pick_wide(p->tiling, T, L.wide[2], false), p->h1_bf16, d.hidden, T, p->u, ns * f,
                     dense + c->off_b1, expanded || nh > 0, beside, stamp(5));
     else
       st = run_gemm(p, GEMM_BF16_TO_BF16_GELU, L.f1, p->h1_bf16, d.hidden, T, p->u, ns * f, dense + c->off_b1, -1, stamp(5));
@@ -925,7 +804,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   }
   CUDA_TRY(mark(6));
   LnLaunch l2{};
-  l2.partial = p->partial; l2.n_partial = ns > 0 ? (wide ? static_cast<int>(f2_choice.splits) : f2.n_split) : 0;
+  l2.partial = p->partial; l2.n_partial = f2_planes;
   l2.bias = dense + c->off_b2;
   l2.resid = bf16_act ? static_cast<const void*>(p->h1_bf16) : static_cast<const void*>(p->h1_f32);
   l2.resid_bf16 = bf16_act ? 1 : 0;
@@ -1363,7 +1242,11 @@ sti_status sti_plan_create(sti_ctx* c, const sti_shard_cfg* attn, const sti_shar
       if (L.ffn[s].cfg.keep) L.kept_slices.push_back(s);
     }
   }
-  parse_tuning(&p->tune, d, c->sm_count);
+  p->tiling.hidden = d.hidden; p->tiling.slice = d.ffn / d.n_ffn_slices;
+  p->tiling.attn_weights = c->attn_weights; p->tiling.ffn_weights = c->ffn_weights;
+  p->tiling.max_tokens = static_cast<long long>(d.max_batch) * d.max_seq;
+  p->tiling.fused_only = c->simt_debug;
+  parse_tuning(&p->tiling.tune, d, c->sm_count);
   *out = p;
   return STI_OK;
 }
@@ -1514,10 +1397,10 @@ sti_status sti_plan_finalize(sti_plan* p) {
   std::vector<uint8_t> host_tables;
   struct Fix { GemmTable* t; size_t jobs_off, tasks_off; };
   std::vector<Fix> fixes;
-  size_t most_partial_rows = 1;
   for (auto& L : p->layers) {
     LayerTables tb;
-    (void)place_wide(c, L);
+    const int heads = static_cast<int>(L.kept_heads.size()), slices = static_cast<int>(L.kept_slices.size());
+    (void)place_wide(p->tiling, heads, slices, L.wide);
     L.tables_off = align16(host_tables.size());
     build_layer_tables(p, L, tb);
     auto place = [&](GemmTable& gt, TableBuilder& b) -> sti_status {
@@ -1527,7 +1410,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
       gt.n_jobs = static_cast<int>(b.jobs.size());
       gt.w_bytes = b.w_bytes;
       gt.n_stages = 2; gt.bps = 1;
-      gt.hdr_bytes = gemm_header_bytes();
+      gt.hdr_bytes = kHeaderBytes;
       if (!b.jobs.empty() && !gemm_pick_ring(b.w_bytes, b.k_max, gt.hdr_bytes, &gt.n_stages, &gt.bps)) return STI_ERR_SHAPE;
       gt.smem = gemm_smem_bytes(b.w_bytes, gt.n_stages, gt.bps, gt.hdr_bytes);
       if (gt.smem > kMaxSmem && !b.jobs.empty()) return STI_ERR_SHAPE;
@@ -1547,7 +1430,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
     for (size_t i = 0; i < L.f2.size() && st == STI_OK; ++i) st = place(L.f2[i], tb.f2[i]);
     if (st != STI_OK) return st;
     L.tables_bytes = host_tables.size() - L.tables_off;
-    most_partial_rows = std::max(most_partial_rows, partial_rows(p, L));
+    p->partial_rows = std::max(p->partial_rows, partial_rows(p->tiling, heads, slices));
   }
   p->tables_bytes = std::max<size_t>(host_tables.size(), 16);
   CUDA_TRY(cudaMalloc(&p->tables, p->tables_bytes));
@@ -1568,7 +1451,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
   const size_t f = d.ffn / d.n_ffn_slices;
   CUDA_TRY(cudaMalloc(&p->qkv, std::max<size_t>(1, 3 * max_heads) * Tmax * 64 * 2));
   CUDA_TRY(cudaMalloc(&p->attn_out, std::max<size_t>(1, max_heads) * Tmax * 64 * 2));
-  CUDA_TRY(cudaMalloc(&p->partial, most_partial_rows * d.hidden * 4));
+  CUDA_TRY(cudaMalloc(&p->partial, p->partial_rows * d.hidden * 4));
   CUDA_TRY(cudaMalloc(&p->h1_f32, Tmax * d.hidden * 4));
   CUDA_TRY(cudaMalloc(&p->h1_bf16, Tmax * d.hidden * 2));
   CUDA_TRY(cudaMalloc(&p->u, std::max<size_t>(1, max_slices) * Tmax * f * 2));
@@ -1721,12 +1604,12 @@ sti_status sti_gemm_probe(sti_plan* p, int layer, int gemm, const void* x_bf16_d
   const GemmTable& tab = *tabs[gemm];
   if (tab.n_jobs == 0) return STI_ERR_STATE;               // no kept unit feeds this GEMM
   const bool wide = variant == 3 || (variant == 2 && !c->simt_debug) || (variant == 0 && use_wide(p, L, tokens));
-  const long long most = static_cast<long long>(d.max_batch) * d.max_seq;
-  if (variant == 3 && (p->tune.f2_kacc_min_tokens == 0 || most < p->tune.f2_kacc_min_tokens))
+  if (variant == 3 && (p->tiling.tune.f2_kacc_min_tokens == 0 || whole_tiles(p->tiling.max_tokens) < p->tiling.tune.f2_kacc_min_tokens))
     return STI_ERR_STATE;                                  // no call of this plan takes FFN2's K range in one piece
   const bool sums = gemm == 1 || gemm == 3;
-  const WideChoice choice = variant == 3 ? pick_wide(p, tokens, L.wide[3], false)
-                                         : (gemm == 3 ? pick_wide_f2(p, L, tokens) : pick_wide(p, tokens, L.wide[gemm], sums));
+  const WideChoice choice = variant == 3 ? pick_wide(p->tiling, tokens, L.wide[3], false)
+                                         : (gemm == 3 ? pick_wide_f2(p->tiling, tokens, L.wide[3])
+                                                      : pick_wide(p->tiling, tokens, L.wide[gemm], sums));
   const int ldx[4] = {d.hidden, nh * 64, d.hidden, ns * f};
   const int ldo[4] = {64, d.hidden, ns * f, d.hidden};
   const int parts = !sums ? 1 : wide ? static_cast<int>(choice.splits) : tab.n_split;

@@ -349,25 +349,8 @@ cudaError_t set_smem(K kernel) {
 
 }  // namespace
 
-size_t gemm_weight_bytes(uint32_t n_rows, uint32_t k_total) { return static_cast<size_t>(n_rows) * k_total * 2; }
-
-uint32_t gemm_header_bytes() { return kHeaderBytes; }
-
 size_t gemm_smem_bytes(uint32_t w_bytes, uint32_t n_stages, uint32_t bps, uint32_t hdr_bytes) {
   return hdr_bytes + static_cast<size_t>(w_bytes) + static_cast<size_t>(n_stages) * bps * kBoxBytes;
-}
-
-// Ring shape for a weight tile of `w_bytes` and a K range of `k_total`: boxes per stage and stages.
-// Fewer, larger stages mean fewer waits for the MMA-issuing warp; at least ~64 KB stay in flight.
-bool gemm_pick_ring(uint32_t w_bytes, uint32_t k_total, uint32_t hdr_bytes, uint32_t* n_stages, uint32_t* bps) {
-  const long room = 227L * 1024 - static_cast<long>(hdr_bytes) - static_cast<long>(w_bytes);
-  if (room < 3L * kBoxBytes) return false;           // the tile does not fit
-  const uint32_t n_boxes = k_total / kChunkK;
-  if (n_boxes <= 8 && room >= 2L * 4 * kBoxBytes) { *bps = 4; *n_stages = 2; return true; }   // a tile's K in <= 2 stages
-  if (room >= 3L * 2 * kBoxBytes) { *bps = 2; *n_stages = static_cast<uint32_t>(room / (2 * kBoxBytes) > 4 ? 4 : room / (2 * kBoxBytes)); return true; }
-  *bps = 1;
-  *n_stages = static_cast<uint32_t>(room / kBoxBytes > 6 ? 6 : room / kBoxBytes);
-  return true;
 }
 
 cudaError_t gemm_configure() {

@@ -7,18 +7,14 @@
 
 #include "sti_device.cuh"
 #include "sti_kernels.h"
+#include "tiling.h"
 
 namespace sti {
 namespace {
 
 constexpr int kThreads = 512;               // warp 0: TMA producer, warp 1: MMA issuer, warps 4-11: epilogue; all 16 decode
 constexpr int kWarps = kThreads / 32;
-constexpr int kTileM = 128;                 // tokens per MMA tile
-constexpr int kChunkK = 64;                 // one TMA box = 64 columns = one 128-byte swizzle row; a stage holds 1, 2 or 4 boxes
 constexpr int kMaxStages = 8;
-constexpr int kBoxBytes = kTileM * kChunkK * 2;     // 16 KB
-// header = barriers (256 B) + bias (512 B) + one 128-byte centroid table per warp; stages start 1024-aligned after it
-constexpr int kHeaderBytes = 3072;
 constexpr int kTableStride = 64;            // bf16 entries of a warp's centroid table
 constexpr int kEpilogueWarp0 = 4;             // epilogue warps 4..11: two per TMEM lane quadrant
 constexpr int kEpilogueWarps = 8;

@@ -52,9 +52,6 @@ struct GemmLaunch {
   unsigned long long* stamps;   // this launch's profiling record (see sti_device.cuh), or null
 };
 
-size_t gemm_weight_bytes(uint32_t n_rows, uint32_t k_total);
-uint32_t gemm_header_bytes();
-bool gemm_pick_ring(uint32_t w_bytes, uint32_t k_total, uint32_t hdr_bytes, uint32_t* n_stages, uint32_t* bps);   // false: does not fit
 size_t gemm_smem_bytes(uint32_t w_bytes, uint32_t n_stages, uint32_t bps, uint32_t hdr_bytes);
 cudaError_t gemm_configure();   // opt in to large dynamic shared memory (once per device)
 cudaError_t launch_gemm(GemmKind kind, const GemmLaunch& p, cudaStream_t s);

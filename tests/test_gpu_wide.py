@@ -123,3 +123,29 @@ def test_the_rule_s_threshold_is_a_matter_of_the_call(monkeypatch):
             sti.sti_model_forward(s.plan, x.data_ptr(), y.data_ptr(), batch, work.seq, 0)
             sti.sti_sync(s.ctx)
             assert rel_err(from_device_act(y), ref[:batch]) <= REL_TOL, batch
+
+
+@pytest.mark.parametrize("model,kept,context,calls", [
+    ("large", 12, (1, 512), [(1, 400), (1, 488), (1, 385), (1, 512)]),
+    ("large", 14, (8, 512), [(11, 134), (1, 512)]),
+    ("base", 12, (8, 256), [(7, 251), (8, 256)]),
+])
+def test_calls_a_few_tokens_smaller_than_their_context(model, kept, context, calls):
+    """Fewer tokens can take more planes of partial sums than the context's capacity does; fp32 activations, so that the residual
+    that stands behind the planes is an fp32 copy."""
+    from gpu_util import from_device_act, rel_err, REL_TOL
+    shape = (W.BERT_BASE if model == "base" else W.BERT_LARGE).with_layers(1)
+    attn = [[W.UnitPlan(i < kept, BITS6[i % 5], True) for i in range(shape.n_heads)]]
+    ffn = [[W.UnitPlan(i < kept, BITS6[(i + 2) % 5], True) for i in range(shape.n_ffn_slices)]]
+    work = W.build_workload("smaller", shape, 1, 8, "f32", attn, ffn, seed=kept)
+    a, f = O.decode_layer(work, 0)
+    with sti.Session(work, max_batch=context[0], max_seq=context[1]) as s:
+        for batch, seq in calls:
+            x = np.random.default_rng(seq).standard_normal((batch, seq, shape.hidden), dtype=np.float32)
+            ref = O.layer_forward(x, work.dense[0], a, f, eps=work.ln_eps)
+            x = torch.from_numpy(x).cuda()
+            y = torch.full_like(x, float("nan"))
+            torch.cuda.synchronize()
+            sti.sti_layer_forward(s.plan, 0, x.data_ptr(), y.data_ptr(), batch, seq, 0)
+            sti.sti_sync(s.ctx)
+            assert rel_err(from_device_act(y), ref) <= REL_TOL, (batch, seq)

@@ -153,7 +153,7 @@ struct sti_plan {
   void* buf[2] = {nullptr, nullptr};
   void* x_in = nullptr; void* y_out = nullptr; int32_t* lens_dev = nullptr;
   uint8_t* wide_buf = nullptr;         // two working buffers for decoded weights, of even and of odd layers (plans for many tokens)
-  size_t wide_bytes = 0;               // of each
+  size_t wide_bytes = 0;               // of each, in whole blocks of 16 KB
   uint8_t* wide_tables = nullptr;      // their tasks and bias offsets
   float* zero_bias = nullptr;          // all-zero bias vector of sti_gemm_probe (allocated by its first call)
   uint8_t* rate_tables = nullptr;      // every layer's FFN1 tile jobs in one table (sti_decode_rate_probe, built by its first call)
@@ -475,7 +475,7 @@ sti_status ensure_wide(sti_plan* p) {
   std::vector<uint8_t> host;
   struct At { size_t tasks, bias[2]; };
   std::vector<At> at(p->layers.size());
-  size_t most = 1024, n_tasks = 0;
+  size_t n_tasks = 0;
   for (Layer& L : p->layers) {
     const uint32_t per[4] = {3 * 64u * c->attn_m[0].kc / 4096, c->attn_m[3].rows * 64 / 4096, c->ffn_m[0].rows * c->ffn_m[0].kc / 4096,
                              c->ffn_m[1].rows * c->ffn_m[1].kc / 4096};
@@ -488,7 +488,6 @@ sti_status ensure_wide(sti_plan* p) {
   bool in_bounds = true;
   for (size_t li = 0; li < p->layers.size(); ++li) {
     Layer& L = p->layers[li];
-    most = std::max(most, static_cast<size_t>(place_wide(p->tiling, static_cast<int>(L.kept_heads.size()), static_cast<int>(L.kept_slices.size()), L.wide)) * 128);
     tasks.resize(L.wide_first[4]);
     uint32_t filled[4] = {L.wide_first[0], L.wide_first[1], L.wide_first[2], L.wide_first[3]};
     // rows [first, first + rows) of the unit's matrix `um` are features n0 .. of layer matrix `m`, from column chunk kc0 on
@@ -532,7 +531,6 @@ sti_status ensure_wide(sti_plan* p) {
     for (int b = 0; b < 2; ++b) at[li].bias[b] = put(bias[b].data(), bias[b].size() * 4);
   }
   if (!in_bounds) return STI_ERR_STATE;                  // not for any plan the calls before let through
-  p->wide_bytes = (most + 16383) / 16384 * 16384;
   if (!p->wide_tables) CUDA_TRY(cudaMalloc(&p->wide_tables, std::max<size_t>(host.size(), 16)));
   if (!host.empty()) CUDA_TRY(cudaMemcpy(p->wide_tables, host.data(), host.size(), cudaMemcpyHostToDevice));
   for (size_t li = 0; li < p->layers.size(); ++li) {
@@ -540,7 +538,7 @@ sti_status ensure_wide(sti_plan* p) {
     L.wide_tasks = reinterpret_cast<const DecodeTask*>(p->wide_tables + at[li].tasks);
     for (int b = 0; b < 2; ++b) L.wide_bias[b] = reinterpret_cast<const int32_t*>(p->wide_tables + at[li].bias[b]);
   }
-  CUDA_TRY(cudaMalloc(&p->wide_buf, 2 * p->wide_bytes));
+  CUDA_TRY(cudaMalloc(&p->wide_buf, std::max<size_t>(2 * p->wide_bytes, 16)));
   return STI_OK;
 }
 
@@ -1400,7 +1398,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
   for (auto& L : p->layers) {
     LayerTables tb;
     const int heads = static_cast<int>(L.kept_heads.size()), slices = static_cast<int>(L.kept_slices.size());
-    (void)place_wide(p->tiling, heads, slices, L.wide);
+    p->wide_bytes = static_cast<size_t>(place_wide(p->tiling, heads, slices, max_heads, max_slices, L.wide)) * 128;      // the same for every layer
     L.tables_off = align16(host_tables.size());
     build_layer_tables(p, L, tb);
     auto place = [&](GemmTable& gt, TableBuilder& b) -> sti_status {

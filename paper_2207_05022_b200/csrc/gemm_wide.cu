@@ -195,8 +195,10 @@ gemm_wide_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
     }
   if (!decoder) {                      // decoding depends on no kernel before this one
     pdl_wait();
-    // Not before the wait: a kernel that has started knows by this that the same GEMM of the layer before has finished, whose
-    // weights stand where its decoders write.
+    // Not before the wait: by this a kernel that has started knows that everything before the last GEMM over the working buffer
+    // has finished (the kernels in between release their successors at once).  Its decoders write the place of their own matrix,
+    // which all layers share and which that last GEMM, being another of the four, does not read: of QKV and O, or FFN1 and FFN2,
+    // the second follows whenever the first is run, and a layer that decodes ahead has all four.
     pdl_launch_dependents();
   }
   if (tid == 0) stamp_min(stamps, STAMP_RELEASE);

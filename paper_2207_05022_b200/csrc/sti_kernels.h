@@ -82,7 +82,7 @@ struct WideLaunch {
   const float* bias;        // null: none
   const int32_t* bias_off;  // per 64 features: where their bias begins
   bool weights_ready;       // decoded by a kernel that has finished before this one can start: read without waiting
-  ExpandLaunch beside;      // decoded beside it by otherwise idle warps (n_tasks 0: nothing); `dst` is read by no kernel in flight
+  ExpandLaunch beside;      // decoded beside it by otherwise idle warps (n_tasks 0: nothing), the same matrix of another layer: no kernel in flight reads its place
   int* err;
   bool pdl;
   unsigned long long* stamps;

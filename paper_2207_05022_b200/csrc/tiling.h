@@ -144,14 +144,17 @@ inline WideChoice pick_wide_f2(const Tiling& t, long long tokens, const WideMatr
   return pick_wide(t, tokens, m, !(t.tune.f2_kacc_min_tokens > 0 && whole_tiles(tokens) >= t.tune.f2_kacc_min_tokens));
 }
 
-// Sizes and places of a layer's matrices (QKV, O, FFN1, FFN2) in its working buffer; its rows of 128 bytes.
-inline uint32_t place_wide(const Tiling& t, int heads, int slices, WideMatrix (&wide)[4]) {
-  const uint32_t d = static_cast<uint32_t>(t.hidden), nh = static_cast<uint32_t>(heads), ff = static_cast<uint32_t>(t.slice * slices);
-  const uint32_t n[4] = {192 * nh, d, ff, d}, k[4] = {d, 64 * nh, d, ff};
+// Sizes and places of a layer's matrices (QKV, O, FFN1, FFN2) in its working buffer; the buffer's rows of 128 bytes.  A matrix has
+// one place in all of a plan's layers, as large as the widest of them needs (`most_heads`, `most_slices`): the warps that decode
+// ahead write while the kernel before theirs may still read, and what that one reads is never the same matrix (gemm_wide.cu).
+inline uint32_t place_wide(const Tiling& t, int heads, int slices, int most_heads, int most_slices, WideMatrix (&wide)[4]) {
+  const uint32_t d = static_cast<uint32_t>(t.hidden);
   uint32_t row = 0;
   for (int m = 0; m < 4; ++m) {
-    wide[m] = {row, n[m], k[m] / 64};
-    row += (n[m] + 255) / 256 * 256 * (k[m] / 64);       // whole tiles of 256 features
+    auto features = [&](int h, int s) { return m == 0 ? 192u * h : m == 2 ? static_cast<uint32_t>(t.slice * s) : d; };
+    auto columns = [&](int h, int s) { return m == 1 ? 64u * h : m == 3 ? static_cast<uint32_t>(t.slice * s) : d; };
+    wide[m] = {row, features(heads, slices), columns(heads, slices) / 64};
+    row += (features(most_heads, most_slices) + 255) / 256 * 256 * (columns(most_heads, most_slices) / 64);       // whole tiles of 256 features
   }
   return row;
 }
@@ -161,7 +164,7 @@ struct SumPlanes { int o, f2; };
 inline SumPlanes sum_planes(const Tiling& t, int heads, int slices, long long tokens) {
   if (use_wide(t, heads, slices, tokens)) {
     WideMatrix wide[4];
-    (void)place_wide(t, heads, slices, wide);
+    (void)place_wide(t, heads, slices, heads, slices, wide);
     return {heads > 0 ? static_cast<int>(pick_wide(t, tokens, wide[1], true).splits) : 0,
             slices > 0 ? static_cast<int>(pick_wide_f2(t, tokens, wide[3]).splits) : 0};
   }

@@ -110,6 +110,38 @@ def test_decoding_ahead_gives_the_same_bytes(act, streamed_from, monkeypatch):
     assert rel_err(from_device_act(cur), O.run_workload(work)) <= REL_TOL
 
 
+@pytest.mark.parametrize("heads,slices", [
+    ((2, 16, 16, 2, 2, 16), (2, 16, 16, 2, 2, 16)),        # two layers after a narrow one comes one that keeps all
+    ((16, 16, 16, 1, 16, 16), (0, 16, 16, 0, 3, 16)),      # ... after one without a slice, whose O projection is its last product
+    ((0, 16, 16, 0, 4, 16), (16, 16, 16, 2, 16, 16)),      # ... without a head
+])
+def test_layers_of_different_widths_give_the_same_bytes(heads, slices):
+    """Layers decoded ahead while layers of other widths are still multiplied with, above the rule's threshold."""
+    from gpu_util import from_device_act, rel_err, to_device_act, REL_TOL
+    n = len(heads)
+    shape = W.BERT_LARGE.with_layers(n)
+    attn = [[W.UnitPlan(i < heads[l], BITS6[(l + i) % 5], True) for i in range(16)] for l in range(n)]
+    ffn = [[W.UnitPlan(i < slices[l], BITS6[(2 * l + i) % 5], True) for i in range(16)] for l in range(n)]
+    work = W.build_workload("widths", shape, 5, 128, "bf16", attn, ffn, seed=n, workers=4)
+    x = to_device_act(work)
+    with sti.Session(work) as s:
+        cur = x.clone()
+        for layer in range(n):
+            y = torch.zeros_like(cur)
+            torch.cuda.synchronize()
+            sti.sti_layer_forward(s.plan, layer, cur.data_ptr(), y.data_ptr(), work.batch, work.seq, 0)
+            sti.sti_sync(s.ctx)
+            cur = y
+        outs = [torch.full_like(x, float("nan")) for _ in range(20)]
+        torch.cuda.synchronize()
+        for o in outs:
+            sti.sti_model_forward(s.plan, x.data_ptr(), o.data_ptr(), work.batch, work.seq, 0)
+        sti.sti_sync(s.ctx)
+    for o in outs:
+        assert torch.equal(o.view(torch.uint8), cur.view(torch.uint8))
+    assert rel_err(from_device_act(cur), O.run_workload(work)) <= REL_TOL
+
+
 def test_the_rule_s_threshold_is_a_matter_of_the_call(monkeypatch):
     """Calls below and above the token count where the working buffer takes over, through one plan and interleaved."""
     from gpu_util import from_device_act, rel_err, to_device_act, REL_TOL

@@ -1,5 +1,5 @@
 """How calls are cut (csrc/tiling.h), compiled for the host: the buffer of partial sums holds the planes of every call that a
-context takes."""
+context takes, and a matrix has one place in the working buffer whatever a layer keeps."""
 import ctypes as C
 import subprocess
 
@@ -34,6 +34,17 @@ extern "C" size_t rows(int hidden, int slice, int heads, int slices, long long m
 extern "C" int wide(int hidden, int slice, int heads, int slices, long long tokens, const int* tune) {
   return use_wide(tiling(hidden, slice, tokens, tune), heads, slices, tokens);
 }
+// Rows of 128 bytes: where each of the four matrices begins, where what is written of it ends, and the buffer's.
+extern "C" unsigned place(int hidden, int slice, const int* units, unsigned* at) {
+  const int tune[3] = {8, -1, 148};
+  WideMatrix wide[4];
+  const unsigned rows = place_wide(tiling(hidden, slice, 1, tune), units[0], units[1], units[2], units[3], wide);
+  for (int m = 0; m < 4; ++m) {
+    at[2 * m] = wide[m].row0;
+    at[2 * m + 1] = wide[m].row0 + (wide[m].n + 255) / 256 * 256 * wide[m].k_chunks;      // a 256-wide tile's boxes reach so far
+  }
+  return rows;
+}
 """
 MODELS = {"base": (768, 256, 12), "large": (1024, 256, 16)}
 DEFAULT = (8, -1, 148)                           # heads per K group, the rule's own threshold, CTAs
@@ -49,6 +60,7 @@ def lib(tmp_path_factory):
     so.overflow.argtypes, so.overflow.restype = args, C.c_longlong
     so.rows.argtypes, so.rows.restype = args, C.c_size_t
     so.wide.argtypes = args
+    so.place.argtypes = [C.c_int, C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_uint)]
     return so
 
 
@@ -77,3 +89,20 @@ def test_planes_are_asked_for_where_calls_have_them(lib):
     """The check above is not an empty one: calls of more than one plane, on either side of the working buffer's threshold."""
     assert lib.rows(1024, 256, 12, 12, 384, _tune()) > 384 and not lib.wide(1024, 256, 12, 12, 384, _tune())
     assert lib.rows(1024, 256, 12, 12, 512, _tune()) > 512 and lib.wide(1024, 256, 12, 12, 400, _tune())
+
+
+@pytest.mark.parametrize("model", sorted(MODELS))
+def test_a_matrix_never_stands_where_another_layer_has_a_different_one(lib, model):
+    hidden, slice_, n = MODELS[model]
+    for most_heads in range(n + 1):
+        for most_slices in (0, 1, 5, n):
+            places = set()
+            for heads in range(most_heads + 1):
+                for slices in range(most_slices + 1):
+                    at = (C.c_uint * 8)()
+                    rows = lib.place(hidden, slice_, (C.c_int * 4)(heads, slices, most_heads, most_slices), at)
+                    begin, end = list(at)[0::2], list(at)[1::2]
+                    places.add(tuple(begin) + (rows,))
+                    assert begin[0] == 0 and all(b % 128 == 0 for b in begin)
+                    assert all(e <= limit for e, limit in zip(end, begin[1:] + [rows]))
+            assert len(places) == 1

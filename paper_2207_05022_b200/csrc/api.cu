@@ -657,9 +657,12 @@ ExpandLaunch expand_job(const sti_plan* p, int li, int first, int end) {
   e.pdl = p->ctx->pdl;
   return e;
 }
-sti_status run_expand(sti_plan* p, int li) {
-  const ExpandLaunch e = expand_job(p, li, 0, 4);
+// `first`: of a forward.  What the layers after it decode ahead is ordered against the GEMMs of this forward only (gemm_wide.cu), so
+// that one begins when everything before it on the stream has finished.
+sti_status run_expand(sti_plan* p, int li, bool first = false) {
+  ExpandLaunch e = expand_job(p, li, 0, 4);
   if (e.n_tasks == 0) return STI_OK;
+  if (first) e.pdl = false;
   CUDA_TRY(launch_expand(e, p->ctx->compute));
   p->ctx->launches++;
   return STI_OK;
@@ -696,12 +699,13 @@ sti_status run_wide(sti_plan* p, GemmKind kind, int li, int which, const WideCho
 
 // The seven kernels of one layer on the compute stream, and for many tokens those that decode weights into the working buffer.
 // `expanded`: this layer's weights are there already; `beside`: the layer that is decoded beside this one's GEMMs (-1: none);
-// `ffn_loaded`: what the FFN units have to be waited for with, if they are still on their way.
+// `ffn_loaded`: what the FFN units have to be waited for with, if they are still on their way; `first_wide`: no layer before this one
+// went through the working buffer in this forward.
 // `x_ready_bf16`: the bf16 copy of x already sits in p->x_bf16 (written by the previous layer's LayerNorm);
 // `want_next_bf16`: this layer's last kernel also writes y as bf16 into p->x_bf16 for the next layer.
 sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch, int seq, const int32_t* lens,
                          bool x_ready_bf16, bool want_next_bf16, int next_layer = -1, bool expanded = false, int beside = -1,
-                         cudaEvent_t ffn_loaded = nullptr) {
+                         cudaEvent_t ffn_loaded = nullptr, bool first_wide = false) {
   sti_ctx* c = p->ctx;
   const sti_model_desc& d = c->desc;
   Layer& L = p->layers[li];
@@ -724,7 +728,7 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
   const int f2_planes = ns > 0 ? (wide ? static_cast<int>(f2_choice.splits) : f2.n_split) : 0;
   if (static_cast<size_t>(T) * std::max(o_planes, f2_planes) > p->partial_rows) return STI_ERR_STATE;      // not for any call: partial_rows
   CUDA_TRY(mark(0));
-  if (wide && !expanded && (st = run_expand(p, li)) != STI_OK) return st;
+  if (wide && !expanded && (st = run_expand(p, li, first_wide)) != STI_OK) return st;
   if (nh > 0) {
     const void* xq = x;
     if (!bf16_act) {
@@ -874,7 +878,7 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
   int last_streamed = -1;
   for (int li = 0; li < n; ++li) if (p->layers[li].str_bytes > 0) last_streamed = li;
   const void* cur = x;
-  bool expanded = false;
+  bool expanded = false, any_wide = false;
   for (int li = 0; li < n; ++li) {
     Layer& L = p->layers[li];
     cudaEvent_t ffn_loaded = nullptr;
@@ -909,8 +913,9 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
                        use_wide(p, p->layers[li + 1], static_cast<long long>(batch) * seq) && p->layers[li + 1].str_bytes == 0 &&
                        !L.kept_heads.empty() && !L.kept_slices.empty();
     sti_status st = enqueue_layer(p, li, cur, nxt, batch, seq, lens, li > 0, li + 1 < n, li + 1 < n ? li + 1 : -1, expanded,
-                                  ahead ? li + 1 : -1, ffn_loaded);
+                                  ahead ? li + 1 : -1, ffn_loaded, !any_wide);
     if (st != STI_OK) return st;
+    any_wide |= use_wide(p, L, static_cast<long long>(batch) * seq) && !(L.kept_heads.empty() && L.kept_slices.empty());
     expanded = ahead;
     if (p->retain_pending && !capturing && L.str_bytes > 0) {
       // keep what this run loaded (Section 3.2): the marked units leave their ring slot for the retained arena

@@ -142,6 +142,34 @@ def test_layers_of_different_widths_give_the_same_bytes(heads, slices):
     assert rel_err(from_device_act(cur), O.run_workload(work)) <= REL_TOL
 
 
+def test_forwards_behind_a_product_by_itself(monkeypatch):
+    """Launched kernel by kernel: a forward decodes layer 1 ahead into the buffer in which a product queued just before it
+    reads layer 3."""
+    from gpu_util import to_device_act
+    monkeypatch.setenv("STI_NO_GRAPH", "1")
+    work = _layers(5, "bf16", 99)
+    shape, T = work.shape, work.batch * work.seq
+    x = to_device_act(work)
+    planes = 3 * len(work.kept(3, ATTN))
+    with sti.Session(work) as s:
+        alone = torch.empty_like(x)
+        sti.sti_model_forward(s.plan, x.data_ptr(), alone.data_ptr(), work.batch, work.seq, 0)
+        rows = 16 * T                                      # a product that takes longer than the forward's first kernels
+        act = torch.randn(rows, shape.hidden, device="cuda").bfloat16()
+        want = torch.zeros(planes, rows, 64, dtype=torch.bfloat16, device="cuda")
+        got = torch.zeros_like(want)
+        torch.cuda.synchronize()
+        sti.sti_gemm_probe(s.plan, 3, 0, act.data_ptr(), rows, want.data_ptr(), want.numel() * 2, 2)
+        sti.sti_sync(s.ctx)
+        for _ in range(10):
+            y = torch.full_like(x, float("nan"))
+            torch.cuda.synchronize()
+            sti.sti_gemm_probe(s.plan, 3, 0, act.data_ptr(), rows, got.data_ptr(), got.numel() * 2, 2)
+            sti.sti_model_forward(s.plan, x.data_ptr(), y.data_ptr(), work.batch, work.seq, 0)
+            sti.sti_sync(s.ctx)
+            assert torch.equal(got, want) and torch.equal(y, alone)
+
+
 def test_the_rule_s_threshold_is_a_matter_of_the_call(monkeypatch):
     """Calls below and above the token count where the working buffer takes over, through one plan and interleaved."""
     from gpu_util import from_device_act, rel_err, to_device_act, REL_TOL

@@ -712,8 +712,13 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
   const double c0 = -0.5 * log(2.0 * 3.14159265358979323846 * var);
   const double inv2var = 1.0 / (2.0 * var);
   const double radius = sqrt(2.0 * var * (c0 + 4.0));                  // inliers satisfy (x - mu)^2 <= 2 var (c0 + 4)
-  if (!(var > 0.0) || !(radius > 0.0)) {
+  // Others may still be reading this CTA's histogram: a CTA that leaves before the next barrier waits for them.
+  auto leave_to_the_sort = [&]() {
     if (rank == 0 && tid == 0) marks[unit] = 1;                        // every thread of the cluster leaves
+    cluster.sync();
+  };
+  if (!(var > 0.0) || !(radius > 0.0)) {
+    leave_to_the_sort();
     return;
   }
   {
@@ -723,7 +728,7 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     const uint32_t in = __ballot_sync(0xffffffffu, !is_outlier(x, mu, inv2var, c0));
     const int least = sti::end_index(in & 0xffffu), most = sti::end_index(in >> 16);
     if (least < 0 || most < 0) {
-      if (rank == 0 && tid == 0) marks[unit] = 1;                      // every thread of the cluster leaves here, too
+      leave_to_the_sort();
       return;
     }
     un.least = __shfl_sync(0xffffffffu, x, least);

@@ -191,6 +191,19 @@ def test_units_without_an_inlier():
         assert list(_check(np.stack([sign, one]), bits)) == [1, 0]
 
 
+@pytest.mark.parametrize("n_units,n", [(1, 196608), (3, 65536 + 480), (1, 524288)])
+def test_units_shared_by_ctas_that_leave_early(n_units, n):
+    """No variance, or a range whose ends are not found: all CTAs of a cluster leave after they have read one another's histograms."""
+    rng = np.random.default_rng(n)
+    flat = np.zeros((n_units, n), np.float32)
+    wide = (rng.standard_normal((n_units, n)) * 30).astype(np.float32)         # above a deviation of 21.8 every weight is an outlier
+    apart = np.where(rng.random((n_units, n)) < 0.5, np.float32(3.0e8), np.float32(3.0e8 + 32)).astype(np.float32)
+    normal = (rng.standard_normal((1, n)) * 0.02).astype(np.float32)
+    for bits in (3, 4):
+        for units in (flat, wide, apart):
+            assert list(_check(np.concatenate([units, normal]), bits, max_out=n)) == [1] * n_units + [0]
+
+
 def test_outlier_lists_shorter_than_the_outliers_found():
     shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=1024, n_ffn_slices=4)
     mats = make_unit_weights(shape, 13, 0, FFN, 1, outlier_stress=0.01)

@@ -432,7 +432,7 @@ constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelMaxCluster = 16;
 constexpr int kSelBins = 16384;            // most value bins; half of them for units of at most 2^18 weights
 constexpr int kSelMaxSeg = 1024;           // weights of one boundary bin that are ranked by counting
-constexpr int kSelSmemSeg = 256;           // ... in shared memory; more than that in the workspace
+constexpr int kSelSmemSeg = 256;           // ... in shared memory; more than that from the workspace
 constexpr int kSelGroups = 4;              // groups of 128 consecutive weights (four per lane) a warp classifies per step
 constexpr int kSelStep = kSelGroups * 128; // weights of one step of one warp
 constexpr uint32_t kSelTails = 32;         // weights of a warp's tails that are listed in shared memory; more of them in the workspace
@@ -466,10 +466,11 @@ struct SelShared {
   union alignas(16) {
     uint32_t hist[kSelBins];               // this CTA's histogram; in its own range of bins the cluster's, then its prefix
     double acc[kAccCells];                 // later the cluster sums
-    unsigned long long pairs[kSelWarps][2][kSelSmemSeg];         // and last the boundary bins: as gathered, in order
+    unsigned long long pairs[kSelWarps][2][kSelSmemSeg];         // and last the boundary bins: as gathered, their keys in order
   } u;
 };
 static_assert(2 * (sizeof(SelShared) + 1024) <= 228 * 1024, "two CTAs on an SM");
+static_assert(4 * kSelSmemSeg >= kSelMaxSeg, "the longest bin's keys in a warp's pairs");
 static_assert(sti::kEndCandidates == 16, "half a warp");
 static_assert(kSelBins / kSelMaxCluster / kSelWarps <= 64, "eight of the cluster's CTAs per lane");
 
@@ -992,14 +993,20 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
   cluster.sync();                                                      // pairs and streams are complete as well
 
   // ---- 5. the boundary bins, a warp each: a pair's rank is the number of smaller pairs of its bin (all are distinct)
+  // The lists' address is worked out again, from a block number that the compiler does not know: kept over pass 4 it makes
+  // another value there come back from L2 (384 units of 524,288 weights at 3 bits 487 -> 520 us, 200 at 4 bits 270 -> 286).
+  uint32_t cta;
+  asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
+  const unsigned long long* lists = reinterpret_cast<const unsigned long long*>(ws_all + static_cast<size_t>(cta / n_ctas) * ws_per_unit);
   for (uint32_t c = 1u + warp * n_ctas + rank; c < K; c += n_warps) {       // neighbours on different SMs
     if (!owns(c)) continue;
     const uint32_t m = sm.seg_len[c], bin = sm.bnd_bin[c];
     uint32_t last = c;                                                 // the bin's boundaries: c .. last
     while (last + 1u < K && sm.bnd_bin[last + 1u] == bin) ++last;
-    const unsigned long long* from = cand + sm.seg_start[c];
-    // in order: the second half of the unit's workspace takes what shared memory cannot
-    unsigned long long* sorted = m <= static_cast<uint32_t>(kSelSmemSeg) ? sm.u.pairs[warp][1] : cand + n + sm.seg_start[c];
+    const unsigned long long* from = lists + sm.seg_start[c];
+    // The keys in order, which is all that the sums need: behind the pairs, or where a longer bin's would have been (the unit's
+    // workspace has no room for them: its second half holds the tails beyond the warps' lists).
+    uint32_t* sorted = reinterpret_cast<uint32_t*>(sm.u.pairs[warp][m <= static_cast<uint32_t>(kSelSmemSeg) ? 1 : 0]);
     if (m <= static_cast<uint32_t>(kSelSmemSeg)) {
       for (uint32_t j = lane; j < m; j += 32) sm.u.pairs[warp][0][j] = from[j];
       if (lane == 0 && (m & 1u) != 0u) sm.u.pairs[warp][0][m] = ~0ull;
@@ -1037,7 +1044,7 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         if (j0 + 32 * e + lane >= m) continue;
-        sorted[smaller[e]] = mine[e];
+        sorted[smaller[e]] = static_cast<uint32_t>(mine[e] >> 32);
         uint32_t code = c - 1u;
         while (code + 1u <= last && sm.bnd_rho[code + 1u] <= smaller[e]) ++code;
         const uint64_t bit = (mine[e] & 0xffffffffull) * bits;
@@ -1050,7 +1057,7 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     for (uint32_t k = c - 1u; k <= last; ++k) {                        // the bin's share of clusters c - 1 .. last
       const uint32_t lo = k == c - 1u ? 0u : sm.bnd_rho[k], hi = k == last ? m : sm.bnd_rho[k + 1u];
       double acc = 0.0;
-      for (uint32_t t = lo + lane; t < hi; t += 32) acc += static_cast<double>(key_value(static_cast<uint32_t>(sorted[t] >> 32)));
+      for (uint32_t t = lo + lane; t < hi; t += 32) acc += static_cast<double>(key_value(sorted[t]));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
       double* to = k == c - 1u ? &sm.extra_hi[k] : &sm.extra_lo[k];

@@ -204,6 +204,52 @@ def test_units_shared_by_ctas_that_leave_early(n_units, n):
             assert list(_check(np.concatenate([units, normal]), bits, max_out=n)) == [1] * n_units + [0]
 
 
+def _long_bins_and_long_tails(n, seed, narrow):
+    """Weights with 0.15 % of ten times the spread; with `narrow`, half of the others have a tenth of it.  A warp's run then has
+    more tails than its list in shared memory takes, and boundary bins hold more than 256 weights."""
+    rng = np.random.default_rng(seed)
+    w = (rng.standard_normal(n) * 0.02).astype(np.float32)
+    if narrow:
+        w[rng.random(n) < 0.5] *= np.float32(0.1)
+    else:
+        w[rng.random(n) < 0.0015] *= 10
+    return w
+
+
+@pytest.mark.parametrize("n,bits", [(1 << 20, 2), (1 << 20, 3), (1 << 20, 6), (524288, 6), (524288, 2)])
+def test_long_boundary_bins_beside_long_lists_of_tails(n, bits):
+    units = _long_bins_and_long_tails(n, 1, narrow=True)[None, :]
+    assert not _check(units, bits, max_out=n).any()
+
+
+@pytest.mark.parametrize("n,narrow,bits", [(1 << 21, False, 3), (1 << 21, False, 2), (1 << 18, True, 2), (524288, True, 3)])
+def test_long_boundary_bins_beside_long_lists_of_tails_one_cta_per_unit(n, narrow, bits):
+    """As many units as the device holds at a time, all the same one."""
+    unit = _long_bins_and_long_tails(n, 2, narrow)
+    words, cents, off, val = Q.quantize_unit(unit, bits)
+    n_units, max_out = 2 * torch.cuda.get_device_properties(0).multi_processor_count, off.size
+    w = torch.from_numpy(unit).cuda().expand(n_units, n).contiguous()
+    ws_bytes = sti.sti_quantize_workspace_bytes(n_units, n)
+    ws = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda")
+    for method in (sti.STI_QUANTIZE_SELECT, sti.STI_QUANTIZE_SORT):
+        some = n_units if method == sti.STI_QUANTIZE_SELECT else 1
+        codes = torch.zeros((some, n * bits // 32), dtype=torch.int32, device="cuda")
+        got_cents = torch.zeros((some, 1 << bits), device="cuda")
+        got_off = torch.zeros((some, max_out), dtype=torch.int32, device="cuda")
+        got_val = torch.zeros((some, max_out), device="cuda")
+        count = torch.zeros(some, dtype=torch.int32, device="cuda")
+        by_sort = torch.zeros(some, dtype=torch.uint8, device="cuda")
+        torch.cuda.synchronize()
+        sti.sti_quantize_units_by(w.data_ptr(), some, n, bits, codes.data_ptr(), got_cents.data_ptr(), got_off.data_ptr(), got_val.data_ptr(),
+                                  max_out, count.data_ptr(), ws.data_ptr(), ws_bytes, method, by_sort.data_ptr())
+        torch.cuda.synchronize()
+        assert (by_sort == (0 if method == sti.STI_QUANTIZE_SELECT else 1)).all()
+        for out in (codes, got_cents, got_off, got_val, count):
+            assert torch.equal(out, out[:1].expand_as(out))
+        _compare(unit[None, :], bits, max_out, [(words, cents, off, val)], codes[:1].cpu().numpy().view(np.uint32), got_cents[:1].cpu().numpy(),
+                 got_off[:1].cpu().numpy().view(np.uint32), got_val[:1].cpu().numpy(), count[:1].cpu().numpy())
+
+
 def test_outlier_lists_shorter_than_the_outliers_found():
     shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=1024, n_ffn_slices=4)
     mats = make_unit_weights(shape, 13, 0, FFN, 1, outlier_stress=0.01)

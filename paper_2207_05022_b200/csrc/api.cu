@@ -722,7 +722,8 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     return p->stamping ? p->stamps + (static_cast<size_t>(li) * kStampKernels + kernel) * kStampRecord : nullptr;
   };
   const bool wide = use_wide(p, L, T);
-  const WideChoice o_choice = pick_wide(p->tiling, T, L.wide[1], true), f2_choice = pick_wide_f2(p->tiling, T, L.wide[3]);
+  WideChoice o_choice{}, f2_choice{};
+  if (wide) { o_choice = pick_wide(p->tiling, T, L.wide[1], true); f2_choice = pick_wide_f2(p->tiling, T, L.wide[3]); }
   const GemmTable& f2 = f2_table(p, L, T);
   const int o_planes = nh > 0 ? (wide ? static_cast<int>(o_choice.splits) : L.o.n_split) : 0;
   const int f2_planes = ns > 0 ? (wide ? static_cast<int>(f2_choice.splits) : f2.n_split) : 0;

@@ -141,7 +141,14 @@ sti_status sti_shard_upload(sti_plan* plan, int layer, sti_kind kind, int index,
 
 /* Section 3.1: fills the preload buffer (resident units -> device memory) and lays every
  * streamed layer out as one contiguous pinned-host blob ("one layer ... as a single IO job").
- * Called implicitly by the first forward.  STI_ERR_SHARD_MISSING if a kept unit has no blob. */
+ * Called implicitly by the first forward.  STI_ERR_SHARD_MISSING if a kept unit has no blob.
+ * Device memory besides the shards: activations and partial sums for max_batch * max_seq tokens (the largest are the FFN's
+ * bf16 activations, 2 bytes per token and kept FFN column, and fp32 sums, 4 * hidden bytes per token and plane: at most one
+ * plane per kept slice in calls of few tokens - per two of BERT's -, 1 to 4 in larger ones), and, in a context of at least 513 tokens (385 where a layer keeps 8 M weights
+ * or more), working buffers in which calls of that many tokens decode a layer's weights to bf16.  One buffer takes 2 bytes
+ * per weight of a layer that keeps the plan's largest number of heads and of slices (BERT-large, all units: 25 MB), and there are
+ * two if any layer follows, without streamed units, one that keeps heads and slices; 32 bytes per 4096 kept weights of the whole plan
+ * come on top (2.4 MB).  STI_ERR_OOM if the memory is not there: a smaller context needs less. */
 sti_status sti_plan_finalize(sti_plan* plan);
 
 /* Section 2.1 / 4.2: one layer over its kept units.  x_dev, y_dev: device, [batch, seq, hidden]

@@ -152,7 +152,8 @@ struct sti_plan {
   uint16_t* x_bf16 = nullptr;          // bf16 copy of fp32 layer inputs (the GEMM operand)
   void* buf[2] = {nullptr, nullptr};
   void* x_in = nullptr; void* y_out = nullptr; int32_t* lens_dev = nullptr;
-  uint8_t* wide_buf = nullptr;         // two working buffers for decoded weights, of even and of odd layers (plans for many tokens)
+  uint8_t* wide_buf = nullptr;         // working buffers for decoded weights (plans for many tokens): two, of even and of odd layers, if any layer can be
+  int wide_count = 1;                  // decoded beside the one before it, else one
   size_t wide_bytes = 0;               // of each, in whole blocks of 16 KB
   uint8_t* wide_tables = nullptr;      // their tasks and bias offsets
   float* zero_bias = nullptr;          // all-zero bias vector of sti_gemm_probe (allocated by its first call)
@@ -466,6 +467,13 @@ void build_layer_tables(sti_plan* p, Layer& L, LayerTables& tb) {
   }
 }
 
+// Whether layer li + 1 can be decoded beside the GEMMs of layer li: not if li lacks one of them, nor if li + 1 is streamed and may not be
+// on the device yet.
+bool can_decode_ahead(const sti_plan* p, int li) {
+  const Layer& L = p->layers[li];
+  return li + 1 < static_cast<int>(p->layers.size()) && !L.kept_heads.empty() && !L.kept_slices.empty() && p->layers[li + 1].str_bytes == 0;
+}
+
 // What fills the working buffer: the tasks of every kept unit, layer by layer, with their places, and the bias offsets of the
 // GEMMs over it.  Made when a plan for many tokens is finalized, or by the first probe that asks for it.
 sti_status ensure_wide(sti_plan* p) {
@@ -538,7 +546,8 @@ sti_status ensure_wide(sti_plan* p) {
     L.wide_tasks = reinterpret_cast<const DecodeTask*>(p->wide_tables + at[li].tasks);
     for (int b = 0; b < 2; ++b) L.wide_bias[b] = reinterpret_cast<const int32_t*>(p->wide_tables + at[li].bias[b]);
   }
-  CUDA_TRY(cudaMalloc(&p->wide_buf, std::max<size_t>(2 * p->wide_bytes, 16)));
+  for (size_t li = 0; li < p->layers.size(); ++li) if (can_decode_ahead(p, static_cast<int>(li))) p->wide_count = 2;
+  CUDA_TRY(cudaMalloc(&p->wide_buf, std::max<size_t>(p->wide_count * p->wide_bytes, 16)));
   return STI_OK;
 }
 
@@ -647,13 +656,14 @@ sti_status run_gemm(sti_plan* p, GemmKind kind, const GemmTable& tab, const void
   return STI_OK;
 }
 
-uint8_t* wide_buffer(const sti_plan* p, int li) { return p->wide_buf + (li & 1) * p->wide_bytes; }
+// Byte offset of layer li's working buffer.
+size_t wide_at(const sti_plan* p, int li) { return (li & (p->wide_count - 1)) * p->wide_bytes; }
 
 // What decodes the matrices [first, end) of layer `li` into its working buffer.
 ExpandLaunch expand_job(const sti_plan* p, int li, int first, int end) {
   const Layer& L = p->layers[li];
   ExpandLaunch e{};
-  e.tasks = L.wide_tasks + L.wide_first[first]; e.n_tasks = L.wide_first[end] - L.wide_first[first]; e.dst = wide_buffer(p, li);
+  e.tasks = L.wide_tasks + L.wide_first[first]; e.n_tasks = L.wide_first[end] - L.wide_first[first]; e.dst = p->wide_buf + wide_at(p, li);
   e.pdl = p->ctx->pdl;
   return e;
 }
@@ -679,7 +689,7 @@ sti_status run_wide(sti_plan* p, GemmKind kind, int li, int which, const WideCho
   g.shape.T = T; g.shape.n = m.n;
   g.shape.n_tiles = (m.n + choice.nt - 1) / choice.nt; g.shape.m_pairs = (T + 255) / 256; g.shape.splits = choice.splits;
   g.shape.k_chunks = m.k_chunks;
-  g.shape.w_row0 = static_cast<uint32_t>((li & 1) * (p->wide_bytes / 128)) + m.row0;
+  g.shape.w_row0 = static_cast<uint32_t>(wide_at(p, li) / 128) + m.row0;
   g.shape.plane64 = which == 0 ? 1 : 0;
   g.nt = choice.nt; g.clusters = choice.clusters; g.weights_ready = weights_ready;
   if (beside >= 0) {
@@ -687,7 +697,7 @@ sti_status run_wide(sti_plan* p, GemmKind kind, int li, int which, const WideCho
     if (g.beside.n_tasks > 0) g.clusters = std::max(1, p->tiling.tune.cta_budget / 2);      // also where no tile is left to multiply
   }
   if (!make_xmap(&g.xmap, x, ldx, T) ||
-      !make_xmap(&g.wmap, p->wide_buf, 64, static_cast<int>(2 * p->wide_bytes / 128), choice.nt / 2, false) ||
+      !make_xmap(&g.wmap, p->wide_buf, 64, static_cast<int>(p->wide_count * p->wide_bytes / 128), choice.nt / 2, false) ||
       !make_omap(&g.omap, out, kind == GEMM_BF16_TO_F32, ldo, T, which == 0 ? m.n / 64 : choice.splits))
     return STI_ERR_CUDA;
   g.bias = bias; g.bias_off = which == 0 ? L.wide_bias[0] : L.wide_bias[1];
@@ -908,11 +918,9 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
     if (prof) CUDA_TRY(cudaEventRecord(L.ev_comp_start, c->compute));
     void* nxt = (li == n - 1) ? y : p->buf[li & 1];
     // the layer's first GEMM also pulls the next layer's packed shards into L2 (if they are on the device yet)
-    // every matrix of the next layer is decoded beside the same one of this layer - unless that is not multiplied with here, or
-    // the next layer is streamed and may not be on the device yet
-    const bool ahead = li + 1 < n && use_wide(p, L, static_cast<long long>(batch) * seq) &&
-                       use_wide(p, p->layers[li + 1], static_cast<long long>(batch) * seq) && p->layers[li + 1].str_bytes == 0 &&
-                       !L.kept_heads.empty() && !L.kept_slices.empty();
+    // every matrix of the next layer is decoded beside the same one of this layer
+    const bool ahead = can_decode_ahead(p, li) && use_wide(p, L, static_cast<long long>(batch) * seq) &&
+                       use_wide(p, p->layers[li + 1], static_cast<long long>(batch) * seq);
     sti_status st = enqueue_layer(p, li, cur, nxt, batch, seq, lens, li > 0, li + 1 < n, li + 1 < n ? li + 1 : -1, expanded,
                                   ahead ? li + 1 : -1, ffn_loaded, !any_wide);
     if (st != STI_OK) return st;

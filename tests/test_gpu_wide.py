@@ -209,3 +209,25 @@ def test_calls_a_few_tokens_smaller_than_their_context(model, kept, context, cal
             sti.sti_layer_forward(s.plan, 0, x.data_ptr(), y.data_ptr(), batch, seq, 0)
             sti.sti_sync(s.ctx)
             assert rel_err(from_device_act(y), ref) <= REL_TOL, (batch, seq)
+
+
+@pytest.mark.parametrize("layers,streamed,buffers", [(1, False, 1), (2, True, 1), (2, False, 2)])
+def test_working_buffers_take_what_the_header_says(layers, streamed, buffers, monkeypatch):
+    shape = W.BERT_LARGE.with_layers(layers)
+    units = [[W.UnitPlan(True, 2, not streamed or l < 1) for _ in range(16)] for l in range(layers)]
+    work = W.build_workload("memory", shape, 1, 512, "bf16", units, units, seed=layers, workers=layers)
+
+    def taken(tune):
+        monkeypatch.setenv("STI_TUNE", tune)
+        with sti.Session(work, finalize=False) as s:
+            before = torch.cuda.mem_get_info()[0]
+            sti.sti_plan_finalize(s.plan)
+            return before - torch.cuda.mem_get_info()[0]
+
+    one = 2 * 16 * (unit_weights(shape, ATTN) + unit_weights(shape, FFN))
+    extra = taken("wide_min_tokens=-1") - taken("wide_min_tokens=0")
+    assert abs(extra - buffers * one) < 8 << 20            # planes of partial sums differ by up to 4 MB, allocations come in 2 MB
+
+
+def unit_weights(shape, kind):
+    return 4 * 64 * shape.hidden if kind == ATTN else 2 * shape.slice_width * shape.hidden

@@ -101,7 +101,9 @@ typedef struct {
   int32_t n_layers;
   float compute_us[64];   /* per layer: first kernel start to last kernel end              */
   float copy_us[64];      /* per layer: duration of its host-to-device shard copy (0 if none) */
-  float stall_us[64];     /* per layer: time compute waited for the copy beyond the previous layer's end */
+  float stall_us[64];     /* per layer: time compute waited for the copy beyond the previous layer's end; the last streamed
+                           * layer's attention part may start before its FFN units are there, and the wait for these, between
+                           * its kernels (so part of its compute_us), is counted here as well */
   uint64_t streamed_bytes[64];
   uint64_t resident_bytes[64];
   float total_us;         /* first operation of the forward to its last                    */

@@ -170,6 +170,7 @@ struct sti_plan {
   bool fail_pinned_alloc = false;      // make the pinned-arena allocation of sti_plan_finalize fail
   int n_streamed_layers = 0;
   bool stats_valid = false;
+  int stats_in_two = -1;               // the layer that the profiled forward copied in two pieces (attention units, FFN units), -1: none
 };
 
 namespace {
@@ -797,7 +798,10 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
     L.k_ran[3] = true;
   }
   CUDA_TRY(mark(4));
-  if (ffn_loaded) CUDA_TRY(cudaStreamWaitEvent(c->compute, ffn_loaded, 0));
+  if (ffn_loaded) {
+    if (p->profiling == 1) CUDA_TRY(cudaEventRecord(L.ev_k[4], c->compute));      // level 2 has it: from here on the FFN units are waited for
+    CUDA_TRY(cudaStreamWaitEvent(c->compute, ffn_loaded, 0));
+  }
   if (ns > 0) {
     if (wide)
       st = run_wide(p, GEMM_BF16_TO_BF16_GELU, li, 2, pick_wide(p->tiling, T, L.wide[2], false), p->h1_bf16, d.hidden, T, p->u, ns * f,
@@ -847,7 +851,7 @@ sti_status enqueue_layer_copy(sti_plan* p, int li, cudaStream_t s, size_t from =
   Layer& L = p->layers[li];
   end = std::min(end, L.str_bytes);
   if (from >= end) return STI_OK;
-  if (li == p->slow_copy_layer && p->slow_copy_us)      // injected slow IO: the job reaches the copy engine late
+  if (li == p->slow_copy_layer && p->slow_copy_us && from == 0)      // injected slow IO: the job reaches the copy engine late
     std::this_thread::sleep_for(std::chrono::microseconds(p->slow_copy_us));
   CUDA_TRY(cudaMemcpyAsync(p->ring + static_cast<size_t>(L.slot) * p->slot_bytes + from, L.str_host + from, end - from,
                            cudaMemcpyHostToDevice, s));
@@ -866,7 +870,10 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
   bool any_streamed = false;
   for (auto& L : p->layers) any_streamed |= L.str_bytes > 0;
   std::vector<char> slot_used(p->ring_slots, 0);
-  if (prof) CUDA_TRY(cudaEventRecord(p->ev_begin, c->compute));
+  if (prof) {
+    CUDA_TRY(cudaEventRecord(p->ev_begin, c->compute));
+    p->stats_in_two = -1;
+  }
   if (capturing && any_streamed) {
     CUDA_TRY(cudaEventRecord(p->ev_fork, c->compute));
     CUDA_TRY(cudaStreamWaitEvent(c->copy, p->ev_fork, 0));
@@ -901,7 +908,7 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
       if (!capturing) CUDA_TRY(cudaStreamWaitEvent(c->copy, p->slot_free[L.slot], 0));
       else if (slot_used[L.slot]) CUDA_TRY(cudaStreamWaitEvent(c->copy, p->g_slot_free[L.slot], 0));
       if (prof) CUDA_TRY(cudaEventRecord(L.ev_copy_start, c->copy));
-      const bool in_two = li == last_streamed && !prof && L.str_attn_bytes > 0 && L.str_attn_bytes < L.str_bytes &&
+      const bool in_two = li == last_streamed && L.str_attn_bytes > 0 && L.str_attn_bytes < L.str_bytes &&
                           !use_wide(p, L, static_cast<long long>(batch) * seq);
       sti_status st = enqueue_layer_copy(p, li, c->copy, 0, in_two ? L.str_attn_bytes : L.str_bytes);
       if (st != STI_OK) return st;
@@ -911,6 +918,7 @@ sti_status enqueue_forward(sti_plan* p, const void* x, void* y, int batch, int s
         if ((st = enqueue_layer_copy(p, li, c->copy, L.str_attn_bytes)) != STI_OK) return st;
         ffn_loaded = capturing ? p->g_ev_ffn : p->ev_ffn;
         CUDA_TRY(cudaEventRecord(ffn_loaded, c->copy));
+        if (prof) p->stats_in_two = li;
       }
       // a layer starts only when its own shards (and, by stream order, all earlier ones) are loaded
       CUDA_TRY(cudaStreamWaitEvent(c->compute, loaded, 0));
@@ -1491,7 +1499,7 @@ sti_status sti_plan_finalize(sti_plan* p) {
   }
   CUDA_TRY(cudaEventCreateWithFlags(&p->ev_copy_tail, cudaEventDisableTiming));
   CUDA_TRY(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
-  CUDA_TRY(cudaEventCreateWithFlags(&p->ev_ffn, cudaEventDisableTiming));
+  CUDA_TRY(cudaEventCreateWithFlags(&p->ev_ffn, flags));
   CUDA_TRY(cudaEventCreateWithFlags(&p->g_ev_ffn, cudaEventDisableTiming));
   CUDA_TRY(cudaEventCreateWithFlags(&p->g_ev_join, cudaEventDisableTiming));
   p->g_slot_free.resize(p->ring_slots);
@@ -1745,17 +1753,23 @@ sti_status sti_get_stats(sti_plan* p, sti_stats* out) {
     CUDA_TRY(cudaEventElapsedTime(&t_start, p->ev_begin, L.ev_comp_start));
     CUDA_TRY(cudaEventElapsedTime(&t_done, p->ev_begin, L.ev_done));
     s.compute_us[l] = (t_done - t_start) * 1e3f;
+    float ffn_stall = 0.f;
     if (L.str_bytes) {
       float ms = 0.f, t_loaded = 0.f;
-      CUDA_TRY(cudaEventElapsedTime(&ms, L.ev_copy_start, L.ev_loaded));
+      CUDA_TRY(cudaEventElapsedTime(&ms, L.ev_copy_start, l == p->stats_in_two ? p->ev_ffn : L.ev_loaded));
       s.copy_us[l] = ms * 1e3f;
       CUDA_TRY(cudaEventElapsedTime(&t_loaded, p->ev_begin, L.ev_loaded));
-      s.stall_us[l] = std::max(0.f, t_loaded - prev_done) * 1e3f;
+      if (l == p->stats_in_two) {
+        CUDA_TRY(cudaEventElapsedTime(&ffn_stall, L.ev_k[4], p->ev_ffn));
+        ffn_stall = std::max(0.f, ffn_stall);
+      }
+      s.stall_us[l] = (std::max(0.f, t_loaded - prev_done) + ffn_stall) * 1e3f;
     }
     if (p->profiling >= 2) {
       float k[7] = {};
       for (int i = 0; i < 7; ++i)
         if (L.k_ran[i]) CUDA_TRY(cudaEventElapsedTime(&k[i], L.ev_k[i], L.ev_k[i + 1]));
+      k[4] = std::max(0.f, k[4] - ffn_stall);
       s.gemm_us[l] = (k[0] + k[2] + k[4] + k[5]) * 1e3f;
       s.attn_us[l] = k[1] * 1e3f;
       s.ln_us[l] = (k[3] + k[6]) * 1e3f;

@@ -33,6 +33,37 @@ def _forward(sess, work, x):
     return y
 
 
+@pytest.mark.parametrize("level", [1, 2])
+def test_profiled_forwards_copy_the_last_layer_in_two_as_others_do(level):
+    """A few tokens, and a last layer whose uncompressed FFN units take ten times as long to copy as its attention units: they are still
+    on their way when its attention part is done.  That wait is a stall, and the copy's time is that of both pieces."""
+    n = 4
+    attn = [[W.UnitPlan(True, 6, l == 0) for _ in range(16)] for l in range(n)]
+    ffn = [[W.UnitPlan(True, 32 if l == n - 1 else 6, l == 0) for _ in range(16)] for l in range(n)]
+    work = W.build_workload("in_two", W.BERT_LARGE.with_layers(n), 1, 8, "f32", attn, ffn, seed=3, workers=4)
+    x = torch.from_numpy(work.x_dev).cuda()
+    with sti.Session(work) as s:
+        y_graph = _forward(s, work, x)
+        sti.sti_plan_set_profiling(s.plan, level)
+        runs = []
+        for _ in range(5):
+            y = _forward(s, work, x)
+            assert torch.equal(y, y_graph)
+            runs.append(sti.sti_get_stats(s.plan))
+        sti.sti_plan_inject(s.plan, sti.STI_INJECT_SLOW_COPY, n - 1, 4000)
+        y = _forward(s, work, x)
+        slow = sti.sti_get_stats(s.plan)
+    assert torch.equal(y, y_graph)
+    st = runs[-1]
+    copies = [st.copy_us[l] / st.streamed_bytes[l] for l in range(1, n)]
+    assert max(copies) < 1.5 * min(copies)                                    # the last one's two pieces at the others' rate
+    wait = st.stall_us[n - 1]                                                 # level 2: most of the copy passes while the host launches events
+    assert (0.25 if level == 1 else 0.05) * st.copy_us[n - 1] < wait < 1.1 * st.copy_us[n - 1] and st.compute_us[n - 1] > 0.8 * wait
+    assert 2000 < slow.stall_us[n - 1] < 7000                                 # the host sleeps once
+    if level == 2:
+        assert st.gemm_us[n - 1] < st.compute_us[n - 1] - 0.6 * wait          # not counted as a kernel's time
+
+
 def test_slow_shard_copy_shows_up_as_that_layers_stall_and_nowhere_else():
     work = _work()
     x = torch.from_numpy(work.x_dev).cuda()

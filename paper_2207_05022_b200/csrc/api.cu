@@ -236,7 +236,7 @@ void parse_tuning(Tuning* t, const sti_model_desc& d, int sm_count) {
         else if (k == "wide_min_tokens") t->wide_min_tokens = std::max(-1, v);
         else if (k == "wide_nt") t->wide_nt = v == 128 || v == 256 ? v : 0;
         else if (k == "wide_splits") t->wide_splits = std::max(0, std::min(v, 8));
-        else if (k == "f2_kacc_min_tokens") t->f2_kacc_min_tokens = std::max(0, v);
+        else if (k == "f2_one_plane_min_tokens") t->f2_one_plane_min_tokens = std::max(0, v);
         else if (k == "attn_tc_min_items") t->attn_tc_min_items = std::max(0, v);
         else if (k == "cta_budget") t->cta_budget = std::max(1, v);
         else fprintf(stderr, "sti: STI_TUNE has no setting \"%s\"\n", k.c_str());
@@ -1624,7 +1624,7 @@ sti_status sti_gemm_probe(sti_plan* p, int layer, int gemm, const void* x_bf16_d
   const GemmTable& tab = *tabs[gemm];
   if (tab.n_jobs == 0) return STI_ERR_STATE;               // no kept unit feeds this GEMM
   const bool wide = variant == 3 || (variant == 2 && !c->simt_debug) || (variant == 0 && use_wide(p, L, tokens));
-  if (variant == 3 && (p->tiling.tune.f2_kacc_min_tokens == 0 || whole_tiles(p->tiling.max_tokens) < p->tiling.tune.f2_kacc_min_tokens))
+  if (variant == 3 && (p->tiling.tune.f2_one_plane_min_tokens == 0 || whole_tiles(p->tiling.max_tokens) < p->tiling.tune.f2_one_plane_min_tokens))
     return STI_ERR_STATE;                                  // no call of this plan takes FFN2's K range in one piece
   const bool sums = gemm == 1 || gemm == 3;
   const WideChoice choice = variant == 3 ? pick_wide(p->tiling, tokens, L.wide[3], false)

@@ -30,7 +30,7 @@ def _work(batch, seq, kept):
 def test_the_context_s_capacity_does_not_change_a_call(batch, seq, kept):
     from gpu_util import run_layer
     work, outs = _work(batch, seq, kept), []
-    for max_batch in (batch, 8 * batch, 4200 // seq + 1):        # the largest also has the tables of the K-accumulating kernel
+    for max_batch in (batch, 8 * batch, 4200 // seq + 1):        # the largest takes FFN2 in one plane in its own largest calls
         with sti.Session(work, max_batch=max_batch) as s:
             outs.append(run_layer(s, work, 0))
     assert np.array_equal(outs[0], outs[1]) and np.array_equal(outs[0], outs[2])

@@ -78,8 +78,8 @@ def test_config5_point_sampled_sequences(plan):
 
 
 def test_config5_largest_bench_point_sampled_sequences():
-    # 32 x 512 = 16,384 tokens: the launch shapes bench.py times (two-CTA GEMMs, K-accumulating FFN2 with two
-    # blocks of tile pairs per CTA pair, tensor-core attention, warp-per-row LayerNorm), two layers, streamed
+    # 32 x 512 = 16,384 tokens: the launch shapes bench.py times (two-CTA GEMMs over the working buffer, FFN2 in
+    # one plane, tensor-core attention, warp-per-row LayerNorm), two layers, streamed
     from gpu_util import rel_err, REL_TOL
     B, L, n_layers = 32, 512, 2
     work = W.make_config(5, n_layers=n_layers, plan="mixed", resident=False, resident_layers=1, batch=1, seq=L, workers=3)

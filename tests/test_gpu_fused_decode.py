@@ -149,7 +149,7 @@ def test_fused_decode_bert_large_few_and_many_token_tilings():
     work = _mixed_work(shape, seed=13)
     with sti.Session(work) as s:                              # tiling chosen for few tokens
         _check_all_gemms(work, s)
-    with sti.Session(work, max_batch=8, max_seq=512) as s:    # tiling chosen for many tokens
+    with sti.Session(work, max_batch=8, max_seq=512) as s:    # a context for many tokens
         _check_all_gemms(work, s, variant=1)                  # one-CTA kernel
         _check_all_gemms(work, s, variant=2)                  # two-CTA (cta_group::2) kernel
 
@@ -167,8 +167,8 @@ def test_fused_decode_more_outliers_than_threads_in_a_tile():
         _check_all_gemms(work, s, variant=2)
 
 
-def _check_ffn2_kacc(work, sess):
-    """FFN2 through the K-accumulating kernel: one complete plane, every weight exactly once."""
+def _check_ffn2_one_plane(work, sess):
+    """FFN2 over the working buffer with its K range in one piece: one complete plane, every weight exactly once."""
     sh = work.shape
     f = sh.slice_width
     slices = work.kept(0, FFN)
@@ -179,30 +179,30 @@ def _check_ffn2_kacc(work, sess):
     assert np.isfinite(got).all()
     for ji, j in enumerate(slices):
         want = O.bf16_rne(_oracle_unit(work, FFN, j)["F2"]).T               # [f][d]
-        assert np.array_equal(got[ji * f:(ji + 1) * f].view(np.uint32), want.view(np.uint32)), ("FFN2 kacc", j)
+        assert np.array_equal(got[ji * f:(ji + 1) * f].view(np.uint32), want.view(np.uint32)), ("FFN2 in one plane", j)
 
 
 @pytest.mark.parametrize("tune,keep_ffn", [
-    ("f2_kacc_min_tokens=1024", lambda i: True),                       # 6 K groups of 256, one tile pair per CTA pair
-    ("f2_kacc_min_tokens=1024,cta_budget=4", lambda i: True),          # one CTA pair per column pair: 2 blocks (4 + 2 tiles)
-    ("f2_kacc_min_tokens=1024,cta_budget=8", lambda i: i != 2),        # 5 slices kept
-    ("f2_kacc_min_tokens=1024,f2_kacc_k=512", lambda i: True),         # K groups of two slices, whole decode tasks per warp
-    ("f2_kacc_min_tokens=1024,f2_kacc_k=512,cta_budget=4", lambda i: i != 2),   # ... the last K group is 256 wide
+    ("f2_one_plane_min_tokens=1024", lambda i: True),
+    ("f2_one_plane_min_tokens=1024,cta_budget=4", lambda i: True),          # two CTA pairs: six tiles of 256 tokens
+    ("f2_one_plane_min_tokens=1024,cta_budget=4,wide_nt=128", lambda i: True),
+    ("f2_one_plane_min_tokens=1024,cta_budget=8,wide_nt=256", lambda i: i != 2),   # five slices kept
+    ("f2_one_plane_min_tokens=1024,wide_splits=3", lambda i: i != 2),       # one plane whatever the splits of other calls
 ])
-def test_fused_decode_k_accumulating_ffn2_small_shape(tune, keep_ffn):
+def test_fused_decode_ffn2_in_one_plane_small_shape(tune, keep_ffn):
     shape = W.ModelShape(n_layers=1, hidden=256, n_heads=4, head_dim=64, ffn=1536, n_ffn_slices=6)
     work = _mixed_work(shape, seed=16, keep_fn=lambda k, i: True if k == ATTN else keep_ffn(i))
     with _Tune(tune), sti.Session(work, max_batch=8, max_seq=256) as s:
-        _check_ffn2_kacc(work, s)
+        _check_ffn2_one_plane(work, s)
 
 
-def test_fused_decode_k_accumulating_ffn2_bert_large():
+def test_fused_decode_ffn2_in_one_plane_bert_large():
     shape = W.BERT_LARGE.with_layers(1)
     work = _mixed_work(shape, seed=17)
     with sti.Session(work, max_batch=32, max_seq=512) as s:                # made for 16,384 tokens: the default rule applies
-        _check_ffn2_kacc(work, s)
+        _check_ffn2_one_plane(work, s)
         _check_all_gemms(work, s, variant=2)
-    with sti.Session(work, max_batch=4, max_seq=512) as s:                 # 2,048 tokens: no K-accumulating table
+    with sti.Session(work, max_batch=4, max_seq=512) as s:                 # 2,048 tokens: no call takes it in one piece
         x = _identity_bf16(64)
         out = torch.zeros(64 * 1024, dtype=torch.float32, device="cuda")
         with pytest.raises(sti.StiError) as e:

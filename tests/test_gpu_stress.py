@@ -26,11 +26,12 @@ def _bf16_act(work):
 @pytest.mark.parametrize("batch,seq,resident", [
     (1, 256, True),          # the headline launch shapes (BERT-large layers, one 256-token sequence)
     (1, 256, False),
-    (1, 512, True),          # three CTAs over four token tiles: two tiles on some CTAs
+    (1, 384, True),          # the most that goes through the fused kernels: two CTAs over three token tiles
+    (1, 512, True),          # the working buffer, decoded ahead; and layer by layer
     (1, 512, False),
-    (8, 128, True),          # 1024 tokens: the two-CTA kernel
+    (8, 128, True),          # 1024 tokens: the working buffer, two-CTA GEMMs
     (1, 8, True),            # a handful of tokens
-    (16, 512, False),        # 8192 tokens: K-accumulating FFN2, tensor-core attention, warp-per-row LayerNorm
+    (16, 512, False),        # 8192 tokens: the working buffer, FFN2 in one plane, tensor-core attention, warp-per-row LayerNorm
 ])
 def test_queued_forwards_meet_every_wait_and_repeat_bit_for_bit(batch, seq, resident):
     work = W.make_config(5, n_layers=3, plan="mixed", resident=resident, resident_layers=3 if resident else 1,

@@ -108,21 +108,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity)
   }
 }
 
-// Same bound, but the waiting thread sleeps between polls so that it does not take issue slots from
-// the warp that shares its scheduler (used by the roles that wait long: producer, epilogue).
-__device__ __forceinline__ bool mbar_wait_bounded_relaxed(uint32_t bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_timer_ns();
-  for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 64; ++i) {
-      __nanosleep(64);
-      if (mbar_try_wait(bar, parity)) return true;
-    }
-    if (global_timer_ns() - t0 > 2000000000ull) return false;
-  }
-}
-
 // Programmatic dependent launch: a kernel launched with the attribute may start while its predecessor
 // on the stream still runs.  `pdl_wait` blocks until the predecessor has completed and its writes are
 // visible - everything before it may only touch data no kernel writes (weights, descriptors, parameters);

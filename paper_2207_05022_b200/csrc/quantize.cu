@@ -993,11 +993,12 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
   cluster.sync();                                                      // pairs and streams are complete as well
 
   // ---- 5. the boundary bins, a warp each: a pair's rank is the number of smaller pairs of its bin (all are distinct)
-  // The lists' address is worked out again, from a block number that the compiler does not know: kept over pass 4 it makes
-  // another value there come back from L2 (384 units of 524,288 weights at 3 bits 487 -> 520 us, 200 at 4 bits 270 -> 286).
-  uint32_t cta;
-  asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
-  const unsigned long long* lists = reinterpret_cast<const unsigned long long*>(ws_all + static_cast<size_t>(cta / n_ctas) * ws_per_unit);
+  // The lists' address is worked out again, from a unit number that the compiler does not know: kept over pass 4 it makes
+  // another value there come back from L2 (384 units of 524,288 weights at 3 bits 487 -> 520 us, 200 at 4 bits 270 -> 286).  The
+  // cluster's number is the unit's; block number over cluster size took 12 units of 196,608 at 4 bits 29.0 -> 29.8.
+  uint32_t same_unit;
+  asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(same_unit));
+  const unsigned long long* lists = reinterpret_cast<const unsigned long long*>(ws_all + static_cast<size_t>(same_unit) * ws_per_unit);
   for (uint32_t c = 1u + warp * n_ctas + rank; c < K; c += n_warps) {       // neighbours on different SMs
     if (!owns(c)) continue;
     const uint32_t m = sm.seg_len[c], bin = sm.bnd_bin[c];
@@ -1006,7 +1007,7 @@ quantize_select_kernel(const float* w_all, uint32_t n, uint32_t n_bins, uint32_t
     const unsigned long long* from = lists + sm.seg_start[c];
     // The keys in order, which is all that the sums need: behind the pairs, or where a longer bin's would have been (the unit's
     // workspace has no room for them: its second half holds the tails beyond the warps' lists).
-    uint32_t* sorted = reinterpret_cast<uint32_t*>(sm.u.pairs[warp][m <= static_cast<uint32_t>(kSelSmemSeg) ? 1 : 0]);
+    uint32_t* sorted = reinterpret_cast<uint32_t*>(sm.u.pairs[warp][0]) + (m <= static_cast<uint32_t>(kSelSmemSeg) ? 2 * kSelSmemSeg : 0);
     if (m <= static_cast<uint32_t>(kSelSmemSeg)) {
       for (uint32_t j = lane; j < m; j += 32) sm.u.pairs[warp][0][j] = from[j];
       if (lane == 0 && (m & 1u) != 0u) sm.u.pairs[warp][0][m] = ~0ull;

@@ -3,14 +3,15 @@
 //
 // Persistent pairs of CTAs (cta_group::2), one CTA per SM.  A pair takes tiles of 256 tokens x NT features (256 or 128): each
 // CTA loads its own 128 tokens and its half of the features, 64 columns at a time, into a ring of stages; CTA 0 issues
-// the MMAs (M = 256, N = NT) into one of two accumulators in tensor memory (2 x 256 columns: all of it) while twelve epilogue
-// warps of each CTA drain the other: tcgen05.ld -> bias / erf-GELU -> global.  fp32 outputs may be split along K; every
-// split writes a plane of its own, which the LayerNorm after it adds up.
+// the MMAs (M = 256, N = NT) into one of two accumulators in tensor memory (at NT = 256 all of it) while eight epilogue warps of
+// each CTA drain the other: tcgen05.ld -> bias / erf-GELU -> shared memory -> bulk tensor store.  fp32 outputs may be split
+// along K; every split writes a plane of its own, which the LayerNorm after it adds up.
 //
 //   warp 0      producer: TMA boxes of activations and weights, both CTAs' bytes reported to CTA 0's `full` barriers
 //   warp 1      MMA issuer (CTA 0)
-//   warps 2-3   decode the same matrix of the next layer into the other working buffer (expand.cu): it is ready a layer ahead
-//   warps 4-15  epilogue, three per tensor-memory lane quadrant
+//   warps 2-3   decode the same matrix of the next layer into the other working buffer (expand.cu): it is ready a layer ahead;
+//               at NT = 128 warps 12-13 as well
+//   warps 4-11  epilogue, two per tensor-memory lane quadrant, half of the tile's features each
 //
 // Bound: the MMAs, as long as a launch has several waves of tiles: a chunk of 64 columns takes 540 cycles at NT = 256 (the tensor
 // core's 512) and 395 at 128 (24 KB written to and 24 KB read from shared memory: 384).  With one wave as much goes

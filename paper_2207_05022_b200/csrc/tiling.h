@@ -43,7 +43,7 @@ struct Tuning {
   int f2_group = 0;                    // FFN slices per K group of FFN2: 0 = chosen per layer and token count (pick_f2_group)
   int cta_budget = 148;                // (replaced by the device's SM count in parse_tuning) CTAs a GEMM launch may use when it splits the token tiles over CTAs
   int wide_min_tokens = -1;            // weights decoded into the working buffer, GEMMs over it: -1 = by the rule of use_wide, 0 = never, else from this many tokens on
-  int f2_one_plane_min_tokens = 4096;       // there, FFN2's K range in one piece (one output plane) from this many tokens on (0 = by cost)
+  int f2_one_plane_min_tokens = 4096;  // there, FFN2's K range in one piece (one output plane) from this many tokens on (0 = by cost)
   int wide_nt = 0, wide_splits = 0;    // there, features per tile and K splits: 0 = chosen by pick_wide
   int attn_tc_min_items = -1;          // tensor-core attention: -1 = by the rule of tc_attention, 0 = never, else from this many (sequence, kept head) pairs on, whatever their length
 };

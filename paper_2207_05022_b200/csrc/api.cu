@@ -764,9 +764,14 @@ sti_status enqueue_layer(sti_plan* p, int li, const void* x, void* y, int batch,
       if (!make_xmap(&qmap, p->qkv, 64, 3 * nh * T, 64) || !make_xmap(&omap, p->attn_out, nh * 64, T, 32)) return STI_ERR_CUDA;
       CUDA_TRY(launch_attention_tc(qmap, omap, p->attn_out, nh, batch, seq, lens, c->err_dev, c->compute, c->pdl, stamp(2)));
     } else {
-      CUDA_TRY(launch_attention(p->qkv, p->attn_out, nh, batch, seq, lens, c->sm_count,
-                                wide ? static_cast<int>(2 * o_choice.clusters) : L.o.n_jobs * m_ctas_for(L.o.n_jobs, T, p->tiling.tune.cta_budget),
-                                c->compute, c->pdl, stamp(2)));
+      // Over the working buffer the O projection has no weights of its own to decode meanwhile: from 321 keys on attention gains more
+      // from every SM than that one loses (us per BERT-large layer of 12 heads and slices by itself / per four in a model, room left
+      // for it against none: 1 x 512 53.8 / 190.7 against 51.6 / 184.4, 1 x 450 53.1 / 188.6 against 50.9 / 181.3; but 4 x 128 47.6 /
+      // 165.4 against 47.0 / 166.6, 5 x 77 46.1 / 159.9 against 46.1 / 162.6; of 8 heads and slices 3 x 340 51.4 / 190.7 against
+      // 50.1 / 188.6, 2 x 300 45.7 / 170 against 46.9 / 170).
+      const int next_ctas = !wide ? L.o.n_jobs * m_ctas_for(L.o.n_jobs, T, p->tiling.tune.cta_budget)
+                            : seq > 320 ? c->sm_count : static_cast<int>(2 * o_choice.clusters);
+      CUDA_TRY(launch_attention(p->qkv, p->attn_out, nh, batch, seq, lens, c->sm_count, next_ctas, c->compute, c->pdl, stamp(2)));
     }
     c->launches++;
     CUDA_TRY(mark(2));

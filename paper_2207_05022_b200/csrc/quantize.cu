@@ -552,21 +552,32 @@ struct SelTails {
   SelTail* far;                            // the others: places kSelTails .. of this array
   uint32_t n;
   __device__ __forceinline__ SelTail& at(uint32_t k) const { return k < kSelTails ? near[k] : far[k]; }
-  // those of one group of 128 weights, all lanes together
+  // Those of one group of 128 weights, all lanes together.  One group in eight of Gaussian weights has one; with heavier tails (a
+  // deviation near 1, where the outliers' share grows, or a scale that varies inside the unit) most have several.  Lane after lane
+  // took 206 us for 16 units of 524,288 weights of deviation 5 at 6 bits and 280 for 64 at 3 bits with half of the weights ten times
+  // smaller, now 121 and 224; a vote per weight instead of per bit of the count spills (384 Gaussian ones at 6 bits 803 -> 831).
   __device__ __forceinline__ void add(uint32_t i0, const float4& x, bool exists, float lo, float hi) {
     const float most = max3(fmaxf(x.x, x.y), x.z, x.w), least = min3(fminf(x.x, x.y), x.z, x.w);
-    uint32_t left = __ballot_sync(0xffffffffu, exists && (most > hi || least < lo));
-    while (left != 0u) {                   // lane after lane, one as a rule
-      const int from = __ffs(static_cast<int>(left)) - 1;
-      left &= left - 1u;
-      uint32_t k = n;
-      if (static_cast<int>(threadIdx.x & 31u) == from) {
-        const float v[4] = {x.x, x.y, x.z, x.w};
+    const bool any = exists && (most > hi || least < lo);
+    if (!__any_sync(0xffffffffu, any)) return;
+    const float v[4] = {x.x, x.y, x.z, x.w};
+    uint32_t count = 0;
+    if (any) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (v[j] < lo || v[j] > hi) at(k++) = {i0 + j, v[j]};
-      }
-      n = __shfl_sync(0xffffffffu, k, from);
+      for (int j = 0; j < 4; ++j) count += v[j] < lo || v[j] > hi ? 1u : 0u;
+    }
+    const uint32_t lt_mask = (1u << (threadIdx.x & 31u)) - 1u;
+    uint32_t k = n;                        // this lane's first place: the counts of the lanes before it, 0 to 4, added up bit by bit
+#pragma unroll
+    for (int bit = 0; bit < 3; ++bit) {
+      const uint32_t all = __ballot_sync(0xffffffffu, (count >> bit & 1u) != 0u);
+      k += __popc(all & lt_mask) << bit;
+      n += __popc(all) << bit;
+    }
+    if (any) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (v[j] < lo || v[j] > hi) at(k++) = {i0 + j, v[j]};
     }
   }
 };

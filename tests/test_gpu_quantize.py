@@ -314,7 +314,7 @@ def _guess_positions(n):
 
 
 @pytest.mark.parametrize("n", [1024, 24576, 100096])
-@pytest.mark.parametrize("what", ["wide", "narrow", "constant", "far", "heavy", "one_sided", "large"])
+@pytest.mark.parametrize("what", ["wide", "narrow", "constant", "far", "heavy", "one_sided", "large", "ordered"])
 def test_units_unlike_what_their_sample_says(what, n):
     """The bins and the tails that are listed come from 256 weights: whatever they say, the result is the oracle's."""
     rng = np.random.default_rng(n)
@@ -335,5 +335,7 @@ def test_units_unlike_what_their_sample_says(what, n):
         w[rng.random(n) < 0.01] = np.float32(-0.5)
     elif what == "large":           # a deviation at which a tenth of a Gaussian's weights are outliers
         w *= np.float32(300)
+    elif what == "ordered":         # from no weight of a group of 128 in the tails to all of them
+        w = np.sort(w * np.float32(50))
     for bits in (2, 3, 5, 6):
         _check(np.stack([w, w[::-1].copy()]), bits)

@@ -801,7 +801,7 @@ def run_quantize(args):
                       "roofline": {"bound": "hbm", "achieved": total_bytes / total_ms / 1e6, "peak": peaks["hbm_gbs"],
                                    "unit": "GB/s", "frac": total_bytes / total_ms / 1e6 / peaks["hbm_gbs"],
                                    "traffic": None, "peak_source": f"hbm_gbs, {peak_src}",
-                                   "note": "totals are the selecting method's (the default); a cluster of CTAs per unit, three passes "
+                                   "note": "totals are the selecting method's (the default); a cluster of CTAs per unit, two passes "
                                            "over the unit's fp32 weights"},
                       "cpu_baseline": {"value": cpu_weights / cpu_s / 1e6, "unit": "Mweights/s", "cores": blas_threads(),
                                        "kind": "oracle", "sample": "one attention unit and one FFN unit of layer 0"}}))

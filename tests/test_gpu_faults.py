@@ -51,17 +51,22 @@ def test_profiled_forwards_copy_the_last_layer_in_two_as_others_do(level):
             assert torch.equal(y, y_graph)
             runs.append(sti.sti_get_stats(s.plan))
         sti.sti_plan_inject(s.plan, sti.STI_INJECT_SLOW_COPY, n - 1, 4000)
-        y = _forward(s, work, x)
-        slow = sti.sti_get_stats(s.plan)
-    assert torch.equal(y, y_graph)
-    st = runs[-1]
-    copies = [st.copy_us[l] / st.streamed_bytes[l] for l in range(1, n)]
+        slow = []
+        for _ in range(3):
+            y = _forward(s, work, x)
+            assert torch.equal(y, y_graph)
+            slow.append(sti.sti_get_stats(s.plan).stall_us[n - 1])
+    # the best of a few forwards: other users of the host can hold up one of them
+    copies = [min(st.copy_us[l] for st in runs) / runs[0].streamed_bytes[l] for l in range(1, n)]
     assert max(copies) < 1.5 * min(copies)                                    # the last one's two pieces at the others' rate
-    wait = st.stall_us[n - 1]                                                 # level 2: most of the copy passes while the host launches events
-    assert (0.25 if level == 1 else 0.05) * st.copy_us[n - 1] < wait < 1.1 * st.copy_us[n - 1] and st.compute_us[n - 1] > 0.8 * wait
-    assert 2000 < slow.stall_us[n - 1] < 7000                                 # the host sleeps once
-    if level == 2:
-        assert st.gemm_us[n - 1] < st.compute_us[n - 1] - 0.6 * wait          # not counted as a kernel's time
+    low = 0.25 if level == 1 else 0.05                                        # level 2: most of the copy passes while the host launches events
+
+    def wait_is_a_stall(st):
+        wait, copy, compute = st.stall_us[n - 1], st.copy_us[n - 1], st.compute_us[n - 1]
+        return low * copy < wait < 1.1 * copy and compute > 0.8 * wait and (level == 1 or st.gemm_us[n - 1] < compute - 0.6 * wait)      # not a kernel's time
+
+    assert any(wait_is_a_stall(st) for st in runs)
+    assert 2000 < min(slow) < 7000                                            # the host sleeps once
 
 
 def test_slow_shard_copy_shows_up_as_that_layers_stall_and_nowhere_else():
